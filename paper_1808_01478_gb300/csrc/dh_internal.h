@@ -23,6 +23,9 @@ constexpr int kBlockLarge = 512;
 constexpr int kBlockHuge = 1024;
 constexpr int kQueueCap = 64;        // deferred pairs per warp queue
 constexpr int kNumVariants = 4;
+constexpr int kListBlock = 512;      // list kernel: threads per block, one block per SM
+constexpr int kRun = 128;            // list kernel: consecutive particles of a species with one bounding box
+constexpr int64_t kListMaxN = (int64_t)1 << 26;  // list kernel: particle and image index share 32 bits
 
 // One frame as seen by the device.  Host fills the first part; the staging and
 // setup kernels fill the second.
@@ -47,7 +50,7 @@ struct FrameDev {
   float rmax_f;      // float32(r_max)
   float S2;          // float32((nbins / r_max)^2)
   float margin;      // triclinic: 1 - 2 r_max / h_min (no-search precondition margin)
-  float tshift[27][3];  // triclinic tile images: -B k rounded once from binary64, k in {-1,0,1}^3
+  float tshift[27][3];  // periodic images: -B k rounded once from binary64, k in {-1,0,1}^3
                         // (index 9 (kx+1) + 3 (ky+1) + (kz+1))
   float tserr[27][3];   // |tshift - (-B k)|, rounded up
   float convf[3];       // binary64 input: per-axis conversion error (conv), rounded up
@@ -58,7 +61,23 @@ struct FrameDev {
   float rr2;            // orthorhombic: (r_max (1 + 2/nbins))^2, rounded up
   double eps_S;      // |S - nbins/r_max| / (nbins/r_max)
   double eps_S2;     // |S2 - (nbins/r_max)^2| / (nbins/r_max)^2
+  // list kernel (null and unset for other frames); lengths in bins: S = nbins / r_max times the caller's
+  float4* P4;         // home positions: x, y, z to a grid (list_grid) and the rest of x,
+  float2* P2;         //   the rest of y and z
+  float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz)
+  float img_h[27][3], img_l[27][3];  // image vectors -B k as double-floats (index as tshift)
+  float period[3];    // a_x, b_y, c_z
   // ---- written on the device
+  int32_t smin[3], smax[3];  // triclinic: the same of the fractional coordinates
+  int32_t wrap;       // the coordinates span more than one cell: P4 is brought home to the first
+  int32_t list_slow;  // list kernel: every pair in binary64 (no trust in the images)
+  int32_t list_all;   // list kernel: every listed pair re-decided (window too wide)
+  float key_lo[3], key_inv;  // spatial order: origin and inverse side of the grid
+  float list_grid;    // list kernel: grid of the positions' high parts (a power of two),
+  float list_c0;      //   constant part of the window (see list_setup),
+  float list_mid;     //   position error of the double-float tier,
+  float list_tie;     //   orthorhombic: distance from half a period re-decided in binary64
+  float cull_abs;     //   absolute slack of the distance bounds
   int32_t cmin[3];   // ordered-integer encodings of the per-axis coordinate min / max
   int32_t cmax[3];
   int32_t bad;       // a non-finite coordinate was seen
@@ -96,6 +115,21 @@ struct Segment {
   int64_t item_base; // segment-local index of that item
 };
 
+// The same for the list kernel: one species pair of one frame and one bin
+// sweep as items of one run of kRun i particles against one run of j particles
+// (or a quarter of it, ListLaunch.split), numbered row by row over (i run, j
+// run); intra-species: j runs not below the i run.  The i side is the larger
+// species.  Launch items [item0, item0 + items) are the segment's items from
+// item_base on.
+struct ListSegment {
+  FrameDev* fd;
+  int32_t intra, h, pass;
+  int32_t n_ti, n_tj;      // runs of the i and the j species
+  int32_t i0, ni, j0, nj;  // frame-local particle ranges
+  int32_t i_run0, j_run0;  // their first runs in the frame's bounds
+  int64_t item0, item_base, items;
+};
+
 // Staging job: one frame's coordinates (n x stride floats) -> float4.
 struct StageJob {
   const float* src;  // n x stride float32, or binary64 when dst64 is set
@@ -107,7 +141,7 @@ struct StageJob {
   int32_t pad;
   int64_t chunk0;    // first staging chunk of this job
 };
-constexpr int kStageChunk = 8192;
+constexpr int kStageChunk = 1024;
 
 // Spatial ordering of one species of one periodic frame: its particles are
 // grouped by cell of a 2^g x 2^g x 2^g grid over the fractional coordinates, in
@@ -118,9 +152,12 @@ struct SortSeg {
   int64_t x0;        // first particle (index into the packed coordinates)
   int32_t n;         // particles
   int32_t g;         // grid bits per axis
-  int64_t key0;      // first counter of this segment (2^(3g) counters)
+  int64_t key0;      // first counter of this segment (2^(3g) counters; a multiple of four)
+  int64_t f0;        // x0 of the frame's first particle
+  int32_t run0;      // first run of this species in the frame's bounds
+  int32_t pad;
 };
-constexpr int kSortChunk = 4096;
+constexpr int kSortChunk = 256;
 
 struct Control {
   unsigned long long next_item;  // dynamic work counter (reset before each launch)
@@ -140,18 +177,42 @@ struct PairLaunch {
   int32_t agg;         // 256-thread blocks, one sweep: warp-aggregated histogram increments (match.any)
 };
 
+// Work counter of one segment of a list-kernel launch (zeroed before it).
+struct SegCounter {
+  unsigned long long next;  // items claimed
+  int32_t attached;         // blocks working on the segment
+  int32_t pad;
+};
+
+struct ListLaunch {
+  const ListSegment* segs;
+  SegCounter* ctr;       // one per segment
+  int32_t n_segs;
+  int32_t hist_width;
+  int64_t n_items;
+  int32_t split;         // items per run pair (1 to 16, a power of two: kRun / split j particles each)
+  int32_t multi;
+};
+
 // ---- launchers (dh_kernels.cu); all enqueue on `stream` and return the launch error
 cudaError_t launch_stage(const StageJob* jobs, int n_jobs, int64_t n_chunks, cudaStream_t stream);
 cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, int pass_hi_max, cudaStream_t stream);
-// counts: zeroed, sum of 2^(3g) over the segments; keys and Xs: one per particle
-// X64 and Xs64 (binary64 copies, same indexing) may be null
-cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, int max_chunks, float4* X, float4* Xs,
-                                double4* X64, double4* Xs64, int32_t* keys, uint32_t* counts,
+// Orders each segment's particles from src (src64) into dst (dst64), and for the
+// list kernel into the frame's P4 and P2 with the bounds of its runs.  counts: n_keys
+// counters, zeroed, then n_keys cursors (n_keys: sort_counters over the segments);
+// keys: one per particle; the binary64 arrays may be null.
+cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, int64_t max_n, const float4* src, float4* dst,
+                                const double4* src64, double4* dst64, int32_t* keys, uint32_t* counts, int64_t n_keys,
                                 cudaStream_t stream);
+int sort_grid_bits(int64_t n);  // grid bits per axis for a species of n particles
 cudaError_t launch_thresholds(double r_max, int32_t nbins, double* T, int32_t* status,
                               cudaStream_t stream);
 // One pair-kernel launch over segments whose frames all have minimum-image variant `variant`.
 cudaError_t launch_pairs(const PairLaunch& p, int variant, int grid, size_t smem, cudaStream_t stream);
+// The list kernel (dh_list.cu): segments of any frames planned for it.
+cudaError_t launch_list(const ListLaunch& p, int grid, cudaStream_t stream);
+size_t list_kernel_smem(int hist_width);
+int list_kernel_max_width();  // widest sweep of the list kernel on the current device
 cudaError_t launch_check_sqrt(unsigned long long* out, cudaStream_t stream);
 cudaError_t launch_check_tiles(const FrameDev* F, int variant, uint64_t n_tiles, uint64_t seed,
                                unsigned long long* out, cudaStream_t stream);

@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "dh_device.h"
 #include "dh_internal.h"
 
 namespace dh {
@@ -36,41 +37,6 @@ namespace dh {
 // another's) is cleared first.  Errors of kernels already running are sticky
 // and still surface at the next synchronisation.
 static inline void clear_stale_error() { (void)cudaGetLastError(); }
-
-// Order-preserving map float -> int32 (for atomicMin/atomicMax on floats).
-__device__ __forceinline__ int32_t ord_of(float f) {
-  int32_t i = __float_as_int(f);
-  return i >= 0 ? i : (i ^ 0x7FFFFFFF);
-}
-__device__ __forceinline__ float float_of_ord(int32_t k) {
-  return __int_as_float(k >= 0 ? k : (k ^ 0x7FFFFFFF));
-}
-
-constexpr float kMagicRound = 12582912.0f;  // 1.5 * 2^23: fma(x, s, M) - M = nint_even(x*s), |x*s| < 2^22
-constexpr float kMagicFloor = 8388608.0f;   // 2^23: fadd.rd(t, 2^23) - 2^23 = floor(t), 0 <= t < 2^23
-constexpr unsigned kFull = 0xffffffffu;
-
-// Relative error bound assumed for sqrt.approx.ftz.f32 (checked exhaustively
-// over two binades by the GPU test suite).
-constexpr double kSqrtRelErr = 8.0 / 16777216.0;  // 8 * 2^-24
-
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-// IEEE minimum that propagates NaN (masked pairs carry NaN and must stay NaN).
-__device__ __forceinline__ float min_nan(float a, float b) {
-  float y;
-  asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-  return y;
-}
-__device__ __forceinline__ float nint_scaled(float x, float s) {
-  return __fadd_rn(__fmaf_rn(x, s, kMagicRound), -kMagicRound);
-}
-__device__ __forceinline__ float nint_f(float x) {
-  return __fadd_rn(__fadd_rn(x, kMagicRound), -kMagicRound);
-}
 
 // ------------------------------------------------------------------ binary64 bin of Alg. 1
 
@@ -154,6 +120,9 @@ __global__ void stage_kernel(const StageJob* __restrict__ jobs, int n_jobs) {
   const int64_t i1 = min(J.n, i0 + (int64_t)kStageChunk);
   float mn0 = INFINITY, mn1 = INFINITY, mn2 = INFINITY;
   float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY;
+  // triclinic: the range of the fractional coordinates too (does the frame span more than one cell?)
+  const bool frac = J.fd->variant == V_TRIC;
+  float sn[3] = {INFINITY, INFINITY, INFINITY}, sx[3] = {-INFINITY, -INFINITY, -INFINITY};
   int bad = 0;
   const float* __restrict__ src = J.src;
   const int stride = J.stride;
@@ -175,67 +144,109 @@ __global__ void stage_kernel(const StageJob* __restrict__ jobs, int n_jobs) {
     J.dst[i] = make_float4(x, y, z, 0.0f);
     mn0 = fminf(mn0, x); mn1 = fminf(mn1, y); mn2 = fminf(mn2, z);
     mx0 = fmaxf(mx0, x); mx1 = fmaxf(mx1, y); mx2 = fmaxf(mx2, z);
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    mn0 = fminf(mn0, __shfl_xor_sync(kFull, mn0, o));
-    mn1 = fminf(mn1, __shfl_xor_sync(kFull, mn1, o));
-    mn2 = fminf(mn2, __shfl_xor_sync(kFull, mn2, o));
-    mx0 = fmaxf(mx0, __shfl_xor_sync(kFull, mx0, o));
-    mx1 = fmaxf(mx1, __shfl_xor_sync(kFull, mx1, o));
-    mx2 = fmaxf(mx2, __shfl_xor_sync(kFull, mx2, o));
-    bad |= __shfl_xor_sync(kFull, bad, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    FrameDev* F = J.fd;
-    if (mn0 <= mx0) {
-      atomicMin(&F->cmin[0], ord_of(mn0)); atomicMin(&F->cmin[1], ord_of(mn1));
-      atomicMin(&F->cmin[2], ord_of(mn2));
-      atomicMax(&F->cmax[0], ord_of(mx0)); atomicMax(&F->cmax[1], ord_of(mx1));
-      atomicMax(&F->cmax[2], ord_of(mx2));
+    if (frac) {
+      const FrameDev* F = J.fd;
+      const float s2 = z * F->invf[2];
+      const float s1 = (y - F->Bf[5] * s2) * F->invf[1];
+      const float s0 = (x - F->Bf[1] * s1 - F->Bf[2] * s2) * F->invf[0];
+      sn[0] = fminf(sn[0], s0); sn[1] = fminf(sn[1], s1); sn[2] = fminf(sn[2], s2);
+      sx[0] = fmaxf(sx[0], s0); sx[1] = fmaxf(sx[1], s1); sx[2] = fmaxf(sx[2], s2);
     }
-    if (bad) atomicExch(&F->bad, 1);
   }
+  // block minima and maxima (maxima as minima of the negated values), one set of
+  // atomics per block
+  float v[12] = {mn0, mn1, mn2, -mx0, -mx1, -mx2, sn[0], sn[1], sn[2], -sx[0], -sx[1], -sx[2]};
+  __shared__ float s_v[8][12];
+  __shared__ int s_bad;
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
+  const int nv = frac ? 12 : 6;
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    if (c >= nv) break;
+    for (int o = 16; o > 0; o >>= 1) v[c] = fminf(v[c], __shfl_xor_sync(kFull, v[c], o));
+    if ((threadIdx.x & 31) == 0) s_v[threadIdx.x >> 5][c] = v[c];
+  }
+  if (bad) s_bad = 1;
+  __syncthreads();
+  if (threadIdx.x < nv) {
+    const int c = threadIdx.x;
+    float m = s_v[0][c];
+    for (int w = 1; w < blockDim.x / 32; ++w) m = fminf(m, s_v[w][c]);
+    FrameDev* F = J.fd;
+    int32_t* const mn = c < 6 ? F->cmin : F->smin;
+    int32_t* const mx = c < 6 ? F->cmax : F->smax;
+    if (c % 6 < 3) {
+      if (m < INFINITY) atomicMin(mn + c % 3, ord_of(m));
+    } else if (m < INFINITY) {
+      atomicMax(mx + c % 3, ord_of(-m));
+    }
+  }
+  if (threadIdx.x == 0 && s_bad) atomicExch(&J.fd->bad, 1);
 }
 
 // ------------------------------------------------------------------ spatial order (staging)
 
-__device__ __forceinline__ uint32_t spread3(uint32_t v) {  // bit k of v -> bit 3k
-  v &= 0x3FFu;
-  v = (v | (v << 16)) & 0x030000FFu;
-  v = (v | (v << 8)) & 0x0300F00Fu;
-  v = (v | (v << 4)) & 0x030C30C3u;
-  v = (v | (v << 2)) & 0x09249249u;
-  return v;
+// Position of cell (x, y, z) of a 2^g grid along the three-dimensional Hilbert
+// curve, by J. Skilling's transpose algorithm (AIP Conf. Proc. 707, 381, 2004).
+// Unlike Morton order its consecutive cells are always neighbours, so runs of
+// consecutive particles have smaller bounding boxes.
+__device__ __forceinline__ uint32_t hilbert_key(uint32_t x, uint32_t y, uint32_t z, int g) {
+  for (uint32_t q = 1u << (g - 1); q > 1; q >>= 1) {  // undo the excess work, axis by axis
+    const uint32_t p = q - 1;
+    if (x & q) x ^= p;
+    if (y & q) {
+      x ^= p;
+    } else {
+      const uint32_t t = (x ^ y) & p;
+      x ^= t;
+      y ^= t;
+    }
+    if (z & q) {
+      x ^= p;
+    } else {
+      const uint32_t t = (x ^ z) & p;
+      x ^= t;
+      z ^= t;
+    }
+  }
+  y ^= x;  // Gray encoding
+  z ^= y;
+  uint32_t t = 0;
+  for (uint32_t q = 1u << (g - 1); q > 1; q >>= 1)
+    if (z & q) t ^= q - 1;
+  x ^= t;
+  y ^= t;
+  z ^= t;
+  uint32_t key = 0;
+  for (int b = g - 1; b >= 0; --b) key = (key << 3) | (((x >> b) & 1u) << 2) | (((y >> b) & 1u) << 1) | ((z >> b) & 1u);
+  return key;
 }
 
-// Morton cell of a particle from its fractional coordinates in the box, or in
-// the frame's bounding box without one (approximate float32; only the order
-// depends on it).
+// A particle's position brought home: minus the lattice vector of its fractional
+// coordinates' integer parts, in binary64 (frames that span several cells).
+__device__ __forceinline__ double3 bring_home(const FrameDev& F, double x, double y, double z) {
+  const double* B = F.B;
+  const double sz = z / B[8], sy = (y - B[5] * sz) / B[4], sx = (x - B[1] * sy - B[2] * sz) / B[0];
+  const double kx = floor(sx), ky = floor(sy), kz = floor(sz);
+  return make_double3(((x - kx * B[0]) - ky * B[1]) - kz * B[2], (y - ky * B[4]) - kz * B[5], z - kz * B[8]);
+}
+
+// Cell of a particle on the curve (only the order depends on it).
 __device__ __forceinline__ uint32_t cell_key(const FrameDev& F, float4 p, int g) {
-  float s[3];
-  if (F.variant == V_NONE) {
-    const float q[3] = {p.x, p.y, p.z};
-    for (int c = 0; c < 3; ++c) {
-      const float lo = float_of_ord(F.cmin[c]), hi = float_of_ord(F.cmax[c]);
-      s[c] = (hi > lo) ? fminf((q[c] - lo) / (hi - lo), 0.999999f) : 0.0f;
-    }
-  } else if (F.variant == V_ORTHO) {
-    s[0] = p.x * F.invf[0];
-    s[1] = p.y * F.invf[1];
-    s[2] = p.z * F.invf[2];
-  } else {
-    s[2] = p.z * F.invf[2];
-    s[1] = (p.y - F.Bf[5] * s[2]) * F.invf[1];
-    s[0] = (p.x - F.Bf[1] * s[1] - F.Bf[2] * s[2]) * F.invf[0];
+  if (g == 0) return 0u;
+  if (F.wrap) {
+    const double3 w = bring_home(F, p.x, p.y, p.z);
+    p.x = (float)w.x;
+    p.y = (float)w.y;
+    p.z = (float)w.z;
   }
   const float G = (float)(1 << g);
-  uint32_t c[3];
-  for (int a = 0; a < 3; ++a) {
-    float f = s[a] - floorf(s[a]);
-    int ci = (int)(f * G);
-    c[a] = (uint32_t)min(max(ci, 0), (1 << g) - 1);
-  }
-  return spread3(c[0]) | (spread3(c[1]) << 1) | (spread3(c[2]) << 2);
+  const int last = (1 << g) - 1;
+  const int cx = (int)((p.x - F.key_lo[0]) * F.key_inv * G), cy = (int)((p.y - F.key_lo[1]) * F.key_inv * G),
+            cz = (int)((p.z - F.key_lo[2]) * F.key_inv * G);
+  return hilbert_key((uint32_t)min(max(cx, 0), last), (uint32_t)min(max(cy, 0), last),
+                     (uint32_t)min(max(cz, 0), last), g);
 }
 
 __global__ void sort_count_kernel(const SortSeg* segs, const float4* __restrict__ X, int32_t* keys,
@@ -250,63 +261,112 @@ __global__ void sort_count_kernel(const SortSeg* segs, const float4* __restrict_
   }
 }
 
-// Exclusive prefix sum of each segment's counters, in place (one block per segment).
-__global__ void sort_scan_kernel(const SortSeg* segs, uint32_t* counts) {
-  const SortSeg S = segs[blockIdx.x];
-  const int64_t m = (int64_t)1 << (3 * S.g);
-  uint32_t* c = counts + S.key0;
-  const int64_t per = (m + blockDim.x - 1) / blockDim.x;
-  const int64_t b = min(m, (int64_t)threadIdx.x * per), e = min(m, b + per);
-  uint32_t local = 0;
-  for (int64_t k = b; k < e; ++k) local += c[k];
-  __shared__ uint32_t warp_sum[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Exclusive prefix sum of each segment's counters (counts -> cursors), one block
+// per kScanTile of them.  A block sums the counters before its tile itself: at
+// most a few MB from L2 in 16-byte loads, cheaper than a second launch or a wait
+// on the blocks before it (a single block per segment took 0.42 ms at 2^18
+// counters, one tenth of what the whole frame's other preparation took).
+constexpr int kScanTile = 4096;
+__global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, const uint32_t* __restrict__ counts,
+                                                         uint32_t* __restrict__ cursors) {
+  const SortSeg S = segs[blockIdx.y];
+  const int m = 1 << (3 * S.g), t0 = blockIdx.x * kScanTile;
+  if (t0 >= m) return;
+  const uint32_t* c = counts + S.key0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ uint32_t s_sum[32];
+  // this thread's four counters (segments below four counters have a whole tile to themselves)
+  uint32_t v[4], local = 0;
+  for (int q = 0; q < 4; ++q) {
+    const int k = t0 + 4 * tid + q;
+    v[q] = k < m ? c[k] : 0u;
+    local += v[q];
+  }
+  // counters before the tile (a multiple of four, 16-byte aligned: see key0)
+  uint32_t before = 0;
+  const uint4* c4 = reinterpret_cast<const uint4*>(c);
+#pragma unroll 4
+  for (int k = tid; k < t0 / 4; k += 1024) {
+    const uint4 x = __ldg(c4 + k);
+    before += (x.x + x.y) + (x.z + x.w);
+  }
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
+  if (lane == 0) s_sum[warp] = before;
+  __syncthreads();
+  uint32_t base = s_sum[lane];
+  for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(kFull, base, o);
+  __syncthreads();
   uint32_t incl = local;
   for (int o = 1; o < 32; o <<= 1) {
-    uint32_t v = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += v;
+    const uint32_t x = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += x;
   }
-  if (lane == 31) warp_sum[warp] = incl;
+  if (lane == 31) s_sum[warp] = incl;
   __syncthreads();
-  if (warp == 0) {
-    const int nw = blockDim.x / 32;
-    uint32_t v = lane < nw ? warp_sum[lane] : 0u, inc = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t t = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += t;
+  uint32_t w = lane < warp ? s_sum[lane] : 0u;
+  for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(kFull, w, o);
+  uint32_t run = base + w + incl - local;
+  for (int q = 0; q < 4; ++q) {
+    const int k = t0 + 4 * tid + q;
+    if (k < m) cursors[S.key0 + k] = run;
+    run += v[q];
+  }
+}
+
+__global__ void sort_scatter_kernel(const SortSeg* segs, const float4* __restrict__ src,
+                                    const double4* __restrict__ src64, const int32_t* __restrict__ keys,
+                                    uint32_t* cursors, float4* dst, double4* dst64) {
+  const SortSeg S = segs[blockIdx.y];
+  const FrameDev& F = *S.fd;
+  const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
+  const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
+  const double to_bins = (double)F.nbins / F.r_max;
+  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    const int64_t pos = S.x0 + atomicAdd(cursors + S.key0 + (uint32_t)keys[S.x0 + i], 1u);
+    const float4 p = src[S.x0 + i];
+    dst[pos] = p;
+    double3 v = make_double3(p.x, p.y, p.z);
+    if (F.X64) {
+      const double4 q = src64[S.x0 + i];
+      dst64[pos] = q;
+      v = make_double3(q.x, q.y, q.z);
     }
-    if (lane < nw) warp_sum[lane] = inc - v;  // exclusive over warps
-  }
-  __syncthreads();
-  uint32_t run = warp_sum[warp] + incl - local;  // exclusive start of this thread's chunk
-  for (int64_t k = b; k < e; ++k) {
-    uint32_t v = c[k];
-    c[k] = run;
-    run += v;
-  }
-}
-
-__global__ void sort_scatter_kernel(const SortSeg* segs, const float4* __restrict__ X,
-                                    const double4* __restrict__ X64, const int32_t* __restrict__ keys,
-                                    uint32_t* cursors, float4* Xs, double4* Xs64) {
-  const SortSeg S = segs[blockIdx.y];
-  const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
-  const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    uint32_t pos = atomicAdd(cursors + S.key0 + (uint32_t)keys[S.x0 + i], 1u);
-    Xs[S.x0 + pos] = X[S.x0 + i];
-    if (X64) Xs64[S.x0 + pos] = X64[S.x0 + i];
+    if (F.P4) {
+      if (F.wrap) v = bring_home(F, v.x, v.y, v.z);
+      v = make_double3(v.x * to_bins, v.y * to_bins, v.z * to_bins);
+      const double g = F.list_grid, ig = 1.0 / g;
+      const float3 h = make_float3((float)(rint(v.x * ig) * g), (float)(rint(v.y * ig) * g), (float)(rint(v.z * ig) * g));
+      F.P4[pos - S.f0] = make_float4(h.x, h.y, h.z, (float)(v.x - (double)h.x));
+      F.P2[pos - S.f0] = make_float2((float)(v.y - (double)h.y), (float)(v.z - (double)h.z));
+    }
   }
 }
 
-__global__ void sort_copy_kernel(const SortSeg* segs, const float4* __restrict__ Xs, float4* X,
-                                 const double4* __restrict__ Xs64, double4* X64) {
+// Bounds of each run of kRun ordered particles (one warp per run), over the
+// positions the list kernel works with.
+__global__ void run_bounds_kernel(const SortSeg* segs) {
   const SortSeg S = segs[blockIdx.y];
-  const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
-  const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    X[S.x0 + i] = Xs[S.x0 + i];
-    if (X64) X64[S.x0 + i] = Xs64[S.x0 + i];
+  const FrameDev& F = *S.fd;
+  const int run = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
+  if (!F.bnd || run * (int64_t)kRun >= S.n) return;
+  float b[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  const int64_t p0 = S.x0 - S.f0;
+  for (int i = run * kRun + lane; i < min(S.n, (run + 1) * kRun); i += 32) {
+    const float4 p = F.P4[p0 + i];
+    const float v[3] = {p.x, p.y, p.z};
+    for (int c = 0; c < 3; ++c) {
+      b[c] = fminf(b[c], v[c]);
+      b[3 + c] = fmaxf(b[3 + c], v[c]);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1)
+    for (int c = 0; c < 3; ++c) {
+      b[c] = fminf(b[c], __shfl_xor_sync(kFull, b[c], o));
+      b[3 + c] = fmaxf(b[3 + c], __shfl_xor_sync(kFull, b[3 + c], o));
+    }
+  if (lane == 0) {
+    F.bnd[2 * (S.run0 + run)] = make_float4(b[0], b[1], b[2], 0.0f);
+    F.bnd[2 * (S.run0 + run) + 1] = make_float4(b[3], b[4], b[5], 0.0f);
   }
 }
 
@@ -319,6 +379,77 @@ __device__ inline double half_ulp_below(double D) {
   int E;
   frexp(D, &E);  // D = m 2^E, m in [1/2, 1): |x| <= D < 2^E
   return ldexp(1.0, E - 25);
+}
+
+// The spatial order's grid and the list kernel's window of one frame.
+//
+// The list kernel works in bins, relative to the centre of an i run: x for the
+// run's particles (|x| <= H, half the diagonal of its bounds), y for an image of
+// a j particle (T = |y|), both double-floats, and evaluates
+//   q = A + (B - 2 x.y),  A = |y|^2, B = |x|^2,
+// A and B rounded once, x and y rounded once for the product, the parenthesis
+// first (three FMAs), A added last.  With u = 2^-24, q errs by at most
+//   x and y rounded for the product         2u TH + 2u TH
+//   A, B                                    u T^2 + u H^2
+//   three FMAs, results below 2 TH + H^2    6u TH + 3u H^2
+//   last add                                u (T + H)^2
+// in all u (2 T^2 + 12 TH + 5 H^2) <= u ((2 + 6l) T^2 + (5 + 6/l) H^2) for any
+// l > 0 (run_window takes l = H over a typical T).  list_c0 covers what the
+// double-floats leave out (a0, 2^-45 of the coordinates) and the binary64
+// definition's own rounding of t.
+__device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
+  const double u = 1.0 / 16777216.0;
+  const double* B = F.B;
+  const double S = (double)F.nbins / F.r_max;
+  int wrap = 0, slow = 0;
+  double lo[3], ext[3], far = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    lo[c] = (F.cmin[c] <= F.cmax[c]) ? (double)float_of_ord(F.cmin[c]) : 0.0;
+    ext[c] = R[c];
+    far = fmax(far, Xm[c]);
+  }
+  if (F.variant != V_NONE) {
+    for (int c = 0; c < 3; ++c) {
+      const double span = F.variant == V_TRIC ? (double)float_of_ord(F.smax[c]) - (double)float_of_ord(F.smin[c])
+                                              : R[c] * (double)F.invf[c];
+      if (span > 1.0 + 1.0 / 16.0) wrap = 1;
+    }
+    if (wrap) {  // the home cell's bounding box
+      ext[0] = B[0] + fabs(B[1]) + fabs(B[2]);
+      ext[1] = B[4] + fabs(B[5]);
+      ext[2] = B[8];
+      lo[0] = fmin(B[1], 0.0) + fmin(B[2], 0.0);
+      lo[1] = fmin(B[5], 0.0);
+      lo[2] = 0.0;
+      // (binary64 still tells the images apart below 2^30 cells)
+      const double sz = Xm[2] / B[8], sy = (Xm[1] + fabs(B[5]) * sz) / B[4],
+                   sx = (Xm[0] + fabs(B[1]) * sy + fabs(B[2]) * sz) / B[0];
+      if (!(fmax(sx, fmax(sy, sz)) < 1e6)) slow = 1;
+    }
+  }
+  const double side = fmax(ext[0], fmax(ext[1], ext[2]));
+  for (int c = 0; c < 3; ++c) F.key_lo[c] = (float)lo[c];
+  F.key_inv = side > 0.0 ? (float)(0.99999 / side) : 0.0f;
+  F.wrap = wrap;
+  F.list_slow = slow;
+  const double cell = F.variant == V_NONE ? 0.0 : B[0] + fabs(B[1]) + fabs(B[2]) + B[4] + fabs(B[5]) + B[8];
+  // positions and image vectors: the largest of them in bins; brought home, the
+  // binary64 subtraction errs by 2^-52 of what is subtracted
+  const double reach = S * ((wrap ? ext[0] + ext[1] + ext[2] : 2.0 * far) + 2.0 * cell);
+  const double a0 = reach * 0x1p-45 + (wrap ? S * far * 0x1p-49 : 0.0);
+  // grid of the high parts: sums of positions, centres and images stay below
+  // 2^23 steps, so they are exact in float32
+  int e = 0;
+  frexp(reach, &e);  // reach < 2^e
+  F.list_grid = (float)ldexp(1.0, max(e - 22, -120));
+  F.cull_abs = __double2float_ru(reach * 9.5367431640625e-07);  // 2^-20
+  F.list_c0 = __double2float_ru(a0 * a0 * 0x1p28 + 0x1p-26);
+  F.list_mid = __double2float_ru(4.0 * a0);
+  F.list_tie = F.variant == V_ORTHO ? __double2float_ru((double)F.tie_eps * S * 1.01 + 4.0 * a0) : 0.0f;
+  // every decision needs the nearest integer of the root right to within one:
+  // window and square-root error below a quarter bin at the far end
+  const double tmax = (double)F.nbins + 40.0;
+  F.list_all = !(8.0 * u * tmax + 4.0 * a0 < 0.25) || !(tmax * 4.76837158203125e-07 < 0.25);
 }
 
 // Derives, for one frame, the bound of the float32 decision and of the
@@ -458,15 +589,6 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
     aw[0][0] = au[0] + half_ulp_below(Dxw) + Kx * dB[0];
     aw[0][1] = au[1];
     aw[0][2] = au[2];
-    for (int m = 0; m < 27; ++m) {
-      const double kx = m / 9 - 1, ky = (m / 3) % 3 - 1, kz = m % 3 - 1;
-      const double v[3] = {-((kx * ax + ky * bx) + kz * cx), -(ky * by + kz * cy), -(kz * cz)};
-      for (int c = 0; c < 3; ++c) {
-        F.tshift[m][c] = (float)v[c];
-        // the binary64 sum itself errs by at most 2^-52 of the row sum
-        F.tserr[m][c] = __double2float_ru(fabs((double)F.tshift[m][c] - v[c]) + fmax(Sx, fmax(Sy, Sz)) * 0x1p-51);
-      }
-    }
     F.kxdb = __double2float_ru(Kx * dB[0]);
     I[0] = D2x + Kx * ax;
     I[1] = D1y + Ky * by;
@@ -527,6 +649,7 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
   F.mid2 = (float)(1.0 / 274877906944.0);                                                   // 2^-38
   F.mid1 = (float)(2.0 * amid / S * 1.01);
   F.tie_eps = (float)tie_eps;
+  list_setup(F, R, Xm);
   F.delta = (float)fmin(delta, 1.0);
   F.alpha_t = (float)alpha;
   F.beta_t = (float)beta;
@@ -686,10 +809,6 @@ __device__ float tile_beta(const FrameDev& F, const float* imin, const float* im
   return __fadd_ru(__fmul_ru(__fmul_ru(F.S, __fsqrt_ru(a2)), 1.0f + 0x1p-12f), tie) + 0x1p-28f;
 }
 
-// Guard words on each side of a shared-memory histogram copy: the increments
-// of pairs outside [lo, hi) land there (see count_or_defer).
-constexpr int kGuard = 36;
-
 struct ItemDesc {
   FrameDev* fd;
   int32_t valid;   // 0: no more work
@@ -751,13 +870,6 @@ __device__ __forceinline__ float wrap_r2(float dx, float dy, float dz, const Fas
   return __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
 }
 
-// ---- packed float32 arithmetic: two pairs per instruction (FFMA2/FADD2/FMUL2)
-
-__device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
 // float32 |d'|^2 of two pairs after the minimum image of the variant; each
 // component is rounded exactly as the scalar sequence of wrap_r2.  In the
 // shifted modes the caller has already subtracted the tile's images from the
@@ -799,40 +911,6 @@ __device__ __forceinline__ float2 wrap_r2_2(float2 dx, float2 dy, float2 dz, con
     return make_float2(wrap_r2<V>(dx.x, dy.x, dz.x, P, amb_a), wrap_r2<V>(dx.y, dy.y, dz.y, P, amb_b));
   }
   return fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-}
-
-// Count one pair, branch free.  With sm = s_c + 1.5*2^23 (s_c the clamped root,
-// bits(sm) - bits(1.5*2^23) = its nearest integer n) and the residual
-// e = n^2 - q (e > 0: t < n, so floor(t) = n - 1; e < 0: floor(t) = n), the
-// bin relative to the sweep is v - kb1 with v = bits(sm) + signbit(e), and the
-// shared-memory address is 4 v + hbase (a shift and an add, which stay off the
-// FMA pipe that the packed float32 arithmetic keeps busy; a multiply-add by 4
-// measured 1-2 % slower).  Every pair increments that word.  The
-// clamp of s_c to [lo - lane, hi + 1 + lane] (integers below 2^22) keeps the
-// relative bin in [-1 - lane, width + 1 + lane]: pairs outside the sweep, and
-// NaN pairs (s_c = hi + 1 + lane, e NaN with a clear sign bit: bin width + lane),
-// land in the guard words, spread over the lanes.  A clamped pair that is
-// decided is decided right: e > bound means t lies within the clamp's integer
-// and the one below, e < -bound that t lies above it, out of the sweep (and
-// the converse at the lower clamp).  A pair with |e| <= bound (false for NaN)
-// also sets the bit `bit` of dmask: it is counted provisionally and re-decided
-// by the drain, which moves its count to the exact bin when the two differ.
-__device__ __forceinline__ void count_or_defer(float sm, float e, float bound, uint32_t hbase, uint32_t bit,
-                                               uint32_t& dmask) {
-  asm volatile(
-      "{\n\t.reg .pred pn;\n\t.reg .u32 eb, sg, v, addr;\n\t.reg .f32 ae;\n\t"
-      "mov.b32 eb, %2;\n\t"
-      "shr.u32 sg, eb, 31;\n\t"
-      "add.u32 v, %1, sg;\n\t"
-      "shl.b32 addr, v, 2;\n\t"
-      "add.u32 addr, addr, %4;\n\t"
-      "abs.f32 ae, %2;\n\t"
-      "setp.gtu.f32 pn, ae, %3;\n\t"
-      "@!pn or.b32 %0, %0, %5;\n\t"
-      "red.shared.add.u32 [addr], 1;\n\t"
-      "}"
-      : "+r"(dmask)
-      : "r"(__float_as_uint(sm)), "f"(e), "f"(bound), "r"(hbase), "r"(bit));
 }
 
 // The same with the increments of the warp aggregated in software (the hybrid
@@ -937,54 +1015,6 @@ __device__ __forceinline__ int provisional_rel(const FastParams& P, float4 pi, f
   return (int)(__float_as_uint(sm) + (__float_as_uint(e) >> 31) - (uint32_t)P.kb1);
 }
 
-// ---- double-float middle tier
-
-struct DF {
-  float h, l;  // unevaluated sum h + l
-};
-
-__device__ __forceinline__ DF two_sum(float a, float b) {
-  float s = __fadd_rn(a, b);
-  float bb = __fsub_rn(s, a);
-  float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return {s, e};
-}
-__device__ __forceinline__ DF two_prod(float a, float b) {
-  float p = __fmul_rn(a, b);
-  return {p, __fmaf_rn(a, b, -p)};
-}
-// v - k (bh + bl) for an integer k, renormalised: after a large image is
-// taken off, the low part of v (the rounding error of a difference of large
-// coordinates) can be far above an ulp of the small result, and the products
-// of df_norm2 are accurate only for a normalised pair (|l| <= ulp(h) / 2)
-__device__ __forceinline__ DF df_sub_kb(DF v, float k, float bh, float bl) {
-  DF p = two_prod(k, bh);
-  DF s = two_sum(v.h, -p.h);
-  float low = __fmaf_rn(-k, bl, __fsub_rn(__fadd_rn(v.l, s.l), p.l));
-  return two_sum(s.h, low);
-}
-__device__ __forceinline__ DF df_norm2(DF x, DF y, DF z) {
-  DF ax = two_prod(x.h, x.h), ay = two_prod(y.h, y.h), az = two_prod(z.h, z.h);
-  DF s1 = two_sum(ax.h, ay.h);
-  DF s2 = two_sum(s1.h, az.h);
-  float low = __fadd_rn(__fadd_rn(__fadd_rn(ax.l, ay.l), __fadd_rn(az.l, s1.l)), s2.l);
-  low = __fmaf_rn(__fadd_rn(x.h, x.h), x.l, low);
-  low = __fmaf_rn(__fadd_rn(y.h, y.h), y.l, low);
-  low = __fmaf_rn(__fadd_rn(z.h, z.h), z.l, low);
-  low = __fmaf_rn(x.l, x.l, __fmaf_rn(y.l, y.l, __fmaf_rn(z.l, z.l, low)));
-  return {s2.h, low};
-}
-
-// xj - xi for binary64 values, as a double-float: each value split into float32
-// high and low parts (x = h + l to about 2^-48 |x|), the high parts subtracted
-// exactly and the low parts added to the error term.
-__device__ __forceinline__ DF df_diff64(double xj, double xi) {
-  const float hj = __double2float_rn(xj), hi = __double2float_rn(xi);
-  const float lj = __double2float_rn(__dsub_rn(xj, (double)hj)), li = __double2float_rn(__dsub_rn(xi, (double)hi));
-  DF s = two_sum(hj, -hi);
-  return two_sum(s.h, __fadd_rn(s.l, __fsub_rn(lj, li)));  // renormalised (see df_sub_kb)
-}
-
 // Bin of a deferred pair from r^2 evaluated in double-float arithmetic (about
 // 44 bits, with the exact coordinate differences (float32 input; binary64
 // input to about 2^-47 of the coordinate magnitude) and the same nearest images
@@ -1051,84 +1081,6 @@ __device__ int mid_bin(const FrameDev& F, int i, int j, float4 pi, float4 pj) {
   float bound = __fmaf_rn(F.mid2, r2.h, __fmul_rn(F.mid1, s));
   if (!(fabsf(diff) > bound)) return -1;
   return diff >= 0.0f ? ni : ni - 1;
-}
-
-// ---- binary64 last resort
-
-// Squared minimum-image distance in binary64, the same operations in the same
-// order as the definition (Alg. 1, Eq. 5, 27 neighbouring shifts); the
-// coordinates are the caller's (float32 promoted exactly, or binary64).
-template <int V>
-__device__ double exact_r2(const FrameDev& F, double3 pi, double3 pj) {
-  double dx = __dsub_rn(pj.x, pi.x);
-  double dy = __dsub_rn(pj.y, pi.y);
-  double dz = __dsub_rn(pj.z, pi.z);
-  const double* B = F.B;
-  if (V == V_ORTHO) {
-    double kx = rint(__dmul_rn(dx, F.Linv[0]));
-    double ky = rint(__dmul_rn(dy, F.Linv[1]));
-    double kz = rint(__dmul_rn(dz, F.Linv[2]));
-    dx = __fma_rn(-kx, B[0], dx);
-    dy = __fma_rn(-ky, B[4], dy);
-    dz = __fma_rn(-kz, B[8], dz);
-  } else if (V == V_TRIC || V == V_TRIC_SEARCH) {
-    const double ax = B[0], bx = B[1], cx = B[2], by = B[4], cy = B[5], cz = B[8];
-    double sz = __ddiv_rn(dz, cz);
-    double sy = __ddiv_rn(__dsub_rn(dy, __dmul_rn(cy, sz)), by);
-    double sx = __ddiv_rn(__dsub_rn(__dsub_rn(dx, __dmul_rn(bx, sy)), __dmul_rn(cx, sz)), ax);
-    double kx = rint(sx), ky = rint(sy), kz = rint(sz);
-    dx = __dsub_rn(__dsub_rn(__dsub_rn(dx, __dmul_rn(ax, kx)), __dmul_rn(bx, ky)), __dmul_rn(cx, kz));
-    dy = __dsub_rn(__dsub_rn(dy, __dmul_rn(by, ky)), __dmul_rn(cy, kz));
-    dz = __dsub_rn(dz, __dmul_rn(cz, kz));
-    // Below half the plane spacing (V_TRIC: r_max <= (1 - 2^-8) h_min / 2) the
-    // shift m = 0 is the minimum of the 27 for every pair inside r_max: the
-    // sequential rounding is Babai's nearest plane in the upper-triangular
-    // basis, exact for vectors shorter than half its smallest Gram-Schmidt
-    // length (cz, by, ax >= h_min), and every other shift is longer than
-    // h_min - r_max > r_max.  Its value is the m = 0 term of the loop, bit for
-    // bit (adding the zero products changes nothing); a pair beyond r_max stays
-    // beyond it under any shift.  So the binary64 bin is the definition's.
-    if (V == V_TRIC) return __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
-    double best = INFINITY;
-#pragma unroll 1
-    for (int mx = -1; mx <= 1; ++mx)
-#pragma unroll 1
-      for (int my = -1; my <= 1; ++my)
-#pragma unroll 1
-        for (int mz = -1; mz <= 1; ++mz) {
-          double ex = __dadd_rn(__dadd_rn(__dadd_rn(dx, __dmul_rn(ax, (double)mx)), __dmul_rn(bx, (double)my)),
-                                __dmul_rn(cx, (double)mz));
-          double ey = __dadd_rn(__dadd_rn(dy, __dmul_rn(by, (double)my)), __dmul_rn(cy, (double)mz));
-          double ez = __dadd_rn(dz, __dmul_rn(cz, (double)mz));
-          double r2 = __fma_rn(ez, ez, __fma_rn(ey, ey, __dmul_rn(ex, ex)));
-          if (r2 < best) best = r2;
-        }
-    return best;
-  }
-  return __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
-}
-
-// Bin of a binary64 r^2 from the threshold table: the largest k with T[k] <= r2
-// (T[0] = 0, T nondecreasing; 0 for NaN).  The float32 estimate S sqrt(r2) is
-// within a bin or two of it; the two walks make the result exact whatever the
-// estimate, with one or two dependent loads instead of a binary search's
-// log2(nbins).
-__device__ __forceinline__ int bin_from_thresholds(const double* __restrict__ T, float S, int nbins, double r2) {
-  if (!(r2 >= 0.0)) return 0;
-  int k = (int)fminf(__fmul_rn(sqrtf(__double2float_rn(r2)), S), (float)nbins);
-  while (k > 0 && __ldg(T + k) > r2) --k;
-  while (k < nbins && __ldg(T + k + 1) <= r2) ++k;
-  return k;
-}
-
-// The caller's coordinates of particle i of a frame, in binary64.
-__device__ __forceinline__ double3 coords64(const FrameDev& F, int i) {
-  if (F.X64) {
-    double4 p = F.X64[i];
-    return make_double3(p.x, p.y, p.z);
-  }
-  float4 p = __ldg(F.X + i);
-  return make_double3((double)p.x, (double)p.y, (double)p.z);
 }
 
 // The binary64 replay of one pair (about one deferred pair in 10^4): out of
@@ -2197,16 +2149,18 @@ cudaError_t launch_stage(const StageJob* jobs, int n_jobs, int64_t n_chunks, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, int max_chunks, float4* X, float4* Xs,
-                                double4* X64, double4* Xs64, int32_t* keys, uint32_t* counts,
+cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, int64_t max_n, const float4* src, float4* dst,
+                                const double4* src64, double4* dst64, int32_t* keys, uint32_t* counts, int64_t n_keys,
                                 cudaStream_t stream) {
   clear_stale_error();
-  if (n_segs <= 0 || max_chunks <= 0) return cudaSuccess;
-  dim3 grid((unsigned)max_chunks, (unsigned)n_segs);
-  sort_count_kernel<<<grid, 256, 0, stream>>>(segs, X, keys, counts);
-  sort_scan_kernel<<<n_segs, 1024, 0, stream>>>(segs, counts);
-  sort_scatter_kernel<<<grid, 256, 0, stream>>>(segs, X, X64, keys, counts, Xs, Xs64);
-  sort_copy_kernel<<<grid, 256, 0, stream>>>(segs, Xs, X, Xs64, X64);
+  if (n_segs <= 0 || max_n <= 0) return cudaSuccess;
+  dim3 grid((unsigned)((max_n + kSortChunk - 1) / kSortChunk), (unsigned)n_segs);
+  sort_count_kernel<<<grid, 256, 0, stream>>>(segs, src, keys, counts);
+  dim3 sgrid((unsigned)((((int64_t)1 << (3 * sort_grid_bits(max_n))) + kScanTile - 1) / kScanTile), (unsigned)n_segs);
+  sort_scan_kernel<<<sgrid, 1024, 0, stream>>>(segs, counts, counts + n_keys);
+  sort_scatter_kernel<<<grid, 256, 0, stream>>>(segs, src, src64, keys, counts + n_keys, dst, dst64);
+  dim3 bgrid((unsigned)((max_n + 8 * kRun - 1) / (8 * kRun)), (unsigned)n_segs);
+  run_bounds_kernel<<<bgrid, 256, 0, stream>>>(segs);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,876 @@
+// The list kernel: pair-distance histograms of spatially ordered species, one
+// warp per run of kRun i particles (sm_103a).
+//
+// Every particle image that can lie in the current bin sweep as seen from the
+// run's bounding box is listed once, and every listed image is evaluated
+// against the whole run with the same arithmetic whatever the box: no nearest
+// image is searched per pair.  With r_max at most half the smallest distance
+// between a particle's images, one image of a pair at most lies inside r_max,
+// and the others are counted as out of range like any other far pair (those
+// whose float32 value comes close to a bin edge are re-decided, and counted
+// only for the image that the binary64 definition picks).  So the periodic
+// frames cost what the frame without a box costs, and particles beyond r_max
+// of the run are dropped one by one, not in tiles.
+//
+// Per pair of float32 lanes: three FMAs and one add give q = t^2 (the run's
+// centre is the origin, so q = |y|^2 + (|x|^2 - 2 x.y) with |y|^2 listed and
+// the parenthesis small), then one square root, two adds and one FMA for the
+// residual, and the counting step of the tiled kernel.  The paper's kernels
+// (Sec. 3.2) evaluate every pair and wrap it per axis (Eq. 5).
+//
+// Warps claim items of one segment (species pair and sweep) straight from its
+// counter; the warps of a block meet only when a segment is exhausted, to merge
+// their shared histogram.
+//
+// What bounds it: without a box the shared-memory pipe (one increment per pair at
+// 3.5 wavefronts on random banks, 90 % busy at N = 200,000), for periodic frames
+// the issue slots (15 instructions per pair and lane, 70 % of the slots used).
+// Pair kernel at 2,070 MHz, 10,000 bins, the tiled kernel before -> now:
+// N = 1,000,000 none 235 -> 230 ms, orthorhombic 254 -> 173, triclinic 284 -> 131;
+// N = 100,000 orthorhombic, two species 4.2 -> 3.1 ms; N = 500,000 clustered
+// triclinic, three species, 20,000 bins 92.6 -> 47 ms; N = 2,000 none, 1,000 bins
+// 118 -> 18 us (items small enough for one per warp).
+// Measured and not kept: three 256-thread blocks of 80 registers (none 13.2 ms at
+// N = 200,000 against 9.6: spills, and the run's factors loaded again per block of
+// images), 384 and 448 threads (10.6 and 10.0 ms), sixteen pairs per lane and turn
+// instead of thirty-two (10.1 ms).
+#include <math.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "dh_device.h"
+#include "dh_internal.h"
+
+namespace dh {
+
+namespace {
+
+constexpr int kBlk = 64;       // listed images evaluated at a time
+constexpr int kCap = 2 * kBlk; // list ring: a block waiting to fill plus one round of 32 appends
+constexpr int kImgShift = 26;  // list reference: particle | image << 26
+constexpr int kHome = 13;      // the image k = 0
+// A claim takes 1/kClaims of a warp's share of the items left.  Items cost from
+// nothing (no image in the sweep) to 16,384 pairs, so a large claim of full items
+// can outlast everything else (2: triclinic N = 200,000 9.9 ms; 3: 8.4; 6: 6.7;
+// 12: 7.3), a small one pays for its run's setup (orthorhombic N = 100,000 2: 3.20,
+// 6: 3.09, 12: 3.72, 24: 3.98 ms).
+constexpr long long kClaims = 6;
+constexpr unsigned kFlushPairs = 1u << 23;  // flush after this many i runs x images (2^30 pairs)
+
+// A position: high parts on the frame's grid, sums of which are exact, and the rest.
+struct Pos {
+  float3 h, l;
+};
+__device__ __forceinline__ Pos unpack(float4 a, float2 b) {
+  return Pos{make_float3(a.x, a.y, a.z), make_float3(a.w, b.x, b.y)};
+}
+// An i run: centre (on the grid), half extents, window W = c1 A + c0 (list_setup).
+struct RunState {
+  float3 c, h;
+  float c1, c0;
+};
+
+// One warp's list: slot s holds y and W - |y|^2 of an image in pair layout (A: x,
+// x', y, y'; B: z, z', and the last for slots 2p, 2p+1), the mask of each group
+// of 8 slots and lane (bit 4 u + r: slot u of the group, i particle lane + 32 r),
+// the queue of pairs to re-decide (reference, i particle), and the current i run.
+struct WarpList {
+  float4 A[kCap / 2];
+  float4 B[kCap / 2];
+  uint32_t ref[kCap];
+  uint32_t mask[kBlk / 8][32];
+  uint2 queue[kQueueCap];
+  RunState R;
+  Pos o;         // the current image's origin,
+  float qm_here; //   its (2 W + 1)^2 where near,
+  float qm;      // and the largest of them in the list
+  unsigned long long uni, axis, cull;  // pairs, for the statistics
+};
+
+// What a block's pairs have in common (its segment), in shared memory.
+struct SegState {
+  FrameDev* F;
+  const float4 *P4i, *P4j, *bi, *bj;  // positions and run bounds of the i and the j species
+  const float2 *P2i, *P2j;
+  int i0, j0, ni, nj, n_ti, n_tj, intra;
+  int lo, hi;             // the sweep's bins
+  float rc_hi2, rc_lo2;   // images kept: nearest distance^2 <= rc_hi2, farthest^2 >= rc_lo2
+  float in_hi2, in_lo2;   // every pair in the sweep: farthest^2 <= in_hi2, nearest^2 >= in_lo2
+  float grid, c0, abs;    // FrameDev list_grid, list_c0, cull_abs
+  int n_img, all, slow;   // images of a particle; FrameDev list_all, list_slow
+  int inner;              // FrameDev in_range: nearly every block is an inner one
+  long long items, item_base;
+  long long claimers;     // claims that share the items left: kClaims per warp of the launch
+  unsigned long long* next;
+};
+
+// The multiple of the grid nearest to v (|v| < 2^22 steps).
+__device__ __forceinline__ float on_grid(float v, float grid) {
+  const float m = kMagicRound * grid;
+  return __fsub_rn(__fadd_rn(v, m), m);
+}
+
+// d + l as a double-float (d a multiple of the grid, |l| about a step at most).
+__device__ __forceinline__ DF renorm(float d, float l) {
+  const float h = __fadd_rn(d, l);
+  return {h, __fadd_rn(__fsub_rn(d, h), l)};
+}
+
+// |v|^2 - sub of a double-float vector, rounded once (to second order).
+__device__ __forceinline__ float norm2_less(DF x, DF y, DF z, float c1, float c0, float& b) {
+  const DF px = two_prod(x.h, x.h), py = two_prod(y.h, y.h), pz = two_prod(z.h, z.h);
+  const DF s1 = two_sum(px.h, py.h);
+  const DF s2 = two_sum(s1.h, pz.h);
+  float low = __fmaf_rn(x.h + x.h, x.l, px.l);
+  low = __fadd_rn(low, __fmaf_rn(y.h + y.h, y.l, py.l));
+  low = __fadd_rn(low, __fmaf_rn(z.h + z.h, z.l, pz.l));
+  low = __fadd_rn(low, __fadd_rn(s1.l, s2.l));
+  b = __fmaf_rn(c1, s2.h, c0);
+  return __fadd_rn(s2.h, __fsub_rn(low, b));
+}
+
+// One run's state from its bounds (explicit roundings: the drain computes it
+// again, and must get the same).  The window takes l of list_setup as
+// H over three quarters of the sweep's end; 2^-7 covers the second-order terms and
+// the rounding of W itself.
+__device__ __forceinline__ RunState run_state(const SegState& G, float4 lo4, float4 hi4) {
+  const float grid = G.grid;
+  RunState r;
+  r.c = make_float3(on_grid(__fmul_rn(0.5f, __fadd_rn(lo4.x, hi4.x)), grid),
+                    on_grid(__fmul_rn(0.5f, __fadd_rn(lo4.y, hi4.y)), grid),
+                    on_grid(__fmul_rn(0.5f, __fadd_rn(lo4.z, hi4.z)), grid));
+  // (the bounds are those of the high parts)
+  r.h = make_float3(__fadd_ru(fmaxf(__fsub_ru(hi4.x, r.c.x), __fsub_ru(r.c.x, lo4.x)), grid),
+                    __fadd_ru(fmaxf(__fsub_ru(hi4.y, r.c.y), __fsub_ru(r.c.y, lo4.y)), grid),
+                    __fadd_ru(fmaxf(__fsub_ru(hi4.z, r.c.z), __fsub_ru(r.c.z, lo4.z)), grid));
+  const float H2 = __fmaf_ru(r.h.z, r.h.z, __fmaf_ru(r.h.y, r.h.y, __fmul_ru(r.h.x, r.h.x)));
+  const float u = 0x1p-24f * (1.0f + 0x1p-7f);
+  const float l = fminf(fmaxf(__fdiv_rn(__fsqrt_rn(H2), __fmul_rn(0.75f, (float)G.hi)), 0.01f), 2.0f);
+  r.c1 = __fadd_rn(__fmul_rn(u, __fmaf_rn(6.0f, l, 2.0f)), 0x1p-27f);
+  r.c0 = __fmaf_rn(__fmul_rn(u, __fadd_rn(5.0f, __fdiv_rn(6.0f, l))), H2, G.c0);
+  return r;
+}
+
+// An i particle relative to the run's centre c: (2 x, -|x|^2), the factors of
+// the FMA chain.
+__device__ __forceinline__ float4 i_factors(const Pos& p, float3 c) {
+  const DF x = renorm(__fsub_rn(p.h.x, c.x), p.l.x), y = renorm(__fsub_rn(p.h.y, c.y), p.l.y),
+           z = renorm(__fsub_rn(p.h.z, c.z), p.l.z);
+  float b;
+  return make_float4(2.0f * x.h, 2.0f * y.h, 2.0f * z.h, -norm2_less(x, y, z, 0.0f, 0.0f, b));
+}
+
+// The vector that takes a home position to image m relative to the centre c
+// (itself on the grid).
+__device__ __forceinline__ Pos image_vector(const FrameDev& F, int m, float grid) {
+  Pos v;
+  v.h = make_float3(on_grid(F.img_h[m][0], grid), on_grid(F.img_h[m][1], grid), on_grid(F.img_h[m][2], grid));
+  v.l = make_float3(__fadd_rn(__fsub_rn(F.img_h[m][0], v.h.x), F.img_l[m][0]),
+                    __fadd_rn(__fsub_rn(F.img_h[m][1], v.h.y), F.img_l[m][1]),
+                    __fadd_rn(__fsub_rn(F.img_h[m][2], v.h.z), F.img_l[m][2]));
+  return v;
+}
+__device__ __forceinline__ Pos image_origin(const FrameDev& F, int m, float3 c, float grid) {
+  Pos o = image_vector(F, m, grid);
+  o.h = make_float3(__fsub_rn(o.h.x, c.x), __fsub_rn(o.h.y, c.y), __fsub_rn(o.h.z, c.z));
+  return o;
+}
+
+// A listed image: (y, W - |y|^2).  With W added, q' = q - W takes the place of q:
+// the sign of e' = n^2 - q' decides as that of n^2 - q does outside the window,
+// and every pair inside it (0 <= e' <= 2 W) is counted one below the edge n.
+__device__ __forceinline__ float4 j_image(const Pos& p, const Pos& o, float c1, float c0) {
+  const DF x = renorm(__fadd_rn(p.h.x, o.h.x), __fadd_rn(p.l.x, o.l.x)),
+           y = renorm(__fadd_rn(p.h.y, o.h.y), __fadd_rn(p.l.y, o.l.y)),
+           z = renorm(__fadd_rn(p.h.z, o.h.z), __fadd_rn(p.l.z, o.l.z));
+  float b;
+  return make_float4(x.h, y.h, z.h, -norm2_less(x, y, z, c1, c0, b));
+}
+
+// ------------------------------------------------------------------ re-decision
+
+// The definition's bin of one pair, counted only when its nearest image is the
+// listed one (displacement d): nbins when it is another.  For the frames whose
+// images are not listed (any), whatever the image.
+template <int V>
+__device__ __forceinline__ int exact_listed(const FrameDev& F, int i, int j, float3 d, bool any) {
+  const double3 pi = coords64(F, i), pj = coords64(F, j);
+  if (V != V_NONE && !any) {
+    const double3 e = exact_image<V>(F, pi, pj);
+    if (!(fabsf((float)e.x * F.S - d.x) < 0.5f * F.period[0] && fabsf((float)e.y * F.S - d.y) < 0.5f * F.period[1] &&
+          fabsf((float)e.z * F.S - d.z) < 0.5f * F.period[2]))
+      return F.nbins;
+  }
+  return bin_from_thresholds(F.T, F.S, F.nbins, exact_r2<V>(F, pi, pj));
+}
+__device__ __noinline__ int exact_listed_bin(const FrameDev& F, int i, int j, float3 d, bool any) {
+  return F.variant == V_NONE    ? exact_listed<V_NONE>(F, i, j, d, any)
+         : F.variant == V_ORTHO ? exact_listed<V_ORTHO>(F, i, j, d, any)
+                                : exact_listed<V_TRIC>(F, i, j, d, any);
+}
+
+// Bin of a re-decided pair from q in double-float arithmetic (about 44 bits) for
+// the listed image m, and the integer n nearest to its root.  The image must be
+// the definition's nearest one: the displacement strictly inside half the periods
+// c_z, b_y, a_x (Babai's step; see exact_r2).  Otherwise, and when q is too close
+// to n^2, the binary64 replay decides.
+__device__ __forceinline__ int listed_bin(const FrameDev& F, int i, int j, int m, float& n, unsigned& nexact) {
+  const Pos a = unpack(__ldg(F.P4 + i), __ldg(F.P2 + i)), b = unpack(__ldg(F.P4 + j), __ldg(F.P2 + j));
+  const float ah[3] = {a.h.x, a.h.y, a.h.z}, al[3] = {a.l.x, a.l.y, a.l.z};
+  const float bh[3] = {b.h.x, b.h.y, b.h.z}, bl[3] = {b.l.x, b.l.y, b.l.z};
+  const Pos v = image_vector(F, m, F.list_grid);
+  const float vh[3] = {v.h.x, v.h.y, v.h.z}, vl[3] = {v.l.x, v.l.y, v.l.z};
+  DF d[3];
+  bool inside = true;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    d[c] = two_sum(__fadd_rn(__fsub_rn(bh[c], ah[c]), vh[c]), __fadd_rn(vl[c], __fsub_rn(bl[c], al[c])));
+    // (orthorhombic: and not where binary64 may round the other way)
+    const float half = 0.5f * F.period[c], w = fabsf(d[c].h);
+    inside = inside && (F.variant == V_NONE || (w < half * (1.0f - 0x1p-18f) && half - w > F.list_tie));
+  }
+  const DF q = df_norm2(d[0], d[1], d[2]);
+  const float s = sqrt_approx(q.h);
+  n = nint_f(s);
+  if (inside) {
+    const DF n2 = two_prod(n, n);
+    const float diff = __fadd_rn(__fsub_rn(q.h, n2.h), __fsub_rn(q.l, n2.l));
+    // 2^-38: the double-float arithmetic and the binary64 rounding of the definition
+    if (fabsf(diff) > __fmaf_rn(0x1p-38f, q.h, F.list_mid * s) + 0x1p-60f || n < 0.5f)
+      return (int)fminf(n, (float)F.nbins + 1.0f) - (diff < 0.0f && n >= 0.5f ? 1 : 0);
+  }
+  ++nexact;
+  return exact_listed_bin(F, i, j, make_float3(d[0].h, d[1].h, d[2].h), false);
+}
+
+// The word in which the pair loop counted a pair close to its run (q' below
+// (2 W + 1)^2 or nearly): the scalar replay of its float32 arithmetic.
+__device__ __noinline__ int replay_rel(const SegState& G, int i, int j, int m) {
+  const FrameDev& F = *G.F;
+  const RunState R = run_state(G, __ldg(G.bi + 2 * (i / kRun)), __ldg(G.bi + 2 * (i / kRun) + 1));
+  const float4 x = i_factors(unpack(__ldg(G.P4i + i), __ldg(G.P2i + i)), R.c);
+  const float4 y = j_image(unpack(__ldg(G.P4j + j), __ldg(G.P2j + j)), image_origin(F, m, R.c, G.grid), R.c1, R.c0);
+  const float nq = __fadd_rn(__fmaf_rn(y.x, x.x, __fmaf_rn(y.y, x.y, __fmaf_rn(y.z, x.z, x.w))), y.w);
+  const int lane = i & 31;
+  float sc = fminf(sqrt_approx(-nq), (float)(G.hi + 1 + lane));
+  if (G.lo > 0) sc = fmaxf(sc, (float)(G.lo - lane));
+  const float sm = __fadd_rn(sc, kMagicRound);
+  const float n = __fadd_rn(sm, -kMagicRound);
+  const float e = __fmaf_rn(n, n, nq);
+  return __float_as_int(sm) + (int)(__float_as_uint(e) >> 31) - (__float_as_int(kMagicRound) + G.lo + 1);
+}
+
+// Decide the first min(32, qcount) queued pairs (reference, i particle), one per
+// lane, and shift the rest of the queue down.  A pair was counted one below its
+// edge n and moves up when it belongs there; close to the run, where the window
+// may hold several edges, the word it was counted in is found by replay.
+constexpr uint32_t kNearPair = 0x80000000u;
+__device__ __noinline__ int list_drain(const SegState& G, WarpList& W, int qcount, uint32_t* sh, int lane) {
+  const FrameDev& F = *G.F;
+  uint2* const q = W.queue;
+  const int count = qcount < 32 ? qcount : 32;
+  unsigned nexact = 0;
+  __syncwarp();
+  if (lane < count) {
+    const uint2 e = q[lane];
+    const int width = G.hi - G.lo, m = (int)(e.x >> kImgShift);
+    const int i = (int)(e.y & ~kNearPair), j = (int)(e.x & ((1u << kImgShift) - 1u));
+    float n;
+    const int bin = listed_bin(F, G.i0 + i, G.j0 + j, m, n, nexact) - G.lo;
+    int prov = (int)n - 1 - G.lo;
+    if (e.y & kNearPair) prov = replay_rel(G, i, j, m);
+    if (bin != prov) {
+      if ((uint32_t)bin < (uint32_t)width) atomicAdd(sh + bin, 1u);
+      if ((uint32_t)prov < (uint32_t)width) atomicAdd(sh + prov, 0xFFFFFFFFu);
+    }
+  }
+  __syncwarp();
+  const int rest = qcount - count;
+  const uint2 keep = lane < rest ? q[32 + lane] : make_uint2(0u, 0u);
+  __syncwarp();
+  if (lane < rest) q[lane] = keep;
+  __syncwarp();
+  for (int o = 16; o > 0; o >>= 1) nexact += __shfl_xor_sync(kFull, nexact, o);
+  if (lane == 0) {
+    atomicAdd(&G.F->deferred, (unsigned long long)count);
+    if (nexact) atomicAdd(&G.F->exact, (unsigned long long)nexact);
+  }
+  return rest;
+}
+
+// ------------------------------------------------------------------ the pair loop
+
+// This lane's four i particles, broadcast to both halves of a float32x2.
+struct IRegs {
+  float2 x[4], y[4], z[4], w[4];
+};
+struct IPos {
+  float4 a[4];
+  float2 b[4];
+};
+__device__ __forceinline__ void fetch_run(const SegState& G, int i_begin, int ni, int lane, IPos& p) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int i = i_begin + min(lane + 32 * r, ni - 1);
+    p.a[r] = __ldg(G.P4i + i);
+    p.b[r] = __ldg(G.P2i + i);
+  }
+}
+__device__ __forceinline__ void load_run(const IPos& p, float3 c, int ni, int lane, IRegs& I) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    float4 x = i_factors(unpack(p.a[r], p.b[r]), c);
+    if (lane + 32 * r >= ni) x = make_float4(NAN, NAN, NAN, NAN);
+    I.x[r] = bc2(x.x);
+    I.y[r] = bc2(x.y);
+    I.z[r] = bc2(x.z);
+    I.w[r] = bc2(x.w);
+  }
+}
+
+// Count one pair: the word of bin n - 1 + signbit(e') of the sweep at byte
+// address 4 v + hbase (v = bits(sm) + signbit), and the mask bit of a pair inside
+// the window: 0 <= e' < w2 as unsigned bits (negative e' compare above, and NaN,
+// e' or both, is not below).  NEAR: and of a pair with -nq < qm.
+template <bool NEAR>
+__device__ __forceinline__ void count_listed(float sm, float e, float nq, uint32_t w2, float nqm, uint32_t hbase,
+                                             uint32_t bit, uint32_t& dmask) {
+  if (NEAR)
+    asm volatile(
+        "{\n\t.reg .pred p, n;\n\t.reg .u32 sg, v, addr;\n\t"
+        "shr.u32 sg, %2, 31;\n\t"
+        "add.u32 v, %1, sg;\n\t"
+        "mad.lo.u32 addr, v, 4, %4;\n\t"
+        "setp.gt.f32 n, %6, %7;\n\t"
+        "setp.lt.or.u32 p, %2, %3, n;\n\t"
+        "@p or.b32 %0, %0, %5;\n\t"
+        "red.shared.add.u32 [addr], 1;\n\t"
+        "}"
+        : "+r"(dmask)
+        : "r"(__float_as_uint(sm)), "r"(__float_as_uint(e)), "r"(w2), "r"(hbase), "r"(bit), "f"(nq), "f"(nqm));
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .u32 sg, v, addr;\n\t"
+        "shr.u32 sg, %2, 31;\n\t"
+        "add.u32 v, %1, sg;\n\t"
+        "mad.lo.u32 addr, v, 4, %4;\n\t"
+        "setp.lt.u32 p, %2, %3;\n\t"
+        "@p or.b32 %0, %0, %5;\n\t"
+        "red.shared.add.u32 [addr], 1;\n\t"
+        "}"
+        : "+r"(dmask)
+        : "r"(__float_as_uint(sm)), "r"(__float_as_uint(e)), "r"(w2), "r"(hbase), "r"(bit));
+}
+
+// Queue the pairs whose mask bits are set (groups: this lane's groups with any;
+// first: the run's first particle and flag):
+// one per lane per turn, each lane from its own first group, so that a block
+// takes two or three turns.
+__device__ __forceinline__ int push_pairs(const SegState& G, WarpList& W, int s0, uint32_t groups, uint32_t first,
+                                          uint32_t* sh, int lane, int qcount) {
+  unsigned bal = __ballot_sync(kFull, groups != 0u);
+  while (bal) {
+    if (groups) {
+      const int g = __ffs(groups) - 1;
+      const uint32_t m = W.mask[g][lane];
+      const int b = __ffs(m) - 1;
+      W.mask[g][lane] = m & (m - 1u);
+      if ((m & (m - 1u)) == 0u) groups &= groups - 1u;
+      W.queue[qcount + __popc(bal & ((1u << lane) - 1u))] =
+          make_uint2(W.ref[s0 + 8 * g + (b >> 2)], first + (uint32_t)(lane + 32 * (b & 3)));
+    }
+    qcount += __popc(bal);
+    if (qcount >= 32) qcount = list_drain(G, W, qcount, sh, lane);
+    bal = __ballot_sync(kFull, groups != 0u);
+  }
+  return qcount;
+}
+
+// Listed images [s0, s0 + n) (multiples of 8, within the ring) against the run of
+// i particles from i_begin.  The root is clamped to the sweep, so that pairs
+// outside it land in guard words, spread over the lanes, and outside the window;
+// NaN (padding) becomes the upper clamp.  INNER: a whole block (no padding) of
+// images all of whose pairs lie in the sweep, no clamp needed.  NEAR: images so near the run that q' may
+// be below qm = (2 W + 1)^2, where the window can hold several edges: those pairs
+// are re-decided too; and with above >= 0, only particles j > above + i (the
+// diagonal item of one species; else above = -2^30).
+enum BlockMode { PLAIN, INNER, NEARBY };
+template <BlockMode MODE, bool MULTI>
+__device__ __forceinline__ int list_block(const SegState& G, const IRegs& I, WarpList& W, int i_begin, int s0, int n,
+                                          float qm, int above, uint32_t* sh, int lane, int qcount) {
+  constexpr bool NEAR = MODE == NEARBY;
+  const int lo = G.lo, hi = G.hi;
+  const uint32_t hbase =
+      (uint32_t)__cvta_generic_to_shared(sh) - 4u * (uint32_t)(__float_as_int(kMagicRound) + lo + 1);
+  const float chi = (float)(hi + 1 + lane), clo = (float)(lo - lane);
+  const float2 M = bc2(kMagicRound), NM = bc2(-kMagicRound);
+  // 2 W from W - A, rounded up: 2 (c1 A + c0) <= w1 (A - W) + w0
+  const float2 w1 = bc2(-2.0f * W.R.c1 * (1.0f + 0x1p-10f)), w0 = bc2(2.0f * W.R.c0 * (1.0f + 0x1p-10f));
+  uint32_t groups = 0u;
+#pragma unroll 1
+  for (int g = 0; g < n; g += 8) {
+    const int sg = s0 + g;
+    uint32_t dmask = 0u;
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      const float4 A = W.A[(sg + u) >> 1], Bv = W.B[(sg + u) >> 1];
+      const float2 yx = make_float2(A.x, A.y), yy = make_float2(A.z, A.w), yz = make_float2(Bv.x, Bv.y),
+                   na = make_float2(Bv.z, Bv.w);
+      const float2 w2 = fma2(na, w1, w0);
+      int ja = 0, jb = 0;
+      if (NEAR) {
+        ja = (int)(W.ref[sg + u] & ((1u << kImgShift) - 1u)) - above - lane;
+        jb = (int)(W.ref[sg + u + 1] & ((1u << kImgShift) - 1u)) - above - lane;
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        float2 nq = add2(fma2(yx, I.x[r], fma2(yy, I.y[r], fma2(yz, I.z[r], I.w[r]))), na);
+        if (NEAR) {
+          if (ja <= 32 * r) nq.x = NAN;
+          if (jb <= 32 * r) nq.y = NAN;
+        }
+        float2 sc = make_float2(sqrt_approx(-nq.x), sqrt_approx(-nq.y));
+        if (MODE != INNER) {
+          sc = make_float2(fminf(sc.x, chi), fminf(sc.y, chi));
+          if (MULTI) sc = make_float2(fmaxf(sc.x, clo), fmaxf(sc.y, clo));
+        }
+        const float2 sm = add2(sc, M);
+        const float2 nn = add2(sm, NM);
+        const float2 e = fma2(nn, nn, nq);
+        count_listed<NEAR>(sm.x, e.x, nq.x, __float_as_uint(w2.x), -qm, hbase, 1u << (u * 4 + r), dmask);
+        count_listed<NEAR>(sm.y, e.y, nq.y, __float_as_uint(w2.y), -qm, hbase, 1u << ((u + 1) * 4 + r), dmask);
+      }
+    }
+    W.mask[g >> 3][lane] = dmask;
+    if (dmask) groups |= 1u << (g >> 3);
+  }
+  return push_pairs(G, W, s0, groups, (uint32_t)i_begin | (NEAR ? kNearPair : 0u), sh, lane, qcount);
+}
+
+// The near form out of line (it loads the run again).
+template <bool MULTI>
+__device__ __noinline__ int list_near(const SegState& G, WarpList& W, int i_begin, int ni, int s0, int n, float qm,
+                                      int above, uint32_t* sh, int lane, int qcount) {
+  IPos p;
+  fetch_run(G, i_begin, ni, lane, p);
+  IRegs I;
+  load_run(p, W.R.c, ni, lane, I);
+  return list_block<NEARBY, MULTI>(G, I, W, i_begin, s0, n, qm, above, sh, lane, qcount);
+}
+
+// Every pair of an item in binary64 (frames whose images cannot be listed).
+__device__ __noinline__ void slow_item(const SegState& G, int ib, int ni, int jbeg, int jend, uint32_t* sh, int lane) {
+  FrameDev* const Fp = G.F;
+  const int nj = jend - jbeg;
+  unsigned long long np = 0;
+  for (int p = lane; p < ni * nj; p += 32) {
+    const int i = ib + p % ni, j = jbeg + p / ni;
+    if (G.intra && j <= i) continue;
+    const int rel = exact_listed_bin(*Fp, G.i0 + i, G.j0 + j, make_float3(0.f, 0.f, 0.f), true) - G.lo;
+    if ((uint32_t)rel < (uint32_t)(G.hi - G.lo)) atomicAdd(sh + rel, 1u);
+    ++np;
+  }
+  for (int o = 16; o > 0; o >>= 1) np += __shfl_xor_sync(kFull, np, o);
+  if (lane == 0 && np) {
+    atomicAdd(&Fp->deferred, np);
+    atomicAdd(&Fp->exact, np);
+  }
+}
+
+// Adds one word's count to the global histogram.  Counts are signed: a
+// provisional count may be moved after the words were flushed.
+__device__ __forceinline__ void merge_count(uint64_t* dst, uint32_t v) {
+  if (v) atomicAdd((unsigned long long*)dst, (unsigned long long)(long long)(int32_t)v);
+}
+
+// One thread fills the block's segment state.
+__device__ void enter_segment(const ListSegment& S, SegCounter* ctr, long long n_items, SegState& G) {
+  FrameDev* const Fp = S.fd;
+  const FrameDev& F = *Fp;
+  G.F = Fp;
+  G.P4i = F.P4 + S.i0;
+  G.P4j = F.P4 + S.j0;
+  G.P2i = F.P2 + S.i0;
+  G.P2j = F.P2 + S.j0;
+  G.bi = F.bnd + 2 * S.i_run0;
+  G.bj = F.bnd + 2 * S.j_run0;
+  G.i0 = S.i0;
+  G.j0 = S.j0;
+  G.ni = S.ni;
+  G.nj = S.nj;
+  G.n_ti = S.n_ti;
+  G.n_tj = S.n_tj;
+  G.intra = S.intra;
+  G.lo = S.pass * F.sweep_width;
+  G.hi = min(F.nbins, G.lo + F.sweep_width);
+  // widened (or narrowed) by 2^-15 and the absolute slack for the float32
+  // roundings of the bounds and the binary64 rounding of the bin
+  const float up = 1.0f + 0x1p-15f, down = 1.0f - 0x1p-15f;
+  const float r_hi = (float)G.hi * up + F.cull_abs, r_lo = fmaxf((float)G.lo * down - F.cull_abs, 0.0f);
+  const float n_hi = fmaxf((float)G.hi * down - F.cull_abs, 0.0f), n_lo = G.lo > 0 ? (float)G.lo * up + F.cull_abs : 0.0f;
+  G.rc_hi2 = r_hi * r_hi;
+  G.rc_lo2 = r_lo * r_lo;
+  G.in_hi2 = n_hi * n_hi;
+  G.in_lo2 = n_lo * n_lo;
+  G.grid = F.list_grid;
+  G.c0 = F.list_c0;
+  G.abs = F.cull_abs;
+  G.n_img = F.variant == V_NONE ? 1 : 27;
+  G.all = F.list_all;
+  G.slow = F.list_slow;
+  // elsewhere the two loops would take turns in the instruction cache, at a loss
+  G.inner = F.in_range;
+  G.items = (G.lo < F.nbins && !F.bad) ? S.items : 0;
+  G.item_base = S.item_base;
+  G.next = &ctr->next;
+  G.claimers = kClaims * (kListBlock / 32) * (long long)gridDim.x;
+}
+
+// Item -> (i run, j run, part).  Row a of a species with itself starts at item
+// a n - a (a - 1) / 2; the row is found from the root of that (the discriminant
+// is exact, its float32 root within a row of the truth).
+__device__ __forceinline__ void item_of(const SegState& G, int split, long long u, int& ri, int& rj, int& sub) {
+  const long long v = u + G.item_base, lid = v / split;
+  sub = (int)(v - lid * split);
+  if (G.intra) {
+    const long long n = G.n_tj, t = 2 * n + 1;
+    int a = (int)(0.5f * ((float)t - sqrtf((float)max(t * t - 8 * lid, 0LL))));
+    a = min(max(a, 0), G.n_ti - 1);
+    while (a > 0 && a * n - (long long)a * (a - 1) / 2 > lid) --a;
+    while (a + 1 < G.n_ti && (a + 1) * n - (long long)(a + 1) * a / 2 <= lid) ++a;
+    ri = a;
+    rj = a + (int)(lid - (a * n - (long long)a * (a - 1) / 2));
+  } else {
+    ri = (int)(lid / G.n_tj);
+    rj = (int)(lid - (long long)ri * G.n_tj);
+  }
+}
+
+// One block of 16 warps with 128 registers per SM: the pair loop and the list
+// state stay in registers, and the SM merges one histogram per segment.
+template <bool MULTI>
+__global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int BLOCK = kListBlock, kWarps = BLOCK / 32;
+  WarpList* lists = reinterpret_cast<WarpList*>(smem);
+  uint32_t* sh = reinterpret_cast<uint32_t*>(smem + sizeof(WarpList) * kWarps) + kGuard;
+  __shared__ int s_seg, s_len;
+  __shared__ unsigned s_since;
+  __shared__ unsigned long long s_best;
+  __shared__ long long s_base, s_first, s_seen;  // first claim, items known to be claimed
+  __shared__ SegState G;
+
+  const int tid = threadIdx.x, warp = tid >> 5;
+  int lane;  // opaque: kept in a register instead of read again from the special register
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  WarpList& W = lists[warp];
+  const unsigned lt_mask = (1u << lane) - 1u;
+  if (tid == 0) {
+    // blocks start spread over the launch's items
+    const long long pos = (long long)((double)L.n_items * ((double)blockIdx.x / (double)gridDim.x));
+    int lo = 0, hi = L.n_segs - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (L.segs[mid].item0 <= pos) lo = mid; else hi = mid - 1;
+    }
+    s_seg = lo;
+  }
+  for (int k = tid; k < L.hist_width + 2 * kGuard; k += BLOCK) sh[k - kGuard] = 0u;
+  __syncthreads();
+
+  for (;;) {
+    const int seg = s_seg;
+    if (seg < 0) break;
+    if (tid == 0) {
+      atomicAdd(&L.ctr[seg].attached, 1);
+      enter_segment(L.segs[seg], L.ctr + seg, L.n_items, G);
+      // the block's first claim, for all its warps; claims shrink with the items
+      // left (a quarter of an even share of them), at first at most the block's
+      // share of the launch
+      const long long part = max(1LL, min(G.items / G.claimers, 1024LL));
+      const long long share = max(1LL, (L.n_items + gridDim.x - 1) / (long long)gridDim.x);
+      const long long want = min(part * kWarps, share);
+      s_len = (int)part;
+      s_first = want;
+      s_base = G.items ? (long long)atomicAdd(G.next, (unsigned long long)want) : 0LL;
+      s_seen = s_base + want;
+      s_since = 0u;
+    }
+    __syncthreads();
+    const FrameDev& F = *G.F;
+    int qcount = 0;
+    if (lane == 0) W.uni = W.axis = W.cull = 0ull;
+    long long u = s_base + (long long)warp * s_len;
+    int len = (int)min((long long)s_len, min(s_first - (long long)warp * s_len, G.items - u));
+
+    for (;;) {
+      if (len <= 0) {
+        if (lane == 0) {
+          const long long part = (G.items - *(volatile long long*)&s_seen) / G.claimers;
+          len = (int)max(1LL, min(part, 1024LL));
+          u = G.items ? (long long)atomicAdd(G.next, (unsigned long long)len) : 0LL;
+          *(volatile long long*)&s_seen = u + len;
+          len = (int)min((long long)len, G.items - u);
+        }
+        len = __shfl_sync(kFull, len, 0);
+        u = __shfl_sync(kFull, u, 0);
+        if (len <= 0) break;
+      }
+
+      unsigned listed = 0;
+      int ri, rj, sub;
+      item_of(G, L.split, u, ri, rj, sub);
+
+      while (len > 0) {
+        const int row = min(len, (G.n_tj - rj) * L.split - sub);
+        len -= row;
+        // ---- the run: state and factors
+        const int i_begin = ri * kRun, ni = min(kRun, G.ni - i_begin), nj = G.nj;
+        const int part = kRun / L.split;
+        IRegs I;
+        int pf = rj * kRun + sub * part;
+        float4 pa = __ldg(G.P4j + min(pf + lane, nj - 1));
+        float2 pb = __ldg(G.P2j + min(pf + lane, nj - 1));
+        {
+          IPos p;
+          fetch_run(G, i_begin, ni, lane, p);
+          const RunState R = run_state(G, __ldg(G.bi + 2 * ri), __ldg(G.bi + 2 * ri + 1));
+          __syncwarp();
+          if (lane == 0) W.R = R;
+          __syncwarp();
+          load_run(p, R.c, ni, lane, I);
+        }
+        int tail = 0, done = 0;
+        // the list's images: none near the run, every pair in the sweep
+        bool near = G.all != 0, inner = true;
+        if (lane == 0) W.qm = 0.0f;
+        for (int t = 0; t < row; ++t) {
+          const bool diag = G.intra && rj == ri;
+          const int jbeg = rj * kRun + sub * part;
+          const int jend = min(nj, jbeg + part);
+          if (G.slow) {
+            if (jbeg < jend) slow_item(G, i_begin, ni, jbeg, jend, sh, lane);
+            listed += kRun;
+          } else {
+            // ---- images of the j run that can lie in the sweep (bounds against bounds)
+            bool keep = false;
+            float g2 = 0.0f, f2 = 0.0f;
+            if (lane < G.n_img && jbeg < jend) {
+              const float4 jlo = __ldg(G.bj + 2 * rj), jhi = __ldg(G.bj + 2 * rj + 1);
+              const int m = G.n_img == 1 ? kHome : lane;
+              const float sx = F.img_h[m][0], sy = F.img_h[m][1], sz = F.img_h[m][2];
+              // ranges of the j run's image around the centre, then out by the half extents
+              const float3 c = W.R.c, h = W.R.h;
+              const float lx = jlo.x + sx - c.x, ux = jhi.x + sx - c.x;
+              const float ly = jlo.y + sy - c.y, uy = jhi.y + sy - c.y;
+              const float lz = jlo.z + sz - c.z, uz = jhi.z + sz - c.z;
+              const float gx = fmaxf(fmaxf(lx, -ux) - h.x, 0.0f), gy = fmaxf(fmaxf(ly, -uy) - h.y, 0.0f),
+                          gz = fmaxf(fmaxf(lz, -uz) - h.z, 0.0f);
+              const float fx = fmaxf(fabsf(lx), fabsf(ux)) + h.x, fy = fmaxf(fabsf(ly), fabsf(uy)) + h.y,
+                          fz = fmaxf(fabsf(lz), fabsf(uz)) + h.z;
+              g2 = gx * gx + gy * gy + gz * gz;
+              f2 = fx * fx + fy * fy + fz * fz;
+              keep = g2 <= G.rc_hi2 && f2 >= G.rc_lo2;
+            }
+            unsigned mask = __ballot_sync(kFull, keep);
+            if (lane == 0) {  // statistics
+              const unsigned long long np = (unsigned long long)max(jend - jbeg, 0) * (unsigned long long)ni;
+              const int nimg = __popc(mask);
+              if (nimg == 0) W.cull += np;
+              if (nimg == 1) W.uni += np;
+              if (nimg == 2) {
+                const int a = __ffs(mask) - 1, b = 31 - __clz(mask);
+                if ((a / 9 != b / 9) + (a / 3 % 3 != b / 3 % 3) + (a % 3 != b % 3) == 1) W.axis += np;
+              }
+            }
+            // one round of 32 j particles of one image per turn; a last turn ends the
+            // list with the row and with the diagonal item
+            const bool ends = t == row - 1 || diag;
+            int m = kHome, jb = jend;
+            bool close = false, in_here = false;
+            for (;;) {
+              int want = kBlk;
+              if (jb >= jend && mask) {
+                const int ml = __ffs(mask) - 1;
+                mask &= mask - 1u;
+                m = G.n_img == 1 ? kHome : ml;
+                // near: some q' may lie below (2 W + 1)^2, W at the farthest corner;
+                // inner: every pair in the sweep
+                const float f2m = __shfl_sync(kFull, f2, ml), g2m = __shfl_sync(kFull, g2, ml);
+                const float wm = 2.0f * __fmaf_rn(W.R.c1, f2m, W.R.c0) + 1.0f;
+                close = sqrtf(g2m) - G.abs < wm + 2.0f || G.all;
+                in_here = f2m <= G.in_hi2 && g2m >= G.in_lo2;
+                near = near || close;
+                inner = inner && in_here;
+                const Pos o = image_origin(F, m, W.R.c, G.grid);
+                __syncwarp();
+                if (lane == 0) {
+                  W.o = o;
+                  W.qm_here = close ? (G.all ? INFINITY : wm * wm) : 0.0f;
+                  W.qm = fmaxf(W.qm, W.qm_here);
+                }
+                __syncwarp();
+                jb = jbeg;
+              }
+              const bool more = jb < jend;
+              if (more) {
+                const int jl = jb + lane;
+                // this round's particle was loaded in the round before (the next
+                // round, image or run is the likely successor); else load it now
+                if (pf != jb) {
+                  pa = __ldg(G.P4j + min(jl, nj - 1));
+                  pb = __ldg(G.P2j + min(jl, nj - 1));
+                }
+                const Pos p = unpack(pa, pb);
+                jb += 32;
+                pf = jb < jend ? jb : (mask ? jbeg : jend);
+                pa = __ldg(G.P4j + min(pf + lane, nj - 1));
+                pb = __ldg(G.P2j + min(pf + lane, nj - 1));
+                const float4 y = j_image(p, W.o, W.R.c1, W.R.c0);
+                const float3 h = W.R.h;
+                const float ax = fabsf(y.x), ay = fabsf(y.y), az = fabsf(y.z);
+                const float gx = fmaxf(ax - h.x, 0.0f), gy = fmaxf(ay - h.y, 0.0f), gz = fmaxf(az - h.z, 0.0f);
+                bool in = jl < jend && gx * gx + gy * gy + gz * gz <= G.rc_hi2;
+                if (MULTI) {
+                  const float fx = ax + h.x, fy = ay + h.y, fz = az + h.z;
+                  in = in && fx * fx + fy * fy + fz * fz >= G.rc_lo2;
+                }
+                const unsigned bal = __ballot_sync(kFull, in);
+                if (in) {
+                  const int s = (tail + __popc(bal & lt_mask)) & (kCap - 1);
+                  float* a = reinterpret_cast<float*>(&W.A[s >> 1]) + (s & 1);
+                  float* b = reinterpret_cast<float*>(&W.B[s >> 1]) + (s & 1);
+                  a[0] = y.x;
+                  a[2] = y.y;
+                  b[0] = y.z;
+                  b[2] = y.w;
+                  W.ref[s] = (uint32_t)jl | ((uint32_t)m << kImgShift);
+                }
+                tail += __popc(bal);
+              } else {
+                if (!ends) break;
+                want = (tail - done + 7) & ~7;  // fewer than a block: padded to whole groups
+                if (want == 0) break;
+                if (lane < done + want - tail) {
+                  const int s = (tail + lane) & (kCap - 1);
+                  reinterpret_cast<float*>(&W.B[s >> 1])[2 + (s & 1)] = NAN;
+                  W.ref[s] = 0u;
+                }
+              }
+              __syncwarp();
+              if (!more || tail - done >= kBlk) {
+                if (near || diag)
+                  qcount = list_near<MULTI>(G, W, i_begin, ni, done & (kCap - 1), want, W.qm, diag ? i_begin : -(1 << 30),
+                                            sh, lane, qcount);
+                else if (inner && more && ni == kRun && G.inner)
+                  qcount = list_block<INNER, MULTI>(G, I, W, i_begin, done & (kCap - 1), kBlk, 0.0f, 0, sh, lane, qcount);
+                else
+                  qcount = list_block<PLAIN, MULTI>(G, I, W, i_begin, done & (kCap - 1), want, 0.0f, 0, sh, lane, qcount);
+                done += kBlk;
+                // what is left was appended in this round
+                near = (more && close) || G.all;
+                inner = !more || in_here;
+                if (lane == 0) W.qm = W.qm_here;
+                __syncwarp();
+              }
+              if (!more) {
+                listed += (unsigned)tail;
+                tail = done = 0;
+                break;
+              }
+            }
+          }
+          if (++sub == L.split) {
+            sub = 0;
+            ++rj;
+          }
+        }
+        if (rj == G.n_tj) {
+          ++ri;
+          rj = G.intra ? ri : 0;
+        }
+      }
+      // flush before a shared count can pass 2^31: the warp that crosses the
+      // mark moves every word (the others keep counting)
+      unsigned before = 0;
+      if (lane == 0) before = atomicAdd(&s_since, listed);
+      before = __shfl_sync(kFull, before, 0);
+      if (before < kFlushPairs && before + listed >= kFlushPairs) {
+        if (lane == 0) atomicSub(&s_since, kFlushPairs);
+        uint64_t* const dst = F.out + (size_t)L.segs[seg].h * F.nbins + G.lo;
+        for (int k = lane; k < G.hi - G.lo; k += 32) merge_count(dst + k, atomicExch(sh + k, 0u));
+      }
+    }
+    while (qcount > 0) qcount = list_drain(G, W, qcount, sh, lane);
+    if (lane == 0) {
+      if (W.uni) atomicAdd(&G.F->uniform_pairs, W.uni);
+      if (W.axis) atomicAdd(&G.F->axis_pairs, W.axis);
+      if (W.cull) atomicAdd(&G.F->culled_pairs, W.cull);
+    }
+
+    __syncthreads();
+    // ---- merge, then attach to the segment with the most work left per block
+    const int width = G.hi - G.lo;
+    if (G.items) {
+      uint64_t* const dst = F.out + (size_t)L.segs[seg].h * F.nbins + G.lo;
+      for (int k = tid; k < width; k += BLOCK) {
+        merge_count(dst + k, sh[k]);
+        sh[k] = 0u;
+      }
+      for (int k = tid; k < 2 * kGuard; k += BLOCK) sh[k < kGuard ? k - kGuard : width + k - kGuard] = 0u;
+    }
+    if (tid == 0) {
+      s_best = 0ull;
+      atomicAdd(&L.ctr[seg].attached, -1);
+      if (!G.items) L.ctr[seg].next = (unsigned long long)L.segs[seg].items;  // nothing to do for anyone
+    }
+    __syncthreads();
+    unsigned long long best = 0ull;
+    for (int k = tid; k < L.n_segs; k += BLOCK) {
+      const unsigned long long nx = *(volatile unsigned long long*)&L.ctr[k].next;
+      const unsigned long long it = (unsigned long long)L.segs[k].items;
+      if (nx >= it) continue;
+      const int att = *(volatile int32_t*)&L.ctr[k].attached;
+      unsigned long long score = (it - nx) * 16ull / (unsigned long long)(1 + max(att, 0));
+      score = min(max(score, 1ull), (1ull << 40) - 1ull);
+      best = max(best, (score << 24) | (unsigned long long)k);
+    }
+    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
+    if (lane == 0 && best) atomicMax(&s_best, best);
+    __syncthreads();
+    if (tid == 0) s_seg = s_best ? (int)(s_best & 0xFFFFFFull) : -1;
+    __syncthreads();
+  }
+}
+
+template <bool MULTI>
+cudaError_t launch_list_t(const ListLaunch& p, int grid, size_t smem, cudaStream_t stream) {
+  cudaError_t e = cudaFuncSetAttribute(list_kernel<MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  list_kernel<MULTI><<<grid, kListBlock, smem, stream>>>(p);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t list_kernel_smem(int hist_width) {
+  return sizeof(WarpList) * (size_t)(kListBlock / 32) + 4 * ((size_t)hist_width + 2 * kGuard);
+}
+
+// The device's shared memory per block, less the kernel's static part.
+int list_kernel_max_width() {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const size_t fixed = list_kernel_smem(0) + 1024;
+  return (size_t)optin <= fixed ? 0 : (int)(((size_t)optin - fixed) / 4) & ~3;
+}
+
+cudaError_t launch_list(const ListLaunch& p, int grid, cudaStream_t stream) {
+  (void)cudaGetLastError();
+  const size_t smem = list_kernel_smem(p.hist_width);
+  return p.multi ? launch_list_t<true>(p, grid, smem, stream) : launch_list_t<false>(p, grid, smem, stream);
+}
+
+}  // namespace dh

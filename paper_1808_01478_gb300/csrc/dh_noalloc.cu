@@ -94,7 +94,7 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   max_width = pair_kernel_max_width();
   if (max_width < 1024) return fail(DH_ERR_CUDA, "not enough shared memory per block");
   PlannedFrame pf;
-  dh_status s = check_frame(frame, pf, max_width);
+  dh_status s = check_frame(frame, pf, max_width, 0);
   if (s != DH_OK) return s;
   unsigned char* base = nullptr;
   s = scratch_for_current_device(&base);

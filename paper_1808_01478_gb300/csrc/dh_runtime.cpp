@@ -161,7 +161,7 @@ int pair_grid(int num_sms, int bps, int64_t n_items) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, n_items));
 }
 
-dh_status check_frame(const dh_frame* f, PlannedFrame& pf, int max_width) {
+dh_status check_frame(const dh_frame* f, PlannedFrame& pf, int max_width, int list_width) {
   if (!f) return fail(DH_ERR_INVALID, "frame is NULL");
   if (f->n < 0 || f->n > (int64_t)0x7FFFFFFF - 2 * kTile)
     return fail(DH_ERR_INVALID, "n = %lld out of range", (long long)f->n);
@@ -210,6 +210,14 @@ dh_status check_frame(const dh_frame* f, PlannedFrame& pf, int max_width) {
     default:
       return fail(DH_ERR_INVALID, "unknown box_type %d", f->box_type);
   }
+  // Two images of a particle are at least the smallest plane spacing apart, so
+  // with r_max up to half of it one image of a pair at most lies inside
+  // (orthorhombic: a tie of two images at exactly L/2 is re-decided, with room
+  // for the rounding of r_max = L/2).
+  pf.list = list_width > 0 && f->n <= kListMaxN &&
+            (pf.variant == V_NONE || pf.variant == V_TRIC ||
+             (pf.variant == V_ORTHO && f->r_max <= 0.5 * std::min(B[0], std::min(B[4], B[8])) * (1.0 + 0x1p-40)));
+  if (pf.list) max_width = std::min(max_width, list_width);
   int64_t S = f->n_species;
   pf.src = f;
   pf.n_hist = (int32_t)(S * (S + 1) / 2);
@@ -265,24 +273,54 @@ void fill_frame_dev(const PlannedFrame& pf, FrameDev& F, const float4* X, uint64
   for (int c = 0; c < 3; ++c) {
     F.cmin[c] = 0x7FFFFFFF;                // ordered encoding of +huge: min starts high
     F.cmax[c] = (int32_t)0x80000000;       // and max starts low
+    F.smin[c] = F.cmin[c];
+    F.smax[c] = F.cmax[c];
+  }
+  if (pf.variant == V_ORTHO || pf.variant == V_TRIC) {
+    // image vectors -B k, in bins as double-floats, and the rounding errors (the
+    // binary64 sum itself errs by at most 2^-52 of the row sum)
+    for (int c = 0; c < 3; ++c) F.period[c] = (float)(S * F.B[4 * c]);
+    const double* B = F.B;
+    const double row = std::max(B[0] + std::fabs(B[1]) + std::fabs(B[2]), std::max(B[4] + std::fabs(B[5]), B[8]));
+    for (int m = 0; m < 27; ++m) {
+      const double kx = m / 9 - 1, ky = (m / 3) % 3 - 1, kz = m % 3 - 1;
+      const double v[3] = {-((kx * B[0] + ky * B[1]) + kz * B[2]), -(ky * B[4] + kz * B[5]), -(kz * B[8])};
+      for (int c = 0; c < 3; ++c) {
+        F.tshift[m][c] = (float)v[c];
+        F.img_h[m][c] = (float)(S * v[c]);
+        F.img_l[m][c] = (float)(S * v[c] - (double)F.img_h[m][c]);
+        const double err = std::fabs((double)F.tshift[m][c] - v[c]) + row * 0x1p-51;
+        F.tserr[m][c] = (float)err;
+        if ((double)F.tserr[m][c] < err) F.tserr[m][c] = std::nextafterf(F.tserr[m][c], INFINITY);
+      }
+    }
   }
 }
 
 int sort_grid_bits(int64_t n) {
-  int g = (int)std::floor(std::log2(std::cbrt((double)n / 16.0)));
-  return std::min(6, std::max(1, g));
+  if (n <= kRun) return 0;  // one run: the order does not matter
+  const int g = (int)std::lround(std::log2(std::cbrt(0.5 * (double)n)));
+  return std::min(7, std::max(1, g));
+}
+
+int64_t frame_runs(const dh_frame* f) {
+  int64_t runs = 0;
+  for (int a = 0; a < f->n_species; ++a)
+    runs += (f->species_offsets[a + 1] - f->species_offsets[a] + kRun - 1) / kRun;
+  return runs;
 }
 
 std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, const FrameDev* fd, int64_t x0, int64_t key0,
-                                        int64_t* keys, int* chunks) {
+                                        int64_t* keys, int64_t* max_n) {
   std::vector<SortSeg> out;
   *keys = 0;
-  *chunks = 0;
+  *max_n = 0;
   if (pf.variant == V_TRIC_SEARCH) return out;
   const int64_t* o = pf.src->species_offsets;
+  int64_t runs = 0;
   for (int a = 0; a < pf.src->n_species; ++a) {
     const int64_t na = o[a + 1] - o[a];
-    if (na < kSortMinParticles) continue;
+    if (na == 0) continue;
     SortSeg g;
     std::memset(&g, 0, sizeof g);
     g.fd = fd;
@@ -290,8 +328,11 @@ std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, const FrameDev* 
     g.n = (int32_t)na;
     g.g = sort_grid_bits(na);
     g.key0 = key0 + *keys;
-    *keys += (int64_t)1 << (3 * g.g);
-    *chunks = std::max<int>(*chunks, (int)((na + kSortChunk - 1) / kSortChunk));
+    g.f0 = x0;
+    g.run0 = (int32_t)runs;
+    runs += (na + kRun - 1) / kRun;
+    *keys += std::max<int64_t>((int64_t)1 << (3 * g.g), 4);
+    *max_n = std::max<int64_t>(*max_n, na);
     out.push_back(g);
   }
   return out;
@@ -363,6 +404,54 @@ int64_t add_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, std::v
   return fill_segments(pf, fd, item0, jm, segs.data() + at, n, &n);
 }
 
+// One segment per species pair and sweep; the larger species is the i side (its
+// runs have the smaller bounds).  Items are numbered from item0.
+int64_t add_list_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, std::vector<ListSegment>& segs,
+                          int split) {
+  const dh_frame* f = pf.src;
+  const int64_t* o = f->species_offsets;
+  const int S = f->n_species;
+  std::vector<int32_t> run0((size_t)S + 1, 0);
+  for (int a = 0; a < S; ++a) run0[a + 1] = run0[a] + (int32_t)((o[a + 1] - o[a] + kRun - 1) / kRun);
+  int64_t items = 0;
+  for (int pass = 0; pass < pf.sweeps; ++pass) {
+    int h = 0;
+    for (int a = 0; a < S; ++a)
+      for (int b = a; b < S; ++b, ++h) {
+        const int64_t na = o[a + 1] - o[a], nb = o[b + 1] - o[b];
+        if (na == 0 || nb == 0 || (a == b && na < 2)) continue;
+        const int i = na >= nb ? a : b, j = na >= nb ? b : a;
+        ListSegment s;
+        std::memset(&s, 0, sizeof s);
+        s.fd = fd;
+        s.intra = a == b;
+        s.h = h;
+        s.pass = pass;
+        s.n_ti = run0[i + 1] - run0[i];
+        s.n_tj = run0[j + 1] - run0[j];
+        s.i0 = (int32_t)o[i];
+        s.ni = (int32_t)(o[i + 1] - o[i]);
+        s.j0 = (int32_t)o[j];
+        s.nj = (int32_t)(o[j + 1] - o[j]);
+        s.i_run0 = run0[i];
+        s.j_run0 = run0[j];
+        s.item0 = item0 + items;
+        s.items = split * (s.intra ? (int64_t)s.n_ti * (s.n_ti + 1) / 2 : (int64_t)s.n_ti * s.n_tj);
+        items += s.items;
+        segs.push_back(s);
+      }
+  }
+  return items;
+}
+
+int list_split_for(double run_pairs, int num_sms) {
+  const double warps = (double)num_sms * (kListBlock / 32);
+  if (run_pairs >= warps) return run_pairs < 8.0 * warps ? 2 : 1;
+  int split = 1;
+  while (split < 16 && run_pairs * 2 * split <= warps) split *= 2;
+  return split;
+}
+
 namespace {
 
 void release_held(dh_ctx* c) {
@@ -373,6 +462,7 @@ void release_held(dh_ctx* c) {
 // The frames of one minimum-image variant in a call, as the autotuner keys them.
 struct VariantSummary {
   int frames = 0, width = 1, multi = 0;
+  int list = 0;  // some frame can run on the list kernel
   double pairs = 0.0;
   TuneKey key() const { return make_tune_key(0, width, frames ? pairs / frames : 0.0, frames); }
 };
@@ -384,6 +474,7 @@ VariantSummary summarize(const std::vector<PlannedFrame>& pfs, int v) {
       ++s.frames;
       s.width = std::max(s.width, pf.sweep_width);
       s.multi |= pf.sweeps > 1;
+      s.list |= pf.list ? 1 : 0;
       s.pairs += (double)pf.pairs;
     }
   return s;
@@ -402,6 +493,7 @@ LaunchParams launch_params(dh_ctx* c, const VariantSummary& s, int v) {
   if (c->tune_forced) return c->tune_force;
   LaunchParams p;
   if (c->tuner.lookup(variant_key(s, v), &p)) return p;
+  p.list = s.list;
   p.block = default_block(v, s.width);
   return p;
 }
@@ -427,8 +519,13 @@ struct CallPlan {
   int max_pass = 1;
   int launched = 0;
   size_t seg_bytes = 0;          // Segment array in the metadata
-  int n_sort = 0;                // spatial-order segments (after the Segments in the metadata)
-  int sort_chunks = 0;           // most staging chunks of one of them
+  size_t lseg_bytes = 0;         // ListSegment array after it
+  int n_lsegs = 0;
+  int64_t litems = 0;            // list-kernel launch: items,
+  int lwidth = 1, lmulti = 0;    //   widest sweep, some sweep above bin 0,
+  int lgrid = 0, lsplit = 1;     //   blocks, items per run pair
+  int n_sort = 0;                // spatial-order segments (after the segments in the metadata)
+  int64_t sort_max = 0;          // largest of them
   int64_t sort_keys = 0;         // counters over all of them
   int64_t sort_particles = 0;    // particles of the frames (index space of keys and the scratch copy)
 };
@@ -455,42 +552,83 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   }
   DH_CUDA_TRY(c->X.ensure(sizeof(float4) * (size_t)std::max<int64_t>(xoff[k], 1)));
   if (P.any_f64) DH_CUDA_TRY(c->X64.ensure(sizeof(double4) * (size_t)std::max<int64_t>(xoff[k], 1)));
+  DH_CUDA_TRY(c->P4.ensure(sizeof(float4) * (size_t)std::max<int64_t>(xoff[k], 1)));
+  DH_CUDA_TRY(c->P2.ensure(sizeof(float2) * (size_t)std::max<int64_t>(xoff[k], 1)));
   if (host_coords) DH_CUDA_TRY(c->raw.ensure(std::max<size_t>(raw_bytes, 16)));
-  DH_CUDA_TRY(c->ctl.ensure(sizeof(Control) * kNumVariants));
-  // device metadata: FrameDev[k] | StageJob[k] | Segment[m], uploaded in one copy;
-  // segments are grouped by minimum-image variant (one pair-kernel launch each)
+  std::vector<int64_t> runs((size_t)k + 1, 0);
+  for (int f = 0; f < k; ++f) runs[f + 1] = runs[f] + frame_runs(pfs[f].src);
+  DH_CUDA_TRY(c->bnd.ensure(2 * sizeof(float4) * (size_t)std::max<int64_t>(runs[k], 1)));
+  // device metadata: FrameDev[k] | StageJob[k] | Segment[m] | ListSegment[l] |
+  // SortSeg[s], uploaded in one copy; segments are grouped by minimum-image
+  // variant (one pair-kernel launch each), those of the list kernel together
   std::vector<Segment> segs;
+  std::vector<ListSegment> lsegs;
   VariantSummary vsum[kNumVariants];
   for (int v = 0; v < kNumVariants; ++v) {
     vsum[v] = summarize(pfs, v);
     P.vparams[v] = launch_params(c, vsum[v], v);
   }
+  // frames the list kernel takes: those it can run, unless a measured shape says otherwise
+  auto on_list = [&](int f) { return pfs[f].list && P.vparams[pfs[f].variant].list; };
+  double lrun_pairs = 0.0;
+  for (int f = 0; f < k; ++f)
+    if (on_list(f)) {
+      P.lwidth = std::max(P.lwidth, pfs[f].sweep_width);
+      P.lmulti |= pfs[f].sweeps > 1;
+      lrun_pairs += (double)pfs[f].pairs / ((double)kRun * kRun) * pfs[f].sweeps;
+    }
+  P.lsplit = list_split_for(lrun_pairs, c->num_sms);
+  VariantSummary told[kNumVariants];  // what the tiled kernel is left with
+  for (int f = 0; f < k; ++f)
+    if (!on_list(f)) {
+      VariantSummary& t = told[pfs[f].variant];
+      t.width = std::max(t.width, pfs[f].sweep_width);
+      t.multi |= pfs[f].sweeps > 1;
+    }
+  for (int v = 0; v < kNumVariants; ++v)
+    if (P.vparams[v].list) {
+      P.vparams[v].block = default_block(v, told[v].width);
+      P.vparams[v].bps = 0;
+    }
   auto plan_segments = [&](FrameDev* dF) {
     segs.clear();
-    P.n_items = 0;
+    lsegs.clear();
+    P.litems = 0;
+    for (int f = 0; f < k; ++f)
+      if (on_list(f)) P.litems += add_list_segments(pfs[f], dF + f, P.litems, lsegs, P.lsplit);
+    if (c->tune_forced && c->tune_cap_pairs > 0.0) {  // a measurement: the first items only
+      int64_t left = (int64_t)std::ceil(c->tune_cap_pairs / ((double)kRun * kRun)) * P.lsplit;
+      P.litems = 0;
+      for (ListSegment& g : lsegs) {
+        g.items = std::min(g.items, left);
+        left -= g.items;
+        P.litems += g.items;
+      }
+    }
+    P.n_lsegs = (int)lsegs.size();
+    P.n_items = P.litems;
     for (int v = 0; v < kNumVariants; ++v) {
       P.vseg0[v] = segs.size();
       P.vitems[v] = 0;
       for (int f = 0; f < k; ++f)
-        if (pfs[f].variant == v)
+        if (pfs[f].variant == v && !on_list(f))
           P.vitems[v] += add_segments(pfs[f], dF + f, P.vitems[v], segs, P.vparams[v].jm);
       P.n_items += P.vitems[v];
     }
     P.vseg0[kNumVariants] = segs.size();
   };
-  // spatial order of the species of periodic frames without the 27-image search
+  // spatial order of the species
   std::vector<SortSeg> sorts;
   auto plan_sorts = [&](FrameDev* dF) {
     sorts.clear();
     P.sort_keys = 0;
-    P.sort_chunks = 0;
+    P.sort_max = 0;
     for (int f = 0; f < k; ++f) {
-      int64_t keys = 0;
-      int chunks = 0;
-      std::vector<SortSeg> fs = plan_spatial_order(pfs[f], dF + f, xoff[f], P.sort_keys, &keys, &chunks);
+      int64_t keys = 0, most = 0;
+      std::vector<SortSeg> fs = plan_spatial_order(pfs[f], dF + f, xoff[f], P.sort_keys, &keys, &most);
       sorts.insert(sorts.end(), fs.begin(), fs.end());
       P.sort_keys += keys;
-      P.sort_chunks = std::max(P.sort_chunks, chunks);
+      P.sort_max = std::max(P.sort_max, most);
     }
     P.n_sort = (int)sorts.size();
     P.sort_particles = xoff[k];
@@ -499,8 +637,10 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   plan_segments((FrameDev*)c->meta.p);
   plan_sorts((FrameDev*)c->meta.p);
   P.seg_bytes = sizeof(Segment) * std::max<size_t>(segs.size(), 1);
-  P.meta_bytes = sizeof(FrameDev) * (size_t)k + sizeof(StageJob) * (size_t)k + P.seg_bytes +
+  P.lseg_bytes = sizeof(ListSegment) * lsegs.size();
+  P.meta_bytes = sizeof(FrameDev) * (size_t)k + sizeof(StageJob) * (size_t)k + P.seg_bytes + P.lseg_bytes +
                  sizeof(SortSeg) * sorts.size();
+  DH_CUDA_TRY(c->ctl.ensure(sizeof(Control) * kNumVariants + sizeof(SegCounter) * lsegs.size()));
   void* before = c->meta.p;
   DH_CUDA_TRY(c->meta.ensure(P.meta_bytes));
   DH_CUDA_TRY(c->hmeta.ensure(P.meta_bytes));
@@ -512,7 +652,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     DH_CUDA_TRY(c->sortX.ensure(sizeof(float4) * (size_t)P.sort_particles));
     if (P.any_f64) DH_CUDA_TRY(c->sortX64.ensure(sizeof(double4) * (size_t)P.sort_particles));
     DH_CUDA_TRY(c->sortK.ensure(sizeof(int32_t) * (size_t)P.sort_particles));
-    DH_CUDA_TRY(c->sortC.ensure(sizeof(uint32_t) * (size_t)P.sort_keys));
+    DH_CUDA_TRY(c->sortC.ensure(2 * sizeof(uint32_t) * (size_t)P.sort_keys));
   }
   FrameDev* dF = (FrameDev*)c->meta.p;
   FrameDev* hF = (FrameDev*)c->hmeta.p;
@@ -525,6 +665,11 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     c->held_tables.push_back(T);
     fill_frame_dev(pfs[f], hF[f], (const float4*)c->X.p + xoff[f], dev_out[f], T);
     if (pfs[f].src->flags & DH_COORDS_F64) hF[f].X64 = (const double4*)c->X64.p + xoff[f];
+    if (on_list(f)) {
+      hF[f].P4 = (float4*)c->P4.p + xoff[f];
+      hF[f].P2 = (float2*)c->P2.p + xoff[f];
+      hF[f].bnd = (float4*)c->bnd.p + 2 * runs[f];
+    }
     P.max_pass = std::max(P.max_pass, pfs[f].sweeps);
   }
   // A1 staging jobs
@@ -537,22 +682,25 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     std::memset(&J, 0, sizeof J);
     J.stride = (fr->flags & DH_COORDS_F4) ? 4 : 3;
     J.src = host_coords ? (const float*)((const unsigned char*)c->raw.p + P.raw_off[f]) : fr->coords;
-    J.dst = (float4*)c->X.p + xoff[f];
-    J.dst64 = (fr->flags & DH_COORDS_F64) ? (double4*)c->X64.p + xoff[f] : nullptr;
+    // staged for the spatial order, or in place where there is none
+    const bool sorted = pfs[f].variant != V_TRIC_SEARCH;
+    J.dst = (float4*)(sorted ? c->sortX.p : c->X.p) + xoff[f];
+    J.dst64 = (fr->flags & DH_COORDS_F64) ? (double4*)(sorted ? c->sortX64.p : c->X64.p) + xoff[f] : nullptr;
     J.fd = dF + f;
     J.n = fr->n;
     J.chunk0 = P.n_chunks;
     P.n_chunks += (fr->n + kStageChunk - 1) / kStageChunk;
   }
   if (!segs.empty()) std::memcpy(hS, segs.data(), sizeof(Segment) * segs.size());
+  if (!lsegs.empty()) std::memcpy((unsigned char*)hS + P.seg_bytes, lsegs.data(), P.lseg_bytes);
   if (!sorts.empty())
-    std::memcpy((unsigned char*)hS + P.seg_bytes, sorts.data(), sizeof(SortSeg) * sorts.size());
+    std::memcpy((unsigned char*)hS + P.seg_bytes + P.lseg_bytes, sorts.data(), sizeof(SortSeg) * sorts.size());
   // launch shapes (occupancy queries and kernel attributes stay outside any stream capture)
   for (int v = 0; v < kNumVariants; ++v) {
     P.vgrid[v] = 0;
     if (P.vitems[v] == 0 || !with_pairs) continue;
-    const int width = vsum[v].width;
-    P.vmulti[v] = vsum[v].multi;
+    const int width = told[v].width;
+    P.vmulti[v] = told[v].multi;
     LaunchParams& lp = P.vparams[v];
     int bps_max = pair_kernel_blocks_per_sm(v, width, lp.depth, lp.block);
     if (bps_max < 1 && lp.depth > 1) {
@@ -568,6 +716,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     P.vwidth[v] = width;
     P.vgrid[v] = pair_grid(c->num_sms, lp.bps, P.vitems[v]);
   }
+  if (with_pairs && P.litems > 0) P.lgrid = pair_grid(c->num_sms, 1, P.litems);
   return DH_OK;
 }
 
@@ -592,29 +741,44 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
     DH_CUDA_TRY(launch_stage(dJ, P.n_jobs, P.n_chunks, st));
     ++launched;
   }
+  DH_CUDA_TRY(launch_frame_setup(dF, k, 0, st));  // the windows, and the grid of the spatial order
+  ++launched;
   if (P.n_sort > 0) {
-    const SortSeg* dSort = (const SortSeg*)((unsigned char*)dS + P.seg_bytes);
+    const SortSeg* dSort = (const SortSeg*)((unsigned char*)dS + P.seg_bytes + P.lseg_bytes);
     DH_CUDA_TRY(cudaMemsetAsync(c->sortC.p, 0, sizeof(uint32_t) * (size_t)P.sort_keys, st));
-    DH_CUDA_TRY(launch_spatial_sort(dSort, P.n_sort, P.sort_chunks, (float4*)c->X.p, (float4*)c->sortX.p,
-                                    P.any_f64 ? (double4*)c->X64.p : nullptr,
-                                    P.any_f64 ? (double4*)c->sortX64.p : nullptr, (int32_t*)c->sortK.p,
-                                    (uint32_t*)c->sortC.p, st));
+    DH_CUDA_TRY(launch_spatial_sort(dSort, P.n_sort, P.sort_max, (const float4*)c->sortX.p, (float4*)c->X.p,
+                                    P.any_f64 ? (const double4*)c->sortX64.p : nullptr,
+                                    P.any_f64 ? (double4*)c->X64.p : nullptr, (int32_t*)c->sortK.p,
+                                    (uint32_t*)c->sortC.p, P.sort_keys, st));
     launched += 4;
   }
-  DH_CUDA_TRY(launch_frame_setup(dF, k, 0, st));
-  ++launched;
   // A2-A8: per variant, one persistent launch over its frames, species pairs and bin sweeps
   int grid = 0, top = -1;
   int64_t top_items = 0;
-  bool any = false;
+  bool any = P.lgrid > 0;
   for (int v = 0; v < kNumVariants; ++v) any |= P.vgrid[v] > 0;
   // timing events: inside a stream capture they must become event-record nodes
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   DH_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
   const unsigned ev_flags = (cs == cudaStreamCaptureStatusActive) ? cudaEventRecordExternal : cudaEventRecordDefault;
   if (any) {
-    DH_CUDA_TRY(cudaMemsetAsync(c->ctl.p, 0, sizeof(Control) * kNumVariants, st));
+    DH_CUDA_TRY(cudaMemsetAsync(c->ctl.p, 0, sizeof(Control) * kNumVariants + sizeof(SegCounter) * (size_t)P.n_lsegs, st));
     if (c->ev_pair0) DH_CUDA_TRY(cudaEventRecordWithFlags(c->ev_pair0, st, ev_flags));
+    if (P.lgrid > 0) {
+      ListLaunch L;
+      std::memset(&L, 0, sizeof L);
+      L.segs = (const ListSegment*)((unsigned char*)dS + P.seg_bytes);
+      L.ctr = (SegCounter*)((unsigned char*)c->ctl.p + sizeof(Control) * kNumVariants);
+      L.n_segs = P.n_lsegs;
+      L.hist_width = P.lwidth;
+      L.n_items = P.litems;
+      L.split = P.lsplit;
+      L.multi = P.lmulti;
+      DH_CUDA_TRY(launch_list(L, P.lgrid, st));
+      ++launched;
+      grid = P.lgrid;
+      top_items = P.litems / P.lsplit / 64;  // in tiles of the other kernel
+    }
     for (int v = 0; v < kNumVariants; ++v) {
       if (P.vgrid[v] == 0) continue;
       PairLaunch L;
@@ -652,6 +816,12 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   S.items = (int32_t)std::min<int64_t>(P.n_items, 0x7FFFFFFF);
   S.kernel_launches = launched + P.launched;
   S.tune_runs = c->tune_runs;
+  if (top < 0 && P.lgrid > 0) {  // the list kernel: one histogram per block, no j tiles of its own
+    S.tile_j = kTile;
+    S.hist_depth = 1;
+    S.blocks_per_sm = 1;
+    S.block_threads = kListBlock;
+  }
   if (top >= 0) {
     S.tile_j = kTile / P.vparams[top].jm;
     S.hist_depth = P.vparams[top].depth;
@@ -707,7 +877,7 @@ dh_status run_frames(dh_ctx* c, const dh_frame* frames, int k, bool wait, bool u
   std::vector<PlannedFrame> pfs((size_t)k);
   bool dev = (frames[0].flags & DH_DEVICE_PTRS) != 0;
   for (int f = 0; f < k; ++f) {
-    dh_status s = check_frame(&frames[f], pfs[f], c->max_width);
+    dh_status s = check_frame(&frames[f], pfs[f], c->max_width, c->list_width);
     if (s != DH_OK) return s;
     if (((frames[f].flags & DH_DEVICE_PTRS) != 0) != dev)
       return fail(DH_ERR_INVALID, "all frames of a batch must use the same pointer kind");
@@ -918,7 +1088,7 @@ dh_status tune_variant(dh_ctx* c, int v, const VariantSummary& vs) {
     double ms = c->stats.pair_kernel_ms;
     double pairs = pairs_one * nf;
     if (c->tune_cap_pairs > 0.0) {  // whole items of the capped launch
-      const double per_item = (double)kTile * (double)(kTile / p.jm);
+      const double per_item = p.list ? (double)kRun * kRun : (double)kTile * (double)(kTile / p.jm);
       pairs = std::min(pairs, std::ceil(c->tune_cap_pairs / per_item) * per_item);
     }
     *gps = ms > 0.0 ? pairs / (ms * 1e6) : 0.0;
@@ -927,6 +1097,7 @@ dh_status tune_variant(dh_ctx* c, int v, const VariantSummary& vs) {
   // the shape used without a measurement is the reference; another shape must
   // beat it by 2 % (single measurements of nearby shapes differ by about 1 %)
   LaunchParams def;
+  def.list = vs.list;
   def.block = default_block(v, vs.width);
   def.bps = pair_kernel_blocks_per_sm(v, vs.width, 1, def.block);
   double g = 0.0;
@@ -956,6 +1127,7 @@ dh_status tune_variant(dh_ctx* c, int v, const VariantSummary& vs) {
   // shape's copies and blocks with the aggregation
   if (s == DH_OK && !vs.multi && def.block == kBlockSmall) {
     LaunchParams p = def;
+    p.list = 0;
     p.agg = 1;
     s = measure(p, &g);
     if (s == DH_OK && g > best.gpairs_s && g > 1.02 * g_def) {
@@ -1014,7 +1186,7 @@ dh_status selfcheck(dh_ctx* c, int32_t what, const dh_frame* frame, uint64_t n_s
   if ((what != DH_CHECK_WINDOW && what != DH_CHECK_TILES) || !frame)
     return fail(DH_ERR_INVALID, "unknown self check %d", what);
   std::vector<PlannedFrame> pfs(1);
-  dh_status s = check_frame(frame, pfs[0], c->max_width);
+  dh_status s = check_frame(frame, pfs[0], c->max_width, c->list_width);
   if (s != DH_OK) return s;
   if (what == DH_CHECK_TILES && ((pfs[0].variant != V_ORTHO && pfs[0].variant != V_TRIC) || frame->n < 2))
     return fail(DH_ERR_INVALID, "the tile check needs an orthorhombic or triclinic frame without search");
@@ -1103,6 +1275,7 @@ dh_status dh_create(const dh_config* config, dh_ctx** out) {
   DH_CUDA_TRY(cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking));
   DH_CUDA_TRY(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   c->max_width = pair_kernel_max_width();
+  c->list_width = list_kernel_max_width();
   if (c->max_width < 1024) return fail(DH_ERR_CUDA, "not enough shared memory per block");
   DH_CUDA_TRY(c->ctl.ensure(sizeof(Control) * kNumVariants));
   DH_CUDA_TRY(c->tstat.ensure(64));
@@ -1140,6 +1313,9 @@ dh_status dh_destroy(dh_ctx* c) {
   c->sortX.release();
   c->sortX64.release();
   c->X64.release();
+  c->P4.release();
+  c->P2.release();
+  c->bnd.release();
   c->sortK.release();
   c->sortC.release();
   c->hmeta.release();

@@ -86,9 +86,11 @@ struct PlannedFrame {
   int32_t sweep_width;
   double margin;
   uint64_t pairs;
+  bool list;  // the list kernel can run it (one image of a pair at most inside r_max)
 };
 
-dh_status check_frame(const dh_frame* f, PlannedFrame& pf, int max_width);
+// list_width: bins per sweep of the list kernel, 0 when the caller has no list path.
+dh_status check_frame(const dh_frame* f, PlannedFrame& pf, int max_width, int list_width);
 void fill_frame_dev(const PlannedFrame& pf, FrameDev& F, const float4* X, uint64_t* out, const double* T);
 // jm: j tiles of kTile/jm particles per i tile of kTile.  fill_segments writes
 // at most cap segments to out and the total to *n_out; add_segments appends all.
@@ -96,8 +98,17 @@ int64_t fill_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, int j
                       int* n_out);
 int64_t add_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, std::vector<Segment>& segs, int jm = 1);
 
+// The same for the list kernel (split: items per run pair, ListLaunch.split).
+int64_t add_list_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, std::vector<ListSegment>& segs,
+                          int split);
+int64_t frame_runs(const dh_frame* f);  // runs of kRun particles over its species
+// Items per run pair: one item per warp where the frames are that small, else
+// enough for an even end.
+int list_split_for(double run_pairs, int num_sms);
+
 // Launch shape of one pair-kernel launch.
 struct LaunchParams {
+  int32_t list = 0;              // the list kernel (the fields below do not apply)
   int32_t jm = 1;                // j tiles per i tile: tile_j = kTile / jm
   int32_t depth = 1;             // private histogram copies per block
   int32_t bps = 0;               // blocks per SM (0: as many as fit)
@@ -124,15 +135,13 @@ TuneKey make_tune_key(int variant, int width, double mean_pairs_per_frame, int f
 // Bytes of a frame's coordinate array (float32 or binary64, 3 or 4 per particle).
 size_t coord_bytes(const dh_frame* f);
 
-// Species of frames without the 27-image search are put in spatial (Morton)
-// order before the pair kernel (no box: over the frame's bounding box), from this many particles on, with about 16
-// particles per cell.  plan_spatial_order lists the species of one frame (its
-// particles from x0 in the packed coordinates, its counters from key0) and
-// returns the counters and most staging chunks they need.
-constexpr int32_t kSortMinParticles = 2048;
-int sort_grid_bits(int64_t n);
+// Species are put in spatial (Hilbert) order before the pair kernel, over the
+// frame's bounding box or its home cell, with about two particles per cell.
+// plan_spatial_order lists the species of one frame (its particles from x0 in
+// the packed coordinates, its counters from key0) and returns the counters they
+// need and the largest species.  Frames of the 27-image search keep their order.
 std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, const FrameDev* fd, int64_t x0, int64_t key0,
-                                        int64_t* keys, int* chunks);
+                                        int64_t* keys, int64_t* max_n);
 
 // Threads per block for a launch without a measured shape: from 16,384 bins on,
 // a 256-thread block's histogram leaves room for at most two blocks per SM, and
@@ -174,6 +183,7 @@ struct dh_ctx {
   std::recursive_mutex mu;
   int num_sms = 0;
   int max_width = 0;
+  int list_width = 0;
   dh_config cfg{};
 
   dh::DevBuf raw;      // caller coordinates copied from the host (n x stride floats)
@@ -186,8 +196,10 @@ struct dh_ctx {
   dh::DevBuf tstat;    // threshold build status
   dh::DevBuf aux;      // small per-call arrays (g(r) pair densities)
   dh::DevBuf X64;      // binary64 input coordinates (double4), when a frame has them
-  dh::DevBuf sortX64;  // spatial order: scratch copy of those,
-  dh::DevBuf sortX;    // of the float32 coordinates,
+  dh::DevBuf P4, P2;   // list kernel: positions in bins (double-floats),
+  dh::DevBuf bnd;      //   bounds of the runs
+  dh::DevBuf sortX64;  // staged in the caller's order: binary64,
+  dh::DevBuf sortX;    // and float32 coordinates,
   dh::DevBuf sortK;    //   cell keys,
   dh::DevBuf sortC;    //   and cell counters
   dh::ThresholdCache tcache;

@@ -135,11 +135,17 @@ struct Request {
   uint64_t* res_pin = nullptr;   // pinned histogram read-back
   size_t res_count = 0;
   double* T = nullptr;
-  std::vector<Segment> segs;     // all segments, items numbered from 0
-  // spatial order of the species (periodic frames): plan, device scratch, pinned upload
+  std::vector<Segment> segs;     // all segments, items numbered from 0: of the tiled kernel,
+  std::vector<ListSegment> lsegs;  // or of the list kernel
+  double pairs_per_item = 1.0;
+  // spatial order of the species: plan, device scratch, pinned upload
   std::vector<SortSeg> sorts;
   int64_t sort_keys = 0;
-  int sort_chunks = 0;
+  int64_t sort_max = 0;
+  int64_t runs = 0;
+  float4* bnd = nullptr;
+  float4* P4 = nullptr;
+  float2* P2 = nullptr;
   SortSeg* sort_dev = nullptr;
   SortSeg* sort_pin = nullptr;
   float4* sort_X = nullptr;
@@ -243,7 +249,7 @@ dh_status Server::start() {
     DH_CUDA_TRY(ln.tstat.ensure(64));
     DH_CUDA_TRY(cudaMemsetAsync(ln.tstat.p, 0, 64, ln.stream));
     for (auto& w : ln.slots) {
-      DH_CUDA_TRY(w.ctl.ensure(sizeof(Control) * kWidthClasses));
+      DH_CUDA_TRY(w.ctl.ensure(sizeof(Control) * kWidthClasses + sizeof(SegCounter) * 1024));
       DH_CUDA_TRY(cudaEventCreate(&w.ev0));
       DH_CUDA_TRY(cudaEventCreate(&w.ev1));
     }
@@ -301,7 +307,7 @@ dh_status Server::submit(const dh_frame* f, uint64_t* ticket) {
   r->frame.species_offsets = r->offs.data();
   if (f->flags & DH_COORDS_F64)
     return fail(DH_ERR_INVALID, "the served path takes float32 coordinates (DH_COORDS_F64: use dh_histogram)");
-  dh_status s = check_frame(&r->frame, r->pf, ctx_->max_width);
+  dh_status s = check_frame(&r->frame, r->pf, ctx_->max_width, ctx_->list_width);
   if (s != DH_OK) return s;
   r->pf.src = &r->frame;
   r->dev_ptrs = (f->flags & DH_DEVICE_PTRS) != 0;
@@ -310,10 +316,12 @@ dh_status Server::submit(const dh_frame* f, uint64_t* ticket) {
   size_t n = (size_t)f->n;
   r->dev_bytes = align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob)) + align_up(16 * std::max<size_t>(n, 1));
   r->pin_bytes = align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob));
-  r->sorts = plan_spatial_order(r->pf, nullptr, 0, 0, &r->sort_keys, &r->sort_chunks);
+  r->sorts = plan_spatial_order(r->pf, nullptr, 0, 0, &r->sort_keys, &r->sort_max);
+  r->runs = frame_runs(&r->frame);
   if (!r->sorts.empty()) {
     r->dev_bytes += align_up(sizeof(SortSeg) * r->sorts.size()) + align_up(16 * n) + align_up(4 * n) +
-                    align_up(4 * (size_t)r->sort_keys);
+                    align_up(8 * (size_t)r->sort_keys);
+    if (r->pf.list) r->dev_bytes += align_up(2 * sizeof(float4) * (size_t)r->runs) + align_up(16 * n) + align_up(8 * n);
     r->pin_bytes += align_up(sizeof(SortSeg) * r->sorts.size());
   }
   if (!r->dev_ptrs) {
@@ -429,7 +437,15 @@ void Server::admit() {
       r.sort_K = (int32_t*)d;
       d += align_up(4 * (size_t)r.frame.n);
       r.sort_C = (uint32_t*)d;
-      d += align_up(4 * (size_t)r.sort_keys);
+      d += align_up(8 * (size_t)r.sort_keys);
+      if (r.pf.list) {
+        r.bnd = (float4*)d;
+        d += align_up(2 * sizeof(float4) * (size_t)r.runs);
+        r.P4 = (float4*)d;
+        d += align_up(16 * (size_t)r.frame.n);
+        r.P2 = (float2*)d;
+        d += align_up(8 * (size_t)r.frame.n);
+      }
       r.sort_pin = (SortSeg*)p;
       p += align_up(sizeof(SortSeg) * r.sorts.size());
     }
@@ -447,7 +463,9 @@ void Server::admit() {
       r.hist = r.frame.out;
     }
     r.segs.clear();
-    r.n_items = add_segments(r.pf, r.fd, 0, r.segs);
+    r.lsegs.clear();
+    r.n_items = r.pf.list ? add_list_segments(r.pf, r.fd, 0, r.lsegs, 1) : add_segments(r.pf, r.fd, 0, r.segs);
+    r.pairs_per_item = r.pf.list ? (double)kRun * kRun : (double)kTile * kTile;
     r.next = 0;
     r.state = Q_ACTIVE;
     queue_.pop_front();
@@ -462,9 +480,12 @@ dh_status Server::prep(Request& r) {
   dh_status s = ctx_->tcache.acquire(r.frame.r_max, r.frame.nbins, st, (int32_t*)ln.tstat.p, &r.T, nullptr);
   if (s != DH_OK) return s;
   fill_frame_dev(r.pf, *r.fd_pin, r.X, r.hist, r.T);
+  r.fd_pin->bnd = r.bnd;
+  r.fd_pin->P4 = r.P4;
+  r.fd_pin->P2 = r.P2;
   std::memset(r.job_pin, 0, sizeof(StageJob));
   r.job_pin->src = r.dev_ptrs ? r.frame.coords : r.raw;
-  r.job_pin->dst = r.X;
+  r.job_pin->dst = r.sorts.empty() ? r.X : r.sort_X;
   r.job_pin->fd = r.fd;
   r.job_pin->n = r.frame.n;
   r.job_pin->stride = r.stride;
@@ -478,6 +499,7 @@ dh_status Server::prep(Request& r) {
     DH_CUDA_TRY(cudaMemsetAsync(r.hist, 0, 8 * r.res_count, st));
   int64_t chunks = (r.frame.n + kStageChunk - 1) / kStageChunk;
   if (chunks > 0) DH_CUDA_TRY(launch_stage(r.job_dev, 1, chunks, st));
+  DH_CUDA_TRY(launch_frame_setup(r.fd, 1, 0, st));
   if (!r.sorts.empty()) {
     for (size_t q = 0; q < r.sorts.size(); ++q) {
       r.sort_pin[q] = r.sorts[q];
@@ -486,10 +508,9 @@ dh_status Server::prep(Request& r) {
     DH_CUDA_TRY(cudaMemcpyAsync(r.sort_dev, r.sort_pin, sizeof(SortSeg) * r.sorts.size(), cudaMemcpyHostToDevice,
                                 st));
     DH_CUDA_TRY(cudaMemsetAsync(r.sort_C, 0, 4 * (size_t)r.sort_keys, st));
-    DH_CUDA_TRY(launch_spatial_sort(r.sort_dev, (int)r.sorts.size(), r.sort_chunks, r.X, r.sort_X, nullptr, nullptr,
-                                    r.sort_K, r.sort_C, st));
+    DH_CUDA_TRY(launch_spatial_sort(r.sort_dev, (int)r.sorts.size(), r.sort_max, r.sort_X, r.X, nullptr, nullptr,
+                                    r.sort_K, r.sort_C, r.sort_keys, st));
   }
-  DH_CUDA_TRY(launch_frame_setup(r.fd, 1, 0, st));
   // marks the end of the preparation: a request cancelled before its first wave
   // keeps its pool memory until this work has finished
   if (!r.done_ev) DH_CUDA_TRY(cudaEventCreateWithFlags(&r.done_ev, cudaEventDisableTiming));
@@ -539,7 +560,6 @@ bool Server::launch_wave(int v) {
   }
   if (run.empty()) return false;
   WaveSlot& W = ln.slots[slot];
-  const double pairs_per_item = (double)kTile * (double)kTile;
   // The wave's pair budget goes to the requests with the least work left
   // first, so small requests finish in the wave they join.  While every
   // admitted request can run (no request waits for admission), the order is
@@ -551,7 +571,10 @@ bool Server::launch_wave(int v) {
   // and equal shares keep the saturated throughput higher (measured).  Every
   // request takes at least one work item per wave.
   std::stable_sort(run.begin(), run.end(),
-                   [](const Request* a, const Request* b) { return a->n_items - a->next < b->n_items - b->next; });
+                   [](const Request* a, const Request* b) {
+                     return (double)(a->n_items - a->next) * a->pairs_per_item <
+                            (double)(b->n_items - b->next) * b->pairs_per_item;
+                   });
   const bool saturated = !queue_.empty();
   double budget_left = ln.rate * wave_seconds_ * (saturated ? kSaturatedWaveFactor : 1.0);
   // segments per histogram-width class: requests of very different widths run
@@ -559,9 +582,11 @@ bool Server::launch_wave(int v) {
   // wide request would otherwise give every request of the wave the shape of
   // the widest histogram: larger blocks and fewer of them per SM)
   std::vector<Segment> csegs[kWidthClasses];
-  int64_t citems[kWidthClasses] = {};
+  std::vector<ListSegment> lsegs[kWidthClasses];
+  int64_t citems[kWidthClasses] = {}, litems[kWidthClasses] = {};
   int cwidth[kWidthClasses], cmulti[kWidthClasses] = {};
-  for (int q = 0; q < kWidthClasses; ++q) cwidth[q] = 1;
+  int lwidth[kWidthClasses], lmulti[kWidthClasses] = {};
+  for (int q = 0; q < kWidthClasses; ++q) cwidth[q] = lwidth[q] = 1;
   int64_t witems = 0;
   double wpairs = 0;
   std::vector<Request*> finishing;
@@ -576,9 +601,9 @@ bool Server::launch_wave(int v) {
       }
     }
     const double share = std::max(0.0, budget_left) / (saturated ? (double)(run.size() - q) : 1.0);
-    int64_t take = std::max<int64_t>(1, (int64_t)(share / pairs_per_item));
+    int64_t take = std::max<int64_t>(1, (int64_t)(share / r->pairs_per_item));
     take = std::min(take, r->n_items - r->next);
-    budget_left -= (double)take * pairs_per_item;
+    budget_left -= (double)take * r->pairs_per_item;
     int64_t lo = r->next, hi = r->next + take;
     const int cl = width_class(r->pf.sweep_width);
     for (const Segment& sg : r->segs) {
@@ -592,18 +617,37 @@ bool Server::launch_wave(int v) {
       witems += b - a;
       csegs[cl].push_back(w);
     }
+    for (const ListSegment& sg : r->lsegs) {
+      int64_t a = std::max(lo, sg.item0), b = std::min(hi, sg.item0 + sg.items);
+      if (a >= b) continue;
+      ListSegment w = sg;
+      w.item0 = litems[cl];
+      w.item_base = a - sg.item0;
+      w.items = b - a;
+      litems[cl] += b - a;
+      witems += b - a;
+      lsegs[cl].push_back(w);
+    }
     r->next = hi;
     r->last_wave = ln.wave_seq + 1;
-    cwidth[cl] = std::max(cwidth[cl], r->pf.sweep_width);
-    cmulti[cl] |= r->pf.sweeps > 1;
-    wpairs += (double)std::min<uint64_t>(r->pf.pairs, (uint64_t)((double)take * pairs_per_item));
+    int& width = r->pf.list ? lwidth[cl] : cwidth[cl];
+    int& multi = r->pf.list ? lmulti[cl] : cmulti[cl];
+    width = std::max(width, r->pf.sweep_width);
+    multi |= r->pf.sweeps > 1;
+    wpairs += (double)std::min<uint64_t>(r->pf.pairs, (uint64_t)((double)take * r->pairs_per_item));
     if (r->next >= r->n_items) finishing.push_back(r);
   }
   if (witems == 0) return false;
-  size_t nseg = 0;
-  for (int q = 0; q < kWidthClasses; ++q) nseg += csegs[q].size();
-  size_t bytes = sizeof(Segment) * nseg;
-  if (W.segs.ensure(bytes) != cudaSuccess || W.hsegs.ensure(bytes) != cudaSuccess) {
+  // descriptors: the tiled kernel's segments, then the list kernel's
+  size_t nseg = 0, nlseg = 0;
+  for (int q = 0; q < kWidthClasses; ++q) {
+    nseg += csegs[q].size();
+    nlseg += lsegs[q].size();
+  }
+  const size_t bytes = sizeof(Segment) * nseg + sizeof(ListSegment) * nlseg;
+  const size_t ctl_bytes = sizeof(Control) * kWidthClasses + sizeof(SegCounter) * nlseg;
+  if (W.segs.ensure(bytes) != cudaSuccess || W.hsegs.ensure(bytes) != cudaSuccess ||
+      W.ctl.ensure(ctl_bytes) != cudaSuccess) {
     thread_error_ = "out of memory for wave descriptors";
     return false;
   }
@@ -612,10 +656,31 @@ bool Server::launch_wave(int v) {
     if (!csegs[q].empty()) std::memcpy((Segment*)W.hsegs.p + at, csegs[q].data(), sizeof(Segment) * csegs[q].size());
     at += csegs[q].size();
   }
+  at = 0;
+  for (int q = 0; q < kWidthClasses; ++q) {
+    ListSegment* hl = (ListSegment*)((Segment*)W.hsegs.p + nseg);
+    if (!lsegs[q].empty()) std::memcpy(hl + at, lsegs[q].data(), sizeof(ListSegment) * lsegs[q].size());
+    at += lsegs[q].size();
+  }
   cudaMemcpyAsync(W.segs.p, W.hsegs.p, bytes, cudaMemcpyHostToDevice, ln.stream);
-  cudaMemsetAsync(W.ctl.p, 0, sizeof(Control) * kWidthClasses, ln.stream);
+  cudaMemsetAsync(W.ctl.p, 0, ctl_bytes, ln.stream);
   cudaEventRecord(W.ev0, ln.stream);
   cudaError_t e = cudaSuccess;
+  at = 0;
+  for (int q = 0; q < kWidthClasses && e == cudaSuccess; ++q) {
+    if (lsegs[q].empty()) continue;
+    ListLaunch L;
+    std::memset(&L, 0, sizeof L);
+    L.segs = (const ListSegment*)((const Segment*)W.segs.p + nseg) + at;
+    L.ctr = (SegCounter*)((Control*)W.ctl.p + kWidthClasses) + at;
+    L.n_segs = (int32_t)lsegs[q].size();
+    L.hist_width = lwidth[q];
+    L.n_items = litems[q];
+    L.split = 1;
+    L.multi = lmulti[q];
+    e = launch_list(L, pair_grid(ctx_->num_sms, 1, litems[q]), ln.stream);
+    at += lsegs[q].size();
+  }
   at = 0;
   for (int q = 0; q < kWidthClasses && e == cudaSuccess; ++q) {
     if (csegs[q].empty()) continue;
