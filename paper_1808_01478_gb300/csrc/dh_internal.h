@@ -67,6 +67,7 @@ struct FrameDev {
   float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz)
   float img_h[27][3], img_l[27][3];  // image vectors -B k as double-floats (index as tshift)
   float period[3];    // a_x, b_y, c_z
+  int32_t pick;       // r_max beyond half the distance between images: the shortest image counts
   // ---- written on the device
   int32_t smin[3], smax[3];  // triclinic: the same of the fractional coordinates
   int32_t wrap;       // the coordinates span more than one cell: P4 is brought home to the first
@@ -192,6 +193,7 @@ struct ListLaunch {
   int64_t n_items;
   int32_t split;         // items per run pair (1 to 16, a power of two: kRun / split j particles each)
   int32_t multi;
+  int32_t pick;          // frames whose pairs take the shortest of several images (FrameDev.pick)
 };
 
 // ---- launchers (dh_kernels.cu); all enqueue on `stream` and return the launch error

@@ -121,7 +121,7 @@ __global__ void stage_kernel(const StageJob* __restrict__ jobs, int n_jobs) {
   float mn0 = INFINITY, mn1 = INFINITY, mn2 = INFINITY;
   float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY;
   // triclinic: the range of the fractional coordinates too (does the frame span more than one cell?)
-  const bool frac = J.fd->variant == V_TRIC;
+  const bool frac = J.fd->variant == V_TRIC || J.fd->variant == V_TRIC_SEARCH;
   float sn[3] = {INFINITY, INFINITY, INFINITY}, sx[3] = {-INFINITY, -INFINITY, -INFINITY};
   int bad = 0;
   const float* __restrict__ src = J.src;
@@ -410,9 +410,10 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
   }
   if (F.variant != V_NONE) {
     for (int c = 0; c < 3; ++c) {
-      const double span = F.variant == V_TRIC ? (double)float_of_ord(F.smax[c]) - (double)float_of_ord(F.smin[c])
-                                              : R[c] * (double)F.invf[c];
-      if (span > 1.0 + 1.0 / 16.0) wrap = 1;
+      const double span = F.variant != V_ORTHO ? (double)float_of_ord(F.smax[c]) - (double)float_of_ord(F.smin[c])
+                                               : R[c] * (double)F.invf[c];
+      // with the search, the nearest image can differ by nearly a cell more (check_frame)
+      if (span > 1.0 + (F.variant == V_TRIC_SEARCH ? 1.0 / 16384.0 : 1.0 / 16.0)) wrap = 1;
     }
     if (wrap) {  // the home cell's bounding box
       ext[0] = B[0] + fabs(B[1]) + fabs(B[2]);

@@ -50,6 +50,9 @@ constexpr int kBlk = 64;       // listed images evaluated at a time
 constexpr int kCap = 2 * kBlk; // list ring: a block waiting to fill plus one round of 32 appends
 constexpr int kImgShift = 26;  // list reference: particle | image << 26
 constexpr int kHome = 13;      // the image k = 0
+constexpr int kPickCap = 64;   // images evaluated at a time in pick_round (at least 27)
+constexpr uint32_t kLastImage = 0x80000000u;
+constexpr uint32_t kAnyImage = 31u << kImgShift;  // reference of a pair whose image is chosen by the drain
 // A claim takes 1/kClaims of a warp's share of the items left.  Items cost from
 // nothing (no image in the sweep) to 16,384 pairs, so a large claim of full items
 // can outlast everything else (2: triclinic N = 200,000 9.9 ms; 3: 8.4; 6: 6.7;
@@ -86,6 +89,10 @@ struct WarpList {
   float qm_here; //   its (2 W + 1)^2 where near,
   float qm;      // and the largest of them in the list
   unsigned long long uni, axis, cull;  // pairs, for the statistics
+  // images of particles whose nearest image differs within the run (pick_round):
+  // y, W - |y|^2, and reference with kLastImage on a particle's last
+  float4 M[kPickCap];
+  uint32_t mref[kPickCap];
 };
 
 // What a block's pairs have in common (its segment), in shared memory.
@@ -207,14 +214,16 @@ __device__ __forceinline__ int exact_listed(const FrameDev& F, int i, int j, flo
 __device__ __noinline__ int exact_listed_bin(const FrameDev& F, int i, int j, float3 d, bool any) {
   return F.variant == V_NONE    ? exact_listed<V_NONE>(F, i, j, d, any)
          : F.variant == V_ORTHO ? exact_listed<V_ORTHO>(F, i, j, d, any)
-                                : exact_listed<V_TRIC>(F, i, j, d, any);
+         : F.variant == V_TRIC ? exact_listed<V_TRIC>(F, i, j, d, any)
+                               : exact_listed<V_TRIC_SEARCH>(F, i, j, d, true);
 }
 
 // Bin of a re-decided pair from q in double-float arithmetic (about 44 bits) for
 // the listed image m, and the integer n nearest to its root.  The image must be
 // the definition's nearest one: the displacement strictly inside half the periods
-// c_z, b_y, a_x (Babai's step; see exact_r2).  Otherwise, and when q is too close
-// to n^2, the binary64 replay decides.
+// c_z, b_y, a_x (Babai's step; see exact_r2), or known to be (F.pick: the listed
+// image is the shortest by a margin).  Otherwise, and when q is too close to n^2,
+// the binary64 replay decides.
 __device__ __forceinline__ int listed_bin(const FrameDev& F, int i, int j, int m, float& n, unsigned& nexact) {
   const Pos a = unpack(__ldg(F.P4 + i), __ldg(F.P2 + i)), b = unpack(__ldg(F.P4 + j), __ldg(F.P2 + j));
   const float ah[3] = {a.h.x, a.h.y, a.h.z}, al[3] = {a.l.x, a.l.y, a.l.z};
@@ -228,7 +237,7 @@ __device__ __forceinline__ int listed_bin(const FrameDev& F, int i, int j, int m
     d[c] = two_sum(__fadd_rn(__fsub_rn(bh[c], ah[c]), vh[c]), __fadd_rn(vl[c], __fsub_rn(bl[c], al[c])));
     // (orthorhombic: and not where binary64 may round the other way)
     const float half = 0.5f * F.period[c], w = fabsf(d[c].h);
-    inside = inside && (F.variant == V_NONE || (w < half * (1.0f - 0x1p-18f) && half - w > F.list_tie));
+    inside = inside && (F.variant == V_NONE || F.pick || (w < half * (1.0f - 0x1p-18f) && half - w > F.list_tie));
   }
   const DF q = df_norm2(d[0], d[1], d[2]);
   const float s = sqrt_approx(q.h);
@@ -241,7 +250,31 @@ __device__ __forceinline__ int listed_bin(const FrameDev& F, int i, int j, int m
       return (int)fminf(n, (float)F.nbins + 1.0f) - (diff < 0.0f && n >= 0.5f ? 1 : 0);
   }
   ++nexact;
-  return exact_listed_bin(F, i, j, make_float3(d[0].h, d[1].h, d[2].h), false);
+  return exact_listed_bin(F, i, j, make_float3(d[0].h, d[1].h, d[2].h), F.pick != 0);
+}
+
+// The same for a pair whose shortest image is not known: the shortest in float32,
+// unless another comes within 2^-16 of it.
+__device__ __noinline__ int picked_bin(const FrameDev& F, int i, int j, unsigned& nexact) {
+  const Pos a = unpack(__ldg(F.P4 + i), __ldg(F.P2 + i)), b = unpack(__ldg(F.P4 + j), __ldg(F.P2 + j));
+  const float dx = b.h.x - a.h.x, dy = b.h.y - a.h.y, dz = b.h.z - a.h.z;
+  float best = INFINITY, next = INFINITY;
+  int m = kHome;
+  for (int k = 0; k < 27; ++k) {
+    const float x = dx + F.img_h[k][0], y = dy + F.img_h[k][1], z = dz + F.img_h[k][2];
+    const float q = x * x + y * y + z * z;
+    next = fminf(next, fmaxf(q, best));
+    if (q < best) {
+      best = q;
+      m = k;
+    }
+  }
+  float n;
+  // (the low parts and the roundings move a distance by less than cull_abs)
+  const float slack = 4.0f * F.cull_abs * (sqrtf(next) + F.cull_abs);
+  if (next - best > best * 0x1p-16f + slack) return listed_bin(F, i, j, m, n, nexact);
+  ++nexact;
+  return exact_listed_bin(F, i, j, make_float3(0.f, 0.f, 0.f), true);
 }
 
 // The word in which the pair loop counted a pair close to its run (q' below
@@ -265,6 +298,7 @@ __device__ __noinline__ int replay_rel(const SegState& G, int i, int j, int m) {
 // lane, and shift the rest of the queue down.  A pair was counted one below its
 // edge n and moves up when it belongs there; close to the run, where the window
 // may hold several edges, the word it was counted in is found by replay.
+// Pairs with kAnyImage were not counted.
 constexpr uint32_t kNearPair = 0x80000000u;
 __device__ __noinline__ int list_drain(const SegState& G, WarpList& W, int qcount, uint32_t* sh, int lane) {
   const FrameDev& F = *G.F;
@@ -277,9 +311,15 @@ __device__ __noinline__ int list_drain(const SegState& G, WarpList& W, int qcoun
     const int width = G.hi - G.lo, m = (int)(e.x >> kImgShift);
     const int i = (int)(e.y & ~kNearPair), j = (int)(e.x & ((1u << kImgShift) - 1u));
     float n;
-    const int bin = listed_bin(F, G.i0 + i, G.j0 + j, m, n, nexact) - G.lo;
-    int prov = (int)n - 1 - G.lo;
-    if (e.y & kNearPair) prov = replay_rel(G, i, j, m);
+    int bin, prov;
+    if (e.x >= kAnyImage) {
+      bin = picked_bin(F, G.i0 + i, G.j0 + j, nexact) - G.lo;
+      prov = -1;
+    } else {
+      bin = listed_bin(F, G.i0 + i, G.j0 + j, m, n, nexact) - G.lo;
+      prov = (int)n - 1 - G.lo;
+      if (e.y & kNearPair) prov = replay_rel(G, i, j, m);
+    }
     if (bin != prov) {
       if ((uint32_t)bin < (uint32_t)width) atomicAdd(sh + bin, 1u);
       if ((uint32_t)prov < (uint32_t)width) atomicAdd(sh + prov, 0xFFFFFFFFu);
@@ -459,6 +499,124 @@ __device__ __noinline__ int list_near(const SegState& G, WarpList& W, int i_begi
   return list_block<NEARBY, MULTI>(G, I, W, i_begin, s0, n, qm, above, sh, lane, qcount);
 }
 
+// Frames whose r_max exceeds half the distance between images (F.pick): a pair's
+// distance is the shortest over the images, so an image of a particle is listed
+// alone only when it is the shortest for every particle of the run.
+//
+// One round of 32 j particles (this lane's at p, index jl, if valid) of a j run of
+// which several images (mask) can be the shortest for some pair.  Per particle,
+// an image whose nearest distance to the run's box exceeds another's farthest
+// cannot be.  Returns the image of a particle left with one, else -1.  The others'
+// images are evaluated here, the smallest q' = q - W taken over them: with W the
+// largest of theirs, the pair's q lies in [q', q' + 2 W], as for a single image.
+// Pairs inside the window or below qm go to a guard word and to the queue, to be
+// counted by the drain.
+template <bool MULTI>
+__device__ __noinline__ int pick_round(const SegState& G, WarpList& W, unsigned mask, Pos p, int jl, bool valid,
+                                       int i_begin, int ni, float qm, int above, uint32_t* sh, int lane, int& qcount) {
+  const FrameDev& F = *G.F;
+  const float3 h = W.R.h;
+  float far = INFINITY;
+  bool below = false;  // some image has every pair below the sweep: so has the shortest
+  for (unsigned k = mask; k; k &= k - 1u) {
+    const Pos o = image_origin(F, __ffs(k) - 1, W.R.c, G.grid);
+    const float x = fabsf(p.h.x + o.h.x) + h.x, y = fabsf(p.h.y + o.h.y) + h.y, z = fabsf(p.h.z + o.h.z) + h.z;
+    const float f = x * x + y * y + z * z;
+    far = fminf(far, f);
+    if (MULTI) below = below || f < G.rc_lo2;
+  }
+  const float reach = sqrtf(far) * (1.0f + 0x1p-15f) + G.abs;
+  const float lim = fminf(reach * reach, G.rc_hi2);
+  unsigned cand = 0u;
+  if (valid && !below)
+    for (unsigned k = mask; k; k &= k - 1u) {
+      const Pos o = image_origin(F, __ffs(k) - 1, W.R.c, G.grid);
+      const float x = fmaxf(fabsf(p.h.x + o.h.x) - h.x, 0.0f), y = fmaxf(fabsf(p.h.y + o.h.y) - h.y, 0.0f),
+                  z = fmaxf(fabsf(p.h.z + o.h.z) - h.z, 0.0f);
+      if (x * x + y * y + z * z <= lim) cand |= k & (0u - k);
+    }
+  const int single = __popc(cand) == 1 ? __ffs(cand) - 1 : -1;
+  if (single >= 0) cand = 0u;
+  if (!__any_sync(kFull, cand != 0u)) return single;
+
+  IPos ip;
+  fetch_run(G, i_begin, ni, lane, ip);
+  IRegs I;
+  load_run(ip, W.R.c, ni, lane, I);
+  float2 x2[2], y2[2], z2[2], w2[2];  // factors of i particles (0, 1) and (2, 3)
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    x2[r] = make_float2(I.x[2 * r].x, I.x[2 * r + 1].x);
+    y2[r] = make_float2(I.y[2 * r].x, I.y[2 * r + 1].x);
+    z2[r] = make_float2(I.z[2 * r].x, I.z[2 * r + 1].x);
+    w2[r] = make_float2(I.w[2 * r].x, I.w[2 * r + 1].x);
+  }
+  const float chi = (float)(G.hi + 1 + lane), clo = (float)(G.lo - lane);
+  const float v1 = -2.0f * W.R.c1 * (1.0f + 0x1p-10f), v0 = 2.0f * W.R.c0 * (1.0f + 0x1p-10f);
+  const int first = __float_as_int(kMagicRound) + G.lo + 1;
+  while (__any_sync(kFull, cand != 0u)) {
+    // as many of the particles left, in lane order, as fit
+    const int c = __popc(cand);
+    int end = c;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(kFull, end, o);
+      if (lane >= o) end += t;
+    }
+    const bool now = c > 0 && end <= kPickCap;
+    const int count = __reduce_max_sync(kFull, end <= kPickCap ? end : 0);
+    if (now) {
+      int s = end - c;
+      for (; cand; cand &= cand - 1u, ++s) {
+        const int m = __ffs(cand) - 1;
+        W.M[s] = j_image(p, image_origin(F, m, W.R.c, G.grid), W.R.c1, W.R.c0);
+        W.mref[s] = (uint32_t)jl | (s == end - 1 ? kLastImage : 0u);
+      }
+    }
+    __syncwarp();
+    float2 nq[2] = {bc2(-INFINITY), bc2(-INFINITY)};
+    float win = 0.0f;
+    for (int s = 0; s < count; ++s) {
+      const float4 y = W.M[s];
+      const uint32_t ref = W.mref[s];
+      win = fmaxf(win, __fmaf_rn(y.w, v1, v0));
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float2 t =
+            add2(fma2(bc2(y.x), x2[r], fma2(bc2(y.y), y2[r], fma2(bc2(y.z), z2[r], w2[r]))), bc2(y.w));
+        nq[r] = make_float2(fmaxf(nq[r].x, t.x), fmaxf(nq[r].y, t.y));
+      }
+      if (!(ref & kLastImage)) continue;
+      const int j = (int)(ref & ~kLastImage);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float v = (r & 1) ? nq[r >> 1].y : nq[r >> 1].x;
+        const int il = lane + 32 * r;
+        const bool ok = il < ni && j > above + il;
+        float sc = fminf(sqrt_approx(fabsf(v)), chi);
+        if (MULTI) sc = fmaxf(sc, clo);
+        const float sm = __fadd_rn(sc, kMagicRound);
+        const float n = __fadd_rn(sm, -kMagicRound);
+        const float e = __fmaf_rn(n, n, v);
+        const bool defer = ok && (-v < qm || __float_as_uint(e) < __float_as_uint(win));
+        const int rel = __float_as_int(sm) + (int)(__float_as_uint(e) >> 31) - first;
+        atomicAdd(sh + (ok && !defer ? rel : G.hi - G.lo + lane), 1u);
+        const unsigned bal = __ballot_sync(kFull, defer);
+        if (bal) {
+          if (defer)
+            W.queue[qcount + __popc(bal & ((1u << lane) - 1u))] =
+                make_uint2((uint32_t)j | kAnyImage, (uint32_t)(i_begin + il));
+          qcount += __popc(bal);
+          if (qcount >= 32) qcount = list_drain(G, W, qcount, sh, lane);
+        }
+      }
+      nq[0] = nq[1] = bc2(-INFINITY);
+      win = 0.0f;
+    }
+    __syncwarp();
+  }
+  return single;
+}
+
 // Every pair of an item in binary64 (frames whose images cannot be listed).
 __device__ __noinline__ void slow_item(const SegState& G, int ib, int ni, int jbeg, int jend, uint32_t* sh, int lane) {
   FrameDev* const Fp = G.F;
@@ -549,7 +707,8 @@ __device__ __forceinline__ void item_of(const SegState& G, int split, long long 
 
 // One block of 16 warps with 128 registers per SM: the pair loop and the list
 // state stay in registers, and the SM merges one histogram per segment.
-template <bool MULTI>
+// PICK: frames whose pairs take the shortest of several images (pick_round).
+template <bool MULTI, bool PICK>
 __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int BLOCK = kListBlock, kWarps = BLOCK / 32;
@@ -671,7 +830,22 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
                           fz = fmaxf(fabsf(lz), fabsf(uz)) + h.z;
               g2 = gx * gx + gy * gy + gz * gz;
               f2 = fx * fx + fy * fy + fz * fz;
-              keep = g2 <= G.rc_hi2 && f2 >= G.rc_lo2;
+              keep = g2 <= G.rc_hi2 && (PICK || f2 >= G.rc_lo2);
+            }
+            unsigned picked = 0u;  // PICK: several images, handled particle by particle
+            float qm_pick = 0.0f;
+            if (PICK) {
+              const bool img = lane < G.n_img && jbeg < jend;
+              float far = img ? f2 : INFINITY, wide = keep ? f2 : 0.0f;
+              for (int o = 16; o > 0; o >>= 1) far = fminf(far, __shfl_xor_sync(kFull, far, o));
+              // only images nearer than the farthest pair of another; none when one puts
+              // every pair below the sweep
+              const float reach = sqrtf(far) * (1.0f + 0x1p-15f) + 2.0f * G.abs;
+              keep = keep && g2 <= reach * reach && far >= G.rc_lo2;
+              wide = keep ? f2 : 0.0f;
+              for (int o = 16; o > 0; o >>= 1) wide = fmaxf(wide, __shfl_xor_sync(kFull, wide, o));
+              const float wm = 2.0f * __fmaf_rn(W.R.c1, wide, W.R.c0) + 1.0f;
+              qm_pick = G.all ? INFINITY : wm * wm;
             }
             unsigned mask = __ballot_sync(kFull, keep);
             if (lane == 0) {  // statistics
@@ -691,9 +865,27 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
             bool close = false, in_here = false;
             for (;;) {
               int want = kBlk;
-              if (jb >= jend && mask) {
+              if (PICK && jb >= jend && (mask & (mask - 1u))) {
+                picked = mask;
+                mask = 0u;
+                // the window bound over all of them, and their nearest
+                float near2 = keep ? g2 : INFINITY;
+                for (int o = 16; o > 0; o >>= 1) near2 = fminf(near2, __shfl_xor_sync(kFull, near2, o));
+                close = !(sqrtf(near2) - G.abs >= sqrtf(qm_pick) + 2.0f);
+                in_here = false;
+                near = near || close;
+                inner = false;
+                __syncwarp();
+                if (lane == 0) {
+                  W.qm_here = close ? qm_pick : 0.0f;
+                  W.qm = fmaxf(W.qm, W.qm_here);
+                }
+                __syncwarp();
+                jb = jbeg;
+              } else if (jb >= jend && mask) {
                 const int ml = __ffs(mask) - 1;
                 mask &= mask - 1u;
+                picked = 0u;
                 m = G.n_img == 1 ? kHome : ml;
                 // near: some q' may lie below (2 W + 1)^2, W at the farthest corner;
                 // inner: every pair in the sweep
@@ -727,12 +919,17 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
                 pf = jb < jend ? jb : (mask ? jbeg : jend);
                 pa = __ldg(G.P4j + min(pf + lane, nj - 1));
                 pb = __ldg(G.P2j + min(pf + lane, nj - 1));
-                const float4 y = j_image(p, W.o, W.R.c1, W.R.c0);
+                if (PICK && picked) {
+                  m = pick_round<MULTI>(G, W, picked, p, jl, jl < jend, i_begin, ni, qm_pick,
+                                        diag ? i_begin : -(1 << 30), sh, lane, qcount);
+                }
+                const float4 y =
+                    j_image(p, PICK && picked ? image_origin(F, max(m, 0), W.R.c, G.grid) : W.o, W.R.c1, W.R.c0);
                 const float3 h = W.R.h;
                 const float ax = fabsf(y.x), ay = fabsf(y.y), az = fabsf(y.z);
                 const float gx = fmaxf(ax - h.x, 0.0f), gy = fmaxf(ay - h.y, 0.0f), gz = fmaxf(az - h.z, 0.0f);
-                bool in = jl < jend && gx * gx + gy * gy + gz * gz <= G.rc_hi2;
-                if (MULTI) {
+                bool in = jl < jend && m >= 0 && gx * gx + gy * gy + gz * gz <= G.rc_hi2;
+                if (MULTI) {  // (for a single image the same as below the sweep)
                   const float fx = ax + h.x, fy = ay + h.y, fz = az + h.z;
                   in = in && fx * fx + fy * fy + fz * fz >= G.rc_lo2;
                 }
@@ -844,11 +1041,12 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
   }
 }
 
-template <bool MULTI>
+template <bool MULTI, bool PICK>
 cudaError_t launch_list_t(const ListLaunch& p, int grid, size_t smem, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(list_kernel<MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e =
+      cudaFuncSetAttribute(list_kernel<MULTI, PICK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  list_kernel<MULTI><<<grid, kListBlock, smem, stream>>>(p);
+  list_kernel<MULTI, PICK><<<grid, kListBlock, smem, stream>>>(p);
   return cudaGetLastError();
 }
 
@@ -870,7 +1068,9 @@ int list_kernel_max_width() {
 cudaError_t launch_list(const ListLaunch& p, int grid, cudaStream_t stream) {
   (void)cudaGetLastError();
   const size_t smem = list_kernel_smem(p.hist_width);
-  return p.multi ? launch_list_t<true>(p, grid, smem, stream) : launch_list_t<false>(p, grid, smem, stream);
+  if (p.pick)
+    return p.multi ? launch_list_t<true, true>(p, grid, smem, stream) : launch_list_t<false, true>(p, grid, smem, stream);
+  return p.multi ? launch_list_t<true, false>(p, grid, smem, stream) : launch_list_t<false, false>(p, grid, smem, stream);
 }
 
 }  // namespace dh

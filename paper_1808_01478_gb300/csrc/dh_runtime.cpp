@@ -213,10 +213,23 @@ dh_status check_frame(const dh_frame* f, PlannedFrame& pf, int max_width, int li
   // Two images of a particle are at least the smallest plane spacing apart, so
   // with r_max up to half of it one image of a pair at most lies inside
   // (orthorhombic: a tie of two images at exactly L/2 is re-decided, with room
-  // for the rounding of r_max = L/2).
-  pf.list = list_width > 0 && f->n <= kListMaxN &&
-            (pf.variant == V_NONE || pf.variant == V_TRIC ||
-             (pf.variant == V_ORTHO && f->r_max <= 0.5 * std::min(B[0], std::min(B[4], B[8])) * (1.0 + 0x1p-40)));
+  // for the rounding of r_max = L/2).  Beyond, the shortest image counts
+  // (pf.pick).  It is the definition's, the shortest of the 27 around the rounded
+  // fractional coordinates, for every orthorhombic box, and for a triclinic one
+  // whose half diagonal of (a_x, b_y, c_z), an upper bound of the shortest image's
+  // length, is below the smallest plane spacing h: the 27 contain Babai's vector
+  // (within that bound), and an image two cells away on some axis is at least
+  // 1.5 h long.  The fractional coordinates of the shortest image are then below 1
+  // in magnitude, so images of home positions differ by at most one cell per axis.
+  const bool in_half =
+      pf.variant == V_NONE || pf.variant == V_TRIC ||
+      (pf.variant == V_ORTHO && f->r_max <= 0.5 * std::min(B[0], std::min(B[4], B[8])) * (1.0 + 0x1p-40));
+  const bool compact =
+      pf.variant == V_ORTHO ||
+      (pf.variant == V_TRIC_SEARCH &&
+       0.5 * std::sqrt(B[0] * B[0] + B[4] * B[4] + B[8] * B[8]) <= 0.9995 * min_plane_spacing(B));
+  pf.list = list_width > 0 && f->n <= kListMaxN && (in_half || compact);
+  pf.pick = !in_half;
   if (pf.list) max_width = std::min(max_width, list_width);
   int64_t S = f->n_species;
   pf.src = f;
@@ -276,7 +289,8 @@ void fill_frame_dev(const PlannedFrame& pf, FrameDev& F, const float4* X, uint64
     F.smin[c] = F.cmin[c];
     F.smax[c] = F.cmax[c];
   }
-  if (pf.variant == V_ORTHO || pf.variant == V_TRIC) {
+  F.pick = pf.pick ? 1 : 0;
+  if (pf.variant != V_NONE) {
     // image vectors -B k, in bins as double-floats, and the rounding errors (the
     // binary64 sum itself errs by at most 2^-52 of the row sum)
     for (int c = 0; c < 3; ++c) F.period[c] = (float)(S * F.B[4 * c]);
@@ -315,7 +329,7 @@ std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, const FrameDev* 
   std::vector<SortSeg> out;
   *keys = 0;
   *max_n = 0;
-  if (pf.variant == V_TRIC_SEARCH) return out;
+  if (pf.variant == V_TRIC_SEARCH && !pf.list) return out;
   const int64_t* o = pf.src->species_offsets;
   int64_t runs = 0;
   for (int a = 0; a < pf.src->n_species; ++a) {
@@ -521,9 +535,14 @@ struct CallPlan {
   size_t seg_bytes = 0;          // Segment array in the metadata
   size_t lseg_bytes = 0;         // ListSegment array after it
   int n_lsegs = 0;
-  int64_t litems = 0;            // list-kernel launch: items,
-  int lwidth = 1, lmulti = 0;    //   widest sweep, some sweep above bin 0,
-  int lgrid = 0, lsplit = 1;     //   blocks, items per run pair
+  // list-kernel launches: frames with one image of a pair inside r_max, and the
+  // others (PlannedFrame.pick): first segment and segments, items, widest sweep,
+  // some sweep above bin 0, blocks, items per run pair
+  struct ListPlan {
+    int seg0 = 0, n_segs = 0;
+    int64_t items = 0;
+    int width = 1, multi = 0, grid = 0, split = 1;
+  } list[2];
   int n_sort = 0;                // spatial-order segments (after the segments in the metadata)
   int64_t sort_max = 0;          // largest of them
   int64_t sort_keys = 0;         // counters over all of them
@@ -570,14 +589,15 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   }
   // frames the list kernel takes: those it can run, unless a measured shape says otherwise
   auto on_list = [&](int f) { return pfs[f].list && P.vparams[pfs[f].variant].list; };
-  double lrun_pairs = 0.0;
+  double lrun_pairs[2] = {0.0, 0.0};
   for (int f = 0; f < k; ++f)
     if (on_list(f)) {
-      P.lwidth = std::max(P.lwidth, pfs[f].sweep_width);
-      P.lmulti |= pfs[f].sweeps > 1;
-      lrun_pairs += (double)pfs[f].pairs / ((double)kRun * kRun) * pfs[f].sweeps;
+      CallPlan::ListPlan& lp = P.list[pfs[f].pick];
+      lp.width = std::max(lp.width, pfs[f].sweep_width);
+      lp.multi |= pfs[f].sweeps > 1;
+      lrun_pairs[pfs[f].pick] += (double)pfs[f].pairs / ((double)kRun * kRun) * pfs[f].sweeps;
     }
-  P.lsplit = list_split_for(lrun_pairs, c->num_sms);
+  for (int g = 0; g < 2; ++g) P.list[g].split = list_split_for(lrun_pairs[g], c->num_sms);
   VariantSummary told[kNumVariants];  // what the tiled kernel is left with
   for (int f = 0; f < k; ++f)
     if (!on_list(f)) {
@@ -593,20 +613,26 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   auto plan_segments = [&](FrameDev* dF) {
     segs.clear();
     lsegs.clear();
-    P.litems = 0;
-    for (int f = 0; f < k; ++f)
-      if (on_list(f)) P.litems += add_list_segments(pfs[f], dF + f, P.litems, lsegs, P.lsplit);
-    if (c->tune_forced && c->tune_cap_pairs > 0.0) {  // a measurement: the first items only
-      int64_t left = (int64_t)std::ceil(c->tune_cap_pairs / ((double)kRun * kRun)) * P.lsplit;
-      P.litems = 0;
-      for (ListSegment& g : lsegs) {
-        g.items = std::min(g.items, left);
-        left -= g.items;
-        P.litems += g.items;
+    P.n_items = 0;
+    for (int g = 0; g < 2; ++g) {
+      CallPlan::ListPlan& lp = P.list[g];
+      lp.seg0 = (int)lsegs.size();
+      lp.items = 0;
+      for (int f = 0; f < k; ++f)
+        if (on_list(f) && (int)pfs[f].pick == g) lp.items += add_list_segments(pfs[f], dF + f, lp.items, lsegs, lp.split);
+      lp.n_segs = (int)lsegs.size() - lp.seg0;
+      if (c->tune_forced && c->tune_cap_pairs > 0.0) {  // a measurement: the first items only
+        int64_t left = (int64_t)std::ceil(c->tune_cap_pairs / ((double)kRun * kRun)) * lp.split;
+        lp.items = 0;
+        for (int q = lp.seg0; q < lp.seg0 + lp.n_segs; ++q) {
+          lsegs[q].items = std::min(lsegs[q].items, left);
+          left -= lsegs[q].items;
+          lp.items += lsegs[q].items;
+        }
       }
+      P.n_items += lp.items;
     }
     P.n_lsegs = (int)lsegs.size();
-    P.n_items = P.litems;
     for (int v = 0; v < kNumVariants; ++v) {
       P.vseg0[v] = segs.size();
       P.vitems[v] = 0;
@@ -683,7 +709,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     J.stride = (fr->flags & DH_COORDS_F4) ? 4 : 3;
     J.src = host_coords ? (const float*)((const unsigned char*)c->raw.p + P.raw_off[f]) : fr->coords;
     // staged for the spatial order, or in place where there is none
-    const bool sorted = pfs[f].variant != V_TRIC_SEARCH;
+    const bool sorted = pfs[f].variant != V_TRIC_SEARCH || pfs[f].list;
     J.dst = (float4*)(sorted ? c->sortX.p : c->X.p) + xoff[f];
     J.dst64 = (fr->flags & DH_COORDS_F64) ? (double4*)(sorted ? c->sortX64.p : c->X64.p) + xoff[f] : nullptr;
     J.fd = dF + f;
@@ -716,7 +742,8 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     P.vwidth[v] = width;
     P.vgrid[v] = pair_grid(c->num_sms, lp.bps, P.vitems[v]);
   }
-  if (with_pairs && P.litems > 0) P.lgrid = pair_grid(c->num_sms, 1, P.litems);
+  for (auto& lp : P.list)
+    if (with_pairs && lp.items > 0) lp.grid = pair_grid(c->num_sms, 1, lp.items);
   return DH_OK;
 }
 
@@ -755,7 +782,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   // A2-A8: per variant, one persistent launch over its frames, species pairs and bin sweeps
   int grid = 0, top = -1;
   int64_t top_items = 0;
-  bool any = P.lgrid > 0;
+  bool any = P.list[0].grid > 0 || P.list[1].grid > 0;
   for (int v = 0; v < kNumVariants; ++v) any |= P.vgrid[v] > 0;
   // timing events: inside a stream capture they must become event-record nodes
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -764,20 +791,23 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   if (any) {
     DH_CUDA_TRY(cudaMemsetAsync(c->ctl.p, 0, sizeof(Control) * kNumVariants + sizeof(SegCounter) * (size_t)P.n_lsegs, st));
     if (c->ev_pair0) DH_CUDA_TRY(cudaEventRecordWithFlags(c->ev_pair0, st, ev_flags));
-    if (P.lgrid > 0) {
+    for (int g = 0; g < 2; ++g) {
+      const CallPlan::ListPlan& lp = P.list[g];
+      if (lp.grid == 0) continue;
       ListLaunch L;
       std::memset(&L, 0, sizeof L);
-      L.segs = (const ListSegment*)((unsigned char*)dS + P.seg_bytes);
-      L.ctr = (SegCounter*)((unsigned char*)c->ctl.p + sizeof(Control) * kNumVariants);
-      L.n_segs = P.n_lsegs;
-      L.hist_width = P.lwidth;
-      L.n_items = P.litems;
-      L.split = P.lsplit;
-      L.multi = P.lmulti;
-      DH_CUDA_TRY(launch_list(L, P.lgrid, st));
+      L.segs = (const ListSegment*)((unsigned char*)dS + P.seg_bytes) + lp.seg0;
+      L.ctr = (SegCounter*)((unsigned char*)c->ctl.p + sizeof(Control) * kNumVariants) + lp.seg0;
+      L.n_segs = lp.n_segs;
+      L.hist_width = lp.width;
+      L.n_items = lp.items;
+      L.split = lp.split;
+      L.multi = lp.multi;
+      L.pick = g;
+      DH_CUDA_TRY(launch_list(L, lp.grid, st));
       ++launched;
-      grid = P.lgrid;
-      top_items = P.litems / P.lsplit / 64;  // in tiles of the other kernel
+      grid = std::max(grid, lp.grid);
+      top_items += lp.items / lp.split / 64;  // in tiles of the other kernel
     }
     for (int v = 0; v < kNumVariants; ++v) {
       if (P.vgrid[v] == 0) continue;
@@ -816,7 +846,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   S.items = (int32_t)std::min<int64_t>(P.n_items, 0x7FFFFFFF);
   S.kernel_launches = launched + P.launched;
   S.tune_runs = c->tune_runs;
-  if (top < 0 && P.lgrid > 0) {  // the list kernel: one histogram per block, no j tiles of its own
+  if (top < 0 && any) {  // the list kernel: one histogram per block, no j tiles of its own
     S.tile_j = kTile;
     S.hist_depth = 1;
     S.blocks_per_sm = 1;

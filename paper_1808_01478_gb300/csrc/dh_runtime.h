@@ -86,7 +86,8 @@ struct PlannedFrame {
   int32_t sweep_width;
   double margin;
   uint64_t pairs;
-  bool list;  // the list kernel can run it (one image of a pair at most inside r_max)
+  bool list;  // the list kernel can run it,
+  bool pick;  //   with the shortest of several images of a pair inside r_max
 };
 
 // list_width: bins per sweep of the list kernel, 0 when the caller has no list path.

@@ -582,11 +582,12 @@ bool Server::launch_wave(int v) {
   // wide request would otherwise give every request of the wave the shape of
   // the widest histogram: larger blocks and fewer of them per SM)
   std::vector<Segment> csegs[kWidthClasses];
-  std::vector<ListSegment> lsegs[kWidthClasses];
-  int64_t citems[kWidthClasses] = {}, litems[kWidthClasses] = {};
+  // (the list kernel's: one image of a pair inside r_max, then the others)
+  std::vector<ListSegment> lsegs[2 * kWidthClasses];
+  int64_t citems[kWidthClasses] = {}, litems[2 * kWidthClasses] = {};
   int cwidth[kWidthClasses], cmulti[kWidthClasses] = {};
-  int lwidth[kWidthClasses], lmulti[kWidthClasses] = {};
-  for (int q = 0; q < kWidthClasses; ++q) cwidth[q] = lwidth[q] = 1;
+  int lwidth[2 * kWidthClasses], lmulti[2 * kWidthClasses] = {};
+  for (int q = 0; q < kWidthClasses; ++q) cwidth[q] = lwidth[q] = lwidth[kWidthClasses + q] = 1;
   int64_t witems = 0;
   double wpairs = 0;
   std::vector<Request*> finishing;
@@ -617,21 +618,22 @@ bool Server::launch_wave(int v) {
       witems += b - a;
       csegs[cl].push_back(w);
     }
+    const int lcl = cl + (r->pf.pick ? kWidthClasses : 0);
     for (const ListSegment& sg : r->lsegs) {
       int64_t a = std::max(lo, sg.item0), b = std::min(hi, sg.item0 + sg.items);
       if (a >= b) continue;
       ListSegment w = sg;
-      w.item0 = litems[cl];
+      w.item0 = litems[lcl];
       w.item_base = a - sg.item0;
       w.items = b - a;
-      litems[cl] += b - a;
+      litems[lcl] += b - a;
       witems += b - a;
-      lsegs[cl].push_back(w);
+      lsegs[lcl].push_back(w);
     }
     r->next = hi;
     r->last_wave = ln.wave_seq + 1;
-    int& width = r->pf.list ? lwidth[cl] : cwidth[cl];
-    int& multi = r->pf.list ? lmulti[cl] : cmulti[cl];
+    int& width = r->pf.list ? lwidth[lcl] : cwidth[cl];
+    int& multi = r->pf.list ? lmulti[lcl] : cmulti[cl];
     width = std::max(width, r->pf.sweep_width);
     multi |= r->pf.sweeps > 1;
     wpairs += (double)std::min<uint64_t>(r->pf.pairs, (uint64_t)((double)take * r->pairs_per_item));
@@ -640,10 +642,8 @@ bool Server::launch_wave(int v) {
   if (witems == 0) return false;
   // descriptors: the tiled kernel's segments, then the list kernel's
   size_t nseg = 0, nlseg = 0;
-  for (int q = 0; q < kWidthClasses; ++q) {
-    nseg += csegs[q].size();
-    nlseg += lsegs[q].size();
-  }
+  for (int q = 0; q < kWidthClasses; ++q) nseg += csegs[q].size();
+  for (const auto& l : lsegs) nlseg += l.size();
   const size_t bytes = sizeof(Segment) * nseg + sizeof(ListSegment) * nlseg;
   const size_t ctl_bytes = sizeof(Control) * kWidthClasses + sizeof(SegCounter) * nlseg;
   if (W.segs.ensure(bytes) != cudaSuccess || W.hsegs.ensure(bytes) != cudaSuccess ||
@@ -657,7 +657,7 @@ bool Server::launch_wave(int v) {
     at += csegs[q].size();
   }
   at = 0;
-  for (int q = 0; q < kWidthClasses; ++q) {
+  for (int q = 0; q < 2 * kWidthClasses; ++q) {
     ListSegment* hl = (ListSegment*)((Segment*)W.hsegs.p + nseg);
     if (!lsegs[q].empty()) std::memcpy(hl + at, lsegs[q].data(), sizeof(ListSegment) * lsegs[q].size());
     at += lsegs[q].size();
@@ -667,7 +667,7 @@ bool Server::launch_wave(int v) {
   cudaEventRecord(W.ev0, ln.stream);
   cudaError_t e = cudaSuccess;
   at = 0;
-  for (int q = 0; q < kWidthClasses && e == cudaSuccess; ++q) {
+  for (int q = 0; q < 2 * kWidthClasses && e == cudaSuccess; ++q) {
     if (lsegs[q].empty()) continue;
     ListLaunch L;
     std::memset(&L, 0, sizeof L);
@@ -678,6 +678,7 @@ bool Server::launch_wave(int v) {
     L.n_items = litems[q];
     L.split = 1;
     L.multi = lmulti[q];
+    L.pick = q >= kWidthClasses;
     e = launch_list(L, pair_grid(ctx_->num_sms, 1, litems[q]), ln.stream);
     at += lsegs[q].size();
   }

@@ -84,3 +84,28 @@ def test_half_box_lattice_and_coincident_particles(oracle_mod):
     x = np.concatenate([x, x[::2]]).copy()
     for nbins in (8, 16, 1024):
         check(oracle_mod, x, [0, 400, len(x)], "lattice", 8.0, nbins)
+
+
+@pytest.mark.parametrize("sizes", [[1, 128], [129, 0, 31], [640, 5], [3000, 129]], ids=lambda s: "-".join(map(str, s)))
+@pytest.mark.parametrize("kind,reach", [("ortho", 1.02), ("ortho", 1.7), ("ortho", 4.0), ("tric", 1.0), ("tric", 1.6),
+                                        ("tric", 3.0)])
+def test_r_max_beyond_half_the_image_distance(oracle_mod, kind, reach, sizes):
+    # several images of a pair inside r_max: the shortest counts
+    offs = np.concatenate([[0], np.cumsum(sizes)])
+    check(oracle_mod, uniform(kind, int(offs[-1]), 15), offs, kind, reach * half(kind), 801)
+
+
+@pytest.mark.parametrize("kind", ["ortho", "tric"])
+@pytest.mark.parametrize("nbins", [2, 50_000, 110_000])
+def test_shortest_image_over_sweeps_and_cells(oracle_mod, kind, nbins):
+    rng = w.rng_for(16)
+    m = w.box_matrix(BOX[kind][1])
+    x = (m @ rng.random((900, 3)).T).T + rng.integers(-3, 4, (900, 3)).astype(np.float64) @ m.T
+    check(oracle_mod, x.astype(np.float32), [0, 350, 900], kind, 1.5 * half(kind), nbins)
+
+
+def test_cells_whose_27_images_can_miss_the_shortest(oracle_mod):
+    # a flat cell: the definition's minimum over 27 shifts is not the lattice's
+    BOX["flat"] = (w.BOX_TRICLINIC, np.array([10.0, 4.0, 4.9, 0.0, 9.0, 4.4, 0.0, 0.0, 2.0]))
+    x = w.uniform_in_cell(w.rng_for(17), 600, BOX["flat"][1])
+    check(oracle_mod, x, [0, 200, 600], "flat", 5.0, 300)
