@@ -224,7 +224,7 @@ __device__ __noinline__ int exact_listed_bin(const FrameDev& F, int i, int j, fl
 // c_z, b_y, a_x (Babai's step; see exact_r2), or known to be (F.pick: the listed
 // image is the shortest by a margin).  Otherwise, and when q is too close to n^2,
 // the binary64 replay decides.
-__device__ __forceinline__ int listed_bin(const FrameDev& F, int i, int j, int m, float& n, unsigned& nexact) {
+__device__ __noinline__ int listed_bin(const FrameDev& F, int i, int j, int m, float& n, unsigned& nexact) {
   const Pos a = unpack(__ldg(F.P4 + i), __ldg(F.P2 + i)), b = unpack(__ldg(F.P4 + j), __ldg(F.P2 + j));
   const float ah[3] = {a.h.x, a.h.y, a.h.z}, al[3] = {a.l.x, a.l.y, a.l.z};
   const float bh[3] = {b.h.x, b.h.y, b.h.z}, bl[3] = {b.l.x, b.l.y, b.l.z};
@@ -277,12 +277,14 @@ __device__ __noinline__ int picked_bin(const FrameDev& F, int i, int j, unsigned
   return exact_listed_bin(F, i, j, make_float3(0.f, 0.f, 0.f), true);
 }
 
+__device__ float4 run_factor(const SegState& G, int i, int end, float3 c);
+
 // The word in which the pair loop counted a pair close to its run (q' below
 // (2 W + 1)^2 or nearly): the scalar replay of its float32 arithmetic.
 __device__ __noinline__ int replay_rel(const SegState& G, int i, int j, int m) {
   const FrameDev& F = *G.F;
   const RunState R = run_state(G, __ldg(G.bi + 2 * (i / kRun)), __ldg(G.bi + 2 * (i / kRun) + 1));
-  const float4 x = i_factors(unpack(__ldg(G.P4i + i), __ldg(G.P2i + i)), R.c);
+  const float4 x = run_factor(G, i, i + 1, R.c);
   const float4 y = j_image(unpack(__ldg(G.P4j + j), __ldg(G.P2j + j)), image_origin(F, m, R.c, G.grid), R.c1, R.c0);
   const float nq = __fadd_rn(__fmaf_rn(y.x, x.x, __fmaf_rn(y.y, x.y, __fmaf_rn(y.z, x.z, x.w))), y.w);
   const int lane = i & 31;
@@ -345,23 +347,17 @@ __device__ __noinline__ int list_drain(const SegState& G, WarpList& W, int qcoun
 struct IRegs {
   float2 x[4], y[4], z[4], w[4];
 };
-struct IPos {
-  float4 a[4];
-  float2 b[4];
-};
-__device__ __forceinline__ void fetch_run(const SegState& G, int i_begin, int ni, int lane, IPos& p) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = i_begin + min(lane + 32 * r, ni - 1);
-    p.a[r] = __ldg(G.P4i + i);
-    p.b[r] = __ldg(G.P2i + i);
-  }
+// The factors of i particle i of the run with centre c, NaN beyond its end.  One
+// copy of the arithmetic: the executed code has to stay in the instruction cache.
+__device__ __noinline__ float4 run_factor(const SegState& G, int i, int end, float3 c) {
+  const int k = min(i, end - 1);
+  const float4 x = i_factors(unpack(__ldg(G.P4i + k), __ldg(G.P2i + k)), c);
+  return i < end ? x : make_float4(NAN, NAN, NAN, NAN);
 }
-__device__ __forceinline__ void load_run(const IPos& p, float3 c, int ni, int lane, IRegs& I) {
+__device__ __forceinline__ void load_run(const SegState& G, float3 c, int i_begin, int ni, int lane, IRegs& I) {
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
-    float4 x = i_factors(unpack(p.a[r], p.b[r]), c);
-    if (lane + 32 * r >= ni) x = make_float4(NAN, NAN, NAN, NAN);
+    const float4 x = run_factor(G, i_begin + lane + 32 * r, i_begin + ni, c);
     I.x[r] = bc2(x.x);
     I.y[r] = bc2(x.y);
     I.z[r] = bc2(x.z);
@@ -434,11 +430,12 @@ __device__ __forceinline__ int push_pairs(const SegState& G, WarpList& W, int s0
 // images all of whose pairs lie in the sweep, no clamp needed.  NEAR: images so near the run that q' may
 // be below qm = (2 W + 1)^2, where the window can hold several edges: those pairs
 // are re-decided too; and with above >= 0, only particles j > above + i (the
-// diagonal item of one species; else above = -2^30).
+// diagonal item of one species; else above = -2^30).  Returns this lane's groups
+// with pairs to re-decide.
 enum BlockMode { PLAIN, INNER, NEARBY };
 template <BlockMode MODE, bool MULTI>
-__device__ __forceinline__ int list_block(const SegState& G, const IRegs& I, WarpList& W, int i_begin, int s0, int n,
-                                          float qm, int above, uint32_t* sh, int lane, int qcount) {
+__device__ __forceinline__ uint32_t list_block(const SegState& G, const IRegs& I, WarpList& W, int s0, int n, float qm,
+                                               int above, uint32_t* sh, int lane) {
   constexpr bool NEAR = MODE == NEARBY;
   const int lo = G.lo, hi = G.hi;
   const uint32_t hbase =
@@ -452,7 +449,7 @@ __device__ __forceinline__ int list_block(const SegState& G, const IRegs& I, War
   for (int g = 0; g < n; g += 8) {
     const int sg = s0 + g;
     uint32_t dmask = 0u;
-#pragma unroll
+#pragma unroll(NEAR ? 1 : 4)
     for (int u = 0; u < 8; u += 2) {
       const float4 A = W.A[(sg + u) >> 1], Bv = W.B[(sg + u) >> 1];
       const float2 yx = make_float2(A.x, A.y), yy = make_float2(A.z, A.w), yz = make_float2(Bv.x, Bv.y),
@@ -485,18 +482,16 @@ __device__ __forceinline__ int list_block(const SegState& G, const IRegs& I, War
     W.mask[g >> 3][lane] = dmask;
     if (dmask) groups |= 1u << (g >> 3);
   }
-  return push_pairs(G, W, s0, groups, (uint32_t)i_begin | (NEAR ? kNearPair : 0u), sh, lane, qcount);
+  return groups;
 }
 
-// The near form out of line (it loads the run again).
+// The near form out of line (it loads the run again) and not unrolled.
 template <bool MULTI>
-__device__ __noinline__ int list_near(const SegState& G, WarpList& W, int i_begin, int ni, int s0, int n, float qm,
-                                      int above, uint32_t* sh, int lane, int qcount) {
-  IPos p;
-  fetch_run(G, i_begin, ni, lane, p);
+__device__ __noinline__ uint32_t list_near(const SegState& G, WarpList& W, int i_begin, int ni, int s0, int n, float qm,
+                                           int above, uint32_t* sh, int lane) {
   IRegs I;
-  load_run(p, W.R.c, ni, lane, I);
-  return list_block<NEARBY, MULTI>(G, I, W, i_begin, s0, n, qm, above, sh, lane, qcount);
+  load_run(G, W.R.c, i_begin, ni, lane, I);
+  return list_block<NEARBY, MULTI>(G, I, W, s0, n, qm, above, sh, lane);
 }
 
 // Frames whose r_max exceeds half the distance between images (F.pick): a pair's
@@ -539,10 +534,8 @@ __device__ __noinline__ int pick_round(const SegState& G, WarpList& W, unsigned 
   if (single >= 0) cand = 0u;
   if (!__any_sync(kFull, cand != 0u)) return single;
 
-  IPos ip;
-  fetch_run(G, i_begin, ni, lane, ip);
   IRegs I;
-  load_run(ip, W.R.c, ni, lane, I);
+  load_run(G, W.R.c, i_begin, ni, lane, I);
   float2 x2[2], y2[2], z2[2], w2[2];  // factors of i particles (0, 1) and (2, 3)
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -792,13 +785,11 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
         float4 pa = __ldg(G.P4j + min(pf + lane, nj - 1));
         float2 pb = __ldg(G.P2j + min(pf + lane, nj - 1));
         {
-          IPos p;
-          fetch_run(G, i_begin, ni, lane, p);
           const RunState R = run_state(G, __ldg(G.bi + 2 * ri), __ldg(G.bi + 2 * ri + 1));
           __syncwarp();
           if (lane == 0) W.R = R;
           __syncwarp();
-          load_run(p, R.c, ni, lane, I);
+          load_run(G, R.c, i_begin, ni, lane, I);
         }
         int tail = 0, done = 0;
         // the list's images: none near the run, every pair in the sweep
@@ -957,13 +948,17 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
               }
               __syncwarp();
               if (!more || tail - done >= kBlk) {
-                if (near || diag)
-                  qcount = list_near<MULTI>(G, W, i_begin, ni, done & (kCap - 1), want, W.qm, diag ? i_begin : -(1 << 30),
-                                            sh, lane, qcount);
-                else if (inner && more && ni == kRun && G.inner)
-                  qcount = list_block<INNER, MULTI>(G, I, W, i_begin, done & (kCap - 1), kBlk, 0.0f, 0, sh, lane, qcount);
-                else
-                  qcount = list_block<PLAIN, MULTI>(G, I, W, i_begin, done & (kCap - 1), want, 0.0f, 0, sh, lane, qcount);
+                const int s0 = done & (kCap - 1);
+                uint32_t groups, first = (uint32_t)i_begin;
+                if (near || diag) {
+                  groups = list_near<MULTI>(G, W, i_begin, ni, s0, want, W.qm, diag ? i_begin : -(1 << 30), sh, lane);
+                  first |= kNearPair;
+                } else if (inner && more && ni == kRun && G.inner) {
+                  groups = list_block<INNER, MULTI>(G, I, W, s0, kBlk, 0.0f, 0, sh, lane);
+                } else {
+                  groups = list_block<PLAIN, MULTI>(G, I, W, s0, want, 0.0f, 0, sh, lane);
+                }
+                qcount = push_pairs(G, W, s0, groups, first, sh, lane, qcount);
                 done += kBlk;
                 // what is left was appended in this round
                 near = (more && close) || G.all;
