@@ -102,6 +102,11 @@ __device__ __forceinline__ DF two_sum(float a, float b) {
   float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
   return {s, e};
 }
+// The multiple of the grid (a power of two) nearest to v (|v| < 2^22 steps).
+__device__ __forceinline__ float on_grid(float v, float grid) {
+  const float m = kMagicRound * grid;
+  return __fsub_rn(__fadd_rn(v, m), m);
+}
 __device__ __forceinline__ DF two_prod(float a, float b) {
   float p = __fmul_rn(a, b);
   return {p, __fmaf_rn(a, b, -p)};

@@ -45,7 +45,7 @@ struct FrameDev {
   float Bf[9];       // float32 copies of B
   float Bl[9];       // float32(B - Bf): B as double-float (Bf + Bl)
   float invf[3];     // float32 reciprocals: ortho 1/Lx,1/Ly,1/Lz; triclinic 1/ax,1/by,1/cz
-  float S;           // float32(nbins / r_max)
+  float S, S_l;      // nbins / r_max as a double-float
   float dr_f;        // float32(r_max / nbins), the bin width
   float rmax_f;      // float32(r_max)
   float S2;          // float32((nbins / r_max)^2)
@@ -71,6 +71,7 @@ struct FrameDev {
   // ---- written on the device
   int32_t smin[3], smax[3];  // triclinic: the same of the fractional coordinates
   int32_t wrap;       // the coordinates span more than one cell: P4 is brought home to the first
+                      // (1: in double-floats; 2: in binary64, from 4,096 cells on)
   int32_t list_slow;  // list kernel: every pair in binary64 (no trust in the images)
   int32_t list_all;   // list kernel: every listed pair re-decided (window too wide)
   float key_lo[3], key_inv;  // spatial order: origin and inverse side of the grid
@@ -139,8 +140,10 @@ struct StageJob {
   FrameDev* fd;
   int64_t n;
   int32_t stride;
-  int32_t pad;
-  int64_t chunk0;    // first staging chunk of this job
+  int32_t chunk0;    // first staging chunk of this job
+  // launch_prep: the frame's species (SortSeg), and the words of its output to clear
+  int32_t sort0, n_sort;
+  int64_t clear;
 };
 constexpr int kStageChunk = 1024;
 
@@ -198,6 +201,12 @@ struct ListLaunch {
 
 // ---- launchers (dh_kernels.cu); all enqueue on `stream` and return the launch error
 cudaError_t launch_stage(const StageJob* jobs, int n_jobs, int64_t n_chunks, cudaStream_t stream);
+// Staging, setup and spatial order of small frames of the list kernel in one
+// launch (jobs: one per frame, n <= max_n <= kPrepMaxN, dst and dst64 the ordered
+// copies; sorts: all their species; counts: their counters, n_keys in all).
+cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, const SortSeg* sorts, uint32_t* counts,
+                        cudaStream_t stream);
+constexpr int64_t kPrepMaxN = 32768, kPrepMaxKeys = 65536;  // particles and counters of a frame
 cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, int pass_hi_max, cudaStream_t stream);
 // Orders each segment's particles from src (src64) into dst (dst64), and for the
 // list kernel into the frame's P4 and P2 with the bounds of its runs.  counts: n_keys

@@ -18,6 +18,7 @@
 // definition (same operations, same order, explicit round-to-nearest
 // intrinsics, no contraction) and comparing r^2 with a table of binary64
 // thresholds T[k] = smallest r^2 whose bin is >= k.
+#include <cooperative_groups.h>
 #include <float.h>
 #include <math.h>
 #include <stdint.h>
@@ -104,6 +105,13 @@ __global__ void thresholds_kernel(double r_max, int32_t nbins, double* T, int32_
 
 // ------------------------------------------------------------------ A1: staging
 
+// Fractional coordinates in float32 (triclinic; orthorhombic too).
+__device__ __forceinline__ float3 frac_coords(const FrameDev& F, float x, float y, float z) {
+  const float s2 = z * F.invf[2];
+  const float s1 = (y - F.Bf[5] * s2) * F.invf[1];
+  return make_float3((x - F.Bf[1] * s1 - F.Bf[2] * s2) * F.invf[0], s1, s2);
+}
+
 // Staging of several frames at once: block b handles chunk b of the job whose
 // chunk range contains it; coords (n x stride floats, or doubles) -> float4
 // (and double4 for binary64 input), per-axis min/max of the float32 values (for
@@ -145,12 +153,9 @@ __global__ void stage_kernel(const StageJob* __restrict__ jobs, int n_jobs) {
     mn0 = fminf(mn0, x); mn1 = fminf(mn1, y); mn2 = fminf(mn2, z);
     mx0 = fmaxf(mx0, x); mx1 = fmaxf(mx1, y); mx2 = fmaxf(mx2, z);
     if (frac) {
-      const FrameDev* F = J.fd;
-      const float s2 = z * F->invf[2];
-      const float s1 = (y - F->Bf[5] * s2) * F->invf[1];
-      const float s0 = (x - F->Bf[1] * s1 - F->Bf[2] * s2) * F->invf[0];
-      sn[0] = fminf(sn[0], s0); sn[1] = fminf(sn[1], s1); sn[2] = fminf(sn[2], s2);
-      sx[0] = fmaxf(sx[0], s0); sx[1] = fmaxf(sx[1], s1); sx[2] = fmaxf(sx[2], s2);
+      const float3 s = frac_coords(*J.fd, x, y, z);
+      sn[0] = fminf(sn[0], s.x); sn[1] = fminf(sn[1], s.y); sn[2] = fminf(sn[2], s.z);
+      sx[0] = fmaxf(sx[0], s.x); sx[1] = fmaxf(sx[1], s.y); sx[2] = fmaxf(sx[2], s.z);
     }
   }
   // block minima and maxima (maxima as minima of the negated values), one set of
@@ -224,7 +229,8 @@ __device__ __forceinline__ uint32_t hilbert_key(uint32_t x, uint32_t y, uint32_t
 }
 
 // A particle's position brought home: minus the lattice vector of its fractional
-// coordinates' integer parts, in binary64 (frames that span several cells).
+// coordinates' integer parts (frames that span several cells). In binary64, of
+// which the SM does two operations per cycle,
 __device__ __forceinline__ double3 bring_home(const FrameDev& F, double x, double y, double z) {
   const double* B = F.B;
   const double sz = z / B[8], sy = (y - B[5] * sz) / B[4], sx = (x - B[1] * sy - B[2] * sz) / B[0];
@@ -232,14 +238,72 @@ __device__ __forceinline__ double3 bring_home(const FrameDev& F, double x, doubl
   return make_double3(((x - kx * B[0]) - ky * B[1]) - kz * B[2], (y - ky * B[4]) - kz * B[5], z - kz * B[8]);
 }
 
+// or in double-floats: the second turn removes what the first one's float32
+// quotients left (they err by a fraction of a cell up to 2^20 cells).  The
+// subtractions err by less than 2^-44 of the coordinates (list_setup).
+struct DF3 {
+  DF x, y, z;
+};
+__device__ __noinline__ DF3 bring_home_df(const FrameDev& F, float x, float y, float z) {
+  DF3 v{{x, 0.0f}, {y, 0.0f}, {z, 0.0f}};
+  for (int turn = 0; turn < 2; ++turn) {
+    const float3 s = frac_coords(F, v.x.h, v.y.h, v.z.h);
+    const float kx = floorf(s.x), ky = floorf(s.y), kz = floorf(s.z);
+    v.x = df_sub_kb(df_sub_kb(df_sub_kb(v.x, kx, F.Bf[0], F.Bl[0]), ky, F.Bf[1], F.Bl[1]), kz, F.Bf[2], F.Bl[2]);
+    v.y = df_sub_kb(df_sub_kb(v.y, ky, F.Bf[4], F.Bl[4]), kz, F.Bf[5], F.Bl[5]);
+    v.z = df_sub_kb(v.z, kz, F.Bf[8], F.Bl[8]);
+  }
+  return v;
+}
+__device__ __forceinline__ float3 home32(const FrameDev& F, float x, float y, float z) {
+  if (F.wrap == 1) {
+    const DF3 v = bring_home_df(F, x, y, z);
+    return make_float3(v.x.h, v.y.h, v.z.h);
+  }
+  const double3 w = bring_home(F, x, y, z);
+  return make_float3((float)w.x, (float)w.y, (float)w.z);
+}
+
+// One coordinate in bins: its high part on the grid, and the rest.
+__device__ __forceinline__ DF to_bins_on_grid(const FrameDev& F, DF v) {
+  const DF p = two_prod(v.h, F.S);
+  const DF s = two_sum(p.h, __fmaf_rn(v.h, F.S_l, __fmaf_rn(v.l, F.S, p.l)));
+  const float h = on_grid(s.h, F.list_grid);
+  return {h, __fadd_rn(__fsub_rn(s.h, h), s.l)};
+}
+// The list kernel's position of a particle (x64: its binary64 input, if it has one).
+__device__ __forceinline__ void list_position(const FrameDev& F, float4 p, const double4* x64, float4& P4, float2& P2) {
+  DF x, y, z;
+  if (x64 || F.wrap == 2) {
+    double3 v = x64 ? make_double3(x64->x, x64->y, x64->z) : make_double3(p.x, p.y, p.z);
+    if (F.wrap) v = bring_home(F, v.x, v.y, v.z);
+    const double s = (double)F.S + (double)F.S_l;
+    const double3 t = make_double3(v.x * s, v.y * s, v.z * s);
+    x.h = on_grid((float)t.x, F.list_grid);
+    y.h = on_grid((float)t.y, F.list_grid);
+    z.h = on_grid((float)t.z, F.list_grid);
+    x.l = (float)(t.x - (double)x.h);
+    y.l = (float)(t.y - (double)y.h);
+    z.l = (float)(t.z - (double)z.h);
+  } else {
+    DF3 v{{p.x, 0.0f}, {p.y, 0.0f}, {p.z, 0.0f}};
+    if (F.wrap) v = bring_home_df(F, p.x, p.y, p.z);
+    x = to_bins_on_grid(F, v.x);
+    y = to_bins_on_grid(F, v.y);
+    z = to_bins_on_grid(F, v.z);
+  }
+  P4 = make_float4(x.h, y.h, z.h, x.l);
+  P2 = make_float2(y.l, z.l);
+}
+
 // Cell of a particle on the curve (only the order depends on it).
 __device__ __forceinline__ uint32_t cell_key(const FrameDev& F, float4 p, int g) {
   if (g == 0) return 0u;
   if (F.wrap) {
-    const double3 w = bring_home(F, p.x, p.y, p.z);
-    p.x = (float)w.x;
-    p.y = (float)w.y;
-    p.z = (float)w.z;
+    const float3 w = home32(F, p.x, p.y, p.z);
+    p.x = w.x;
+    p.y = w.y;
+    p.z = w.z;
   }
   const float G = (float)(1 << g);
   const int last = (1 << g) - 1;
@@ -320,39 +384,23 @@ __global__ void sort_scatter_kernel(const SortSeg* segs, const float4* __restric
   const FrameDev& F = *S.fd;
   const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
   const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
-  const double to_bins = (double)F.nbins / F.r_max;
   for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
     const int64_t pos = S.x0 + atomicAdd(cursors + S.key0 + (uint32_t)keys[S.x0 + i], 1u);
     const float4 p = src[S.x0 + i];
     dst[pos] = p;
-    double3 v = make_double3(p.x, p.y, p.z);
-    if (F.X64) {
-      const double4 q = src64[S.x0 + i];
-      dst64[pos] = q;
-      v = make_double3(q.x, q.y, q.z);
-    }
-    if (F.P4) {
-      if (F.wrap) v = bring_home(F, v.x, v.y, v.z);
-      v = make_double3(v.x * to_bins, v.y * to_bins, v.z * to_bins);
-      const double g = F.list_grid, ig = 1.0 / g;
-      const float3 h = make_float3((float)(rint(v.x * ig) * g), (float)(rint(v.y * ig) * g), (float)(rint(v.z * ig) * g));
-      F.P4[pos - S.f0] = make_float4(h.x, h.y, h.z, (float)(v.x - (double)h.x));
-      F.P2[pos - S.f0] = make_float2((float)(v.y - (double)h.y), (float)(v.z - (double)h.z));
-    }
+    double4 q;
+    if (F.X64) dst64[pos] = q = src64[S.x0 + i];
+    if (F.P4) list_position(F, p, F.X64 ? &q : nullptr, F.P4[pos - S.f0], F.P2[pos - S.f0]);
   }
 }
 
-// Bounds of each run of kRun ordered particles (one warp per run), over the
-// positions the list kernel works with.
-__global__ void run_bounds_kernel(const SortSeg* segs) {
-  const SortSeg S = segs[blockIdx.y];
-  const FrameDev& F = *S.fd;
-  const int run = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
-  if (!F.bnd || run * (int64_t)kRun >= S.n) return;
+// Bounds of one run of kRun ordered particles (by one warp), over the positions
+// the list kernel works with.
+__device__ __forceinline__ void run_bounds(const FrameDev& F, const SortSeg& S, int run, int lane) {
   float b[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
   const int64_t p0 = S.x0 - S.f0;
   for (int i = run * kRun + lane; i < min(S.n, (run + 1) * kRun); i += 32) {
-    const float4 p = F.P4[p0 + i];
+    const float4 p = __ldcg(F.P4 + p0 + i);
     const float v[3] = {p.x, p.y, p.z};
     for (int c = 0; c < 3; ++c) {
       b[c] = fminf(b[c], v[c]);
@@ -369,6 +417,11 @@ __global__ void run_bounds_kernel(const SortSeg* segs) {
     F.bnd[2 * (S.run0 + run) + 1] = make_float4(b[3], b[4], b[5], 0.0f);
   }
 }
+__global__ void run_bounds_kernel(const SortSeg* segs) {
+  const SortSeg S = segs[blockIdx.y];
+  const int run = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  if (S.fd->bnd && run * (int64_t)kRun < S.n) run_bounds(*S.fd, S, run, threadIdx.x & 31);
+}
 
 // ------------------------------------------------------------------ per-frame error window
 
@@ -379,6 +432,16 @@ __device__ inline double half_ulp_below(double D) {
   int E;
   frexp(D, &E);  // D = m 2^E, m in [1/2, 1): |x| <= D < 2^E
   return ldexp(1.0, E - 25);
+}
+
+// Orthorhombic: float32 and binary64 can round d/L to different images only within
+// eta of a half integer; both images then have |d'_c| within eta L of L/2.  2 eta L:
+__device__ __forceinline__ double ortho_tie(const FrameDev& F, int c, double R, double conv) {
+  const double L = F.B[4 * c];
+  return 2.0 * (half_ulp_below(R) + conv + R * fabs((double)F.invf[c] - F.Linv[c]) + 1e-15 * (R + L));
+}
+__device__ __forceinline__ double ortho_tie_eps(const FrameDev& F, const double* tie_c) {
+  return 2.0 * fmax(tie_c[0], fmax(tie_c[1], tie_c[2])) + 1e-12 * fmin(F.B[0], fmin(F.B[4], F.B[8]));
 }
 
 // The spatial order's grid and the list kernel's window of one frame.
@@ -395,12 +458,12 @@ __device__ inline double half_ulp_below(double D) {
 //   last add                                u (T + H)^2
 // in all u (2 T^2 + 12 TH + 5 H^2) <= u ((2 + 6l) T^2 + (5 + 6/l) H^2) for any
 // l > 0 (run_window takes l = H over a typical T).  list_c0 covers what the
-// double-floats leave out (a0, 2^-45 of the coordinates) and the binary64
-// definition's own rounding of t.
+// double-floats leave out (a0: positions, 2^-47 each and per axis, the products
+// with S and the image vectors) and the binary64 definition's own rounding of t.
 __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
   const double u = 1.0 / 16777216.0;
   const double* B = F.B;
-  const double S = (double)F.nbins / F.r_max;
+  const double S = (double)F.S + (double)F.S_l;
   int wrap = 0, slow = 0;
   double lo[3], ext[3], far = 0.0;
   for (int c = 0; c < 3; ++c) {
@@ -425,7 +488,9 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
       // (binary64 still tells the images apart below 2^30 cells)
       const double sz = Xm[2] / B[8], sy = (Xm[1] + fabs(B[5]) * sz) / B[4],
                    sx = (Xm[0] + fabs(B[1]) * sy + fabs(B[2]) * sz) / B[0];
-      if (!(fmax(sx, fmax(sy, sz)) < 1e6)) slow = 1;
+      const double cells = fmax(sx, fmax(sy, sz));
+      if (!(cells < 1e6)) slow = 1;
+      if (!(cells < 4096.0)) wrap = 2;
     }
   }
   const double side = fmax(ext[0], fmax(ext[1], ext[2]));
@@ -435,9 +500,10 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
   F.list_slow = slow;
   const double cell = F.variant == V_NONE ? 0.0 : B[0] + fabs(B[1]) + fabs(B[2]) + B[4] + fabs(B[5]) + B[8];
   // positions and image vectors: the largest of them in bins; brought home, the
-  // binary64 subtraction errs by 2^-52 of what is subtracted
+  // subtraction errs by 2^-52 (binary64) or 2^-45 (double-floats) of what is
+  // subtracted, per axis and position
   const double reach = S * ((wrap ? ext[0] + ext[1] + ext[2] : 2.0 * far) + 2.0 * cell);
-  const double a0 = reach * 0x1p-45 + (wrap ? S * far * 0x1p-49 : 0.0);
+  const double a0 = reach * 0x1p-44 + (wrap ? S * far * (wrap == 1 ? 0x1p-43 : 0x1p-49) : 0.0);
   // grid of the high parts: sums of positions, centres and images stay below
   // 2^23 steps, so they are exact in float32
   int e = 0;
@@ -451,6 +517,13 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
   // window and square-root error below a quarter bin at the far end
   const double tmax = (double)F.nbins + 40.0;
   F.list_all = !(8.0 * u * tmax + 4.0 * a0 < 0.25) || !(tmax * 4.76837158203125e-07 < 0.25);
+}
+
+// No box, one sweep: the largest distance D maps below nbins + 1 even after the
+// float32 roundings of q and of its square root (relative 2^-18 covers them).
+__device__ __forceinline__ bool inside_one_sweep(const FrameDev& F, double D) {
+  return F.variant == V_NONE && F.sweep_width >= F.nbins &&
+         ((double)F.S + (double)F.S_l) * D * (1.0 + 1.0 / 262144.0) < (double)F.nbins + 1.0;
 }
 
 // Derives, for one frame, the bound of the float32 decision and of the
@@ -534,11 +607,7 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
       I[c] = R[c] + K * L;
       if (R[c] / L > 1048576.0) all_defer = 1;  // nearest integer via the 1.5*2^23 trick needs |d/L| < 2^22
       Lmin = fmin(Lmin, L);
-      // float32 and binary64 can round d/L to different images only within eta of a
-      // half integer; both images then have |d'_c| within eta L of L/2
-      double eta = (half_ulp_below(R[c]) + conv[c] + R[c] * fabs((double)F.invf[c] - 1.0 / L)) / L +
-                   1e-15 * (R[c] / L + 1.0);
-      tie_c[c] = 2.0 * eta * L;
+      tie_c[c] = ortho_tie(F, c, R[c], conv[c]);
     }
     // components that can sit at L_c/2 while t <= nbins + 1 (r <= r_max (1 + 1/nbins))
     double rr = F.r_max * (1.0 + 2.0 / (double)F.nbins);
@@ -548,7 +617,7 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
       double t3 = sqrt(tie_c[0] * tie_c[0] + tie_c[1] * tie_c[1] + tie_c[2] * tie_c[2]);
       tie = S * (m >= 3 ? t3 : (m == 2 ? fmin(t3, 1.4142135623730951 * t1) : t1)) * 1.01;
     }
-    tie_eps = 2.0 * fmax(tie_c[0], fmax(tie_c[1], tie_c[2])) + 1e-12 * Lmin;
+    tie_eps = ortho_tie_eps(F, tie_c);
     // uniform-image tiles: the image is subtracted exactly (|k| <= 1), so d'_c
     // errs only by the float32 box entry; the tie term is not needed where the
     // tile's difference range, widened by tie_m = 4 eta L, keeps one image
@@ -658,15 +727,221 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
   for (int w = 0; w < 3; ++w) F.beta_w[w] = (float)beta_w[w];
   F.eps_s = eps_s;
   F.all_defer = all_defer;
-  // No box, one sweep: the largest possible distance, sqrt(sum R_c^2), maps below
-  // nbins + 1 even after the float32 roundings of q and of its square root
-  // (relative 2^-18 covers them), so no pair's root reaches the clamp.
+  // no pair's root reaches the clamp: the largest possible distance is sqrt(sum R_c^2)
   {
     const double D = sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]);
-    F.in_range = F.variant == V_NONE && F.sweep_width >= F.nbins && !all_defer &&
-                 S * D * (1.0 + 1.0 / 262144.0) < (double)F.nbins + 1.0;
+    F.in_range = !all_defer && inside_one_sweep(F, D);
     // no box: bounding tiles pays only when some tile can miss a sweep
     F.cull_ok = F.variant == V_NONE && (F.sweep_width < F.nbins || F.r_max < D);
+  }
+}
+
+// ------------------------------------------------------------------ small frames: one launch
+
+// Staging, list_setup and spatial order of one frame per cluster, for frames of
+// which only the list kernel is run (the tiled kernel's window is not derived).
+// A small frame's preparation is a chain of short steps, each over all of its
+// particles: as kernels of their own (stage, setup, count, scan, scatter, bounds and
+// two fills) they took 62 us at any size up to N = 5,000, most of it launches, first
+// touches and one thread's binary64 arithmetic.  Here the steps meet at cluster
+// barriers, the particles stay in registers, and the frame's descriptor is read into
+// shared memory once.  Whole call, before -> now: N = 2,000 without a box 91 -> 64 us,
+// N = 8,000 triclinic 159 -> 127 us, N = 32,000 orthorhombic 429 -> 411 us; larger
+// frames have work for more SMs than a cluster's and keep the separate kernels.
+constexpr int kPrepBlock = 1024, kPrepPer = 4, kPrepCluster = 8, kPrepScan = 8;
+static_assert((int64_t)kPrepBlock * kPrepPer * kPrepCluster == kPrepMaxN, "particles per cluster");
+__global__ void __launch_bounds__(kPrepBlock, 1)
+    prep_kernel(const StageJob* __restrict__ jobs, const SortSeg* __restrict__ sorts, uint32_t* counts) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int slot = rank * kPrepBlock + tid, slots = C * kPrepBlock;
+  __shared__ StageJob J;
+  __shared__ __align__(16) FrameDev F;
+  __shared__ float s_red[32][12];
+  __shared__ float s_part[13];  // this block's minima (negated maxima), then 1 if a coordinate is not finite
+  __shared__ float s_all[13];
+  __shared__ uint32_t s_sum[32], s_total, s_base[kPrepCluster];
+  __shared__ int s_bad;
+  static_assert(sizeof(FrameDev) % 4 == 0 && sizeof(FrameDev) / 4 <= kPrepBlock, "one word per thread");
+  const StageJob& job = jobs[blockIdx.x / C];
+  if (tid == 0) {
+    J = job;
+    s_bad = 0;
+  }
+  FrameDev* const dev = job.fd;
+  const int fwords = (int)(sizeof(FrameDev) / 4);
+  if (tid < fwords) reinterpret_cast<uint32_t*>(&F)[tid] = reinterpret_cast<const uint32_t*>(dev)[tid];
+  __syncthreads();
+  const SortSeg* const S = sorts + J.sort0;
+  const int64_t key0 = S[0].key0;
+  const int keys = (int)(S[J.n_sort - 1].key0 - key0) + max(1 << (3 * S[J.n_sort - 1].g), 4);
+  for (int k = slot; k < keys; k += slots) counts[key0 + k] = 0u;
+  for (int64_t k = slot; k < J.clear; k += slots) F.out[k] = 0ull;
+
+  // ---- coordinates and their ranges
+  const int n = (int)J.n, stride = J.stride;
+  const double* const src64 = J.dst64 ? reinterpret_cast<const double*>(J.src) : nullptr;
+  const bool frac = F.variant == V_TRIC || F.variant == V_TRIC_SEARCH;
+  float3 p[kPrepPer];
+  float v[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) v[c] = INFINITY;
+  bool bad = false;
+#pragma unroll
+  for (int q = 0; q < kPrepPer; ++q) {
+    const int i = slot + q * slots;
+    p[q] = make_float3(0.0f, 0.0f, 0.0f);
+    if (i >= n) continue;
+    if (src64) {
+      const double* x = src64 + (int64_t)i * stride;
+      p[q] = make_float3(__double2float_rn(x[0]), __double2float_rn(x[1]), __double2float_rn(x[2]));
+    } else {
+      const float* x = J.src + (int64_t)i * stride;
+      p[q] = make_float3(x[0], x[1], x[2]);
+    }
+    const float3 a = p[q];
+    bad |= !(isfinite(a.x) && isfinite(a.y) && isfinite(a.z));
+    v[0] = fminf(v[0], a.x); v[1] = fminf(v[1], a.y); v[2] = fminf(v[2], a.z);
+    v[3] = fminf(v[3], -a.x); v[4] = fminf(v[4], -a.y); v[5] = fminf(v[5], -a.z);
+    if (frac) {
+      const float3 s = frac_coords(F, a.x, a.y, a.z);
+      v[6] = fminf(v[6], s.x); v[7] = fminf(v[7], s.y); v[8] = fminf(v[8], s.z);
+      v[9] = fminf(v[9], -s.x); v[10] = fminf(v[10], -s.y); v[11] = fminf(v[11], -s.z);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    if (c >= 6 && !frac) break;
+    for (int o = 16; o > 0; o >>= 1) v[c] = fminf(v[c], __shfl_xor_sync(kFull, v[c], o));
+    if (lane == 0) s_red[warp][c] = v[c];
+  }
+  if (bad) s_bad = 1;
+  __syncthreads();
+  if (warp < 12) {
+    float m = INFINITY;
+    if (warp < 6 || frac) m = s_red[lane][warp];
+    for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(kFull, m, o));
+    if (lane == 0) s_part[warp] = m;
+  }
+  if (tid == 0) s_part[12] = s_bad ? -1.0f : 0.0f;
+  cluster.sync();
+  if (tid < 13) {
+    float m = INFINITY;
+    for (int b = 0; b < C; ++b) m = fminf(m, cluster.map_shared_rank(s_part, b)[tid]);
+    s_all[tid] = m;
+  }
+  __syncthreads();
+
+  // ---- the frame's window and grid, by every block for itself
+  if (tid == 0) {
+    double R[3], Xm[3], tie_c[3];
+    for (int c = 0; c < 3; ++c) {
+      const float lo = s_all[c], hi = -s_all[3 + c];
+      // (a frame without one finite coordinate keeps the initial, empty range)
+      if (lo < INFINITY) F.cmin[c] = ord_of(lo);
+      if (hi > -INFINITY) F.cmax[c] = ord_of(hi);
+      if (frac && s_all[6 + c] < INFINITY) F.smin[c] = ord_of(s_all[6 + c]);
+      if (frac && s_all[9 + c] < INFINITY) F.smax[c] = ord_of(-s_all[9 + c]);
+    }
+    F.bad = s_all[12] < 0.0f;
+    const bool any = F.cmin[0] <= F.cmax[0];
+    for (int c = 0; c < 3; ++c) {
+      const double lo = any ? (double)float_of_ord(F.cmin[c]) : 0.0, hi = any ? (double)float_of_ord(F.cmax[c]) : 0.0;
+      R[c] = hi - lo;
+      Xm[c] = fmax(fabs(lo), fabs(hi));
+      if (F.variant == V_ORTHO) tie_c[c] = ortho_tie(F, c, R[c], F.X64 ? 2.0 * half_ulp_below(Xm[c]) : 0.0);
+    }
+    F.tie_eps = F.variant == V_ORTHO ? (float)ortho_tie_eps(F, tie_c) : 0.0f;
+    list_setup(F, R, Xm);
+    F.in_range = inside_one_sweep(F, sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]));
+  }
+  __syncthreads();
+  if (rank == 0 && tid < fwords) reinterpret_cast<uint32_t*>(dev)[tid] = reinterpret_cast<const uint32_t*>(&F)[tid];
+
+  // ---- cells, and each particle's place in its cell
+  uint32_t cell[kPrepPer], place[kPrepPer];
+#pragma unroll
+  for (int q = 0; q < kPrepPer; ++q) {
+    const int i = slot + q * slots;
+    cell[q] = place[q] = 0u;
+    if (i >= n) continue;
+    int a = 0, hi = J.n_sort - 1;
+    while (a < hi) {
+      const int mid = (a + hi + 1) >> 1;
+      if (S[mid].x0 - S[mid].f0 <= i) a = mid; else hi = mid - 1;
+    }
+    cell[q] = (uint32_t)(S[a].key0 - key0) + cell_key(F, make_float4(p[q].x, p[q].y, p[q].z, 0.0f), S[a].g);
+    place[q] = atomicAdd(counts + key0 + cell[q], 1u);
+  }
+  cluster.sync();
+
+  // ---- prefix sum over the frame's cells, species after species: within the block,
+  // then of the blocks' totals
+  const int each = (keys + slots - 1) / slots, k0 = slot * each;
+  uint32_t c[kPrepScan], sum = 0u;
+#pragma unroll
+  for (int q = 0; q < kPrepScan; ++q) {
+    c[q] = (q < each && k0 + q < keys) ? __ldcg(counts + key0 + k0 + q) : 0u;
+    sum += c[q];
+  }
+  uint32_t incl = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += x;
+  }
+  if (lane == 31) s_sum[warp] = incl;
+  __syncthreads();
+  uint32_t before = s_sum[lane];
+  if (warp == 0) {
+    uint32_t t = before;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+    if (lane == 0) s_total = t;
+  }
+  if (lane >= warp) before = 0u;
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
+  uint32_t at = before + incl - sum;
+#pragma unroll
+  for (int q = 0; q < kPrepScan; ++q) {
+    if (q < each && k0 + q < keys) __stcg(counts + key0 + k0 + q, at);
+    at += c[q];
+  }
+  cluster.sync();
+  if (tid < C) {
+    uint32_t b = 0u;
+    for (int r = 0; r < tid; ++r) b += *cluster.map_shared_rank(&s_total, r);
+    s_base[tid] = b;
+  }
+  __syncthreads();
+
+  // ---- the ordered copies
+  const int per_block = each * kPrepBlock;
+#pragma unroll
+  for (int q = 0; q < kPrepPer; ++q) {
+    const int i = slot + q * slots;
+    if (i >= n) continue;
+    const int pos = (int)(s_base[cell[q] / per_block] + __ldcg(counts + key0 + cell[q]) + place[q]);
+    const float4 a = make_float4(p[q].x, p[q].y, p[q].z, 0.0f);
+    J.dst[pos] = a;
+    double4 d;
+    if (src64) {
+      const double* x = src64 + (int64_t)i * stride;
+      J.dst64[pos] = d = make_double4(x[0], x[1], x[2], 0.0);
+    }
+    list_position(F, a, src64 ? &d : nullptr, F.P4[pos], F.P2[pos]);
+  }
+  cluster.sync();
+
+  // ---- bounds of the runs
+  const int runs = S[J.n_sort - 1].run0 + (S[J.n_sort - 1].n + kRun - 1) / kRun;
+  for (int r = rank * 32 + warp; r < runs; r += C * 32) {
+    int a = 0, hi = J.n_sort - 1;
+    while (a < hi) {
+      const int mid = (a + hi + 1) >> 1;
+      if (S[mid].run0 <= r) a = mid; else hi = mid - 1;
+    }
+    run_bounds(F, S[a], r - S[a].run0, lane);
   }
 }
 
@@ -2163,6 +2438,27 @@ cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, int64_t max_n, 
   dim3 bgrid((unsigned)((max_n + 8 * kRun - 1) / (8 * kRun)), (unsigned)n_segs);
   run_bounds_kernel<<<bgrid, 256, 0, stream>>>(segs);
   return cudaGetLastError();
+}
+
+cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, const SortSeg* sorts, uint32_t* counts,
+                        cudaStream_t stream) {
+  clear_stale_error();
+  if (n_jobs <= 0) return cudaSuccess;
+  // one particle per thread up to the largest portable cluster (two or four per
+  // thread: N = 4,000 without a box 72 and 80 us instead of 65)
+  unsigned blocks = 1;
+  while (blocks < (unsigned)kPrepCluster && (int64_t)blocks * kPrepBlock < max_n) blocks *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks * (unsigned)n_jobs);
+  cfg.blockDim = dim3(kPrepBlock);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = blocks;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, prep_kernel, jobs, sorts, counts);
 }
 
 cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, int, cudaStream_t stream) {

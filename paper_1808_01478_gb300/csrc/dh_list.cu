@@ -112,12 +112,6 @@ struct SegState {
   unsigned long long* next;
 };
 
-// The multiple of the grid nearest to v (|v| < 2^22 steps).
-__device__ __forceinline__ float on_grid(float v, float grid) {
-  const float m = kMagicRound * grid;
-  return __fsub_rn(__fadd_rn(v, m), m);
-}
-
 // d + l as a double-float (d a multiple of the grid, |l| about a step at most).
 __device__ __forceinline__ DF renorm(float d, float l) {
   const float h = __fadd_rn(d, l);

@@ -277,6 +277,7 @@ void fill_frame_dev(const PlannedFrame& pf, FrameDev& F, const float4* X, uint64
   }
   double S = (double)f->nbins / f->r_max;
   F.S = (float)S;
+  F.S_l = (float)(S - (double)F.S);
   F.dr_f = (float)(f->r_max / (double)f->nbins);
   F.rmax_f = (float)f->r_max;
   F.eps_S = std::fabs((double)F.S - S) / S;
@@ -533,7 +534,8 @@ struct CallPlan {
   int max_pass = 1;
   int launched = 0;
   size_t seg_bytes = 0;          // Segment array in the metadata
-  size_t lseg_bytes = 0;         // ListSegment array after it
+  size_t lseg_bytes = 0;         // ListSegment array after it,
+  size_t sort_bytes = 0;         // then the SortSeg array and a zeroed SegCounter per list segment
   int n_lsegs = 0;
   // list-kernel launches: frames with one image of a pair inside r_max, and the
   // others (PlannedFrame.pick): first segment and segments, items, widest sweep,
@@ -543,6 +545,7 @@ struct CallPlan {
     int64_t items = 0;
     int width = 1, multi = 0, grid = 0, split = 1;
   } list[2];
+  bool prep = false;             // frames prepared by one launch (launch_prep)
   int n_sort = 0;                // spatial-order segments (after the segments in the metadata)
   int64_t sort_max = 0;          // largest of them
   int64_t sort_keys = 0;         // counters over all of them
@@ -578,7 +581,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   for (int f = 0; f < k; ++f) runs[f + 1] = runs[f] + frame_runs(pfs[f].src);
   DH_CUDA_TRY(c->bnd.ensure(2 * sizeof(float4) * (size_t)std::max<int64_t>(runs[k], 1)));
   // device metadata: FrameDev[k] | StageJob[k] | Segment[m] | ListSegment[l] |
-  // SortSeg[s], uploaded in one copy; segments are grouped by minimum-image
+  // SortSeg[s] | SegCounter[l], uploaded in one copy; segments are grouped by minimum-image
   // variant (one pair-kernel launch each), those of the list kernel together
   std::vector<Segment> segs;
   std::vector<ListSegment> lsegs;
@@ -645,16 +648,21 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   };
   // spatial order of the species
   std::vector<SortSeg> sorts;
+  std::vector<int> sort0((size_t)k + 1, 0);
   auto plan_sorts = [&](FrameDev* dF) {
     sorts.clear();
     P.sort_keys = 0;
     P.sort_max = 0;
+    P.prep = with_pairs;
     for (int f = 0; f < k; ++f) {
       int64_t keys = 0, most = 0;
       std::vector<SortSeg> fs = plan_spatial_order(pfs[f], dF + f, xoff[f], P.sort_keys, &keys, &most);
       sorts.insert(sorts.end(), fs.begin(), fs.end());
       P.sort_keys += keys;
       P.sort_max = std::max(P.sort_max, most);
+      sort0[f + 1] = (int)sorts.size();
+      P.prep = P.prep && on_list(f) && xoff[f + 1] - xoff[f] >= 1 && xoff[f + 1] - xoff[f] <= kPrepMaxN &&
+               keys <= kPrepMaxKeys;
     }
     P.n_sort = (int)sorts.size();
     P.sort_particles = xoff[k];
@@ -664,9 +672,9 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   plan_sorts((FrameDev*)c->meta.p);
   P.seg_bytes = sizeof(Segment) * std::max<size_t>(segs.size(), 1);
   P.lseg_bytes = sizeof(ListSegment) * lsegs.size();
+  P.sort_bytes = sizeof(SortSeg) * sorts.size();
   P.meta_bytes = sizeof(FrameDev) * (size_t)k + sizeof(StageJob) * (size_t)k + P.seg_bytes + P.lseg_bytes +
-                 sizeof(SortSeg) * sorts.size();
-  DH_CUDA_TRY(c->ctl.ensure(sizeof(Control) * kNumVariants + sizeof(SegCounter) * lsegs.size()));
+                 P.sort_bytes + sizeof(SegCounter) * lsegs.size();
   void* before = c->meta.p;
   DH_CUDA_TRY(c->meta.ensure(P.meta_bytes));
   DH_CUDA_TRY(c->hmeta.ensure(P.meta_bytes));
@@ -674,7 +682,9 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     plan_segments((FrameDev*)c->meta.p);
     plan_sorts((FrameDev*)c->meta.p);
   }
-  if (P.n_sort > 0) {
+  if (P.prep) {
+    DH_CUDA_TRY(c->sortC.ensure(sizeof(uint32_t) * (size_t)P.sort_keys));
+  } else if (P.n_sort > 0) {
     DH_CUDA_TRY(c->sortX.ensure(sizeof(float4) * (size_t)P.sort_particles));
     if (P.any_f64) DH_CUDA_TRY(c->sortX64.ensure(sizeof(double4) * (size_t)P.sort_particles));
     DH_CUDA_TRY(c->sortK.ensure(sizeof(int32_t) * (size_t)P.sort_particles));
@@ -689,6 +699,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     dh_status s = c->tcache.acquire(pfs[f].src->r_max, pfs[f].src->nbins, st, (int32_t*)c->tstat.p, &T, &P.launched);
     if (s != DH_OK) return s;
     c->held_tables.push_back(T);
+    c->tstat_new |= P.launched > 0;
     fill_frame_dev(pfs[f], hF[f], (const float4*)c->X.p + xoff[f], dev_out[f], T);
     if (pfs[f].src->flags & DH_COORDS_F64) hF[f].X64 = (const double4*)c->X64.p + xoff[f];
     if (on_list(f)) {
@@ -709,18 +720,22 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     J.stride = (fr->flags & DH_COORDS_F4) ? 4 : 3;
     J.src = host_coords ? (const float*)((const unsigned char*)c->raw.p + P.raw_off[f]) : fr->coords;
     // staged for the spatial order, or in place where there is none
-    const bool sorted = pfs[f].variant != V_TRIC_SEARCH || pfs[f].list;
+    const bool sorted = !P.prep && (pfs[f].variant != V_TRIC_SEARCH || pfs[f].list);
     J.dst = (float4*)(sorted ? c->sortX.p : c->X.p) + xoff[f];
     J.dst64 = (fr->flags & DH_COORDS_F64) ? (double4*)(sorted ? c->sortX64.p : c->X64.p) + xoff[f] : nullptr;
     J.fd = dF + f;
     J.n = fr->n;
-    J.chunk0 = P.n_chunks;
+    J.sort0 = sort0[f];
+    J.n_sort = sort0[f + 1] - sort0[f];
+    J.clear = host_coords || !(fr->flags & DH_ACCUMULATE) ? (int64_t)pfs[f].n_hist * fr->nbins : 0;
+    J.chunk0 = (int32_t)P.n_chunks;
     P.n_chunks += (fr->n + kStageChunk - 1) / kStageChunk;
   }
   if (!segs.empty()) std::memcpy(hS, segs.data(), sizeof(Segment) * segs.size());
   if (!lsegs.empty()) std::memcpy((unsigned char*)hS + P.seg_bytes, lsegs.data(), P.lseg_bytes);
   if (!sorts.empty())
     std::memcpy((unsigned char*)hS + P.seg_bytes + P.lseg_bytes, sorts.data(), sizeof(SortSeg) * sorts.size());
+  std::memset((unsigned char*)hS + P.seg_bytes + P.lseg_bytes + P.sort_bytes, 0, sizeof(SegCounter) * lsegs.size());
   // launch shapes (occupancy queries and kernel attributes stay outside any stream capture)
   for (int v = 0; v < kNumVariants; ++v) {
     P.vgrid[v] = 0;
@@ -764,14 +779,21 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
                                   cudaMemcpyHostToDevice, st));
     }
   DH_CUDA_TRY(cudaMemcpyAsync(dF, c->hmeta.p, P.meta_bytes, cudaMemcpyHostToDevice, st));
-  if (P.n_jobs > 0) {
-    DH_CUDA_TRY(launch_stage(dJ, P.n_jobs, P.n_chunks, st));
+  const SortSeg* dSort = (const SortSeg*)((unsigned char*)dS + P.seg_bytes + P.lseg_bytes);
+  if (P.prep) {
+    int64_t max_n = 0;
+    for (auto& pf : pfs) max_n = std::max(max_n, pf.src->n);
+    DH_CUDA_TRY(launch_prep(dJ, k, max_n, dSort, (uint32_t*)c->sortC.p, st));
+    ++launched;
+  } else {
+    if (P.n_jobs > 0) {
+      DH_CUDA_TRY(launch_stage(dJ, P.n_jobs, P.n_chunks, st));
+      ++launched;
+    }
+    DH_CUDA_TRY(launch_frame_setup(dF, k, 0, st));  // the windows, and the grid of the spatial order
     ++launched;
   }
-  DH_CUDA_TRY(launch_frame_setup(dF, k, 0, st));  // the windows, and the grid of the spatial order
-  ++launched;
-  if (P.n_sort > 0) {
-    const SortSeg* dSort = (const SortSeg*)((unsigned char*)dS + P.seg_bytes + P.lseg_bytes);
+  if (!P.prep && P.n_sort > 0) {
     DH_CUDA_TRY(cudaMemsetAsync(c->sortC.p, 0, sizeof(uint32_t) * (size_t)P.sort_keys, st));
     DH_CUDA_TRY(launch_spatial_sort(dSort, P.n_sort, P.sort_max, (const float4*)c->sortX.p, (float4*)c->X.p,
                                     P.any_f64 ? (const double4*)c->sortX64.p : nullptr,
@@ -789,7 +811,9 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   DH_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
   const unsigned ev_flags = (cs == cudaStreamCaptureStatusActive) ? cudaEventRecordExternal : cudaEventRecordDefault;
   if (any) {
-    DH_CUDA_TRY(cudaMemsetAsync(c->ctl.p, 0, sizeof(Control) * kNumVariants + sizeof(SegCounter) * (size_t)P.n_lsegs, st));
+    bool tiled = false;
+    for (int v = 0; v < kNumVariants; ++v) tiled |= P.vgrid[v] > 0;
+    if (tiled) DH_CUDA_TRY(cudaMemsetAsync(c->ctl.p, 0, sizeof(Control) * kNumVariants, st));
     if (c->ev_pair0) DH_CUDA_TRY(cudaEventRecordWithFlags(c->ev_pair0, st, ev_flags));
     for (int g = 0; g < 2; ++g) {
       const CallPlan::ListPlan& lp = P.list[g];
@@ -797,7 +821,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
       ListLaunch L;
       std::memset(&L, 0, sizeof L);
       L.segs = (const ListSegment*)((unsigned char*)dS + P.seg_bytes) + lp.seg0;
-      L.ctr = (SegCounter*)((unsigned char*)c->ctl.p + sizeof(Control) * kNumVariants) + lp.seg0;
+      L.ctr = (SegCounter*)((unsigned char*)dSort + P.sort_bytes) + lp.seg0;
       L.n_segs = lp.n_segs;
       L.hist_width = lp.width;
       L.n_items = lp.items;
@@ -875,11 +899,16 @@ dh_status finish_frames(dh_ctx* c, int k) {
   FrameDev* hF = (FrameDev*)c->hmeta.p;
   DH_CUDA_TRY(cudaMemcpyAsync(hF, c->meta.p, sizeof(FrameDev) * (size_t)k, cudaMemcpyDeviceToHost, c->stream()));
   int32_t tstat = 0;
-  DH_CUDA_TRY(cudaMemcpyAsync(&tstat, c->tstat.p, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream()));
+  if (c->tstat_new)
+    DH_CUDA_TRY(cudaMemcpyAsync(&tstat, c->tstat.p, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream()));
   cudaError_t e = cudaStreamSynchronize(c->stream());
   release_held(c);
   DH_CUDA_TRY(e);
-  if (tstat != 0) return fail(DH_ERR_CUDA, "bin threshold table did not converge");
+  c->tstat_new = false;
+  if (tstat != 0) {
+    DH_CUDA_TRY(cudaMemsetAsync(c->tstat.p, 0, sizeof(int32_t), c->stream()));
+    return fail(DH_ERR_CUDA, "bin threshold table did not converge");
+  }
   if (c->timed) {
     float ms = 0.0f;
     DH_CUDA_TRY(cudaEventElapsedTime(&ms, c->ev_pair0, c->ev_pair1));
@@ -928,7 +957,6 @@ dh_status run_frames(dh_ctx* c, const dh_frame* frames, int k, bool wait, bool u
     DH_CUDA_TRY(c->hist.ensure(sizeof(uint64_t) * std::max<size_t>(hoff[k], 1)));
     for (int f = 0; f < k; ++f) dev_out[f] = (uint64_t*)c->hist.p + hoff[f];
   }
-  DH_CUDA_TRY(cudaMemsetAsync(c->tstat.p, 0, sizeof(int32_t), st));
   CallPlan P;
   dh_status s = prepare_frames(c, pfs, dev_out, !dev, true, P);
   if (s == DH_OK && graph) {
@@ -937,7 +965,9 @@ dh_status run_frames(dh_ctx* c, const dh_frame* frames, int k, bool wait, bool u
   }
   if (s == DH_OK) {
     cudaError_t e = cudaSuccess;
-    if (dev) {
+    if (P.prep) {
+      // cleared by the preparation
+    } else if (dev) {
       for (int f = 0; f < k && e == cudaSuccess; ++f)
         if (!(frames[f].flags & DH_ACCUMULATE))
           e = cudaMemsetAsync(frames[f].out, 0, sizeof(uint64_t) * (hoff[f + 1] - hoff[f]), st);
@@ -1309,6 +1339,7 @@ dh_status dh_create(const dh_config* config, dh_ctx** out) {
   if (c->max_width < 1024) return fail(DH_ERR_CUDA, "not enough shared memory per block");
   DH_CUDA_TRY(c->ctl.ensure(sizeof(Control) * kNumVariants));
   DH_CUDA_TRY(c->tstat.ensure(64));
+  DH_CUDA_TRY(cudaMemset(c->tstat.p, 0, sizeof(int32_t)));
   if (c->cfg.flags & DH_CFG_TIMING) {
     DH_CUDA_TRY(cudaEventCreate(&c->ev_pair0));
     DH_CUDA_TRY(cudaEventCreate(&c->ev_pair1));

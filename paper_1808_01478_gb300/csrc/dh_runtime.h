@@ -194,7 +194,8 @@ struct dh_ctx {
   dh::DevBuf ctl;      // Control
   dh::HostBuf hmeta;   // pinned staging for meta
   dh::HostBuf hout;    // pinned staging for accumulate-on-host
-  dh::DevBuf tstat;    // threshold build status
+  dh::DevBuf tstat;    // threshold build status,
+  bool tstat_new = false;  //   to be read after the call: a table was built
   dh::DevBuf aux;      // small per-call arrays (g(r) pair densities)
   dh::DevBuf X64;      // binary64 input coordinates (double4), when a frame has them
   dh::DevBuf P4, P2;   // list kernel: positions in bins (double-floats),

@@ -423,6 +423,11 @@ void Server::admit() {
     d += align_up(sizeof(FrameDev));
     r.job_dev = (StageJob*)d;
     d += align_up(sizeof(StageJob));
+    // (descriptors in the order of the pinned copies: one upload)
+    if (!r.sorts.empty()) {
+      r.sort_dev = (SortSeg*)d;
+      d += align_up(sizeof(SortSeg) * r.sorts.size());
+    }
     r.X = (float4*)d;
     d += align_up(16 * std::max<size_t>((size_t)r.frame.n, 1));
     r.fd_pin = (FrameDev*)p;
@@ -430,8 +435,6 @@ void Server::admit() {
     r.job_pin = (StageJob*)p;
     p += align_up(sizeof(StageJob));
     if (!r.sorts.empty()) {
-      r.sort_dev = (SortSeg*)d;
-      d += align_up(sizeof(SortSeg) * r.sorts.size());
       r.sort_X = (float4*)d;
       d += align_up(16 * (size_t)r.frame.n);
       r.sort_K = (int32_t*)d;
@@ -485,31 +488,38 @@ dh_status Server::prep(Request& r) {
   r.fd_pin->P2 = r.P2;
   std::memset(r.job_pin, 0, sizeof(StageJob));
   r.job_pin->src = r.dev_ptrs ? r.frame.coords : r.raw;
-  r.job_pin->dst = r.sorts.empty() ? r.X : r.sort_X;
+  // a small frame of the list kernel is prepared by one launch, which also clears the output
+  const bool clear = !r.dev_ptrs || !(r.frame.flags & DH_ACCUMULATE);
+  const bool fused = r.pf.list && r.frame.n > 0 && r.frame.n <= kPrepMaxN && r.sort_keys <= kPrepMaxKeys;
+  r.job_pin->dst = r.sorts.empty() || fused ? r.X : r.sort_X;
+  r.job_pin->n_sort = (int32_t)r.sorts.size();
+  r.job_pin->clear = clear ? (int64_t)r.res_count : 0;
   r.job_pin->fd = r.fd;
   r.job_pin->n = r.frame.n;
   r.job_pin->stride = r.stride;
   r.job_pin->chunk0 = 0;
-  DH_CUDA_TRY(cudaMemcpyAsync(r.fd, r.fd_pin, sizeof(FrameDev), cudaMemcpyHostToDevice, st));
-  DH_CUDA_TRY(cudaMemcpyAsync(r.job_dev, r.job_pin, sizeof(StageJob), cudaMemcpyHostToDevice, st));
+  for (size_t q = 0; q < r.sorts.size(); ++q) {
+    r.sort_pin[q] = r.sorts[q];
+    r.sort_pin[q].fd = r.fd;
+  }
+  DH_CUDA_TRY(cudaMemcpyAsync(r.fd, r.fd_pin,
+                              align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob)) + sizeof(SortSeg) * r.sorts.size(),
+                              cudaMemcpyHostToDevice, st));
   if (!r.dev_ptrs && r.frame.n > 0)
     DH_CUDA_TRY(cudaMemcpyAsync(r.raw, r.raw_pin, 4 * (size_t)r.stride * (size_t)r.frame.n,
                                 cudaMemcpyHostToDevice, st));
-  if (!r.dev_ptrs || !(r.frame.flags & DH_ACCUMULATE))
-    DH_CUDA_TRY(cudaMemsetAsync(r.hist, 0, 8 * r.res_count, st));
-  int64_t chunks = (r.frame.n + kStageChunk - 1) / kStageChunk;
-  if (chunks > 0) DH_CUDA_TRY(launch_stage(r.job_dev, 1, chunks, st));
-  DH_CUDA_TRY(launch_frame_setup(r.fd, 1, 0, st));
-  if (!r.sorts.empty()) {
-    for (size_t q = 0; q < r.sorts.size(); ++q) {
-      r.sort_pin[q] = r.sorts[q];
-      r.sort_pin[q].fd = r.fd;
+  if (fused) {
+    DH_CUDA_TRY(launch_prep(r.job_dev, 1, r.frame.n, r.sort_dev, r.sort_C, st));
+  } else {
+    if (clear) DH_CUDA_TRY(cudaMemsetAsync(r.hist, 0, 8 * r.res_count, st));
+    int64_t chunks = (r.frame.n + kStageChunk - 1) / kStageChunk;
+    if (chunks > 0) DH_CUDA_TRY(launch_stage(r.job_dev, 1, chunks, st));
+    DH_CUDA_TRY(launch_frame_setup(r.fd, 1, 0, st));
+    if (!r.sorts.empty()) {
+      DH_CUDA_TRY(cudaMemsetAsync(r.sort_C, 0, 4 * (size_t)r.sort_keys, st));
+      DH_CUDA_TRY(launch_spatial_sort(r.sort_dev, (int)r.sorts.size(), r.sort_max, r.sort_X, r.X, nullptr, nullptr,
+                                      r.sort_K, r.sort_C, r.sort_keys, st));
     }
-    DH_CUDA_TRY(cudaMemcpyAsync(r.sort_dev, r.sort_pin, sizeof(SortSeg) * r.sorts.size(), cudaMemcpyHostToDevice,
-                                st));
-    DH_CUDA_TRY(cudaMemsetAsync(r.sort_C, 0, 4 * (size_t)r.sort_keys, st));
-    DH_CUDA_TRY(launch_spatial_sort(r.sort_dev, (int)r.sorts.size(), r.sort_max, r.sort_X, r.X, nullptr, nullptr,
-                                    r.sort_K, r.sort_C, r.sort_keys, st));
   }
   // marks the end of the preparation: a request cancelled before its first wave
   // keeps its pool memory until this work has finished

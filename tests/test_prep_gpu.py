@@ -1,0 +1,69 @@
+"""Preparation of small frames in one launch, against the FP64 oracle bin for bin.
+
+The frames sit on the edges of the launch: one particle, one thread's, one
+block's and one cluster's worth and one more (the general path), species of few
+particles and empty ones, coordinates of several cells brought home in
+double-floats or in binary64 (from 4,096 cells on), both input types and strides,
+outputs that are cleared and outputs that are added to.
+"""
+import numpy as np
+import pytest
+
+import paper_1808_01478_gb300 as dh
+import workloads as w
+
+pytestmark = pytest.mark.gpu
+
+BOXES = {
+    "none": (w.BOX_NONE, np.zeros(9)),
+    "ortho": (w.BOX_ORTHO, w.ortho_box(11.0, 12.0, 13.0)),
+    "triclinic": (w.BOX_TRICLINIC, w.triclinic_box(12.0, 12.0, 12.0, *w.C3_ANGLES)),
+}
+
+
+@pytest.fixture(scope="module")
+def torch_mod():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch
+
+
+@pytest.mark.parametrize("box", list(BOXES))
+@pytest.mark.parametrize("n,cells,dtype,stride", [
+    (1, 0, "f4", 3), (2, 0, "f4", 4), (129, 3, "f4", 3), (1024, 0, "f8", 3), (1025, 6000, "f4", 3), (4097, 40, "f4", 4),
+    (8192, 2, "f8", 4), (8193, 2000, "f4", 3), (32768, 0, "f4", 3), (32769, 5, "f4", 3)])
+def test_small_frames_match_oracle(torch_mod, oracle_mod, box, n, cells, dtype, stride):
+    box_type, B = BOXES[box]
+    rng = w.rng_for(5000 + n)
+    x = rng.random((n, 3))
+    if box_type == w.BOX_NONE:
+        x = x * 12.0 + 5.0
+    else:
+        m = w.box_matrix(B)
+        x = (x + (rng.integers(-cells, cells + 1, size=(n, 3)) if cells else 0)) @ m.T
+    xs = np.zeros((n, stride), dtype)
+    xs[:, :3] = x
+    cuts = sorted(min(n, k) for k in (1, 1, 130))  # one particle, none, fewer than a run or two, the rest
+    offs = np.array([0, *cuts, n], dtype=np.int64)
+    r_max, nbins = 5.0, 777
+    want = oracle_mod.histogram(np.ascontiguousarray(xs[:, :3]), offs, box_type, B, r_max, nbins)
+    with dh.Context(0) as ctx:
+        dev = torch_mod.from_numpy(xs).cuda()
+        out = torch_mod.full(want.shape, 7, dtype=torch_mod.int64, device="cuda")
+        ctx.histogram(dev, offs, box_type, B, r_max, nbins, out)
+        assert np.array_equal(out.cpu().numpy().view(np.uint64), want)
+        ctx.histogram(dev, offs, box_type, B, r_max, nbins, out, accumulate=True)
+        assert np.array_equal(out.cpu().numpy().view(np.uint64), 2 * want)
+        assert np.array_equal(ctx.histogram(xs, offs, box_type, B, r_max, nbins), want)
+
+
+def test_many_species(torch_mod, oracle_mod):
+    # a counter group per species, more of them than one thread's share of particles
+    n = 300
+    x = w.rng_for(77).random((n, 3)).astype(np.float32) * 9.0
+    offs = np.arange(n + 1, dtype=np.int64)
+    want = oracle_mod.histogram(x, offs, w.BOX_NONE, np.zeros(9), 8.0, 3)
+    with dh.Context(0) as ctx:
+        got = ctx.histogram(torch_mod.from_numpy(x).cuda(), offs, w.BOX_NONE, None, 8.0, 3)
+    assert np.array_equal(got.cpu().numpy().view(np.uint64), want)
