@@ -78,7 +78,6 @@ struct FrameDev {
   float list_grid;    // list kernel: grid of the positions' high parts (a power of two),
   float list_c0;      //   constant part of the window (see list_setup),
   float list_mid;     //   position error of the double-float tier,
-  float list_tie;     //   orthorhombic: distance from half a period re-decided in binary64
   float cull_abs;     //   absolute slack of the distance bounds
   int32_t cmin[3];   // ordered-integer encodings of the per-axis coordinate min / max
   int32_t cmax[3];
@@ -222,8 +221,8 @@ cudaError_t launch_thresholds(double r_max, int32_t nbins, double* T, int32_t* s
 cudaError_t launch_pairs(const PairLaunch& p, int variant, int grid, size_t smem, cudaStream_t stream);
 // The list kernel (dh_list.cu): segments of any frames planned for it.
 cudaError_t launch_list(const ListLaunch& p, int grid, cudaStream_t stream);
-size_t list_kernel_smem(int hist_width);
-int list_kernel_max_width();  // widest sweep of the list kernel on the current device
+int list_kernel_max_width();  // widest sweep of the list kernel on the current device,
+constexpr int kPickWords = 12288;  //   less these bins for frames that need the shortest image
 cudaError_t launch_check_sqrt(unsigned long long* out, cudaStream_t stream);
 cudaError_t launch_check_tiles(const FrameDev* F, int variant, uint64_t n_tiles, uint64_t seed,
                                unsigned long long* out, cudaStream_t stream);

@@ -434,16 +434,6 @@ __device__ inline double half_ulp_below(double D) {
   return ldexp(1.0, E - 25);
 }
 
-// Orthorhombic: float32 and binary64 can round d/L to different images only within
-// eta of a half integer; both images then have |d'_c| within eta L of L/2.  2 eta L:
-__device__ __forceinline__ double ortho_tie(const FrameDev& F, int c, double R, double conv) {
-  const double L = F.B[4 * c];
-  return 2.0 * (half_ulp_below(R) + conv + R * fabs((double)F.invf[c] - F.Linv[c]) + 1e-15 * (R + L));
-}
-__device__ __forceinline__ double ortho_tie_eps(const FrameDev& F, const double* tie_c) {
-  return 2.0 * fmax(tie_c[0], fmax(tie_c[1], tie_c[2])) + 1e-12 * fmin(F.B[0], fmin(F.B[4], F.B[8]));
-}
-
 // The spatial order's grid and the list kernel's window of one frame.
 //
 // The list kernel works in bins, relative to the centre of an i run: x for the
@@ -512,7 +502,6 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
   F.cull_abs = __double2float_ru(reach * 9.5367431640625e-07);  // 2^-20
   F.list_c0 = __double2float_ru(a0 * a0 * 0x1p28 + 0x1p-26);
   F.list_mid = __double2float_ru(4.0 * a0);
-  F.list_tie = F.variant == V_ORTHO ? __double2float_ru((double)F.tie_eps * S * 1.01 + 4.0 * a0) : 0.0f;
   // every decision needs the nearest integer of the root right to within one:
   // window and square-root error below a quarter bin at the far end
   const double tmax = (double)F.nbins + 40.0;
@@ -607,7 +596,11 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
       I[c] = R[c] + K * L;
       if (R[c] / L > 1048576.0) all_defer = 1;  // nearest integer via the 1.5*2^23 trick needs |d/L| < 2^22
       Lmin = fmin(Lmin, L);
-      tie_c[c] = ortho_tie(F, c, R[c], conv[c]);
+      // float32 and binary64 can round d/L to different images only within eta of a
+      // half integer; both images then have |d'_c| within eta L of L/2
+      double eta = (half_ulp_below(R[c]) + conv[c] + R[c] * fabs((double)F.invf[c] - 1.0 / L)) / L +
+                   1e-15 * (R[c] / L + 1.0);
+      tie_c[c] = 2.0 * eta * L;
     }
     // components that can sit at L_c/2 while t <= nbins + 1 (r <= r_max (1 + 1/nbins))
     double rr = F.r_max * (1.0 + 2.0 / (double)F.nbins);
@@ -617,7 +610,7 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
       double t3 = sqrt(tie_c[0] * tie_c[0] + tie_c[1] * tie_c[1] + tie_c[2] * tie_c[2]);
       tie = S * (m >= 3 ? t3 : (m == 2 ? fmin(t3, 1.4142135623730951 * t1) : t1)) * 1.01;
     }
-    tie_eps = ortho_tie_eps(F, tie_c);
+    tie_eps = 2.0 * fmax(tie_c[0], fmax(tie_c[1], tie_c[2])) + 1e-12 * Lmin;
     // uniform-image tiles: the image is subtracted exactly (|k| <= 1), so d'_c
     // errs only by the float32 box entry; the tie term is not needed where the
     // tile's difference range, widened by tie_m = 4 eta L, keeps one image
@@ -836,7 +829,7 @@ __global__ void __launch_bounds__(kPrepBlock, 1)
 
   // ---- the frame's window and grid, by every block for itself
   if (tid == 0) {
-    double R[3], Xm[3], tie_c[3];
+    double R[3], Xm[3];
     for (int c = 0; c < 3; ++c) {
       const float lo = s_all[c], hi = -s_all[3 + c];
       // (a frame without one finite coordinate keeps the initial, empty range)
@@ -851,9 +844,7 @@ __global__ void __launch_bounds__(kPrepBlock, 1)
       const double lo = any ? (double)float_of_ord(F.cmin[c]) : 0.0, hi = any ? (double)float_of_ord(F.cmax[c]) : 0.0;
       R[c] = hi - lo;
       Xm[c] = fmax(fabs(lo), fabs(hi));
-      if (F.variant == V_ORTHO) tie_c[c] = ortho_tie(F, c, R[c], F.X64 ? 2.0 * half_ulp_below(Xm[c]) : 0.0);
     }
-    F.tie_eps = F.variant == V_ORTHO ? (float)ortho_tie_eps(F, tie_c) : 0.0f;
     list_setup(F, R, Xm);
     F.in_range = inside_one_sweep(F, sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]));
   }

@@ -230,7 +230,19 @@ dh_status check_frame(const dh_frame* f, PlannedFrame& pf, int max_width, int li
        0.5 * std::sqrt(B[0] * B[0] + B[4] * B[4] + B[8] * B[8]) <= 0.9995 * min_plane_spacing(B));
   pf.list = list_width > 0 && f->n <= kListMaxN && (in_half || compact);
   pf.pick = !in_half;
-  if (pf.list) max_width = std::min(max_width, list_width);
+  if (pf.list) {
+    const int width = std::min(max_width, list_width - (pf.pick ? kPickWords : 0));
+    // Without a box the tiled kernel, whose sweeps are a little wider, is the faster one
+    // where it needs a single sweep and the list kernel two (51,000 bins: N = 20,000
+    // 223 against 253 us, N = 250,000 19.5 against 21.0 ms), but not with three against
+    // its two (100,000 bins: 381 against 314 us, 32.2 against 24.7 ms), nor with a box,
+    // where each sweep evaluates mostly its own pairs (N = 50,000 orthorhombic 1.54
+    // against 1.16 ms).
+    if (pf.variant == V_NONE && f->nbins > width && f->nbins <= max_width)
+      pf.list = false;
+    else
+      max_width = width;
+  }
   int64_t S = f->n_species;
   pf.src = f;
   pf.n_hist = (int32_t)(S * (S + 1) / 2);
