@@ -45,7 +45,7 @@ struct FrameDev {
   float Bf[9];       // float32 copies of B
   float Bl[9];       // float32(B - Bf): B as double-float (Bf + Bl)
   float invf[3];     // float32 reciprocals: ortho 1/Lx,1/Ly,1/Lz; triclinic 1/ax,1/by,1/cz
-  float S, S_l;      // nbins / r_max as a double-float
+  float S;           // float32(nbins / r_max)
   float dr_f;        // float32(r_max / nbins), the bin width
   float rmax_f;      // float32(r_max)
   float S2;          // float32((nbins / r_max)^2)
@@ -61,24 +61,7 @@ struct FrameDev {
   float rr2;            // orthorhombic: (r_max (1 + 2/nbins))^2, rounded up
   double eps_S;      // |S - nbins/r_max| / (nbins/r_max)
   double eps_S2;     // |S2 - (nbins/r_max)^2| / (nbins/r_max)^2
-  // list kernel (null and unset for other frames); lengths in bins: S = nbins / r_max times the caller's
-  float4* P4;         // home positions: x, y, z to a grid (list_grid) and the rest of x,
-  float2* P2;         //   the rest of y and z
-  float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz)
-  float img_h[27][3], img_l[27][3];  // image vectors -B k as double-floats (index as tshift)
-  float period[3];    // a_x, b_y, c_z
-  int32_t pick;       // r_max beyond half the distance between images: the shortest image counts
   // ---- written on the device
-  int32_t smin[3], smax[3];  // triclinic: the same of the fractional coordinates
-  int32_t wrap;       // the coordinates span more than one cell: P4 is brought home to the first
-                      // (1: in double-floats; 2: in binary64, from 4,096 cells on)
-  int32_t list_slow;  // list kernel: every pair in binary64 (no trust in the images)
-  int32_t list_all;   // list kernel: every listed pair re-decided (window too wide)
-  float key_lo[3], key_inv;  // spatial order: origin and inverse side of the grid
-  float list_grid;    // list kernel: grid of the positions' high parts (a power of two),
-  float list_c0;      //   constant part of the window (see list_setup),
-  float list_mid;     //   position error of the double-float tier,
-  float cull_abs;     //   absolute slack of the distance bounds
   int32_t cmin[3];   // ordered-integer encodings of the per-axis coordinate min / max
   int32_t cmax[3];
   int32_t bad;       // a non-finite coordinate was seen
@@ -98,6 +81,26 @@ struct FrameDev {
   unsigned long long uniform_pairs;  // pairs of (warp i run, j tile) blocks with one nearest image for all
   unsigned long long axis_pairs;     // pairs of such blocks whose image is uniform on all axes but one
   unsigned long long culled_pairs;   // pairs of blocks skipped: no pair of them has its bin in the sweep
+  // ---- spatial order and list kernel (P4 null for other frames); lengths in bins:
+  // S + S_l = nbins / r_max times the caller's.  From the host:
+  float4* P4;         // home positions: x, y, z to a grid (list_grid) and the rest of x,
+  float2* P2;         //   the rest of y and z
+  float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz)
+  float S_l;          // nbins / r_max - S
+  float img_h[27][3], img_l[27][3];  // image vectors -B k as double-floats (index as tshift)
+  float period[3];    // a_x, b_y, c_z
+  int32_t pick;       // r_max beyond half the distance between images: the shortest image counts
+  // ... and from the device
+  int32_t smin[3], smax[3];  // triclinic: range of the fractional coordinates, as cmin and cmax
+  int32_t wrap;       // the coordinates span more than one cell: P4 is brought home to the first
+                      // (1: in double-floats; 2: in binary64, from 4,096 cells on)
+  int32_t list_slow;  // every pair in binary64 (no trust in the images)
+  int32_t list_all;   // every listed pair re-decided (window too wide)
+  float key_lo[3], key_inv;  // spatial order: origin and inverse side of the grid
+  float list_grid;    // grid of the positions' high parts (a power of two),
+  float list_c0;      //   constant part of the window (see list_setup),
+  float list_mid;     //   position error of the double-float tier,
+  float cull_abs;     //   absolute slack of the distance bounds
 };
 
 // One species pair (a,b) of one frame and one bin sweep, cut into kTile x kTile
@@ -205,8 +208,14 @@ cudaError_t launch_stage(const StageJob* jobs, int n_jobs, int64_t n_chunks, cud
 // copies; sorts: all their species; counts: their counters, n_keys in all).
 cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, const SortSeg* sorts, uint32_t* counts,
                         cudaStream_t stream);
-constexpr int64_t kPrepMaxN = 32768, kPrepMaxKeys = 65536;  // particles and counters of a frame
-cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, int pass_hi_max, cudaStream_t stream);
+constexpr int64_t kPrepMaxN = 65536;
+// Within reach of launch_prep: particles and counters of a frame.
+constexpr bool prep_fits(int64_t n, int64_t keys) { return n >= 1 && n <= kPrepMaxN && keys <= 2 * (n <= kPrepMaxN / 2 ? kPrepMaxN / 2 : kPrepMaxN); }
+// ... and better there than with the separate kernels, which use the whole chip.
+constexpr int64_t kPrepBestN = 32768;
+// order: the spatial order's grid and the list kernel's window too; windows: the tiled
+// kernel's window also for frames of the list kernel.
+cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, bool order, bool windows, cudaStream_t stream);
 // Orders each segment's particles from src (src64) into dst (dst64), and for the
 // list kernel into the frame's P4 and P2 with the bounds of its runs.  counts: n_keys
 // counters, zeroed, then n_keys cursors (n_keys: sort_counters over the segments);

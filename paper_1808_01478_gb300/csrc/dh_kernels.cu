@@ -434,6 +434,13 @@ __device__ inline double half_ulp_below(double D) {
   return ldexp(1.0, E - 25);
 }
 
+// No box, one sweep: the largest distance D maps below nbins + 1 even after the
+// float32 roundings of q and of its square root (relative 2^-18 covers them).
+__device__ __forceinline__ bool inside_one_sweep(const FrameDev& F, double D) {
+  return F.variant == V_NONE && F.sweep_width >= F.nbins &&
+         ((double)F.S + (double)F.S_l) * D * (1.0 + 1.0 / 262144.0) < (double)F.nbins + 1.0;
+}
+
 // The spatial order's grid and the list kernel's window of one frame.
 //
 // The list kernel works in bins, relative to the centre of an i run: x for the
@@ -506,13 +513,7 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
   // window and square-root error below a quarter bin at the far end
   const double tmax = (double)F.nbins + 40.0;
   F.list_all = !(8.0 * u * tmax + 4.0 * a0 < 0.25) || !(tmax * 4.76837158203125e-07 < 0.25);
-}
-
-// No box, one sweep: the largest distance D maps below nbins + 1 even after the
-// float32 roundings of q and of its square root (relative 2^-18 covers them).
-__device__ __forceinline__ bool inside_one_sweep(const FrameDev& F, double D) {
-  return F.variant == V_NONE && F.sweep_width >= F.nbins &&
-         ((double)F.S + (double)F.S_l) * D * (1.0 + 1.0 / 262144.0) < (double)F.nbins + 1.0;
+  F.in_range = inside_one_sweep(F, sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]));
 }
 
 // Derives, for one frame, the bound of the float32 decision and of the
@@ -545,24 +546,13 @@ __device__ __forceinline__ bool inside_one_sweep(const FrameDev& F, double D) {
 // beta also carries 2^-28 for the binary64 rounding of t itself (< 2^-29 for t < 2^22).
 // If a precondition of the float32 path fails (nearest-integer range,
 // triclinic margin) or the t-space bound reaches 1/4, every pair is deferred.
-__global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
-  int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= n_frames) return;
-  FrameDev& F = frames[f];
+__device__ void window_setup(FrameDev& F, const double* R, const double* Xm) {
   const double u = 1.0 / 16777216.0;
-  double R[3] = {0, 0, 0};
   // binary64 input: the float32 path starts from coordinates rounded to float32,
   // each within half an ulp of the largest magnitude on its axis
   double conv[3] = {0, 0, 0};
-  double Xm[3] = {0, 0, 0};  // largest coordinate magnitude per axis
-  if (F.n > 0 && F.cmin[0] <= F.cmax[0]) {
-    for (int c = 0; c < 3; ++c) {
-      double lo = float_of_ord(F.cmin[c]), hi = float_of_ord(F.cmax[c]);
-      R[c] = hi - lo;
-      Xm[c] = fmax(fabs(lo), fabs(hi));
-      if (F.X64) conv[c] = 2.0 * half_ulp_below(Xm[c]);
-    }
-  }
+  if (F.X64)
+    for (int c = 0; c < 3; ++c) conv[c] = 2.0 * half_ulp_below(Xm[c]);
   double S = (double)F.nbins / F.r_max;
   double alpha = 3.0 * u + 0.5 * F.eps_S2;
   double a[3] = {0, 0, 0};
@@ -712,7 +702,6 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
   F.mid2 = (float)(1.0 / 274877906944.0);                                                   // 2^-38
   F.mid1 = (float)(2.0 * amid / S * 1.01);
   F.tie_eps = (float)tie_eps;
-  list_setup(F, R, Xm);
   F.delta = (float)fmin(delta, 1.0);
   F.alpha_t = (float)alpha;
   F.beta_t = (float)beta;
@@ -729,6 +718,37 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
   }
 }
 
+// Coordinate ranges and largest magnitudes per axis (zero for a frame without a finite coordinate).
+__device__ __forceinline__ void frame_ranges(const FrameDev& F, double* R, double* Xm) {
+  const bool any = F.n > 0 && F.cmin[0] <= F.cmax[0];
+  for (int c = 0; c < 3; ++c) {
+    const double lo = any ? (double)float_of_ord(F.cmin[c]) : 0.0, hi = any ? (double)float_of_ord(F.cmax[c]) : 0.0;
+    R[c] = hi - lo;
+    Xm[c] = fmax(fabs(lo), fabs(hi));
+  }
+}
+
+// One block per frame: its descriptor in shared memory, where one thread's chain of
+// dependent accesses costs a tenth of what it does in global memory, and of the two
+// setups those that the frame needs: order (spatial order, list kernel) and the
+// window of the tiled kernel, of which frames of the list kernel go without unless
+// asked for (windows).
+__global__ void frame_setup_kernel(FrameDev* frames, int order, int windows) {
+  __shared__ __align__(16) FrameDev F;
+  uint32_t* const dev = reinterpret_cast<uint32_t*>(frames + blockIdx.x);
+  uint32_t* const own = reinterpret_cast<uint32_t*>(&F);
+  for (int k = threadIdx.x; k < (int)(sizeof(FrameDev) / 4); k += blockDim.x) own[k] = dev[k];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double R[3], Xm[3];
+    frame_ranges(F, R, Xm);
+    if (order) list_setup(F, R, Xm);
+    if (windows || !F.P4) window_setup(F, R, Xm);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < (int)(sizeof(FrameDev) / 4); k += blockDim.x) dev[k] = own[k];
+}
+
 // ------------------------------------------------------------------ small frames: one launch
 
 // Staging, list_setup and spatial order of one frame per cluster, for frames of
@@ -741,12 +761,14 @@ __global__ void frame_setup_kernel(FrameDev* frames, int n_frames) {
 // shared memory once.  Whole call, before -> now: N = 2,000 without a box 91 -> 64 us,
 // N = 8,000 triclinic 159 -> 127 us, N = 32,000 orthorhombic 429 -> 411 us; larger
 // frames have work for more SMs than a cluster's and keep the separate kernels.
-constexpr int kPrepBlock = 1024, kPrepPer = 4, kPrepCluster = 8, kPrepScan = 8;
-static_assert((int64_t)kPrepBlock * kPrepPer * kPrepCluster == kPrepMaxN, "particles per cluster");
+constexpr int kPrepBlock = 1024, kPrepCluster = 8;
+static_assert((int64_t)kPrepBlock * 8 * kPrepCluster == kPrepMaxN, "particles per cluster");
+template <int PER>  // particles per thread, at most; twice as many counters
 __global__ void __launch_bounds__(kPrepBlock, 1)
     prep_kernel(const StageJob* __restrict__ jobs, const SortSeg* __restrict__ sorts, uint32_t* counts) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
+  constexpr int kPrepPer = PER, kPrepScan = 2 * PER;
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int slot = rank * kPrepBlock + tid, slots = C * kPrepBlock;
@@ -839,14 +861,8 @@ __global__ void __launch_bounds__(kPrepBlock, 1)
       if (frac && s_all[9 + c] < INFINITY) F.smax[c] = ord_of(-s_all[9 + c]);
     }
     F.bad = s_all[12] < 0.0f;
-    const bool any = F.cmin[0] <= F.cmax[0];
-    for (int c = 0; c < 3; ++c) {
-      const double lo = any ? (double)float_of_ord(F.cmin[c]) : 0.0, hi = any ? (double)float_of_ord(F.cmax[c]) : 0.0;
-      R[c] = hi - lo;
-      Xm[c] = fmax(fabs(lo), fabs(hi));
-    }
+    frame_ranges(F, R, Xm);
     list_setup(F, R, Xm);
-    F.in_range = inside_one_sweep(F, sqrt(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]));
   }
   __syncthreads();
   if (rank == 0 && tid < fwords) reinterpret_cast<uint32_t*>(dev)[tid] = reinterpret_cast<const uint32_t*>(&F)[tid];
@@ -2449,13 +2465,14 @@ cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, const S
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, prep_kernel, jobs, sorts, counts);
+  return max_n * 2 <= kPrepMaxN ? cudaLaunchKernelEx(&cfg, prep_kernel<4>, jobs, sorts, counts)
+                                : cudaLaunchKernelEx(&cfg, prep_kernel<8>, jobs, sorts, counts);
 }
 
-cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, int, cudaStream_t stream) {
+cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, bool order, bool windows, cudaStream_t stream) {
   clear_stale_error();
   if (n_frames <= 0) return cudaSuccess;
-  frame_setup_kernel<<<(n_frames + 63) / 64, 64, 0, stream>>>(frames, n_frames);
+  frame_setup_kernel<<<n_frames, 128, 0, stream>>>(frames, order, windows);
   return cudaGetLastError();
 }
 

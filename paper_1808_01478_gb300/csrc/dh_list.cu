@@ -110,7 +110,8 @@ struct SegState {
   int lo, hi;             // the sweep's bins
   float rc_hi2, rc_lo2;   // images kept: nearest distance^2 <= rc_hi2, farthest^2 >= rc_lo2
   float in_hi2, in_lo2;   // every pair in the sweep: farthest^2 <= in_hi2, nearest^2 >= in_lo2
-  float grid, c0, abs;    // FrameDev list_grid, list_c0, cull_abs
+  float grid, c0, abs, mid;  // FrameDev list_grid, list_c0, cull_abs, list_mid
+  float nbins;
   int n_img, all, slow;   // images of a particle; FrameDev list_all, list_slow
   int inner;              // FrameDev in_range: nearly every block is an inner one
   long long items, item_base;
@@ -220,14 +221,13 @@ __device__ __noinline__ int exact_listed_bin(const FrameDev& F, int i, int j, fl
                                : exact_listed<V_TRIC_SEARCH>(F, i, j, d, true);
 }
 
-// Bin of a re-decided pair from q in double-float arithmetic (about 44 bits) for
+// Bin of a re-decided pair (particles i and j of the segment's species) from q in double-float arithmetic (about 44 bits) for
 // the listed image m, and the integer n nearest to its root.  An image inside r_max
 // is the definition's: the shortest by a margin (F.pick), else the only one there
 // (check_frame), up to ties of two at r_max itself.  When q is too close to n^2, or the
 // image is not known (m < 0), the binary64 replay decides.
-__device__ __forceinline__ int listed_bin(const SegState& G, const FrameDev& F, int i, int j, int m, float& n,
-                                          unsigned& nexact) {
-  const Pos a = unpack(__ldg(F.P4 + i), __ldg(F.P2 + i)), b = unpack(__ldg(F.P4 + j), __ldg(F.P2 + j));
+__device__ __forceinline__ int listed_bin(const SegState& G, int i, int j, int m, float& n, unsigned& nexact) {
+  const Pos a = unpack(__ldg(G.P4i + i), __ldg(G.P2i + i)), b = unpack(__ldg(G.P4j + j), __ldg(G.P2j + j));
   const float ah[3] = {a.h.x, a.h.y, a.h.z}, al[3] = {a.l.x, a.l.y, a.l.z};
   const float bh[3] = {b.h.x, b.h.y, b.h.z}, bl[3] = {b.l.x, b.l.y, b.l.z};
   const Pos v = unpack(G.V4[max(m, 0)], G.V2[max(m, 0)]);
@@ -244,11 +244,11 @@ __device__ __forceinline__ int listed_bin(const SegState& G, const FrameDev& F, 
   const float diff = __fadd_rn(__fsub_rn(q.h, n2.h), __fsub_rn(q.l, n2.l));
   // 2^-38: the double-float arithmetic and the binary64 rounding of the definition;
   // at r_max also the images that tie at half a period, 2^-40 of it within r_max (check_frame)
-  const float rel = n >= (float)F.nbins ? 0x1p-36f : 0x1p-38f;
-  if (m >= 0 && (fabsf(diff) > __fmaf_rn(rel, q.h, F.list_mid * s) + 0x1p-60f || n < 0.5f))
-    return (int)fminf(n, (float)F.nbins + 1.0f) - (diff < 0.0f && n >= 0.5f ? 1 : 0);
+  const float rel = n >= G.nbins ? 0x1p-36f : 0x1p-38f;
+  if (m >= 0 && (fabsf(diff) > __fmaf_rn(rel, q.h, G.mid * s) + 0x1p-60f || n < 0.5f))
+    return (int)fminf(n, G.nbins + 1.0f) - (diff < 0.0f && n >= 0.5f ? 1 : 0);
   ++nexact;
-  return exact_listed_bin(F, i, j, make_float3(d[0].h, d[1].h, d[2].h), F.pick != 0);
+  return exact_listed_bin(*G.F, G.i0 + i, G.j0 + j, make_float3(d[0].h, d[1].h, d[2].h), G.F->pick != 0);
 }
 
 // The shortest image of a pair in float32, -1 if another comes within 2^-16 of it.
@@ -304,7 +304,6 @@ __device__ __noinline__ int replay_rel(const SegState& G, int i, int j, int m) {
 // Pairs with kAnyImage were not counted.
 constexpr uint32_t kNearPair = 0x80000000u;
 __device__ __noinline__ int list_drain(const SegState& G, uint2* q, int qcount, uint32_t* sh, int lane) {
-  const FrameDev& F = *G.F;
   const int count = qcount < 32 ? qcount : 32;
   unsigned nexact = 0;
   __syncwarp();
@@ -316,8 +315,8 @@ __device__ __noinline__ int list_drain(const SegState& G, uint2* q, int qcount, 
     float n;
     int bin, prov;
     const bool any = e.x >= kAnyImage;
-    if (any) m = picked_image(F, G.i0 + i, G.j0 + j);
-    bin = listed_bin(G, F, G.i0 + i, G.j0 + j, m, n, nexact) - G.lo;
+    if (any) m = picked_image(*G.F, G.i0 + i, G.j0 + j);
+    bin = listed_bin(G, i, j, m, n, nexact) - G.lo;
     prov = any ? -1 : (int)n - 1 - G.lo;
     if (e.y & kNearPair) prov = replay_rel(G, i, j, m);
     if (bin != prov) {
@@ -670,6 +669,8 @@ __device__ void enter_segment(const ListSegment& S, SegCounter* ctr, long long n
   G.grid = F.list_grid;
   G.c0 = F.list_c0;
   G.abs = F.cull_abs;
+  G.mid = F.list_mid;
+  G.nbins = (float)F.nbins;
   G.n_img = F.variant == V_NONE ? 1 : 27;
   G.all = F.list_all;
   G.slow = F.list_slow;

@@ -20,6 +20,7 @@
 
 #include <cstring>
 #include <mutex>
+#include <vector>
 
 #include "dh_runtime.h"
 
@@ -45,6 +46,46 @@ static_assert(sizeof(FrameDev) <= kNaFrame && sizeof(StageJob) <= kNaJob && size
               "scratch slots too small");
 constexpr int kNaMaxSegs = (int)(kNaSegs / sizeof(Segment));
 constexpr int kNaMaxDevices = 64;
+
+// Frames of the list kernel share the scratch out anew, in one upload up to T:
+//   Control | FrameDev | StageJob | SortSeg[] | ListSegment[] | SegCounter[] |
+//   T | run bounds | P4 | P2 | ordered coordinates | cell counters
+// (about 46 bytes per particle and 16 per bin: 60,000 particles with 10,000 bins).
+struct NaListPlan {
+  PlannedFrame pf;
+  std::vector<SortSeg> sorts;
+  std::vector<ListSegment> segs;
+  int64_t items = 0;
+  int split = 1;
+  size_t sort_at = 0, seg_at = 0, ctr_at = 0, T_at = 0, bnd_at = 0, P4_at = 0, P2_at = 0, X_at = 0, cells_at = 0;
+};
+
+// False when the frame is not one for the list kernel or does not fit: the tiled kernel takes it.
+bool plan_list(const dh_frame* f, int max_width, int num_sms, unsigned char* base, NaListPlan& p) {
+  if (check_frame(f, p.pf, max_width, list_kernel_max_width()) != DH_OK || !p.pf.list) return false;
+  FrameDev* fd = (FrameDev*)(base + kNaOffFrame);
+  int64_t keys = 0, most = 0;
+  p.sorts = plan_spatial_order(p.pf, fd, 0, 0, &keys, &most);
+  if (!prep_fits(f->n, keys)) return false;
+  p.split = list_split_for((double)p.pf.pairs / ((double)kRun * kRun) * p.pf.sweeps, num_sms);
+  p.items = add_list_segments(p.pf, fd, 0, p.segs, p.split);
+  size_t at = kNaOffSegs;
+  auto part = [&at](size_t bytes) {
+    const size_t here = at;
+    at += (bytes + 255) & ~(size_t)255;
+    return here;
+  };
+  p.sort_at = part(sizeof(SortSeg) * p.sorts.size());
+  p.seg_at = part(sizeof(ListSegment) * p.segs.size());
+  p.ctr_at = part(sizeof(SegCounter) * p.segs.size());
+  p.T_at = part(16 * ((size_t)f->nbins + 1));
+  p.bnd_at = part(2 * sizeof(float4) * (size_t)frame_runs(f));
+  p.P4_at = part(sizeof(float4) * (size_t)f->n);
+  p.P2_at = part(sizeof(float2) * (size_t)f->n);
+  p.X_at = part(sizeof(float4) * (size_t)f->n);
+  p.cells_at = part(sizeof(uint32_t) * (size_t)keys);
+  return at <= kNaBytes;
+}
 
 // The scratch itself.  Host code must not pass this name to a kernel: on the
 // host it is only a stand-in; its device address comes from cudaGetSymbolAddress.
@@ -105,8 +146,6 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   FrameDev* fd = (FrameDev*)(base + kNaOffFrame);
   StageJob* job = (StageJob*)(base + kNaOffJob);
   Segment* segs = (Segment*)(base + kNaOffSegs);
-  double* T = (double*)(base + kNaOffT);
-  float4* X = (float4*)(base + kNaOffX);
 
   // Every host-side check comes before the first enqueued operation, so that a
   // call that fails leaves the caller's output and the shared scratch untouched.
@@ -120,48 +159,77 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   const int bps = n_items > 0 ? pair_kernel_blocks_per_sm(pf.variant, pf.sweep_width, 1, block) : 1;
   if (bps < 1) return fail(DH_ERR_INVALID, "histogram of %d bins does not fit in shared memory", pf.sweep_width);
 
-  // Host-side descriptors live on the stack; the copies below read them before returning.
-  FrameDev hF;
-  fill_frame_dev(pf, hF, X, frame->out, T);
-  StageJob hJ;
-  std::memset(&hJ, 0, sizeof hJ);
+  // Small frames go the way of dh_histogram: ordered by launch_prep and counted by
+  // the list kernel (N = 30,000 triclinic, two species, 8,192 bins: 595 -> 421 us).
+  NaListPlan lp;
+  const bool list = plan_list(frame, max_width, num_sms, base, lp);
+  double* T = (double*)(base + (list ? lp.T_at : kNaOffT));
+  float4* X = (float4*)(base + (list ? lp.X_at : kNaOffX));
+  const bool clear = !(frame->flags & DH_ACCUMULATE);
+  const size_t out_words = (size_t)pf.n_hist * (size_t)frame->nbins;
+
+  // The descriptors, uploaded in one copy that has read them when it returns; what
+  // must start at zero is part of it.
+  std::vector<unsigned char> up(list ? lp.T_at : kNaOffSegs + sizeof(Segment) * (size_t)n_segs, 0);
+  FrameDev& hF = *(FrameDev*)(up.data() + kNaOffFrame);
+  fill_frame_dev(list ? lp.pf : pf, hF, X, frame->out, T);
+  StageJob& hJ = *(StageJob*)(up.data() + kNaOffJob);
   hJ.src = frame->coords;
   hJ.dst = X;
   hJ.fd = fd;
   hJ.n = frame->n;
   hJ.stride = (frame->flags & DH_COORDS_F4) ? 4 : 3;
-  hJ.chunk0 = 0;
-  size_t out_bytes = sizeof(uint64_t) * (size_t)pf.n_hist * (size_t)frame->nbins;
-
-  // Clear what must start at zero, upload descriptors, build the table, stage, run.
-  DH_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Control), st));
-  DH_CUDA_TRY(cudaMemcpyAsync(fd, &hF, sizeof(FrameDev), cudaMemcpyHostToDevice, st));
-  DH_CUDA_TRY(cudaMemcpyAsync(job, &hJ, sizeof(StageJob), cudaMemcpyHostToDevice, st));
-  if (n_segs > 0) DH_CUDA_TRY(cudaMemcpyAsync(segs, hS, sizeof(Segment) * n_segs, cudaMemcpyHostToDevice, st));
-  if (!(frame->flags & DH_ACCUMULATE)) DH_CUDA_TRY(cudaMemsetAsync(frame->out, 0, out_bytes, st));
-  DH_CUDA_TRY(launch_thresholds(frame->r_max, frame->nbins, T, &ctl->status, st));
-  int64_t chunks = (frame->n + kStageChunk - 1) / kStageChunk;
-  if (chunks > 0) DH_CUDA_TRY(launch_stage(job, 1, chunks, st));
-  DH_CUDA_TRY(launch_frame_setup(fd, 1, 0, st));
-  if (n_items > 0) {
-    PairLaunch L;
-    std::memset(&L, 0, sizeof L);
-    L.block = block;
-    L.segs = segs;
-    L.n_segs = n_segs;
-    L.n_items = n_items;
-    L.hist_width = pf.sweep_width;
-    L.multi = pf.sweeps > 1;
-    L.ctl = ctl;
-    DH_CUDA_TRY(launch_pairs(L, pf.variant, pair_grid(num_sms, bps, n_items),
-                             pair_kernel_smem(pf.sweep_width, 1, block), st));
+  if (list) {
+    hF.bnd = (float4*)(base + lp.bnd_at);
+    hF.P4 = (float4*)(base + lp.P4_at);
+    hF.P2 = (float2*)(base + lp.P2_at);
+    hJ.n_sort = (int32_t)lp.sorts.size();
+    hJ.clear = clear ? (int64_t)out_words : 0;
+    std::memcpy(up.data() + lp.sort_at, lp.sorts.data(), sizeof(SortSeg) * lp.sorts.size());
+    if (!lp.segs.empty()) std::memcpy(up.data() + lp.seg_at, lp.segs.data(), sizeof(ListSegment) * lp.segs.size());
+  } else if (n_segs > 0) {
+    std::memcpy(up.data() + kNaOffSegs, hS, sizeof(Segment) * (size_t)n_segs);
   }
-  // Read back the flags into stack memory and wait.
-  int32_t status = 0, bad = 0;
-  DH_CUDA_TRY(cudaMemcpyAsync(&status, &ctl->status, sizeof status, cudaMemcpyDeviceToHost, st));
-  DH_CUDA_TRY(cudaMemcpyAsync(&bad, &fd->bad, sizeof bad, cudaMemcpyDeviceToHost, st));
+  DH_CUDA_TRY(cudaMemcpyAsync(base, up.data(), up.size(), cudaMemcpyHostToDevice, st));
+  DH_CUDA_TRY(launch_thresholds(frame->r_max, frame->nbins, T, &ctl->status, st));
+  if (list) {
+    DH_CUDA_TRY(launch_prep(job, 1, frame->n, (const SortSeg*)(base + lp.sort_at), (uint32_t*)(base + lp.cells_at), st));
+    if (lp.items > 0) {
+      ListLaunch L;
+      std::memset(&L, 0, sizeof L);
+      L.segs = (const ListSegment*)(base + lp.seg_at);
+      L.ctr = (SegCounter*)(base + lp.ctr_at);
+      L.n_segs = (int32_t)lp.segs.size();
+      L.hist_width = lp.pf.sweep_width;
+      L.n_items = lp.items;
+      L.split = lp.split;
+      L.multi = lp.pf.sweeps > 1;
+      L.pick = lp.pf.pick;
+      DH_CUDA_TRY(launch_list(L, pair_grid(num_sms, 1, lp.items), st));
+    }
+  } else {
+    if (clear) DH_CUDA_TRY(cudaMemsetAsync(frame->out, 0, sizeof(uint64_t) * out_words, st));
+    int64_t chunks = (frame->n + kStageChunk - 1) / kStageChunk;
+    if (chunks > 0) DH_CUDA_TRY(launch_stage(job, 1, chunks, st));
+    DH_CUDA_TRY(launch_frame_setup(fd, 1, false, false, st));
+    if (n_items > 0) {
+      PairLaunch L;
+      std::memset(&L, 0, sizeof L);
+      L.block = block;
+      L.segs = segs;
+      L.n_segs = n_segs;
+      L.n_items = n_items;
+      L.hist_width = pf.sweep_width;
+      L.multi = pf.sweeps > 1;
+      L.ctl = ctl;
+      DH_CUDA_TRY(launch_pairs(L, pf.variant, pair_grid(num_sms, bps, n_items),
+                               pair_kernel_smem(pf.sweep_width, 1, block), st));
+    }
+  }
+  // Read back the flags (in Control and FrameDev) and wait.
+  DH_CUDA_TRY(cudaMemcpyAsync(up.data(), base, kNaOffJob, cudaMemcpyDeviceToHost, st));
   DH_CUDA_TRY(cudaStreamSynchronize(st));
-  if (status != 0) return fail(DH_ERR_CUDA, "bin threshold table did not converge");
-  if (bad) return fail(DH_ERR_INVALID, "frame has non-finite coordinates");
+  if (((const Control*)up.data())->status != 0) return fail(DH_ERR_CUDA, "bin threshold table did not converge");
+  if (hF.bad) return fail(DH_ERR_INVALID, "frame has non-finite coordinates");
   return DH_OK;
 }

@@ -673,8 +673,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
       P.sort_keys += keys;
       P.sort_max = std::max(P.sort_max, most);
       sort0[f + 1] = (int)sorts.size();
-      P.prep = P.prep && on_list(f) && xoff[f + 1] - xoff[f] >= 1 && xoff[f + 1] - xoff[f] <= kPrepMaxN &&
-               keys <= kPrepMaxKeys;
+      P.prep = P.prep && on_list(f) && xoff[f + 1] - xoff[f] <= kPrepBestN && prep_fits(xoff[f + 1] - xoff[f], keys);
     }
     P.n_sort = (int)sorts.size();
     P.sort_particles = xoff[k];
@@ -802,7 +801,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
       DH_CUDA_TRY(launch_stage(dJ, P.n_jobs, P.n_chunks, st));
       ++launched;
     }
-    DH_CUDA_TRY(launch_frame_setup(dF, k, 0, st));  // the windows, and the grid of the spatial order
+    DH_CUDA_TRY(launch_frame_setup(dF, k, true, !P.with_pairs, st));  // the windows, and the grid of the spatial order
     ++launched;
   }
   if (!P.prep && P.n_sort > 0) {

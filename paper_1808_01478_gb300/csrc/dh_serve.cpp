@@ -490,7 +490,7 @@ dh_status Server::prep(Request& r) {
   r.job_pin->src = r.dev_ptrs ? r.frame.coords : r.raw;
   // a small frame of the list kernel is prepared by one launch, which also clears the output
   const bool clear = !r.dev_ptrs || !(r.frame.flags & DH_ACCUMULATE);
-  const bool fused = r.pf.list && r.frame.n > 0 && r.frame.n <= kPrepMaxN && r.sort_keys <= kPrepMaxKeys;
+  const bool fused = r.pf.list && r.frame.n <= kPrepBestN && prep_fits(r.frame.n, r.sort_keys);
   r.job_pin->dst = r.sorts.empty() || fused ? r.X : r.sort_X;
   r.job_pin->n_sort = (int32_t)r.sorts.size();
   r.job_pin->clear = clear ? (int64_t)r.res_count : 0;
@@ -514,7 +514,7 @@ dh_status Server::prep(Request& r) {
     if (clear) DH_CUDA_TRY(cudaMemsetAsync(r.hist, 0, 8 * r.res_count, st));
     int64_t chunks = (r.frame.n + kStageChunk - 1) / kStageChunk;
     if (chunks > 0) DH_CUDA_TRY(launch_stage(r.job_dev, 1, chunks, st));
-    DH_CUDA_TRY(launch_frame_setup(r.fd, 1, 0, st));
+    DH_CUDA_TRY(launch_frame_setup(r.fd, 1, true, false, st));
     if (!r.sorts.empty()) {
       DH_CUDA_TRY(cudaMemsetAsync(r.sort_C, 0, 4 * (size_t)r.sort_keys, st));
       DH_CUDA_TRY(launch_spatial_sort(r.sort_dev, (int)r.sorts.size(), r.sort_max, r.sort_X, r.X, nullptr, nullptr,

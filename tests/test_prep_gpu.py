@@ -67,3 +67,22 @@ def test_many_species(torch_mod, oracle_mod):
     with dh.Context(0) as ctx:
         got = ctx.histogram(torch_mod.from_numpy(x).cuda(), offs, w.BOX_NONE, None, 8.0, 3)
     assert np.array_equal(got.cpu().numpy().view(np.uint64), want)
+
+
+@pytest.mark.parametrize("box", list(BOXES))
+@pytest.mark.parametrize("n,nbins", [(1, 5), (2, 5), (129, 60000), (8193, 9000), (32769, 700), (65536, 700),
+                                     (65536, 20000), (65537, 700)])
+def test_allocation_free_frames_match_dh_histogram(torch_mod, box, n, nbins):
+    # both ways through the fixed scratch: ordered for the list kernel where everything
+    # fits (not with 65,536 particles and 20,000 bins, nor with 65,537), and in place
+    box_type, B = BOXES[box]
+    m = np.eye(3) * 12.0 if box_type == w.BOX_NONE else w.box_matrix(B)
+    x = torch_mod.from_numpy((w.rng_for(6000 + n).random((n, 3)) @ m.T).astype(np.float32)).cuda()
+    offs = np.array([0, n // 3, n // 3, n], dtype=np.int64)
+    with dh.Context(0) as ctx:
+        want = ctx.histogram(x, offs, box_type, B, 5.0, nbins)
+    out = torch_mod.full((6, nbins), 7, dtype=torch_mod.int64, device="cuda")
+    dh.dh_histogram_noalloc(dh.FrameArgs(x, offs, box_type, B, 5.0, nbins, out).frame)
+    assert torch_mod.equal(out, want)
+    dh.dh_histogram_noalloc(dh.FrameArgs(x, offs, box_type, B, 5.0, nbins, out, True).frame)
+    assert torch_mod.equal(out, 2 * want)
