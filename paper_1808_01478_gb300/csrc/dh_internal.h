@@ -145,24 +145,34 @@ struct StageJob {
   int32_t chunk0;    // first staging chunk of this job
   // launch_prep: the frame's species (SortSeg), and the words of its output to clear
   int32_t sort0, n_sort;
+  int32_t strips, pad;  // some species is ordered in strips
   int64_t clear;
 };
 constexpr int kStageChunk = 1024;
 
-// Spatial ordering of one species of one periodic frame: its particles are
-// grouped by cell of a 2^g x 2^g x 2^g grid over the fractional coordinates, in
-// Morton order, so that tiles of consecutive particles are compact in space.
-// The histogram does not depend on the order of particles within a species.
+// Spatial ordering of one species, by counting sorts whose cells are the keys; the
+// histogram does not depend on the order of particles within a species.  Either in
+// one pass along a Hilbert curve over 2^g cells per axis, which keeps any number of
+// consecutive particles compact; or (nb > 0) in slabs of equal counts along x, each
+// in columns along y, each along z, in three passes over cells of each axis: runs of
+// kRun particles become boxes as near to cubes as can be.
 struct SortSeg {
   const FrameDev* fd;
   int64_t x0;        // first particle (index into the packed coordinates)
-  int32_t n;         // particles
-  int32_t g;         // grid bits per axis
-  int64_t key0;      // first counter of this segment (2^(3g) counters; a multiple of four)
   int64_t f0;        // x0 of the frame's first particle
+  int64_t key0[3];   // first counter of each pass (Hilbert: of the last, the others have none)
+  int32_t n;         // particles
+  int32_t g;         // Hilbert: grid bits per axis
+  int32_t nb[3];     // strips: cells along x, y and z, multiples of four
+  int32_t n_slab, n_col;   // slabs, columns per slab
+  int32_t slab, col;       // particles per slab and per column, multiples of kRun
   int32_t run0;      // first run of this species in the frame's bounds
-  int32_t pad;
 };
+// Counters of a pass.
+__host__ __device__ inline int64_t sort_keys(const SortSeg& S, int pass) {
+  if (S.nb[0] == 0) return pass < 2 ? 0 : S.g > 0 ? (int64_t)1 << (3 * S.g) : 4;
+  return (int64_t)S.nb[pass] * (pass == 0 ? 1 : pass == 1 ? S.n_slab : S.n_slab * S.n_col);
+}
 constexpr int kSortChunk = 256;
 
 struct Control {
@@ -205,25 +215,46 @@ struct ListLaunch {
 cudaError_t launch_stage(const StageJob* jobs, int n_jobs, int64_t n_chunks, cudaStream_t stream);
 // Staging, setup and spatial order of small frames of the list kernel in one
 // launch (jobs: one per frame, n <= max_n <= kPrepMaxN, dst and dst64 the ordered
-// copies; sorts: all their species; counts: their counters, n_keys in all).
-cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, const SortSeg* sorts, uint32_t* counts,
-                        cudaStream_t stream);
+// copies; strips: some species is ordered so; sorts: all their species; counts:
+// their counters).
+cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, bool strips, const SortSeg* sorts,
+                        uint32_t* counts, cudaStream_t stream);
 constexpr int64_t kPrepMaxN = 65536;
 // Within reach of launch_prep: particles and counters of a frame.
-constexpr bool prep_fits(int64_t n, int64_t keys) { return n >= 1 && n <= kPrepMaxN && keys <= 2 * (n <= kPrepMaxN / 2 ? kPrepMaxN / 2 : kPrepMaxN); }
+constexpr int kPrepBlock = 1024, kPrepCluster = 8;
+inline int prep_blocks(int64_t max_n) {
+  // one particle per thread up to the largest portable cluster (two or four per
+  // thread: N = 4,000 without a box 72 and 80 us a call instead of 65)
+  int blocks = 1;
+  while (blocks < kPrepCluster && (int64_t)blocks * kPrepBlock < max_n) blocks *= 2;
+  return blocks;
+}
+inline bool prep_fits(int64_t n, int64_t keys) {
+  return n >= 1 && n <= kPrepMaxN && keys <= (int64_t)prep_blocks(n) * kPrepBlock * (2 * n <= kPrepMaxN ? 8 : 16);
+}
 // ... and better there than with the separate kernels, which use the whole chip.
 constexpr int64_t kPrepBestN = 32768;
 // order: the spatial order's grid and the list kernel's window too; windows: the tiled
 // kernel's window also for frames of the list kernel.
 cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, bool order, bool windows, cudaStream_t stream);
+// What a set of SortSeg needs.
+struct SortPlan {
+  int64_t keys = 0;               // counters of all passes
+  int64_t max_n = 0;              // the largest species,
+  int64_t max_keys[3] = {0, 0, 0};  // and the most counters of one in each pass
+  void add(const SortPlan& o) {
+    keys += o.keys;
+    max_n = o.max_n > max_n ? o.max_n : max_n;
+    for (int p = 0; p < 3; ++p) max_keys[p] = o.max_keys[p] > max_keys[p] ? o.max_keys[p] : max_keys[p];
+  }
+};
 // Orders each segment's particles from src (src64) into dst (dst64), and for the
-// list kernel into the frame's P4 and P2 with the bounds of its runs.  counts: n_keys
-// counters, zeroed, then n_keys cursors (n_keys: sort_counters over the segments);
-// keys: one per particle; the binary64 arrays may be null.
-cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, int64_t max_n, const float4* src, float4* dst,
-                                const double4* src64, double4* dst64, int32_t* keys, uint32_t* counts, int64_t n_keys,
+// list kernel into the frame's P4 and P2 with the bounds of its runs.  counts:
+// plan.keys counters, zeroed, then as many cursors; keys: two per particle; the
+// binary64 arrays may be null.
+cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, const SortPlan& plan, const float4* src, float4* dst,
+                                const double4* src64, double4* dst64, int2* keys, uint32_t* counts,
                                 cudaStream_t stream);
-int sort_grid_bits(int64_t n);  // grid bits per axis for a species of n particles
 cudaError_t launch_thresholds(double r_max, int32_t nbins, double* T, int32_t* status,
                               cudaStream_t stream);
 // One pair-kernel launch over segments whose frames all have minimum-image variant `variant`.

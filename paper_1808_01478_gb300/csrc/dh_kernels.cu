@@ -296,32 +296,48 @@ __device__ __forceinline__ void list_position(const FrameDev& F, float4 p, const
   P2 = make_float2(y.l, z.l);
 }
 
-// Cell of a particle on the curve (only the order depends on it).
-__device__ __forceinline__ uint32_t cell_key(const FrameDev& F, float4 p, int g) {
-  if (g == 0) return 0u;
+// Cell of a particle in a pass of the spatial order (only the order depends on it):
+// on the curve, or its slab's (pass 1) or column's (pass 2) cell along the pass's
+// axis.  rank: its place after the pass before.
+__device__ __forceinline__ int sort_cell(const FrameDev& F, const SortSeg& S, float4 p, int pass, int rank) {
+  if (S.nb[0] == 0 && S.g == 0) return 0;
   if (F.wrap) {
     const float3 w = home32(F, p.x, p.y, p.z);
     p.x = w.x;
     p.y = w.y;
     p.z = w.z;
   }
-  const float G = (float)(1 << g);
-  const int last = (1 << g) - 1;
+  if (S.nb[0]) {
+    const int nb = S.nb[pass];
+    const float v = pass == 0 ? p.x - F.key_lo[0] : pass == 1 ? p.y - F.key_lo[1] : p.z - F.key_lo[2];
+    int group = 0;
+    if (pass > 0) group = rank / S.slab;
+    if (pass > 1) group = group * S.n_col + (rank - group * S.slab) / S.col;
+    return group * nb + min(max((int)(v * F.key_inv * (float)nb), 0), nb - 1);
+  }
+  const float G = (float)(1 << S.g);
+  const int last = (1 << S.g) - 1;
   const int cx = (int)((p.x - F.key_lo[0]) * F.key_inv * G), cy = (int)((p.y - F.key_lo[1]) * F.key_inv * G),
             cz = (int)((p.z - F.key_lo[2]) * F.key_inv * G);
-  return hilbert_key((uint32_t)min(max(cx, 0), last), (uint32_t)min(max(cy, 0), last),
-                     (uint32_t)min(max(cz, 0), last), g);
+  return (int)hilbert_key((uint32_t)min(max(cx, 0), last), (uint32_t)min(max(cy, 0), last),
+                          (uint32_t)min(max(cz, 0), last), S.g);
 }
 
-__global__ void sort_count_kernel(const SortSeg* segs, const float4* __restrict__ X, int32_t* keys,
-                                  uint32_t* counts) {
+// One pass: each particle's cell and its place in the cell (keys), the cells' counts.
+__global__ void sort_count_kernel(const SortSeg* segs, int pass, const float4* __restrict__ X, int2* keys,
+                                  uint32_t* counts, const uint32_t* __restrict__ cursors) {
   const SortSeg S = segs[blockIdx.y];
+  if (pass < 2 && S.nb[0] == 0) return;
   const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
   const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
   for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    uint32_t k = cell_key(*S.fd, X[S.x0 + i], S.g);
-    keys[S.x0 + i] = (int32_t)k;
-    atomicAdd(counts + S.key0 + k, 1u);
+    int rank = 0;
+    if (pass > 0 && S.nb[0]) {
+      const int2 k = keys[S.x0 + i];
+      rank = (int)cursors[S.key0[pass - 1] + k.x] + k.y;
+    }
+    const int cell = sort_cell(*S.fd, S, X[S.x0 + i], pass, rank);
+    keys[S.x0 + i] = make_int2(cell, (int)atomicAdd(counts + S.key0[pass] + cell, 1u));
   }
 }
 
@@ -331,12 +347,13 @@ __global__ void sort_count_kernel(const SortSeg* segs, const float4* __restrict_
 // on the blocks before it (a single block per segment took 0.42 ms at 2^18
 // counters, one tenth of what the whole frame's other preparation took).
 constexpr int kScanTile = 4096;
-__global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, const uint32_t* __restrict__ counts,
+__global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, int pass,
+                                                         const uint32_t* __restrict__ counts,
                                                          uint32_t* __restrict__ cursors) {
   const SortSeg S = segs[blockIdx.y];
-  const int m = 1 << (3 * S.g), t0 = blockIdx.x * kScanTile;
+  const int m = (int)sort_keys(S, pass), t0 = blockIdx.x * kScanTile;
   if (t0 >= m) return;
-  const uint32_t* c = counts + S.key0;
+  const uint32_t* c = counts + S.key0[pass];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ uint32_t s_sum[32];
   // this thread's four counters (segments below four counters have a whole tile to themselves)
@@ -372,20 +389,21 @@ __global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, co
   uint32_t run = base + w + incl - local;
   for (int q = 0; q < 4; ++q) {
     const int k = t0 + 4 * tid + q;
-    if (k < m) cursors[S.key0 + k] = run;
+    if (k < m) cursors[S.key0[pass] + k] = run;
     run += v[q];
   }
 }
 
 __global__ void sort_scatter_kernel(const SortSeg* segs, const float4* __restrict__ src,
-                                    const double4* __restrict__ src64, const int32_t* __restrict__ keys,
-                                    uint32_t* cursors, float4* dst, double4* dst64) {
+                                    const double4* __restrict__ src64, const int2* __restrict__ keys,
+                                    const uint32_t* __restrict__ cursors, float4* dst, double4* dst64) {
   const SortSeg S = segs[blockIdx.y];
   const FrameDev& F = *S.fd;
   const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
   const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
   for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    const int64_t pos = S.x0 + atomicAdd(cursors + S.key0 + (uint32_t)keys[S.x0 + i], 1u);
+    const int2 k = keys[S.x0 + i];
+    const int64_t pos = S.x0 + cursors[S.key0[2] + k.x] + k.y;
     const float4 p = src[S.x0 + i];
     dst[pos] = p;
     double4 q;
@@ -761,17 +779,19 @@ __global__ void frame_setup_kernel(FrameDev* frames, int order, int windows) {
 // shared memory once.  Whole call, before -> now: N = 2,000 without a box 91 -> 64 us,
 // N = 8,000 triclinic 159 -> 127 us, N = 32,000 orthorhombic 429 -> 411 us; larger
 // frames have work for more SMs than a cluster's and keep the separate kernels.
-constexpr int kPrepBlock = 1024, kPrepCluster = 8;
 static_assert((int64_t)kPrepBlock * 8 * kPrepCluster == kPrepMaxN, "particles per cluster");
-template <int PER>  // particles per thread, at most; twice as many counters
+// PER: particles per thread, at most, and half the counters of a pass; STRIPS: some
+// species of some frame is ordered in strips (without, one pass straight through:
+// three passes' code costs the smallest frames 5 us).
+template <int PER, bool STRIPS>
 __global__ void __launch_bounds__(kPrepBlock, 1)
     prep_kernel(const StageJob* __restrict__ jobs, const SortSeg* __restrict__ sorts, uint32_t* counts) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int kPrepPer = PER, kPrepScan = 2 * PER;
-  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int C = (int)cluster.num_blocks(), block = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int slot = rank * kPrepBlock + tid, slots = C * kPrepBlock;
+  const int slot = block * kPrepBlock + tid, slots = C * kPrepBlock;
   __shared__ StageJob J;
   __shared__ __align__(16) FrameDev F;
   __shared__ float s_red[32][12];
@@ -790,9 +810,12 @@ __global__ void __launch_bounds__(kPrepBlock, 1)
   if (tid < fwords) reinterpret_cast<uint32_t*>(&F)[tid] = reinterpret_cast<const uint32_t*>(dev)[tid];
   __syncthreads();
   const SortSeg* const S = sorts + J.sort0;
-  const int64_t key0 = S[0].key0;
-  const int keys = (int)(S[J.n_sort - 1].key0 - key0) + max(1 << (3 * S[J.n_sort - 1].g), 4);
-  for (int k = slot; k < keys; k += slots) counts[key0 + k] = 0u;
+  const SortSeg& last = S[J.n_sort - 1];
+  const int first_pass = STRIPS && J.strips ? 0 : 2;
+  {
+    const int64_t k0 = S[0].key0[first_pass], k1 = last.key0[2] + sort_keys(last, 2);
+    for (int64_t k = k0 + slot; k < k1; k += slots) counts[k] = 0u;
+  }
   for (int64_t k = slot; k < J.clear; k += slots) F.out[k] = 0ull;
 
   // ---- coordinates and their ranges
@@ -865,70 +888,92 @@ __global__ void __launch_bounds__(kPrepBlock, 1)
     list_setup(F, R, Xm);
   }
   __syncthreads();
-  if (rank == 0 && tid < fwords) reinterpret_cast<uint32_t*>(dev)[tid] = reinterpret_cast<const uint32_t*>(&F)[tid];
+  if (block == 0 && tid < fwords) reinterpret_cast<uint32_t*>(dev)[tid] = reinterpret_cast<const uint32_t*>(&F)[tid];
 
-  // ---- cells, and each particle's place in its cell
-  uint32_t cell[kPrepPer], place[kPrepPer];
+  // ---- the passes of the spatial order
+  int rank[kPrepPer], spec[kPrepPer];
 #pragma unroll
   for (int q = 0; q < kPrepPer; ++q) {
-    const int i = slot + q * slots;
-    cell[q] = place[q] = 0u;
-    if (i >= n) continue;
     int a = 0, hi = J.n_sort - 1;
     while (a < hi) {
       const int mid = (a + hi + 1) >> 1;
-      if (S[mid].x0 - S[mid].f0 <= i) a = mid; else hi = mid - 1;
+      if (S[mid].x0 - S[mid].f0 <= slot + q * slots) a = mid; else hi = mid - 1;
     }
-    cell[q] = (uint32_t)(S[a].key0 - key0) + cell_key(F, make_float4(p[q].x, p[q].y, p[q].z, 0.0f), S[a].g);
-    place[q] = atomicAdd(counts + key0 + cell[q], 1u);
+    spec[q] = a;
+    rank[q] = 0;
   }
-  cluster.sync();
-
-  // ---- prefix sum over the frame's cells, species after species: within the block,
-  // then of the blocks' totals
-  const int each = (keys + slots - 1) / slots, k0 = slot * each;
-  uint32_t c[kPrepScan], sum = 0u;
+#pragma unroll 1
+  for (int pass = STRIPS ? first_pass : 2; pass < 3; ++pass) {
+    // cells, and each particle's place in its cell
+    const int64_t key0 = S[0].key0[pass];
+    const int keys = (int)(last.key0[pass] + sort_keys(last, pass) - key0);
+    int cell[kPrepPer], place[kPrepPer];
 #pragma unroll
-  for (int q = 0; q < kPrepScan; ++q) {
-    c[q] = (q < each && k0 + q < keys) ? __ldcg(counts + key0 + k0 + q) : 0u;
-    sum += c[q];
-  }
-  uint32_t incl = sum;
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t x = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += x;
-  }
-  if (lane == 31) s_sum[warp] = incl;
-  __syncthreads();
-  uint32_t before = s_sum[lane];
-  if (warp == 0) {
-    uint32_t t = before;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-    if (lane == 0) s_total = t;
-  }
-  if (lane >= warp) before = 0u;
-  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
-  uint32_t at = before + incl - sum;
+    for (int q = 0; q < kPrepPer; ++q) {
+      cell[q] = -1;
+      place[q] = 0;
+      const SortSeg& T = S[spec[q]];
+      if (slot + q * slots >= n || (pass < 2 && T.nb[0] == 0)) continue;
+      cell[q] = (int)(T.key0[pass] - key0) + sort_cell(F, T, make_float4(p[q].x, p[q].y, p[q].z, 0.0f), pass, rank[q]);
+      place[q] = (int)atomicAdd(counts + key0 + cell[q], 1u);
+    }
+    cluster.sync();
+    // prefix sum over the cells, species after species: within the block, then of
+    // the blocks' totals
+    const int each = (keys + slots - 1) / slots, k0 = slot * each;
+    uint32_t c[kPrepScan], sum = 0u;
 #pragma unroll
-  for (int q = 0; q < kPrepScan; ++q) {
-    if (q < each && k0 + q < keys) __stcg(counts + key0 + k0 + q, at);
-    at += c[q];
+    for (int q = 0; q < kPrepScan; ++q) {
+      c[q] = (q < each && k0 + q < keys) ? __ldcg(counts + key0 + k0 + q) : 0u;
+      sum += c[q];
+    }
+    uint32_t incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += x;
+    }
+    if (lane == 31) s_sum[warp] = incl;
+    __syncthreads();
+    uint32_t before = s_sum[lane];
+    if (warp == 0) {
+      uint32_t t = before;
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+      if (lane == 0) s_total = t;
+    }
+    if (lane >= warp) before = 0u;
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
+    uint32_t at = before + incl - sum;
+#pragma unroll
+    for (int q = 0; q < kPrepScan; ++q) {
+      if (q < each && k0 + q < keys) __stcg(counts + key0 + k0 + q, at);
+      at += c[q];
+    }
+    cluster.sync();
+    if (tid < C) {
+      uint32_t b = 0u;
+      for (int r = 0; r < tid; ++r) b += *cluster.map_shared_rank(&s_total, r);
+      s_base[tid] = b;
+    }
+    __syncthreads();
+    // ranks within the species (without strips, within the frame)
+    const int per_block = each * kPrepBlock;
+#pragma unroll
+    for (int q = 0; q < kPrepPer; ++q) {
+      if (cell[q] < 0) continue;
+      rank[q] = (int)(s_base[cell[q] / per_block] + __ldcg(counts + key0 + cell[q])) + place[q];
+      if (STRIPS) {
+        const int t0 = (int)(S[spec[q]].key0[pass] - key0);
+        rank[q] -= (int)(s_base[t0 / per_block] + __ldcg(counts + key0 + t0));
+      }
+    }
   }
-  cluster.sync();
-  if (tid < C) {
-    uint32_t b = 0u;
-    for (int r = 0; r < tid; ++r) b += *cluster.map_shared_rank(&s_total, r);
-    s_base[tid] = b;
-  }
-  __syncthreads();
 
   // ---- the ordered copies
-  const int per_block = each * kPrepBlock;
 #pragma unroll
   for (int q = 0; q < kPrepPer; ++q) {
     const int i = slot + q * slots;
     if (i >= n) continue;
-    const int pos = (int)(s_base[cell[q] / per_block] + __ldcg(counts + key0 + cell[q]) + place[q]);
+    const int pos = (STRIPS ? (int)(S[spec[q]].x0 - S[spec[q]].f0) : 0) + rank[q];
     const float4 a = make_float4(p[q].x, p[q].y, p[q].z, 0.0f);
     J.dst[pos] = a;
     double4 d;
@@ -941,8 +986,8 @@ __global__ void __launch_bounds__(kPrepBlock, 1)
   cluster.sync();
 
   // ---- bounds of the runs
-  const int runs = S[J.n_sort - 1].run0 + (S[J.n_sort - 1].n + kRun - 1) / kRun;
-  for (int r = rank * 32 + warp; r < runs; r += C * 32) {
+  const int runs = last.run0 + (last.n + kRun - 1) / kRun;
+  for (int r = block * 32 + warp; r < runs; r += C * 32) {
     int a = 0, hi = J.n_sort - 1;
     while (a < hi) {
       const int mid = (a + hi + 1) >> 1;
@@ -2432,29 +2477,30 @@ cudaError_t launch_stage(const StageJob* jobs, int n_jobs, int64_t n_chunks, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, int64_t max_n, const float4* src, float4* dst,
-                                const double4* src64, double4* dst64, int32_t* keys, uint32_t* counts, int64_t n_keys,
+cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, const SortPlan& plan, const float4* src, float4* dst,
+                                const double4* src64, double4* dst64, int2* keys, uint32_t* counts,
                                 cudaStream_t stream) {
   clear_stale_error();
-  if (n_segs <= 0 || max_n <= 0) return cudaSuccess;
-  dim3 grid((unsigned)((max_n + kSortChunk - 1) / kSortChunk), (unsigned)n_segs);
-  sort_count_kernel<<<grid, 256, 0, stream>>>(segs, src, keys, counts);
-  dim3 sgrid((unsigned)((((int64_t)1 << (3 * sort_grid_bits(max_n))) + kScanTile - 1) / kScanTile), (unsigned)n_segs);
-  sort_scan_kernel<<<sgrid, 1024, 0, stream>>>(segs, counts, counts + n_keys);
-  sort_scatter_kernel<<<grid, 256, 0, stream>>>(segs, src, src64, keys, counts + n_keys, dst, dst64);
-  dim3 bgrid((unsigned)((max_n + 8 * kRun - 1) / (8 * kRun)), (unsigned)n_segs);
+  if (n_segs <= 0 || plan.max_n <= 0) return cudaSuccess;
+  uint32_t* const cursors = counts + plan.keys;
+  const dim3 grid((unsigned)((plan.max_n + kSortChunk - 1) / kSortChunk), (unsigned)n_segs);
+  for (int pass = 0; pass < 3; ++pass) {
+    if (plan.max_keys[pass] == 0) continue;
+    sort_count_kernel<<<grid, 256, 0, stream>>>(segs, pass, src, keys, counts, cursors);
+    const dim3 sgrid((unsigned)((plan.max_keys[pass] + kScanTile - 1) / kScanTile), (unsigned)n_segs);
+    sort_scan_kernel<<<sgrid, 1024, 0, stream>>>(segs, pass, counts, cursors);
+  }
+  sort_scatter_kernel<<<grid, 256, 0, stream>>>(segs, src, src64, keys, cursors, dst, dst64);
+  const dim3 bgrid((unsigned)((plan.max_n + 8 * kRun - 1) / (8 * kRun)), (unsigned)n_segs);
   run_bounds_kernel<<<bgrid, 256, 0, stream>>>(segs);
   return cudaGetLastError();
 }
 
-cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, const SortSeg* sorts, uint32_t* counts,
-                        cudaStream_t stream) {
+cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, bool strips, const SortSeg* sorts,
+                        uint32_t* counts, cudaStream_t stream) {
   clear_stale_error();
   if (n_jobs <= 0) return cudaSuccess;
-  // one particle per thread up to the largest portable cluster (two or four per
-  // thread: N = 4,000 without a box 72 and 80 us instead of 65)
-  unsigned blocks = 1;
-  while (blocks < (unsigned)kPrepCluster && (int64_t)blocks * kPrepBlock < max_n) blocks *= 2;
+  const unsigned blocks = (unsigned)prep_blocks(max_n);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks * (unsigned)n_jobs);
   cfg.blockDim = dim3(kPrepBlock);
@@ -2465,8 +2511,9 @@ cudaError_t launch_prep(const StageJob* jobs, int n_jobs, int64_t max_n, const S
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return max_n * 2 <= kPrepMaxN ? cudaLaunchKernelEx(&cfg, prep_kernel<4>, jobs, sorts, counts)
-                                : cudaLaunchKernelEx(&cfg, prep_kernel<8>, jobs, sorts, counts);
+  if (max_n * 2 > kPrepMaxN) return cudaLaunchKernelEx(&cfg, prep_kernel<8, true>, jobs, sorts, counts);
+  return strips ? cudaLaunchKernelEx(&cfg, prep_kernel<4, true>, jobs, sorts, counts)
+                : cudaLaunchKernelEx(&cfg, prep_kernel<4, false>, jobs, sorts, counts);
 }
 
 cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, bool order, bool windows, cudaStream_t stream) {

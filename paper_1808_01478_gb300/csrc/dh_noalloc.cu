@@ -56,7 +56,7 @@ struct NaListPlan {
   std::vector<SortSeg> sorts;
   std::vector<ListSegment> segs;
   int64_t items = 0;
-  int split = 1;
+  int split = 1, strips = 0;
   size_t sort_at = 0, seg_at = 0, ctr_at = 0, T_at = 0, bnd_at = 0, P4_at = 0, P2_at = 0, X_at = 0, cells_at = 0;
 };
 
@@ -64,9 +64,10 @@ struct NaListPlan {
 bool plan_list(const dh_frame* f, int max_width, int num_sms, unsigned char* base, NaListPlan& p) {
   if (check_frame(f, p.pf, max_width, list_kernel_max_width()) != DH_OK || !p.pf.list) return false;
   FrameDev* fd = (FrameDev*)(base + kNaOffFrame);
-  int64_t keys = 0, most = 0;
-  p.sorts = plan_spatial_order(p.pf, fd, 0, 0, &keys, &most);
-  if (!prep_fits(f->n, keys)) return false;
+  SortPlan sort;
+  p.sorts = plan_spatial_order(p.pf, true, fd, 0, 0, &sort);
+  p.strips = sort.max_keys[0] > 0;
+  if (!prep_fits(f->n, sort.keys)) return false;
   p.split = list_split_for((double)p.pf.pairs / ((double)kRun * kRun) * p.pf.sweeps, num_sms);
   p.items = add_list_segments(p.pf, fd, 0, p.segs, p.split);
   size_t at = kNaOffSegs;
@@ -83,7 +84,7 @@ bool plan_list(const dh_frame* f, int max_width, int num_sms, unsigned char* bas
   p.P4_at = part(sizeof(float4) * (size_t)f->n);
   p.P2_at = part(sizeof(float2) * (size_t)f->n);
   p.X_at = part(sizeof(float4) * (size_t)f->n);
-  p.cells_at = part(sizeof(uint32_t) * (size_t)keys);
+  p.cells_at = part(sizeof(uint32_t) * (size_t)sort.keys);
   return at <= kNaBytes;
 }
 
@@ -184,6 +185,7 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
     hF.P4 = (float4*)(base + lp.P4_at);
     hF.P2 = (float2*)(base + lp.P2_at);
     hJ.n_sort = (int32_t)lp.sorts.size();
+    hJ.strips = lp.strips;
     hJ.clear = clear ? (int64_t)out_words : 0;
     std::memcpy(up.data() + lp.sort_at, lp.sorts.data(), sizeof(SortSeg) * lp.sorts.size());
     if (!lp.segs.empty()) std::memcpy(up.data() + lp.seg_at, lp.segs.data(), sizeof(ListSegment) * lp.segs.size());
@@ -193,7 +195,7 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   DH_CUDA_TRY(cudaMemcpyAsync(base, up.data(), up.size(), cudaMemcpyHostToDevice, st));
   DH_CUDA_TRY(launch_thresholds(frame->r_max, frame->nbins, T, &ctl->status, st));
   if (list) {
-    DH_CUDA_TRY(launch_prep(job, 1, frame->n, (const SortSeg*)(base + lp.sort_at), (uint32_t*)(base + lp.cells_at), st));
+    DH_CUDA_TRY(launch_prep(job, 1, frame->n, lp.strips != 0, (const SortSeg*)(base + lp.sort_at), (uint32_t*)(base + lp.cells_at), st));
     if (lp.items > 0) {
       ListLaunch L;
       std::memset(&L, 0, sizeof L);

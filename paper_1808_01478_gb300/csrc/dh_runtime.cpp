@@ -324,11 +324,35 @@ void fill_frame_dev(const PlannedFrame& pf, FrameDev& F, const float4* X, uint64
   }
 }
 
+namespace {
+// Cells of the Hilbert order: about two particles each.
 int sort_grid_bits(int64_t n) {
   if (n <= kRun) return 0;  // one run: the order does not matter
   const int g = (int)std::lround(std::log2(std::cbrt(0.5 * (double)n)));
   return std::min(7, std::max(1, g));
 }
+
+// Slabs, columns and cells of the strip order of a species of n particles in a box
+// with sides L (any scale): runs of about equal sides, with 32 to 64 cells along each
+// (the blur of a run's ends), and at most 1.5 counters per particle.
+void plan_strips(SortSeg& g, int64_t n, const double* L) {
+  const double runs = (double)((n + kRun - 1) / kRun), side = std::cbrt(L[0] * L[1] * L[2] / runs);
+  const double n_slab = std::min(runs, std::max(1.0, std::round(L[0] / side)));
+  const double slab = std::ceil(runs / n_slab);
+  const double n_col = std::min(slab, std::max(1.0, std::round(std::sqrt(slab * L[1] / L[2]))));
+  const double col = std::ceil(slab / n_col);
+  g.slab = (int32_t)(kRun * slab);
+  g.col = (int32_t)(kRun * col);
+  g.n_slab = (int32_t)std::ceil(runs / slab);
+  g.n_col = (int32_t)std::ceil(slab / col);
+  const double most = 1.5 * (double)n / ((double)g.n_slab * g.n_col);
+  const double want = 32.0 * std::max(L[0], std::max(L[1], L[2])) / side;
+  g.nb[2] = 32;
+  while (g.nb[2] < 4096 && g.nb[2] < want && 2.0 * g.nb[2] <= most) g.nb[2] *= 2;
+  g.nb[1] = std::min(4 * g.nb[2], 4096);  // few slabs, few counters: more cells, not more increments of each
+  g.nb[0] = std::min(16 * g.nb[2], 8192);
+}
+}  // namespace
 
 int64_t frame_runs(const dh_frame* f) {
   int64_t runs = 0;
@@ -337,13 +361,15 @@ int64_t frame_runs(const dh_frame* f) {
   return runs;
 }
 
-std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, const FrameDev* fd, int64_t x0, int64_t key0,
-                                        int64_t* keys, int64_t* max_n) {
+std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, bool list, const FrameDev* fd, int64_t x0, int64_t key0,
+                                        SortPlan* plan) {
   std::vector<SortSeg> out;
-  *keys = 0;
-  *max_n = 0;
+  *plan = SortPlan();
   if (pf.variant == V_TRIC_SEARCH && !pf.list) return out;
   const int64_t* o = pf.src->species_offsets;
+  const double* B = pf.src->box;
+  const double cube[3] = {1.0, 1.0, 1.0}, box[3] = {B[0], B[4], B[8]};
+  const bool strips = list && pf.src->n >= (pf.variant == V_NONE ? kStripMinNoBoxN : kStripMinN);
   int64_t runs = 0;
   for (int a = 0; a < pf.src->n_species; ++a) {
     const int64_t na = o[a + 1] - o[a];
@@ -353,15 +379,24 @@ std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, const FrameDev* 
     g.fd = fd;
     g.x0 = x0 + o[a];
     g.n = (int32_t)na;
-    g.g = sort_grid_bits(na);
-    g.key0 = key0 + *keys;
     g.f0 = x0;
     g.run0 = (int32_t)runs;
     runs += (na + kRun - 1) / kRun;
-    *keys += std::max<int64_t>((int64_t)1 << (3 * g.g), 4);
-    *max_n = std::max<int64_t>(*max_n, na);
+    if (strips && na >= kStripMinSpecies)
+      plan_strips(g, na, pf.variant == V_NONE ? cube : box);
+    else
+      g.g = sort_grid_bits(na);
+    plan->max_n = std::max<int64_t>(plan->max_n, na);
     out.push_back(g);
   }
+  // a frame's counters: pass by pass, species after species
+  for (int p = 0; p < 3; ++p)
+    for (SortSeg& g : out) {
+      const int64_t m = sort_keys(g, p);
+      g.key0[p] = key0 + plan->keys;
+      plan->keys += m;
+      plan->max_keys[p] = std::max(plan->max_keys[p], m);
+    }
   return out;
 }
 
@@ -559,8 +594,7 @@ struct CallPlan {
   } list[2];
   bool prep = false;             // frames prepared by one launch (launch_prep)
   int n_sort = 0;                // spatial-order segments (after the segments in the metadata)
-  int64_t sort_max = 0;          // largest of them
-  int64_t sort_keys = 0;         // counters over all of them
+  SortPlan sort;                 // what they need
   int64_t sort_particles = 0;    // particles of the frames (index space of keys and the scratch copy)
 };
 
@@ -660,20 +694,19 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   };
   // spatial order of the species
   std::vector<SortSeg> sorts;
-  std::vector<int> sort0((size_t)k + 1, 0);
+  std::vector<int> sort0((size_t)k + 1, 0), strips((size_t)k, 0);
   auto plan_sorts = [&](FrameDev* dF) {
     sorts.clear();
-    P.sort_keys = 0;
-    P.sort_max = 0;
+    P.sort = SortPlan();
     P.prep = with_pairs;
     for (int f = 0; f < k; ++f) {
-      int64_t keys = 0, most = 0;
-      std::vector<SortSeg> fs = plan_spatial_order(pfs[f], dF + f, xoff[f], P.sort_keys, &keys, &most);
+      SortPlan fp;
+      std::vector<SortSeg> fs = plan_spatial_order(pfs[f], on_list(f), dF + f, xoff[f], P.sort.keys, &fp);
       sorts.insert(sorts.end(), fs.begin(), fs.end());
-      P.sort_keys += keys;
-      P.sort_max = std::max(P.sort_max, most);
+      P.sort.add(fp);
+      strips[f] = fp.max_keys[0] > 0;
       sort0[f + 1] = (int)sorts.size();
-      P.prep = P.prep && on_list(f) && xoff[f + 1] - xoff[f] <= kPrepBestN && prep_fits(xoff[f + 1] - xoff[f], keys);
+      P.prep = P.prep && on_list(f) && xoff[f + 1] - xoff[f] <= kPrepBestN && prep_fits(xoff[f + 1] - xoff[f], fp.keys);
     }
     P.n_sort = (int)sorts.size();
     P.sort_particles = xoff[k];
@@ -694,12 +727,12 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     plan_sorts((FrameDev*)c->meta.p);
   }
   if (P.prep) {
-    DH_CUDA_TRY(c->sortC.ensure(sizeof(uint32_t) * (size_t)P.sort_keys));
+    DH_CUDA_TRY(c->sortC.ensure(sizeof(uint32_t) * (size_t)P.sort.keys));
   } else if (P.n_sort > 0) {
     DH_CUDA_TRY(c->sortX.ensure(sizeof(float4) * (size_t)P.sort_particles));
     if (P.any_f64) DH_CUDA_TRY(c->sortX64.ensure(sizeof(double4) * (size_t)P.sort_particles));
-    DH_CUDA_TRY(c->sortK.ensure(sizeof(int32_t) * (size_t)P.sort_particles));
-    DH_CUDA_TRY(c->sortC.ensure(2 * sizeof(uint32_t) * (size_t)P.sort_keys));
+    DH_CUDA_TRY(c->sortK.ensure(sizeof(int2) * (size_t)P.sort_particles));
+    DH_CUDA_TRY(c->sortC.ensure(2 * sizeof(uint32_t) * (size_t)P.sort.keys));
   }
   FrameDev* dF = (FrameDev*)c->meta.p;
   FrameDev* hF = (FrameDev*)c->hmeta.p;
@@ -738,6 +771,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     J.n = fr->n;
     J.sort0 = sort0[f];
     J.n_sort = sort0[f + 1] - sort0[f];
+    J.strips = strips[f];
     J.clear = host_coords || !(fr->flags & DH_ACCUMULATE) ? (int64_t)pfs[f].n_hist * fr->nbins : 0;
     J.chunk0 = (int32_t)P.n_chunks;
     P.n_chunks += (fr->n + kStageChunk - 1) / kStageChunk;
@@ -794,7 +828,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   if (P.prep) {
     int64_t max_n = 0;
     for (auto& pf : pfs) max_n = std::max(max_n, pf.src->n);
-    DH_CUDA_TRY(launch_prep(dJ, k, max_n, dSort, (uint32_t*)c->sortC.p, st));
+    DH_CUDA_TRY(launch_prep(dJ, k, max_n, P.sort.max_keys[0] > 0, dSort, (uint32_t*)c->sortC.p, st));
     ++launched;
   } else {
     if (P.n_jobs > 0) {
@@ -805,12 +839,13 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
     ++launched;
   }
   if (!P.prep && P.n_sort > 0) {
-    DH_CUDA_TRY(cudaMemsetAsync(c->sortC.p, 0, sizeof(uint32_t) * (size_t)P.sort_keys, st));
-    DH_CUDA_TRY(launch_spatial_sort(dSort, P.n_sort, P.sort_max, (const float4*)c->sortX.p, (float4*)c->X.p,
+    DH_CUDA_TRY(cudaMemsetAsync(c->sortC.p, 0, sizeof(uint32_t) * (size_t)P.sort.keys, st));
+    DH_CUDA_TRY(launch_spatial_sort(dSort, P.n_sort, P.sort, (const float4*)c->sortX.p, (float4*)c->X.p,
                                     P.any_f64 ? (const double4*)c->sortX64.p : nullptr,
-                                    P.any_f64 ? (double4*)c->X64.p : nullptr, (int32_t*)c->sortK.p,
-                                    (uint32_t*)c->sortC.p, P.sort_keys, st));
-    launched += 4;
+                                    P.any_f64 ? (double4*)c->X64.p : nullptr, (int2*)c->sortK.p,
+                                    (uint32_t*)c->sortC.p, st));
+    launched += 2;
+    for (int64_t m : P.sort.max_keys) launched += m > 0 ? 2 : 0;
   }
   // A2-A8: per variant, one persistent launch over its frames, species pairs and bin sweeps
   int grid = 0, top = -1;

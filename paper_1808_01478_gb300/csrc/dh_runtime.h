@@ -136,13 +136,22 @@ TuneKey make_tune_key(int variant, int width, double mean_pairs_per_frame, int f
 // Bytes of a frame's coordinate array (float32 or binary64, 3 or 4 per particle).
 size_t coord_bytes(const dh_frame* f);
 
-// Species are put in spatial (Hilbert) order before the pair kernel, over the
-// frame's bounding box or its home cell, with about two particles per cell.
-// plan_spatial_order lists the species of one frame (its particles from x0 in
-// the packed coordinates, its counters from key0) and returns the counters they
-// need and the largest species.  Frames of the 27-image search keep their order.
-std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, const FrameDev* fd, int64_t x0, int64_t key0,
-                                        int64_t* keys, int64_t* max_n);
+// Species are put in spatial order before the pair kernel, over the frame's
+// bounding box or its home cell (SortSeg).  plan_spatial_order lists the species of
+// one frame (its particles from x0 in the packed coordinates, its counters from
+// key0); frames of the search that are not for the list kernel keep their order.
+// list: the list kernel runs the frame, and its larger species are ordered in strips.
+std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, bool list, const FrameDev* fd, int64_t x0, int64_t key0,
+                                        SortPlan* plan);
+// Strips instead of the Hilbert curve: the runs' boxes are smaller, so that fewer pairs
+// beyond r_max are evaluated and fewer pairs re-decided (whole call, orthorhombic
+// N = 32,000 422 -> 406 us, N = 100,000 2.43 -> 2.27 ms, pair kernel at N = 1,000,000
+// 170.2 -> 162.4 ms; N = 200,000 with 100,000 bins 15.8 -> 14.2 ms), for two passes more
+// (10 us in launch_prep, 20 as kernels): at N = 16,000 188 against 182 us triclinic and
+// 190 against 191 orthorhombic, at N = 12,000 144 against 153.  Without a box nothing is
+// gained where r_max holds the whole frame: N = 60,000 1.01 against 1.03 ms, from
+// N = 200,000 on even.  Species of a few runs have nothing to gain either way.
+constexpr int64_t kStripMinN = 16000, kStripMinNoBoxN = 200000, kStripMinSpecies = 2048;
 
 // Threads per block for a launch without a measured shape: from 16,384 bins on,
 // a 256-thread block's histogram leaves room for at most two blocks per SM, and

@@ -140,8 +140,7 @@ struct Request {
   double pairs_per_item = 1.0;
   // spatial order of the species: plan, device scratch, pinned upload
   std::vector<SortSeg> sorts;
-  int64_t sort_keys = 0;
-  int64_t sort_max = 0;
+  SortPlan sort;
   int64_t runs = 0;
   float4* bnd = nullptr;
   float4* P4 = nullptr;
@@ -149,7 +148,7 @@ struct Request {
   SortSeg* sort_dev = nullptr;
   SortSeg* sort_pin = nullptr;
   float4* sort_X = nullptr;
-  int32_t* sort_K = nullptr;
+  int2* sort_K = nullptr;
   uint32_t* sort_C = nullptr;
   int64_t n_items = 0, next = 0;
   bool prepped = false, finalize_enqueued = false, cancel = false;
@@ -316,11 +315,11 @@ dh_status Server::submit(const dh_frame* f, uint64_t* ticket) {
   size_t n = (size_t)f->n;
   r->dev_bytes = align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob)) + align_up(16 * std::max<size_t>(n, 1));
   r->pin_bytes = align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob));
-  r->sorts = plan_spatial_order(r->pf, nullptr, 0, 0, &r->sort_keys, &r->sort_max);
+  r->sorts = plan_spatial_order(r->pf, r->pf.list, nullptr, 0, 0, &r->sort);
   r->runs = frame_runs(&r->frame);
   if (!r->sorts.empty()) {
-    r->dev_bytes += align_up(sizeof(SortSeg) * r->sorts.size()) + align_up(16 * n) + align_up(4 * n) +
-                    align_up(8 * (size_t)r->sort_keys);
+    r->dev_bytes += align_up(sizeof(SortSeg) * r->sorts.size()) + align_up(16 * n) + align_up(8 * n) +
+                    align_up(8 * (size_t)r->sort.keys);
     if (r->pf.list) r->dev_bytes += align_up(2 * sizeof(float4) * (size_t)r->runs) + align_up(16 * n) + align_up(8 * n);
     r->pin_bytes += align_up(sizeof(SortSeg) * r->sorts.size());
   }
@@ -437,10 +436,10 @@ void Server::admit() {
     if (!r.sorts.empty()) {
       r.sort_X = (float4*)d;
       d += align_up(16 * (size_t)r.frame.n);
-      r.sort_K = (int32_t*)d;
-      d += align_up(4 * (size_t)r.frame.n);
+      r.sort_K = (int2*)d;
+      d += align_up(8 * (size_t)r.frame.n);
       r.sort_C = (uint32_t*)d;
-      d += align_up(8 * (size_t)r.sort_keys);
+      d += align_up(8 * (size_t)r.sort.keys);
       if (r.pf.list) {
         r.bnd = (float4*)d;
         d += align_up(2 * sizeof(float4) * (size_t)r.runs);
@@ -490,9 +489,10 @@ dh_status Server::prep(Request& r) {
   r.job_pin->src = r.dev_ptrs ? r.frame.coords : r.raw;
   // a small frame of the list kernel is prepared by one launch, which also clears the output
   const bool clear = !r.dev_ptrs || !(r.frame.flags & DH_ACCUMULATE);
-  const bool fused = r.pf.list && r.frame.n <= kPrepBestN && prep_fits(r.frame.n, r.sort_keys);
+  const bool fused = r.pf.list && r.frame.n <= kPrepBestN && prep_fits(r.frame.n, r.sort.keys);
   r.job_pin->dst = r.sorts.empty() || fused ? r.X : r.sort_X;
   r.job_pin->n_sort = (int32_t)r.sorts.size();
+  r.job_pin->strips = r.sort.max_keys[0] > 0;
   r.job_pin->clear = clear ? (int64_t)r.res_count : 0;
   r.job_pin->fd = r.fd;
   r.job_pin->n = r.frame.n;
@@ -509,16 +509,16 @@ dh_status Server::prep(Request& r) {
     DH_CUDA_TRY(cudaMemcpyAsync(r.raw, r.raw_pin, 4 * (size_t)r.stride * (size_t)r.frame.n,
                                 cudaMemcpyHostToDevice, st));
   if (fused) {
-    DH_CUDA_TRY(launch_prep(r.job_dev, 1, r.frame.n, r.sort_dev, r.sort_C, st));
+    DH_CUDA_TRY(launch_prep(r.job_dev, 1, r.frame.n, r.sort.max_keys[0] > 0, r.sort_dev, r.sort_C, st));
   } else {
     if (clear) DH_CUDA_TRY(cudaMemsetAsync(r.hist, 0, 8 * r.res_count, st));
     int64_t chunks = (r.frame.n + kStageChunk - 1) / kStageChunk;
     if (chunks > 0) DH_CUDA_TRY(launch_stage(r.job_dev, 1, chunks, st));
     DH_CUDA_TRY(launch_frame_setup(r.fd, 1, true, false, st));
     if (!r.sorts.empty()) {
-      DH_CUDA_TRY(cudaMemsetAsync(r.sort_C, 0, 4 * (size_t)r.sort_keys, st));
-      DH_CUDA_TRY(launch_spatial_sort(r.sort_dev, (int)r.sorts.size(), r.sort_max, r.sort_X, r.X, nullptr, nullptr,
-                                      r.sort_K, r.sort_C, r.sort_keys, st));
+      DH_CUDA_TRY(cudaMemsetAsync(r.sort_C, 0, 4 * (size_t)r.sort.keys, st));
+      DH_CUDA_TRY(launch_spatial_sort(r.sort_dev, (int)r.sorts.size(), r.sort, r.sort_X, r.X, nullptr, nullptr,
+                                      r.sort_K, r.sort_C, st));
     }
   }
   // marks the end of the preparation: a request cancelled before its first wave

@@ -86,3 +86,35 @@ def test_allocation_free_frames_match_dh_histogram(torch_mod, box, n, nbins):
     assert torch_mod.equal(out, want)
     dh.dh_histogram_noalloc(dh.FrameArgs(x, offs, box_type, B, 5.0, nbins, out, True).frame)
     assert torch_mod.equal(out, 2 * want)
+
+
+@pytest.mark.parametrize("n,cuts,box,shape", [
+    (15999, [], "ortho", "uniform"),               # one particle short of the strips: the curve
+    (16000, [], "ortho", "uniform"),
+    (16000, [2047, 4095], "triclinic", "uniform"),  # one species in the curve's order, two in strips
+    (20001, [1, 1, 3000], "ortho", "flat"),        # a plane: every particle in one cell of an axis
+    (32768, [16384], "triclinic", "point"),        # half of them in one place
+    (33025, [129], "ortho", "long"),               # general path, sides 1 : 1 : 60
+    (33025, [], "triclinic", "cells"),             # ... brought home from several cells
+    (200000, [], "none", "uniform"),
+])
+def test_strip_order(torch_mod, oracle_mod, n, cuts, box, shape):
+    box_type, B = BOXES[box]
+    if shape == "long":
+        B = w.ortho_box(6.0, 6.0, 360.0)
+    rng = w.rng_for(7000 + n)
+    x = rng.random((n, 3))
+    if shape == "flat":
+        x[:, 1] = 0.25
+    if shape == "point":
+        x[: n // 2] = 0.5 + 1e-4 * x[: n // 2]
+    if shape == "cells":
+        x += rng.integers(-3, 4, size=(n, 3))
+    m = np.eye(3) * 12.0 if box_type == w.BOX_NONE else w.box_matrix(B)
+    x = (x @ m.T).astype(np.float32)
+    offs = np.array([0, *cuts, n], dtype=np.int64)
+    r_max, nbins = (2.9 if shape == "long" else 5.0), 600
+    want = oracle_mod.histogram(x, offs, box_type, B, r_max, nbins)
+    with dh.Context(0) as ctx:
+        got = ctx.histogram(torch_mod.from_numpy(x).cuda(), offs, box_type, B, r_max, nbins)
+    assert np.array_equal(got.cpu().numpy().view(np.uint64), want)
