@@ -313,26 +313,38 @@ dh_status Server::submit(const dh_frame* f, uint64_t* ticket) {
   r->stride = (f->flags & DH_COORDS_F4) ? 4 : 3;
   r->res_count = (size_t)r->pf.n_hist * (size_t)f->nbins;
   size_t n = (size_t)f->n;
-  r->dev_bytes = align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob)) + align_up(16 * std::max<size_t>(n, 1));
+  size_t least = align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob)) + align_up(16 * std::max<size_t>(n, 1));
   r->pin_bytes = align_up(sizeof(FrameDev)) + align_up(sizeof(StageJob));
+  if (!r->dev_ptrs) {
+    least += align_up(4 * (size_t)r->stride * n) + align_up(8 * r->res_count);
+    r->pin_bytes += align_up(4 * (size_t)r->stride * n) + align_up(8 * r->res_count);
+  }
+  r->dev_bytes = least;
+  // what the pool has to hold for a request to be taken: these, and an order of the species
+  if (r->pf.variant != V_TRIC_SEARCH) least += align_up(16 * n) + align_up(4 * n) + align_up(n / 4);
   r->sorts = plan_spatial_order(r->pf, r->pf.list, nullptr, 0, 0, &r->sort);
   r->runs = frame_runs(&r->frame);
   if (!r->sorts.empty()) {
-    r->dev_bytes += align_up(sizeof(SortSeg) * r->sorts.size()) + align_up(16 * n) + align_up(8 * n) +
-                    align_up(8 * (size_t)r->sort.keys);
-    if (r->pf.list) r->dev_bytes += align_up(2 * sizeof(float4) * (size_t)r->runs) + align_up(16 * n) + align_up(8 * n);
-    r->pin_bytes += align_up(sizeof(SortSeg) * r->sorts.size());
-  }
-  if (!r->dev_ptrs) {
-    r->dev_bytes += align_up(4 * (size_t)r->stride * n) + align_up(8 * r->res_count);
-    r->pin_bytes += align_up(4 * (size_t)r->stride * n) + align_up(8 * r->res_count);
+    size_t more = align_up(sizeof(SortSeg) * r->sorts.size()) + align_up(16 * n) + align_up(8 * n) +
+                  align_up(8 * (size_t)r->sort.keys);
+    if (r->pf.list) more += align_up(2 * sizeof(float4) * (size_t)r->runs) + align_up(16 * n) + align_up(8 * n);
+    if (least <= dev_arena_.capacity() && r->dev_bytes + more > dev_arena_.capacity()) {
+      // no room for the ordered copies (about 60 bytes a particle): the tiled kernel, in the caller's order
+      s = check_frame(&r->frame, r->pf, ctx_->max_width, 0);
+      if (s != DH_OK) return s;
+      r->sorts.clear();
+      r->sort = SortPlan();
+    } else {
+      r->dev_bytes += more;
+      r->pin_bytes += align_up(sizeof(SortSeg) * r->sorts.size());
+    }
   }
   std::lock_guard<std::mutex> g(mu_);
   if (stop_) return fail(DH_ERR_CANCELLED, "server is shutting down");
   if (!thread_error_.empty()) return fail(DH_ERR_CUDA, "%s", thread_error_.c_str());
-  if (r->dev_bytes > dev_arena_.capacity() || r->pin_bytes > pin_arena_.capacity())
+  if (std::max(least, r->dev_bytes) > dev_arena_.capacity() || r->pin_bytes > pin_arena_.capacity())
     return fail(DH_ERR_NOMEM, "request needs %zu device / %zu pinned bytes, pool holds %zu / %zu",
-                r->dev_bytes, r->pin_bytes, dev_arena_.capacity(), pin_arena_.capacity());
+                std::max(least, r->dev_bytes), r->pin_bytes, dev_arena_.capacity(), pin_arena_.capacity());
   r->ticket = next_ticket_++;
   r->t_submit = Clock::now();
   *ticket = r->ticket;

@@ -118,3 +118,21 @@ def test_strip_order(torch_mod, oracle_mod, n, cuts, box, shape):
     with dh.Context(0) as ctx:
         got = ctx.histogram(torch_mod.from_numpy(x).cuda(), offs, box_type, B, r_max, nbins)
     assert np.array_equal(got.cpu().numpy().view(np.uint64), want)
+
+
+@pytest.mark.parametrize("box", list(BOXES))
+def test_served_request_without_room_for_the_order(torch_mod, box):
+    # 36 bytes a particle are enough for a request to be taken, 60 for its ordered copies
+    box_type, B = BOXES[box]
+    n, nbins = 45_000, 600
+    x = torch_mod.from_numpy((w.rng_for(91).random((n, 3)) * 10.0).astype(np.float32)).cuda()
+    offs = np.array([0, n // 2, n], dtype=np.int64)
+    with dh.Context(0, pool_bytes=2 << 20, max_inflight=2) as c:
+        want = c.histogram(x, offs, box_type, B, 5.0, nbins)
+        fa = dh.FrameArgs(x, offs, box_type, B, 5.0, nbins)
+        assert c.wait(c.submit(fa)) == dh.DH_OK
+        assert torch_mod.equal(fa.out, want)
+        big = torch_mod.zeros((60_000, 3), device="cuda")
+        with pytest.raises(dh.DHError) as e:
+            c.submit(dh.FrameArgs(big, [0, 60_000], box_type, B, 5.0, nbins))
+        assert e.value.status == dh.DH_ERR_NOMEM
