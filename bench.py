@@ -51,25 +51,14 @@ METRIC = "Gpairs/s binned at N=1M (plain vs batched/served) + p50/p99 frame late
 UNIT = "Gpairs/s"
 BOXES = (w.BOX_NONE, w.BOX_ORTHO, w.BOX_TRICLINIC)
 
-# Per-pair arithmetic of the pair kernel on the float32 (FMA) pipe, by tile mode,
-# as lane operations of each packed kind (FADD2, FMUL2, FFMA2 count two lanes).
-# Every mode: d = xj - xi (3 add), r^2 (1 mul, 2 fma), q = S^2 r^2 (1 mul), the
-# nearest integer of the root and its residual (2 add, 1 fma), the near-edge
-# bound (1 fma).  Orthorhombic tiles with a uniform image shift the j's by the
-# image (3 packed adds per 2 j x 4 i: 0.75 lanes per pair; 0.5 with one axis
-# wrapped per pair).  A wrapped axis adds a nearest integer and an fma (1 add,
-# 2 fma); the per-pair triclinic wrap rounds along c, b, a (3 add, 9 fma).  The
+# Per-pair arithmetic of the pair kernel (the list kernel) on the float32 (FMA)
+# pipe, as lane operations of each packed kind (FADD2, FFMA2 count two lanes): the
+# squared distance in bins relative to the run's centre (3 fma, 1 add), the
+# nearest integer of its root and the residual (2 add, 1 fma), for every box.  The
 # square root is one MUFU operation per pair and the histogram update one
-# shared-memory atomic per pair (the clamp of out-of-range roots runs on the
-# integer ALU).
-BASE_OPS = {"fadd": 5.0, "fmul": 2.0, "ffma": 4.0}
-MODE_OPS = {
-    (w.BOX_NONE, "uni"): {}, (w.BOX_NONE, "pair"): {},
-    (w.BOX_ORTHO, "uni"): {"fadd": 0.75}, (w.BOX_ORTHO, "axis"): {"fadd": 1.5, "ffma": 2.0},
-    (w.BOX_ORTHO, "pair"): {"fadd": 3.0, "ffma": 6.0},
-    (w.BOX_TRICLINIC, "uni"): {}, (w.BOX_TRICLINIC, "axis"): {"fadd": 1.0, "ffma": 2.0},
-    (w.BOX_TRICLINIC, "pair"): {"fadd": 3.0, "ffma": 9.0},
-}
+# shared-memory atomic per pair (the clamp of out-of-range roots, the address and
+# the deferral test run on the integer ALU).
+PAIR_OPS = {"fadd": 3.0, "ffma": 4.0}
 SM_COUNT = 152
 PIPE_SET = ("ffma2", "fadd2", "fmul2", "ffma", "sqrt", "frnd", "f2i", "lop3", "iadd", "imad", "dfma", "match",
             "smem_atomic_clustered", "smem_atomic_same", "smem_atomic_sequential")
@@ -94,62 +83,25 @@ def measure_pipes(device: int, widths) -> dict:
     return out
 
 
-def fp32_lane_ops(box_type: int, f_uni: float, f_axis: float) -> dict:
-    """Float32 lane operations per pair of each kind, averaged over the tile modes
-    with the fractions of pairs the kernel evaluated in each."""
-    f_pair = max(0.0, 1.0 - f_uni - f_axis)
-    ops = dict(BASE_OPS)
-    for mode, frac in (("uni", f_uni), ("axis", f_axis), ("pair", f_pair)):
-        for k, v in MODE_OPS.get((box_type, mode), {}).items():
-            ops[k] += frac * v
-    return ops
-
-
-def bank_load(f_in: float, trials: int = 4000) -> float:
-    """Expected largest number of distinct words one bank receives in a warp's
-    shared-memory increment when a fraction f_in of its 32 lanes hits uniform
-    random bins and the others their own guard words (one bank each: the
-    clamp sends lane l's out-of-range pairs to the word hi + 1 + l)."""
-    rng = np.random.default_rng(12345)
-    inr = rng.random((trials, 32)) < f_in
-    banks = np.where(inr, rng.integers(0, 32, (trials, 32)), np.arange(32)[None, :])
-    loads = np.zeros((trials, 32))
-    np.add.at(loads, (np.repeat(np.arange(trials), 32), banks.ravel()), 1.0)
-    return float(loads.max(axis=1).mean())
-
-
-def atomic_rate(width: int, f_in: float, pipes: dict) -> float:
-    """Shared-memory increments per clock per SM for a histogram of `width`
-    bins when a fraction f_in of the pairs is inside r_max: the measured rate
-    on uniform random bins (every lane in range), scaled by the expected bank
-    load relative to that case, but never above the conflict-free rate."""
+def pair_bound(width: int, pipes: dict) -> dict:
+    """Roofline of the pair kernel in pairs inside r_max per clock per SM: the
+    minimum over pipes of measured rate / operations per pair (float32 FMA pipe,
+    MUFU square root, shared-memory atomic on random bins at the frame's width).
+    Pairs beyond r_max need not be evaluated, so none are counted."""
     key = f"smem_atomic_random@{width}"
-    if key not in pipes:
-        return float("nan")
-    r_rand, r_free = pipes[key]["per_clk_sm"], pipes["smem_atomic_sequential"]["per_clk_sm"]
-    return min(r_free, r_rand * bank_load(1.0) / bank_load(min(1.0, max(0.0, f_in))))
-
-
-def pair_bound(box_type: int, width: int, f_uni: float, f_axis: float, pipes: dict, f_in: float = 1.0) -> dict:
-    """Roofline of the pair kernel for one frame in pairs per clock per SM: the
-    minimum over pipes of measured rate / operations per pair (float32 FMA
-    pipe, MUFU square root, shared-memory atomic at the frame's width and
-    fraction f_in of pairs inside r_max)."""
-    ops = fp32_lane_ops(box_type, f_uni, f_axis)
-    fp32_clk = (ops["fadd"] / pipes["fadd2"]["per_clk_sm"] + ops["fmul"] / pipes["fmul2"]["per_clk_sm"]
-                + ops["ffma"] / pipes["ffma2"]["per_clk_sm"])
-    bounds = {"fp32": 1.0 / fp32_clk, "mufu": pipes["sqrt"]["per_clk_sm"],
-              "smem_atomic": atomic_rate(width, f_in, pipes)}
+    bounds = {"fp32": 1.0 / (PAIR_OPS["fadd"] / pipes["fadd2"]["per_clk_sm"]
+                             + PAIR_OPS["ffma"] / pipes["ffma2"]["per_clk_sm"]),
+              "mufu": pipes["sqrt"]["per_clk_sm"],
+              "smem_atomic": pipes[key]["per_clk_sm"] if key in pipes else float("nan")}
     binding = min((v, k) for k, v in bounds.items() if v == v)[1]
     return {"pairs_per_clk_sm": bounds[binding], "binding": binding,
-            "fp32_lane_ops_per_pair": round(sum(ops.values()), 3),
+            "fp32_lane_ops_per_pair": round(sum(PAIR_OPS.values()), 3),
             "bounds_pairs_per_clk_sm": {k: round(v, 3) for k, v in bounds.items()}}
 
 
 def roofline_entry(pairs: float, seconds: float, mhz: float, bound: dict) -> dict:
     """Achieved pairs per clock per SM (at the SM clock sampled under load)
-    against the frame's bound; `pairs` are the pairs the kernel evaluated (its
-    tiles skipped as out of range or out of the sweep are not counted)."""
+    against the frame's bound; `pairs` are the pairs inside r_max, those counted."""
     achieved = pairs / seconds / (SM_COUNT * mhz * 1e6)
     return {"achieved_pairs_per_clk_sm": round(achieved, 3), "bound_pairs_per_clk_sm": round(bound["pairs_per_clk_sm"], 3),
             "frac": round(achieved / bound["pairs_per_clk_sm"], 4), "binding": bound["binding"],
@@ -432,13 +384,14 @@ def run_configs(ctx, stream, dev, args, pipes, mhz, flush_l2):
         ev = pairs * (1.0 - f_cull)
         fu = st["uniform_pairs"] / max(1.0, ev)
         fa_ = st["axis_pairs"] / max(1.0, ev)
-        bound = pair_bound(f.box_type, f.nbins, fu, fa_, pipes, int(o.sum().item()) / max(1.0, ev))
+        inside = int(o.sum().item())
+        bound = pair_bound(f.nbins, pipes)
         out[name] = {"workload": f.name, "pairs": pairs, "gpairs_s": round(pairs / (statistics.median(ts) / 1e3) / 1e9, 3),
                      "ms": round(statistics.median(ts), 4), "pair_kernel_ms": round(statistics.median(pk), 4),
                      "deferred_frac": round(st["deferred"] / max(1, st["pairs"]), 6),
                      "binary64_frac": round(st["exact_fallback"] / max(1, st["pairs"]), 8),
                      "tile_image_frac": round(fu, 4), "axis_image_frac": round(fa_, 4), "culled_frac": round(f_cull, 4),
-                     "roofline": roofline_entry(ev, statistics.median(pk) / 1e3, mhz, bound)}
+                     "roofline": roofline_entry(inside, statistics.median(pk) / 1e3, mhz, bound)}
         del x, o
     return out
 
@@ -748,7 +701,7 @@ def run_gpu(args, world, rank, local):
     # ---- plain per-frame path (and the pair kernel's own device time per frame)
     plain = {}
     bounds = {}
-    evaluated = {}
+    inside = {}
     for k, f in enumerate(frames):
         ctx.histogram(X[k], f.offsets, f.box_type, f.box, f.r_max, f.nbins, OUT[k])
         ts, pk = [], []
@@ -766,10 +719,9 @@ def run_gpu(args, world, rank, local):
         fu = st["uniform_pairs"] / max(1, st["pairs"])
         fa_ = st["axis_pairs"] / max(1, st["pairs"])
         f_cull = st["culled_pairs"] / max(1, st["pairs"] * st["sweeps"])  # of the pairs of all sweeps
-        evaluated[k] = pairs[k] * (1.0 - f_cull)
-        f_in = int(OUT[k].sum().item()) / max(1.0, evaluated[k])  # evaluated pairs inside r_max
+        inside[k] = int(OUT[k].sum().item())  # pairs inside r_max
         fu, fa_ = fu / (1.0 - f_cull) if f_cull < 1 else 0.0, fa_ / (1.0 - f_cull) if f_cull < 1 else 0.0
-        bounds[k] = pair_bound(f.box_type, f.nbins, fu, fa_, pipes, f_in)
+        bounds[k] = pair_bound(f.nbins, pipes)
         plain[w.BOX_NAMES[f.box_type]] = {
             "gpairs_s": round(pairs[k] / (statistics.mean(ts) / 1e3) / 1e9, 3),
             "ms": round(statistics.mean(ts), 3),
@@ -778,7 +730,7 @@ def run_gpu(args, world, rank, local):
             "tile_image_frac": round(fu, 4),
             "axis_image_frac": round(fa_, 4),
             "culled_frac": round(f_cull, 4),
-            "roofline": roofline_entry(evaluated[k], statistics.mean(pk) / 1e3, mhz, bounds[k]),
+            "roofline": roofline_entry(inside[k], statistics.mean(pk) / 1e3, mhz, bounds[k]),
         }
 
     # ---- roofline of the pair kernel in the timed batched steps: pairs per
@@ -786,24 +738,24 @@ def run_gpu(args, world, rank, local):
     # the step's frames, min over pipes of measured rate / operations per pair,
     # scaled by the SMs and the median SM clock sampled during the timed steps
     mean_pair_s = statistics.mean(pair_ms) / 1e3
-    eval_step = sum(evaluated.values())
-    clk_per_step = sum(evaluated[k] / bounds[k]["pairs_per_clk_sm"] for k in range(len(pairs)))  # SM-clocks
-    peak_gpairs = eval_step / clk_per_step * SM_COUNT * mhz * 1e6 / 1e9
-    achieved_gpairs = eval_step / mean_pair_s / 1e9
+    in_step = sum(inside.values())
+    clk_per_step = sum(inside[k] / bounds[k]["pairs_per_clk_sm"] for k in range(len(pairs)))  # SM-clocks
+    peak_gpairs = in_step / clk_per_step * SM_COUNT * mhz * 1e6 / 1e9
+    achieved_gpairs = in_step / mean_pair_s / 1e9
     headline_size = (args.n, args.nbins) == (1_000_000, 10_000)
     traffic = committed_traffic() if headline_size else None
     roofline = {"bound": "alu", "achieved": round(achieved_gpairs, 3), "peak": round(peak_gpairs, 3),
                 "unit": "Gpairs/s",
-                "achieved_basis": ("pairs the pair kernel evaluated (tiles skipped as outside the bins are not "
-                                   "counted) over the CUDA-event time of its launches in the timed steps"),
+                "achieved_basis": ("pairs inside r_max, those that have to be counted, over the CUDA-event time "
+                                   "of the pair kernel's launches in the timed steps"),
                 "frac": round(achieved_gpairs / peak_gpairs, 4), "traffic": traffic,
-                "traffic_basis": ("DRAM bytes read + written by the step's three pair-kernel launches (ncu, "
-                                  f"{TRAFFIC_FILE}); algorithmic: 3 x (16 B x N + 8 B x nbins)"
+                "traffic_basis": ("DRAM bytes read + written by the step's pair-kernel launch (ncu, "
+                                  f"{TRAFFIC_FILE}); algorithmic: 3 x (24 B x N + 8 B x nbins)"
                                   if traffic else None),
-                "kernel": "dh::pair_kernel",
+                "kernel": "dh::list_kernel",
                 "per_frame": {w.BOX_NAMES[f.box_type]: plain[w.BOX_NAMES[f.box_type]]["roofline"] for f in frames},
                 "peak_basis": (f"per frame min over pipes of measured rate (dh_pipe_rate, ops/clk/SM) / ops per "
-                               f"pair (float32 FMA pipe by tile mode, MUFU sqrt, shared atomic at the width), "
+                               f"pair (float32 FMA pipe, MUFU sqrt, shared atomic on random bins at the width), "
                                f"combined over the step's frames, x {SM_COUNT} SMs x {mhz:.0f} MHz (median SM "
                                f"clock sampled during the timed steps)")}
 

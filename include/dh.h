@@ -121,7 +121,7 @@ typedef struct {
   uint64_t exact_fallback; /* deferred pairs that needed the binary64 replay */
   int32_t sweeps;          /* passes over the pairs (histogram wider than shared memory) */
   int32_t blocks;          /* CUDA blocks launched for the pair kernel */
-  int32_t items;           /* work items (tile pairs) */
+  int32_t items;           /* work items (pairs of runs or tiles) */
   int32_t kernel_launches; /* kernels launched by the call */
   int32_t graph_replays;   /* 1 when the call ran as a replayed CUDA graph */
   int32_t tune_runs;       /* autotuner measurement launches made before the call (DH_CFG_AUTOTUNE) */
@@ -130,12 +130,14 @@ typedef struct {
   int32_t hist_depth;      /*   private histogram copies per block (warp w uses copy w mod depth), */
   int32_t blocks_per_sm;   /*   blocks per SM */
   int32_t block_threads;   /*   and threads per block */
-  uint64_t uniform_pairs;  /* pairs evaluated with one nearest image for their whole tile (no per-pair rounding) */
-  uint64_t axis_pairs;     /* pairs whose tile image is uniform on all axes but one (that axis wrapped per pair) */
+  uint64_t uniform_pairs;  /* pairs of blocks of particles of which one image can lie in the sweep's bins (list
+                              kernel), or with one nearest image for all (tiled kernel) */
+  uint64_t axis_pairs;     /* pairs of blocks with two such images along one axis, or with a nearest image
+                              uniform on all axes but one (tiled kernel: that axis wrapped per pair) */
   int32_t warp_agg;        /* 1 when the largest launch aggregated its increments per warp (tune cache agg) */
   int32_t reserved;
-  uint64_t culled_pairs;   /* pairs (counted once per bin sweep) of tiles skipped because their distance
-                              bounds put no pair in the sweep's bins (periodic frames) */
+  uint64_t culled_pairs;   /* pairs (counted once per bin sweep) of blocks skipped because their distance
+                              bounds put no pair in the sweep's bins */
 } dh_stats;
 
 /* Create a context on config->device (NULL: device 0, defaults).  Owns a CUDA

@@ -26,9 +26,9 @@
 // 3.5 wavefronts on random banks, 90 % busy at N = 200,000), for periodic frames
 // the issue slots (15 instructions per pair and lane, 70 % of the slots used).
 // Pair kernel at 2,070 MHz, 10,000 bins, the tiled kernel before -> now:
-// N = 1,000,000 none 235 -> 229 ms, orthorhombic 254 -> 170, triclinic 284 -> 130;
-// N = 100,000 orthorhombic, two species 4.2 -> 2.8 ms; N = 500,000 clustered
-// triclinic, three species, 20,000 bins 92.6 -> 44 ms; N = 2,000 none, 1,000 bins
+// N = 1,000,000 none 235 -> 229 ms, orthorhombic 254 -> 162, triclinic 284 -> 125;
+// N = 100,000 orthorhombic, two species 4.2 -> 2.6 ms; N = 500,000 clustered
+// triclinic, three species, 20,000 bins 92.6 -> 43 ms; N = 2,000 none, 1,000 bins
 // 118 -> 18 us (items small enough for one per warp).
 // Measured and not kept: three 256-thread blocks of 80 registers (none 13.2 ms at
 // N = 200,000 against 9.6: spills, and the run's factors loaded again per block of
@@ -127,8 +127,8 @@ __device__ __forceinline__ DF renorm(float d, float l) {
   return {h, __fadd_rn(__fsub_rn(d, h), l)};
 }
 
-// |v|^2 - sub of a double-float vector, rounded once (to second order).
-__device__ __forceinline__ float norm2_less(DF x, DF y, DF z, float c1, float c0, float& b) {
+// |v|^2 - (c1 |v|^2 + c0) of a double-float vector, rounded once (to second order).
+__device__ __forceinline__ float norm2_less(DF x, DF y, DF z, float c1, float c0) {
   const DF px = two_prod(x.h, x.h), py = two_prod(y.h, y.h), pz = two_prod(z.h, z.h);
   const DF s1 = two_sum(px.h, py.h);
   const DF s2 = two_sum(s1.h, pz.h);
@@ -136,8 +136,7 @@ __device__ __forceinline__ float norm2_less(DF x, DF y, DF z, float c1, float c0
   low = __fadd_rn(low, __fmaf_rn(y.h + y.h, y.l, py.l));
   low = __fadd_rn(low, __fmaf_rn(z.h + z.h, z.l, pz.l));
   low = __fadd_rn(low, __fadd_rn(s1.l, s2.l));
-  b = __fmaf_rn(c1, s2.h, c0);
-  return __fadd_rn(s2.h, __fsub_rn(low, b));
+  return __fadd_rn(s2.h, __fsub_rn(low, __fmaf_rn(c1, s2.h, c0)));
 }
 
 // One run's state from its bounds (explicit roundings: the drain computes it
@@ -167,8 +166,7 @@ __device__ __forceinline__ RunState run_state(const SegState& G, float4 lo4, flo
 __device__ __forceinline__ float4 i_factors(const Pos& p, float3 c) {
   const DF x = renorm(__fsub_rn(p.h.x, c.x), p.l.x), y = renorm(__fsub_rn(p.h.y, c.y), p.l.y),
            z = renorm(__fsub_rn(p.h.z, c.z), p.l.z);
-  float b;
-  return make_float4(2.0f * x.h, 2.0f * y.h, 2.0f * z.h, -norm2_less(x, y, z, 0.0f, 0.0f, b));
+  return make_float4(2.0f * x.h, 2.0f * y.h, 2.0f * z.h, -norm2_less(x, y, z, 0.0f, 0.0f));
 }
 
 // The vector that takes a home position to image m relative to the centre c
@@ -194,8 +192,7 @@ __device__ __forceinline__ float4 j_image(const Pos& p, const Pos& o, float c1, 
   const DF x = renorm(__fadd_rn(p.h.x, o.h.x), __fadd_rn(p.l.x, o.l.x)),
            y = renorm(__fadd_rn(p.h.y, o.h.y), __fadd_rn(p.l.y, o.l.y)),
            z = renorm(__fadd_rn(p.h.z, o.h.z), __fadd_rn(p.l.z, o.l.z));
-  float b;
-  return make_float4(x.h, y.h, z.h, -norm2_less(x, y, z, c1, c0, b));
+  return make_float4(x.h, y.h, z.h, -norm2_less(x, y, z, c1, c0));
 }
 
 // ------------------------------------------------------------------ re-decision
@@ -638,7 +635,7 @@ __device__ __forceinline__ void merge_count(uint64_t* dst, uint32_t v) {
 }
 
 // One thread fills the block's segment state.
-__device__ void enter_segment(const ListSegment& S, SegCounter* ctr, long long n_items, SegState& G) {
+__device__ void enter_segment(const ListSegment& S, SegCounter* ctr, SegState& G) {
   FrameDev* const Fp = S.fd;
   const FrameDev& F = *Fp;
   G.F = Fp;
@@ -742,7 +739,7 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
     if (seg < 0) break;
     if (tid == 0) {
       atomicAdd(&L.ctr[seg].attached, 1);
-      enter_segment(L.segs[seg], L.ctr + seg, L.n_items, G);
+      enter_segment(L.segs[seg], L.ctr + seg, G);
       // the block's first claim, for all its warps; claims shrink with the items
       // left (a quarter of an even share of them), at first at most the block's
       // share of the launch

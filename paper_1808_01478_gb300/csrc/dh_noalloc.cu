@@ -161,7 +161,7 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   if (bps < 1) return fail(DH_ERR_INVALID, "histogram of %d bins does not fit in shared memory", pf.sweep_width);
 
   // Small frames go the way of dh_histogram: ordered by launch_prep and counted by
-  // the list kernel (N = 30,000 triclinic, two species, 8,192 bins: 595 -> 421 us).
+  // the list kernel (N = 30,000 triclinic, two species, 8,192 bins: 595 -> 389 us).
   NaListPlan lp;
   const bool list = plan_list(frame, max_width, num_sms, base, lp);
   double* T = (double*)(base + (list ? lp.T_at : kNaOffT));

@@ -211,7 +211,7 @@ struct dh_ctx {
   dh::DevBuf bnd;      //   bounds of the runs
   dh::DevBuf sortX64;  // staged in the caller's order: binary64,
   dh::DevBuf sortX;    // and float32 coordinates,
-  dh::DevBuf sortK;    //   cell keys,
+  dh::DevBuf sortK;    //   each particle's cell and place in it,
   dh::DevBuf sortC;    //   and cell counters
   dh::ThresholdCache tcache;
   std::vector<const double*> held_tables;  // tables referenced by work not yet finished
