@@ -750,7 +750,7 @@ __device__ __forceinline__ void frame_ranges(const FrameDev& F, double* R, doubl
 // dependent accesses costs a tenth of what it does in global memory, and of the two
 // setups those that the frame needs: order (spatial order, list kernel) and the
 // window of the tiled kernel, of which frames of the list kernel go without unless
-// asked for (windows).
+// asked for (windows): 7 us for them, 24 with the window (24 with either before).
 __global__ void frame_setup_kernel(FrameDev* frames, int order, int windows) {
   __shared__ __align__(16) FrameDev F;
   uint32_t* const dev = reinterpret_cast<uint32_t*>(frames + blockIdx.x);
