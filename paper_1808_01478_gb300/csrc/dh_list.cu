@@ -60,7 +60,7 @@ constexpr uint32_t kAnyImage = 31u << kImgShift;  // reference of a pair whose i
 // 12: 7.3), a small one pays for its run's setup (orthorhombic N = 100,000 2: 3.20,
 // 6: 3.09, 12: 3.72, 24: 3.98 ms).
 constexpr long long kClaims = 6;
-constexpr unsigned kFlushPairs = 1u << 23;  // flush after this many i runs x images (2^30 pairs)
+constexpr unsigned kFlushPairs = 1u << 23;  // flush after this many i runs x images (2^30 pairs); a power of two
 
 // A position: high parts on the frame's grid, sums of which are exact, and the rest.
 struct Pos {
@@ -898,6 +898,7 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
                 if constexpr (PICK) if (picked) {
                   m = pick_round<MULTI>(G, W, picks[warp], picked, p, jl, jl < jend, i_begin, ni,
                                         diag ? i_begin : -(1 << 30), sh, lane, qcount);
+                  listed += 32u;  // (particles whose pairs it counted are not listed)
                 }
                 const float4 y =
                     j_image(p, PICK && picked ? image_origin(G, max(m, 0), W.R.c) : W.o, W.R.c1, W.R.c0);
@@ -970,13 +971,12 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
           rj = G.intra ? ri : 0;
         }
       }
-      // flush before a shared count can pass 2^31: the warp that crosses the
-      // mark moves every word (the others keep counting)
+      // flush before a shared count can pass 2^31: a warp that takes the total past a
+      // multiple of kFlushPairs moves every word (the others keep counting)
       unsigned before = 0;
       if (lane == 0) before = atomicAdd(&s_since, listed);
       before = __shfl_sync(kFull, before, 0);
-      if (before < kFlushPairs && before + listed >= kFlushPairs) {
-        if (lane == 0) atomicSub(&s_since, kFlushPairs);
+      if ((before ^ (before + listed)) >= kFlushPairs) {
         uint64_t* const dst = F.out + (size_t)L.segs[seg].h * F.nbins + G.lo;
         for (int k = lane; k < G.hi - G.lo; k += 32) merge_count(dst + k, atomicExch(sh + k, 0u));
       }
