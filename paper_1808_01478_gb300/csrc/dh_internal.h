@@ -85,7 +85,8 @@ struct FrameDev {
   // S + S_l = nbins / r_max times the caller's.  From the host:
   float4* P4;         // home positions: x, y, z to a grid (list_grid) and the rest of x,
   float2* P2;         //   the rest of y and z
-  float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz)
+  float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz; w of the
+                      // first: 1 if some coordinate is beyond list_far)
   float S_l;          // nbins / r_max - S
   float img_h[27][3], img_l[27][3];  // image vectors -B k as double-floats (index as tshift)
   float period[3];    // a_x, b_y, c_z
@@ -94,13 +95,14 @@ struct FrameDev {
   int32_t smin[3], smax[3];  // triclinic: range of the fractional coordinates, as cmin and cmax
   int32_t wrap;       // the coordinates span more than one cell: P4 is brought home to the first
                       // (1: in double-floats; 2: in binary64, from 4,096 cells on)
-  int32_t list_slow;  // every pair in binary64 (no trust in the images)
+  int32_t list_slow;  // every pair in binary64 (no trust in the images, or distances beyond float32)
   int32_t list_all;   // every listed pair re-decided (window too wide)
   float key_lo[3], key_inv;  // spatial order: origin and inverse side of the grid
   float list_grid;    // grid of the positions' high parts (a power of two),
   float list_c0;      //   constant part of the window (see list_setup),
   float list_mid;     //   position error of the double-float tier,
   float cull_abs;     //   absolute slack of the distance bounds
+  float list_far;     // no box: runs with a coordinate from here on (bins) are compared in binary64
 };
 
 // One species pair (a,b) of one frame and one bin sweep, cut into kTile x kTile

@@ -264,9 +264,14 @@ __device__ __forceinline__ float3 home32(const FrameDev& F, float x, float y, fl
   return make_float3((float)w.x, (float)w.y, (float)w.z);
 }
 
+// Bins beyond which a far coordinate is moved in to, so that sums of squares stay
+// finite.  Differences only get smaller by it: bounds of such runs remain lower bounds.
+constexpr float kFarthest = 0x1p60f;
+
 // One coordinate in bins: its high part on the grid, and the rest.
 __device__ __forceinline__ DF to_bins_on_grid(const FrameDev& F, DF v) {
   const DF p = two_prod(v.h, F.S);
+  if (fabsf(p.h) >= F.list_far) return {fminf(fmaxf(p.h, -kFarthest), kFarthest), 0.0f};
   const DF s = two_sum(p.h, __fmaf_rn(v.h, F.S_l, __fmaf_rn(v.l, F.S, p.l)));
   const float h = on_grid(s.h, F.list_grid);
   return {h, __fadd_rn(__fsub_rn(s.h, h), s.l)};
@@ -278,7 +283,12 @@ __device__ __forceinline__ void list_position(const FrameDev& F, float4 p, const
     double3 v = x64 ? make_double3(x64->x, x64->y, x64->z) : make_double3(p.x, p.y, p.z);
     if (F.wrap) v = bring_home(F, v.x, v.y, v.z);
     const double s = (double)F.S + (double)F.S_l;
-    const double3 t = make_double3(v.x * s, v.y * s, v.z * s);
+    double3 t = make_double3(v.x * s, v.y * s, v.z * s);
+    if (F.list_far < INFINITY) {
+      t.x = fmin(fmax(t.x, -(double)kFarthest), (double)kFarthest);
+      t.y = fmin(fmax(t.y, -(double)kFarthest), (double)kFarthest);
+      t.z = fmin(fmax(t.z, -(double)kFarthest), (double)kFarthest);
+    }
     x.h = on_grid((float)t.x, F.list_grid);
     y.h = on_grid((float)t.y, F.list_grid);
     z.h = on_grid((float)t.z, F.list_grid);
@@ -431,7 +441,8 @@ __device__ __forceinline__ void run_bounds(const FrameDev& F, const SortSeg& S, 
       b[3 + c] = fmaxf(b[3 + c], __shfl_xor_sync(kFull, b[3 + c], o));
     }
   if (lane == 0) {
-    F.bnd[2 * (S.run0 + run)] = make_float4(b[0], b[1], b[2], 0.0f);
+    const float most = fmaxf(fmaxf(fmaxf(-b[0], b[3]), fmaxf(-b[1], b[4])), fmaxf(-b[2], b[5]));
+    F.bnd[2 * (S.run0 + run)] = make_float4(b[0], b[1], b[2], most >= F.list_far ? 1.0f : 0.0f);
     F.bnd[2 * (S.run0 + run) + 1] = make_float4(b[3], b[4], b[5], 0.0f);
   }
 }
@@ -508,16 +519,29 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
       if (!(cells < 4096.0)) wrap = 2;
     }
   }
+  // No box: one particle far away must not cost the others their precision, nor squares
+  // of bins their finite range.  From 2^16 r_max on, where float32 coordinates are a
+  // 256th of r_max apart, a run's pairs are compared in binary64 and the others' grid
+  // does not reach; frames within 2^17 r_max, wherever they are, need none of this.
+  // One particle of N = 100,000 parked at 1e8: pair kernel 16.0 -> 5.6 ms; at 1e20, where
+  // every pair was replayed and many were lost, 200.8 -> 5.6 ms.
+  F.list_far = INFINITY;
+  if (F.variant == V_NONE && fmax(R[0], fmax(R[1], R[2])) > 131072.0 * F.r_max) {
+    F.list_far = 65536.0f * (float)F.nbins;
+    far = fmin(far, 65536.0 * F.r_max);
+  }
   const double side = fmax(ext[0], fmax(ext[1], ext[2]));
   for (int c = 0; c < 3; ++c) F.key_lo[c] = (float)lo[c];
   F.key_inv = side > 0.0 ? (float)(0.99999 / side) : 0.0f;
   F.wrap = wrap;
-  F.list_slow = slow;
   const double cell = F.variant == V_NONE ? 0.0 : B[0] + fabs(B[1]) + fabs(B[2]) + B[4] + fabs(B[5]) + B[8];
   // positions and image vectors: the largest of them in bins; brought home, the
   // subtraction errs by 2^-52 (binary64) or 2^-45 (double-floats) of what is
   // subtracted, per axis and position
   const double reach = S * ((wrap ? ext[0] + ext[1] + ext[2] : 2.0 * far) + 2.0 * cell);
+  // bins so narrow that squares of the frame's extent pass float32's range (or S itself does)
+  if (!(reach < 0x1p60)) slow = 1;
+  F.list_slow = slow;
   const double a0 = reach * 0x1p-44 + (wrap ? S * far * (wrap == 1 ? 0x1p-43 : 0x1p-49) : 0.0);
   // grid of the high parts: sums of positions, centres and images stay below
   // 2^23 steps, so they are exact in float32

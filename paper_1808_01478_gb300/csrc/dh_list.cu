@@ -112,7 +112,7 @@ struct SegState {
   float in_hi2, in_lo2;   // every pair in the sweep: farthest^2 <= in_hi2, nearest^2 >= in_lo2
   float grid, c0, abs, mid;  // FrameDev list_grid, list_c0, cull_abs, list_mid
   float nbins;
-  int n_img, all, slow;   // images of a particle; FrameDev list_all, list_slow
+  int n_img, all, slow;   // images of a particle; FrameDev list_all; 1: list_slow, 2: some runs are far (far_item)
   int inner;              // FrameDev in_range: nearly every block is an inner one
   long long items, item_base;
   long long claimers;     // claims that share the items left: kClaims per warp of the launch
@@ -628,6 +628,23 @@ __device__ __noinline__ void slow_item(const SegState& G, int ib, int ni, int jb
   }
 }
 
+// How an item of a frame with far runs (FrameDev.list_far) is done: 0 as any other,
+// when neither run is one; 2 not at all, when the gap between their bounds puts every
+// pair beyond the sweep (2^-20 of the coordinates for the rounding of the bounds); else
+// 1, in binary64.
+__device__ __noinline__ int far_item(const SegState& G, int ri, int rj) {
+  const float4 ilo = __ldg(G.bi + 2 * ri), ihi = __ldg(G.bi + 2 * ri + 1);
+  const float4 jlo = __ldg(G.bj + 2 * rj), jhi = __ldg(G.bj + 2 * rj + 1);
+  if (ilo.w == 0.0f && jlo.w == 0.0f) return 0;
+  auto gap = [](float il, float ih, float jl, float jh) {
+    const float size = fmaxf(fmaxf(fabsf(il), fabsf(ih)), fmaxf(fabsf(jl), fabsf(jh)));
+    return fmaxf(fmaxf(jl - ih, il - jh) - size * 0x1p-20f, 0.0f);
+  };
+  const float gx = gap(ilo.x, ihi.x, jlo.x, jhi.x), gy = gap(ilo.y, ihi.y, jlo.y, jhi.y),
+              gz = gap(ilo.z, ihi.z, jlo.z, jhi.z);
+  return gx * gx + gy * gy + gz * gz > G.rc_hi2 ? 2 : 1;
+}
+
 // Adds one word's count to the global histogram.  Counts are signed: a
 // provisional count may be moved after the words were flushed.
 __device__ __forceinline__ void merge_count(uint64_t* dst, uint32_t v) {
@@ -670,7 +687,7 @@ __device__ void enter_segment(const ListSegment& S, SegCounter* ctr, SegState& G
   G.nbins = (float)F.nbins;
   G.n_img = F.variant == V_NONE ? 1 : 27;
   G.all = F.list_all;
-  G.slow = F.list_slow;
+  G.slow = F.list_slow ? 1 : F.list_far < INFINITY ? 2 : 0;
   // elsewhere the two loops would take turns in the instruction cache, at a loss
   G.inner = F.in_range;
   G.items = (G.lo < F.nbins && !F.bad) ? S.items : 0;
@@ -807,14 +824,17 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
           const bool diag = G.intra && rj == ri;
           const int jbeg = rj * kRun + sub * part;
           const int jend = min(nj, jbeg + part);
-          if (G.slow) {
+          int slow = G.slow;
+          if (slow == 2) slow = far_item(G, ri, rj);
+          if (slow == 1) {
             if (jbeg < jend) slow_item(G, i_begin, ni, jbeg, jend, sh, lane);
             listed += kRun;
-          } else {
+          }
+          if (G.slow != 1) {
             // ---- images of the j run that can lie in the sweep (bounds against bounds)
             bool keep = false;
             float g2 = 0.0f, f2 = 0.0f;
-            if (lane < G.n_img && jbeg < jend) {
+            if (lane < G.n_img && jbeg < jend && slow == 0) {
               const float4 jlo = __ldg(G.bj + 2 * rj), jhi = __ldg(G.bj + 2 * rj + 1);
               const int m = G.n_img == 1 ? kHome : lane;
               const float4 V = G.V4[m];
@@ -843,7 +863,7 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
               keep = keep && g2 <= reach * reach && far >= G.rc_lo2;
             }
             unsigned mask = __ballot_sync(kFull, keep);
-            if (lane == 0) {  // statistics
+            if (lane == 0 && slow != 1) {  // statistics
               const unsigned long long np = (unsigned long long)max(jend - jbeg, 0) * (unsigned long long)ni;
               const int nimg = __popc(mask);
               if (nimg == 0) W.cull += np;

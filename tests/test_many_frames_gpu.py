@@ -1,0 +1,42 @@
+"""Batches of very many frames: more species than a launch dimension holds, and
+frames that need another preparation than the rest.
+"""
+import numpy as np
+import pytest
+
+import paper_1808_01478_gb300 as dh
+import workloads as w
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_mod():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch
+
+
+@pytest.mark.parametrize("odd", ["none", "empty", "large", "wide"])
+def test_more_species_than_a_launch_dimension(torch_mod, oracle_mod, odd):
+    # 66,000 frames of three particles, and one that the one-launch preparation cannot take
+    frames, nbins, r_max = 66_000, 2, 2.0
+    rng = w.rng_for(41)
+    x = torch_mod.from_numpy(rng.random((frames * 3, 3)).astype(np.float32)).cuda()
+    out = torch_mod.full((frames, 1, nbins), 9, dtype=torch_mod.int64, device="cuda")
+    fas = [dh.FrameArgs(x[3 * k:3 * k + 3], [0, 3], w.BOX_NONE, None, r_max, nbins, out[k]) for k in range(frames)]
+    if odd != "none":
+        n, bins = {"empty": (0, 3), "large": (40_000, 50), "wide": (2000, 50_000)}[odd]
+        y = (rng.random((n, 3)) * 5.0).astype(np.float32)
+        want = oracle_mod.histogram(y, np.array([0, n // 3, n]), w.BOX_NONE, np.zeros(9), 4.0, bins)
+        fas.insert(frames // 2, dh.FrameArgs(torch_mod.from_numpy(y).cuda(), [0, n // 3, n], w.BOX_NONE, None, 4.0, bins))
+    with dh.Context(0) as ctx:
+        ctx.histogram_batch(fas)
+    got = out.cpu().numpy()
+    d = np.linalg.norm(np.diff(np.concatenate([x.cpu().numpy().astype(np.float64).reshape(-1, 3, 3)] * 2, 1)[:, :4], axis=1),
+                       axis=2)  # the three distances
+    near = (d < r_max / 2).sum(1)
+    assert np.array_equal(got[:, 0, 0], near) and np.array_equal(got[:, 0, 1], 3 - near)
+    if odd != "none":
+        assert np.array_equal(fas[frames // 2].out.cpu().numpy().view(np.uint64), want)
