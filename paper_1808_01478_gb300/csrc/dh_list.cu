@@ -112,7 +112,7 @@ struct SegState {
   float in_hi2, in_lo2;   // every pair in the sweep: farthest^2 <= in_hi2, nearest^2 >= in_lo2
   float grid, c0, abs, mid;  // FrameDev list_grid, list_c0, cull_abs, list_mid
   float nbins;
-  int n_img, all, slow;   // images of a particle; FrameDev list_all; 1: list_slow, 2: some runs are far (far_item)
+  int n_img, all, slow;   // images of a particle; FrameDev list_all; 1: list_slow, 2: some runs are far (slow_item)
   int inner;              // FrameDev in_range: nearly every block is an inner one
   long long items, item_base;
   long long claimers;     // claims that share the items left: kClaims per warp of the launch
@@ -609,10 +609,30 @@ __device__ __noinline__ int pick_round(const SegState& G, WarpList<kBlk>& W, Pic
   return single;
 }
 
-// Every pair of an item in binary64 (frames whose images cannot be listed).
-__device__ __noinline__ void slow_item(const SegState& G, int ib, int ni, int jbeg, int jend, uint32_t* sh, int lane) {
+// Of two runs of which one is far (FrameDev.list_far): the gap between their bounds puts
+// every pair beyond the sweep (2^-20 of the coordinates for the rounding of the bounds).
+__device__ __forceinline__ bool far_apart(const SegState& G, float4 ilo, float4 ihi, float4 jlo, float4 jhi) {
+  auto gap = [](float il, float ih, float jl, float jh) {
+    const float size = fmaxf(fmaxf(fabsf(il), fabsf(ih)), fmaxf(fabsf(jl), fabsf(jh)));
+    return fmaxf(fmaxf(jl - ih, il - jh) - size * 0x1p-20f, 0.0f);
+  };
+  const float gx = gap(ilo.x, ihi.x, jlo.x, jhi.x), gy = gap(ilo.y, ihi.y, jlo.y, jhi.y),
+              gz = gap(ilo.z, ihi.z, jlo.z, jhi.z);
+  return gx * gx + gy * gy + gz * gz > G.rc_hi2;
+}
+
+// Every pair of an item in binary64, in frames whose images cannot be listed (G.slow 1)
+// or for a far run (G.slow 2, i run ri and j run rj).  Returns the images that the item
+// counts for towards the flush, -1 for an item of two runs that are not far: nothing done.
+__device__ __noinline__ int slow_item(const SegState& G, int ri, int rj, int ni, int jbeg, int jend, uint32_t* sh, int lane) {
+  if (G.slow == 2) {
+    const float4 ilo = __ldg(G.bi + 2 * ri), ihi = __ldg(G.bi + 2 * ri + 1);
+    const float4 jlo = __ldg(G.bj + 2 * rj), jhi = __ldg(G.bj + 2 * rj + 1);
+    if (ilo.w == 0.0f && jlo.w == 0.0f) return -1;
+    if (far_apart(G, ilo, ihi, jlo, jhi)) return 0;
+  }
   FrameDev* const Fp = G.F;
-  const int nj = jend - jbeg;
+  const int ib = ri * kRun, nj = jend - jbeg;
   unsigned long long np = 0;
   for (int p = lane; p < ni * nj; p += 32) {
     const int i = ib + p % ni, j = jbeg + p / ni;
@@ -626,23 +646,7 @@ __device__ __noinline__ void slow_item(const SegState& G, int ib, int ni, int jb
     atomicAdd(&Fp->deferred, np);
     atomicAdd(&Fp->exact, np);
   }
-}
-
-// How an item of a frame with far runs (FrameDev.list_far) is done: 0 as any other,
-// when neither run is one; 2 not at all, when the gap between their bounds puts every
-// pair beyond the sweep (2^-20 of the coordinates for the rounding of the bounds); else
-// 1, in binary64.
-__device__ __noinline__ int far_item(const SegState& G, int ri, int rj) {
-  const float4 ilo = __ldg(G.bi + 2 * ri), ihi = __ldg(G.bi + 2 * ri + 1);
-  const float4 jlo = __ldg(G.bj + 2 * rj), jhi = __ldg(G.bj + 2 * rj + 1);
-  if (ilo.w == 0.0f && jlo.w == 0.0f) return 0;
-  auto gap = [](float il, float ih, float jl, float jh) {
-    const float size = fmaxf(fmaxf(fabsf(il), fabsf(ih)), fmaxf(fabsf(jl), fabsf(jh)));
-    return fmaxf(fmaxf(jl - ih, il - jh) - size * 0x1p-20f, 0.0f);
-  };
-  const float gx = gap(ilo.x, ihi.x, jlo.x, jhi.x), gy = gap(ilo.y, ihi.y, jlo.y, jhi.y),
-              gz = gap(ilo.z, ihi.z, jlo.z, jhi.z);
-  return gx * gx + gy * gy + gz * gz > G.rc_hi2 ? 2 : 1;
+  return kRun;
 }
 
 // Adds one word's count to the global histogram.  Counts are signed: a
@@ -823,162 +827,161 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
         for (int t = 0; t < row; ++t) {
           const bool diag = G.intra && rj == ri;
           const int jbeg = rj * kRun + sub * part;
-          const int jend = min(nj, jbeg + part);
-          int slow = G.slow;
-          if (slow == 2) slow = far_item(G, ri, rj);
-          if (slow == 1) {
-            if (jbeg < jend) slow_item(G, i_begin, ni, jbeg, jend, sh, lane);
-            listed += kRun;
+          int jend = min(nj, jbeg + part);
+          if (G.slow) {
+            const int counted = slow_item(G, ri, rj, ni, jbeg, jend, sh, lane);
+            if (counted >= 0) {
+              listed += (unsigned)counted;
+              jend = jbeg;  // nothing to list
+            }
           }
-          if (G.slow != 1) {
-            // ---- images of the j run that can lie in the sweep (bounds against bounds)
-            bool keep = false;
-            float g2 = 0.0f, f2 = 0.0f;
-            if (lane < G.n_img && jbeg < jend && slow == 0) {
-              const float4 jlo = __ldg(G.bj + 2 * rj), jhi = __ldg(G.bj + 2 * rj + 1);
-              const int m = G.n_img == 1 ? kHome : lane;
-              const float4 V = G.V4[m];
-              const float sx = V.x, sy = V.y, sz = V.z;
-              // ranges of the j run's image around the centre, then out by the half extents
-              const float3 c = W.R.c, h = W.R.h;
-              const float lx = jlo.x + sx - c.x, ux = jhi.x + sx - c.x;
-              const float ly = jlo.y + sy - c.y, uy = jhi.y + sy - c.y;
-              const float lz = jlo.z + sz - c.z, uz = jhi.z + sz - c.z;
-              const float gx = fmaxf(fmaxf(lx, -ux) - h.x, 0.0f), gy = fmaxf(fmaxf(ly, -uy) - h.y, 0.0f),
-                          gz = fmaxf(fmaxf(lz, -uz) - h.z, 0.0f);
-              const float fx = fmaxf(fabsf(lx), fabsf(ux)) + h.x, fy = fmaxf(fabsf(ly), fabsf(uy)) + h.y,
-                          fz = fmaxf(fabsf(lz), fabsf(uz)) + h.z;
-              g2 = gx * gx + gy * gy + gz * gz;
-              f2 = fx * fx + fy * fy + fz * fz;
-              keep = g2 <= G.rc_hi2 && (PICK || f2 >= G.rc_lo2);
+          // ---- images of the j run that can lie in the sweep (bounds against bounds)
+          bool keep = false;
+          float g2 = 0.0f, f2 = 0.0f;
+          if (lane < G.n_img && jbeg < jend) {
+            const float4 jlo = __ldg(G.bj + 2 * rj), jhi = __ldg(G.bj + 2 * rj + 1);
+            const int m = G.n_img == 1 ? kHome : lane;
+            const float4 V = G.V4[m];
+            const float sx = V.x, sy = V.y, sz = V.z;
+            // ranges of the j run's image around the centre, then out by the half extents
+            const float3 c = W.R.c, h = W.R.h;
+            const float lx = jlo.x + sx - c.x, ux = jhi.x + sx - c.x;
+            const float ly = jlo.y + sy - c.y, uy = jhi.y + sy - c.y;
+            const float lz = jlo.z + sz - c.z, uz = jhi.z + sz - c.z;
+            const float gx = fmaxf(fmaxf(lx, -ux) - h.x, 0.0f), gy = fmaxf(fmaxf(ly, -uy) - h.y, 0.0f),
+                        gz = fmaxf(fmaxf(lz, -uz) - h.z, 0.0f);
+            const float fx = fmaxf(fabsf(lx), fabsf(ux)) + h.x, fy = fmaxf(fabsf(ly), fabsf(uy)) + h.y,
+                        fz = fmaxf(fabsf(lz), fabsf(uz)) + h.z;
+            g2 = gx * gx + gy * gy + gz * gz;
+            f2 = fx * fx + fy * fy + fz * fz;
+            keep = g2 <= G.rc_hi2 && (PICK || f2 >= G.rc_lo2);
+          }
+          unsigned picked = 0u;  // PICK: several images, handled particle by particle
+          if (PICK) {
+            const bool img = lane < G.n_img && jbeg < jend;
+            float far = img ? f2 : INFINITY;
+            for (int o = 16; o > 0; o >>= 1) far = fminf(far, __shfl_xor_sync(kFull, far, o));
+            // only images nearer than the farthest pair of another; none when one puts
+            // every pair below the sweep
+            const float reach = sqrtf(far) * (1.0f + 0x1p-15f) + 2.0f * G.abs;
+            keep = keep && g2 <= reach * reach && far >= G.rc_lo2;
+          }
+          unsigned mask = __ballot_sync(kFull, keep);
+          if (lane == 0) {  // statistics
+            const unsigned long long np = (unsigned long long)max(jend - jbeg, 0) * (unsigned long long)ni;
+            const int nimg = __popc(mask);
+            if (nimg == 0) W.cull += np;
+            if (nimg == 1) W.uni += np;
+            if (nimg == 2) {
+              const int a = __ffs(mask) - 1, b = 31 - __clz(mask);
+              if ((a / 9 != b / 9) + (a / 3 % 3 != b / 3 % 3) + (a % 3 != b % 3) == 1) W.axis += np;
             }
-            unsigned picked = 0u;  // PICK: several images, handled particle by particle
-            if (PICK) {
-              const bool img = lane < G.n_img && jbeg < jend;
-              float far = img ? f2 : INFINITY;
-              for (int o = 16; o > 0; o >>= 1) far = fminf(far, __shfl_xor_sync(kFull, far, o));
-              // only images nearer than the farthest pair of another; none when one puts
-              // every pair below the sweep
-              const float reach = sqrtf(far) * (1.0f + 0x1p-15f) + 2.0f * G.abs;
-              keep = keep && g2 <= reach * reach && far >= G.rc_lo2;
-            }
-            unsigned mask = __ballot_sync(kFull, keep);
-            if (lane == 0 && slow != 1) {  // statistics
-              const unsigned long long np = (unsigned long long)max(jend - jbeg, 0) * (unsigned long long)ni;
-              const int nimg = __popc(mask);
-              if (nimg == 0) W.cull += np;
-              if (nimg == 1) W.uni += np;
-              if (nimg == 2) {
-                const int a = __ffs(mask) - 1, b = 31 - __clz(mask);
-                if ((a / 9 != b / 9) + (a / 3 % 3 != b / 3 % 3) + (a % 3 != b % 3) == 1) W.axis += np;
-              }
-            }
-            // one round of 32 j particles of one image per turn; a last turn ends the
-            // list with the row and with the diagonal item
-            const bool ends = t == row - 1 || diag;
-            int m = kHome, jb = jend;
-            bool in_here = false, near_here = false;
-            for (;;) {
-              int want = BLK;
-              if (PICK && jb >= jend && (mask & (mask - 1u))) {
-                picked = mask;
-                mask = 0u;
-                in_here = inner = false;
-                jb = jbeg;
-              } else if (jb >= jend && mask) {
-                const int ml = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                picked = 0u;
-                m = G.n_img == 1 ? kHome : ml;
-                // inner: every pair in the sweep
-                const float f2m = __shfl_sync(kFull, f2, ml), g2m = __shfl_sync(kFull, g2, ml);
-                in_here = f2m <= G.in_hi2 && g2m >= G.in_lo2;
-                inner = inner && in_here;
-                const Pos o = image_origin(G, m, W.R.c);
-                __syncwarp();
-                if (lane == 0) W.o = o;
-                __syncwarp();
-                jb = jbeg;
-              }
-              const bool more = jb < jend;
-              near_here = false;
-              if (more) {
-                const int jl = jb + lane;
-                // this round's particle was loaded in the round before (the next
-                // round, image or run is the likely successor); else load it now
-                if (pf != jb) {
-                  pa = __ldg(G.P4j + min(jl, nj - 1));
-                  pb = __ldg(G.P2j + min(jl, nj - 1));
-                }
-                const Pos p = unpack(pa, pb);
-                jb += 32;
-                pf = jb < jend ? jb : (mask ? jbeg : jend);
-                pa = __ldg(G.P4j + min(pf + lane, nj - 1));
-                pb = __ldg(G.P2j + min(pf + lane, nj - 1));
-                if constexpr (PICK) if (picked) {
-                  m = pick_round<MULTI>(G, W, picks[warp], picked, p, jl, jl < jend, i_begin, ni,
-                                        diag ? i_begin : -(1 << 30), sh, lane, qcount);
-                  listed += 32u;  // (particles whose pairs it counted are not listed)
-                }
-                const float4 y =
-                    j_image(p, PICK && picked ? image_origin(G, max(m, 0), W.R.c) : W.o, W.R.c1, W.R.c0);
-                const float3 h = W.R.h;
-                const float ax = fabsf(y.x), ay = fabsf(y.y), az = fabsf(y.z);
-                const float gx = fmaxf(ax - h.x, 0.0f), gy = fmaxf(ay - h.y, 0.0f), gz = fmaxf(az - h.z, 0.0f);
-                bool in = jl < jend && m >= 0 && gx * gx + gy * gy + gz * gz <= G.rc_hi2;
-                if (MULTI) {  // (for a single image the same as below the sweep)
-                  const float fx = ax + h.x, fy = ay + h.y, fz = az + h.z;
-                  in = in && fx * fx + fy * fy + fz * fz >= G.rc_lo2;
-                }
-                const unsigned bal = __ballot_sync(kFull, in);
-                // this round's own particles: near the run's box for their own W?
-                const float w = __fmaf_rn(2.0f * W.R.c1, ax * ax + ay * ay + az * az, 2.0f * W.R.c0 + 3.0f + G.abs);
-                near_here = __any_sync(kFull, in && gx * gx + gy * gy + gz * gz < w * w);
-                near = near || near_here;
-                if (in) {
-                  const int s = (tail + __popc(bal & lt_mask)) & (kCap - 1);
-                  float* a = reinterpret_cast<float*>(&W.A[s >> 1]) + (s & 1);
-                  float* b = reinterpret_cast<float*>(&W.B[s >> 1]) + (s & 1);
-                  a[0] = y.x;
-                  a[2] = y.y;
-                  b[0] = y.z;
-                  b[2] = y.w;
-                  W.ref[s] = (uint32_t)jl | ((uint32_t)m << kImgShift);
-                }
-                tail += __popc(bal);
-              } else {
-                if (!ends) break;
-                want = (tail - done + 7) & ~7;  // fewer than a block: padded to whole groups
-                if (want == 0) break;
-                if (lane < done + want - tail) {
-                  const int s = (tail + lane) & (kCap - 1);
-                  reinterpret_cast<float*>(&W.B[s >> 1])[2 + (s & 1)] = NAN;
-                  W.ref[s] = 0u;
-                }
-              }
+          }
+          // one round of 32 j particles of one image per turn; a last turn ends the
+          // list with the row and with the diagonal item
+          const bool ends = t == row - 1 || diag;
+          int m = kHome, jb = jend;
+          bool in_here = false, near_here = false;
+          for (;;) {
+            int want = BLK;
+            if (PICK && jb >= jend && (mask & (mask - 1u))) {
+              picked = mask;
+              mask = 0u;
+              in_here = inner = false;
+              jb = jbeg;
+            } else if (jb >= jend && mask) {
+              const int ml = __ffs(mask) - 1;
+              mask &= mask - 1u;
+              picked = 0u;
+              m = G.n_img == 1 ? kHome : ml;
+              // inner: every pair in the sweep
+              const float f2m = __shfl_sync(kFull, f2, ml), g2m = __shfl_sync(kFull, g2, ml);
+              in_here = f2m <= G.in_hi2 && g2m >= G.in_lo2;
+              inner = inner && in_here;
+              const Pos o = image_origin(G, m, W.R.c);
               __syncwarp();
-              if (!more || tail - done >= BLK) {
-                const int s0 = done & (kCap - 1);
-                uint32_t groups, first = (uint32_t)i_begin;
-                if (near || diag) {
-                  groups = list_near<MULTI>(G, W, i_begin, ni, s0, want, diag ? i_begin : -(1 << 30), sh, lane);
-                  first |= kNearPair;
-                } else if (inner && more && ni == kRun && G.inner) {
-                  groups = list_block<INNER, MULTI>(G, I, W, s0, BLK, 0, sh, lane);
-                } else {
-                  groups = list_block<PLAIN, MULTI>(G, I, W, s0, want, 0, sh, lane);
-                }
-                qcount = push_pairs(G, W, s0, groups, first, sh, lane, qcount);
-                done += BLK;
-                // what is left was appended in this round
-                near = near_here || G.all;
-                inner = !more || in_here;
+              if (lane == 0) W.o = o;
+              __syncwarp();
+              jb = jbeg;
+            }
+            const bool more = jb < jend;
+            near_here = false;
+            if (more) {
+              const int jl = jb + lane;
+              // this round's particle was loaded in the round before (the next
+              // round, image or run is the likely successor); else load it now
+              if (pf != jb) {
+                pa = __ldg(G.P4j + min(jl, nj - 1));
+                pb = __ldg(G.P2j + min(jl, nj - 1));
               }
-              if (!more) {
-                listed += (unsigned)tail;
-                tail = done = 0;
-                break;
+              const Pos p = unpack(pa, pb);
+              jb += 32;
+              pf = jb < jend ? jb : (mask ? jbeg : jend);
+              pa = __ldg(G.P4j + min(pf + lane, nj - 1));
+              pb = __ldg(G.P2j + min(pf + lane, nj - 1));
+              if constexpr (PICK) if (picked) {
+                m = pick_round<MULTI>(G, W, picks[warp], picked, p, jl, jl < jend, i_begin, ni,
+                                      diag ? i_begin : -(1 << 30), sh, lane, qcount);
+                listed += 32u;  // (particles whose pairs it counted are not listed)
               }
+              const float4 y =
+                  j_image(p, PICK && picked ? image_origin(G, max(m, 0), W.R.c) : W.o, W.R.c1, W.R.c0);
+              const float3 h = W.R.h;
+              const float ax = fabsf(y.x), ay = fabsf(y.y), az = fabsf(y.z);
+              const float gx = fmaxf(ax - h.x, 0.0f), gy = fmaxf(ay - h.y, 0.0f), gz = fmaxf(az - h.z, 0.0f);
+              bool in = jl < jend && m >= 0 && gx * gx + gy * gy + gz * gz <= G.rc_hi2;
+              if (MULTI) {  // (for a single image the same as below the sweep)
+                const float fx = ax + h.x, fy = ay + h.y, fz = az + h.z;
+                in = in && fx * fx + fy * fy + fz * fz >= G.rc_lo2;
+              }
+              const unsigned bal = __ballot_sync(kFull, in);
+              // this round's own particles: near the run's box for their own W?
+              const float w = __fmaf_rn(2.0f * W.R.c1, ax * ax + ay * ay + az * az, 2.0f * W.R.c0 + 3.0f + G.abs);
+              near_here = __any_sync(kFull, in && gx * gx + gy * gy + gz * gz < w * w);
+              near = near || near_here;
+              if (in) {
+                const int s = (tail + __popc(bal & lt_mask)) & (kCap - 1);
+                float* a = reinterpret_cast<float*>(&W.A[s >> 1]) + (s & 1);
+                float* b = reinterpret_cast<float*>(&W.B[s >> 1]) + (s & 1);
+                a[0] = y.x;
+                a[2] = y.y;
+                b[0] = y.z;
+                b[2] = y.w;
+                W.ref[s] = (uint32_t)jl | ((uint32_t)m << kImgShift);
+              }
+              tail += __popc(bal);
+            } else {
+              if (!ends) break;
+              want = (tail - done + 7) & ~7;  // fewer than a block: padded to whole groups
+              if (want == 0) break;
+              if (lane < done + want - tail) {
+                const int s = (tail + lane) & (kCap - 1);
+                reinterpret_cast<float*>(&W.B[s >> 1])[2 + (s & 1)] = NAN;
+                W.ref[s] = 0u;
+              }
+            }
+            __syncwarp();
+            if (!more || tail - done >= BLK) {
+              const int s0 = done & (kCap - 1);
+              uint32_t groups, first = (uint32_t)i_begin;
+              if (near || diag) {
+                groups = list_near<MULTI>(G, W, i_begin, ni, s0, want, diag ? i_begin : -(1 << 30), sh, lane);
+                first |= kNearPair;
+              } else if (inner && more && ni == kRun && G.inner) {
+                groups = list_block<INNER, MULTI>(G, I, W, s0, BLK, 0, sh, lane);
+              } else {
+                groups = list_block<PLAIN, MULTI>(G, I, W, s0, want, 0, sh, lane);
+              }
+              qcount = push_pairs(G, W, s0, groups, first, sh, lane, qcount);
+              done += BLK;
+              // what is left was appended in this round
+              near = near_here || G.all;
+              inner = !more || in_here;
+            }
+            if (!more) {
+              listed += (unsigned)tail;
+              tail = done = 0;
+              break;
             }
           }
           if (++sub == L.split) {
