@@ -169,13 +169,16 @@ struct SortSeg {
   int32_t n_slab, n_col;   // slabs, columns per slab
   int32_t slab, col;       // particles per slab and per column, multiples of kRun
   int32_t run0;      // first run of this species in the frame's bounds
+  int32_t chunk0, tile0[3], bblock0;  // first block of the launches (number_sort_blocks)
 };
 // Counters of a pass.
 __host__ __device__ inline int64_t sort_keys(const SortSeg& S, int pass) {
   if (S.nb[0] == 0) return pass < 2 ? 0 : S.g > 0 ? (int64_t)1 << (3 * S.g) : 4;
   return (int64_t)S.nb[pass] * (pass == 0 ? 1 : pass == 1 ? S.n_slab : S.n_slab * S.n_col);
 }
-constexpr int kSortChunk = 256;
+constexpr int kSortChunk = 256;   // particles per block,
+constexpr int kScanTile = 4096;   //   counters per block,
+constexpr int kBoundRuns = 8;     //   runs per block of the order's launches
 
 struct Control {
   unsigned long long next_item;  // dynamic work counter (reset before each launch)
@@ -242,14 +245,30 @@ cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, bool order, bool 
 // What a set of SortSeg needs.
 struct SortPlan {
   int64_t keys = 0;               // counters of all passes
-  int64_t max_n = 0;              // the largest species,
-  int64_t max_keys[3] = {0, 0, 0};  // and the most counters of one in each pass
+  int64_t max_keys[3] = {0, 0, 0};  // most counters of one in each pass
+  int64_t chunks = 0, tiles[3] = {0, 0, 0}, bblocks = 0;  // blocks of the launches
   void add(const SortPlan& o) {
     keys += o.keys;
-    max_n = o.max_n > max_n ? o.max_n : max_n;
     for (int p = 0; p < 3; ++p) max_keys[p] = o.max_keys[p] > max_keys[p] ? o.max_keys[p] : max_keys[p];
   }
 };
+// Numbers the blocks of the segments' launches one after another, so that each block
+// has work whatever the sizes, and any number of species fits a launch.
+inline void number_sort_blocks(SortSeg* segs, size_t n, SortPlan& plan) {
+  plan.chunks = plan.bblocks = 0;
+  for (int64_t& t : plan.tiles) t = 0;
+  for (size_t q = 0; q < n; ++q) {
+    SortSeg& g = segs[q];
+    g.chunk0 = (int32_t)plan.chunks;
+    g.bblock0 = (int32_t)plan.bblocks;
+    plan.chunks += (g.n + kSortChunk - 1) / kSortChunk;
+    plan.bblocks += (g.n + (int64_t)kBoundRuns * kRun - 1) / ((int64_t)kBoundRuns * kRun);
+    for (int p = 0; p < 3; ++p) {
+      g.tile0[p] = (int32_t)plan.tiles[p];
+      plan.tiles[p] += (sort_keys(g, p) + kScanTile - 1) / kScanTile;
+    }
+  }
+}
 // Orders each segment's particles from src (src64) into dst (dst64), and for the
 // list kernel into the frame's P4 and P2 with the bounds of its runs.  counts:
 // plan.keys counters, zeroed, then as many cursors; keys: two per particle; the

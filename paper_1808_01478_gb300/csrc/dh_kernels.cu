@@ -333,12 +333,23 @@ __device__ __forceinline__ int sort_cell(const FrameDev& F, const SortSeg& S, fl
                           (uint32_t)min(max(cz, 0), last), S.g);
 }
 
+// The segment of this block: the last whose first block (first(segment)) is not above it.
+template <typename First>
+__device__ __forceinline__ const SortSeg& segment_of_block(const SortSeg* segs, int n_segs, First first) {
+  int lo = 0, hi = n_segs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (first(segs[mid]) <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  return segs[lo];
+}
+
 // One pass: each particle's cell and its place in the cell (keys), the cells' counts.
-__global__ void sort_count_kernel(const SortSeg* segs, int pass, const float4* __restrict__ X, int2* keys,
+__global__ void sort_count_kernel(const SortSeg* segs, int n_segs, int pass, const float4* __restrict__ X, int2* keys,
                                   uint32_t* counts, const uint32_t* __restrict__ cursors) {
-  const SortSeg S = segs[blockIdx.y];
+  const SortSeg S = segment_of_block(segs, n_segs, [](const SortSeg& s) { return s.chunk0; });
   if (pass < 2 && S.nb[0] == 0) return;
-  const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
+  const int64_t i0 = (int64_t)((int)blockIdx.x - S.chunk0) * kSortChunk;
   const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
   for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
     int rank = 0;
@@ -356,12 +367,11 @@ __global__ void sort_count_kernel(const SortSeg* segs, int pass, const float4* _
 // most a few MB from L2 in 16-byte loads, cheaper than a second launch or a wait
 // on the blocks before it (a single block per segment took 0.42 ms at 2^18
 // counters, one tenth of what the whole frame's other preparation took).
-constexpr int kScanTile = 4096;
-__global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, int pass,
+__global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, int n_segs, int pass,
                                                          const uint32_t* __restrict__ counts,
                                                          uint32_t* __restrict__ cursors) {
-  const SortSeg S = segs[blockIdx.y];
-  const int m = (int)sort_keys(S, pass), t0 = blockIdx.x * kScanTile;
+  const SortSeg S = segment_of_block(segs, n_segs, [pass](const SortSeg& s) { return s.tile0[pass]; });
+  const int m = (int)sort_keys(S, pass), t0 = ((int)blockIdx.x - S.tile0[pass]) * kScanTile;
   if (t0 >= m) return;
   const uint32_t* c = counts + S.key0[pass];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -404,12 +414,12 @@ __global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, in
   }
 }
 
-__global__ void sort_scatter_kernel(const SortSeg* segs, const float4* __restrict__ src,
+__global__ void sort_scatter_kernel(const SortSeg* segs, int n_segs, const float4* __restrict__ src,
                                     const double4* __restrict__ src64, const int2* __restrict__ keys,
                                     const uint32_t* __restrict__ cursors, float4* dst, double4* dst64) {
-  const SortSeg S = segs[blockIdx.y];
+  const SortSeg S = segment_of_block(segs, n_segs, [](const SortSeg& s) { return s.chunk0; });
   const FrameDev& F = *S.fd;
-  const int64_t i0 = (int64_t)blockIdx.x * kSortChunk;
+  const int64_t i0 = (int64_t)((int)blockIdx.x - S.chunk0) * kSortChunk;
   const int64_t i1 = min((int64_t)S.n, i0 + kSortChunk);
   for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
     const int2 k = keys[S.x0 + i];
@@ -446,9 +456,9 @@ __device__ __forceinline__ void run_bounds(const FrameDev& F, const SortSeg& S, 
     F.bnd[2 * (S.run0 + run) + 1] = make_float4(b[3], b[4], b[5], 0.0f);
   }
 }
-__global__ void run_bounds_kernel(const SortSeg* segs) {
-  const SortSeg S = segs[blockIdx.y];
-  const int run = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+__global__ void run_bounds_kernel(const SortSeg* segs, int n_segs) {
+  const SortSeg S = segment_of_block(segs, n_segs, [](const SortSeg& s) { return s.bblock0; });
+  const int run = ((int)blockIdx.x - S.bblock0) * kBoundRuns + threadIdx.x / 32;
   if (S.fd->bnd && run * (int64_t)kRun < S.n) run_bounds(*S.fd, S, run, threadIdx.x & 31);
 }
 
@@ -2505,18 +2515,16 @@ cudaError_t launch_spatial_sort(const SortSeg* segs, int n_segs, const SortPlan&
                                 const double4* src64, double4* dst64, int2* keys, uint32_t* counts,
                                 cudaStream_t stream) {
   clear_stale_error();
-  if (n_segs <= 0 || plan.max_n <= 0) return cudaSuccess;
+  if (n_segs <= 0 || plan.chunks <= 0) return cudaSuccess;
   uint32_t* const cursors = counts + plan.keys;
-  const dim3 grid((unsigned)((plan.max_n + kSortChunk - 1) / kSortChunk), (unsigned)n_segs);
+  const unsigned chunks = (unsigned)plan.chunks;
   for (int pass = 0; pass < 3; ++pass) {
-    if (plan.max_keys[pass] == 0) continue;
-    sort_count_kernel<<<grid, 256, 0, stream>>>(segs, pass, src, keys, counts, cursors);
-    const dim3 sgrid((unsigned)((plan.max_keys[pass] + kScanTile - 1) / kScanTile), (unsigned)n_segs);
-    sort_scan_kernel<<<sgrid, 1024, 0, stream>>>(segs, pass, counts, cursors);
+    if (plan.tiles[pass] == 0) continue;
+    sort_count_kernel<<<chunks, 256, 0, stream>>>(segs, n_segs, pass, src, keys, counts, cursors);
+    sort_scan_kernel<<<(unsigned)plan.tiles[pass], 1024, 0, stream>>>(segs, n_segs, pass, counts, cursors);
   }
-  sort_scatter_kernel<<<grid, 256, 0, stream>>>(segs, src, src64, keys, cursors, dst, dst64);
-  const dim3 bgrid((unsigned)((plan.max_n + 8 * kRun - 1) / (8 * kRun)), (unsigned)n_segs);
-  run_bounds_kernel<<<bgrid, 256, 0, stream>>>(segs);
+  sort_scatter_kernel<<<chunks, 256, 0, stream>>>(segs, n_segs, src, src64, keys, cursors, dst, dst64);
+  run_bounds_kernel<<<(unsigned)plan.bblocks, 32 * kBoundRuns, 0, stream>>>(segs, n_segs);
   return cudaGetLastError();
 }
 

@@ -386,7 +386,6 @@ std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, bool list, const
       plan_strips(g, na, pf.variant == V_NONE ? cube : box);
     else
       g.g = sort_grid_bits(na);
-    plan->max_n = std::max<int64_t>(plan->max_n, na);
     out.push_back(g);
   }
   // a frame's counters: pass by pass, species after species
@@ -397,6 +396,7 @@ std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, bool list, const
       plan->keys += m;
       plan->max_keys[p] = std::max(plan->max_keys[p], m);
     }
+  number_sort_blocks(out.data(), out.size(), *plan);
   return out;
 }
 
@@ -709,6 +709,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
       P.prep = P.prep && on_list(f) && xoff[f + 1] - xoff[f] <= kPrepBestN && prep_fits(xoff[f + 1] - xoff[f], fp.keys);
     }
     P.n_sort = (int)sorts.size();
+    number_sort_blocks(sorts.data(), sorts.size(), P.sort);
     P.sort_particles = xoff[k];
   };
   DH_CUDA_TRY(c->meta.ensure(sizeof(FrameDev) * (size_t)k + sizeof(StageJob) * (size_t)k));
