@@ -508,11 +508,23 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
     far = fmax(far, Xm[c]);
   }
   if (F.variant != V_NONE) {
+    // What the span may be off by, in cells: binary64 input was rounded to float32 at both
+    // ends, and the fractional coordinates of a triclinic cell come from a chain of less
+    // than 14 roundings of magnitudes up to the coordinates'.
+    double off[3] = {0.0, 0.0, 0.0};
+    if (F.X64 || F.variant != V_ORTHO) {
+      const double per = F.variant != V_ORTHO ? 32.0 * u : 0.0;
+      double e[3];
+      for (int c = 0; c < 3; ++c) e[c] = per * Xm[c] + (F.X64 ? 2.0 * half_ulp_below(Xm[c]) : 0.0);
+      off[2] = e[2] * (double)F.invf[2];
+      off[1] = (e[1] + fabs(B[5]) * off[2]) * (double)F.invf[1];
+      off[0] = (e[0] + fabs(B[1]) * off[1] + fabs(B[2]) * off[2]) * (double)F.invf[0];
+    }
     for (int c = 0; c < 3; ++c) {
       const double span = F.variant != V_ORTHO ? (double)float_of_ord(F.smax[c]) - (double)float_of_ord(F.smin[c])
                                                : R[c] * (double)F.invf[c];
       // with the search, the nearest image can differ by nearly a cell more (check_frame)
-      if (span > 1.0 + (F.variant == V_TRIC_SEARCH ? 1.0 / 16384.0 : 1.0 / 16.0)) wrap = 1;
+      if (!(span + off[c] <= 1.0 + (F.variant == V_TRIC_SEARCH ? 1.0 / 16384.0 : 1.0 / 16.0))) wrap = 1;
     }
     if (wrap) {  // the home cell's bounding box
       ext[0] = B[0] + fabs(B[1]) + fabs(B[2]);
