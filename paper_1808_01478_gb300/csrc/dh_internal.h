@@ -123,7 +123,7 @@ struct Segment {
 
 // The same for the list kernel: one species pair of one frame and one bin
 // sweep as items of one run of kRun i particles against one run of j particles
-// (or a quarter of it, ListLaunch.split), numbered row by row over (i run, j
+// (or a part of it, split_log2), numbered row by row over (i run, j
 // run); intra-species: j runs not below the i run.  The i side is the larger
 // species.  Launch items [item0, item0 + items) are the segment's items from
 // item_base on.
@@ -133,6 +133,7 @@ struct ListSegment {
   int32_t n_ti, n_tj;      // runs of the i and the j species
   int32_t i0, ni, j0, nj;  // frame-local particle ranges
   int32_t i_run0, j_run0;  // their first runs in the frame's bounds
+  int32_t split_log2;      // log2 of the items per run pair (0 to 4: kRun >> split_log2 j particles each)
   int64_t item0, item_base, items;
 };
 
@@ -198,7 +199,8 @@ struct PairLaunch {
   int32_t agg;         // 256-thread blocks, one sweep: warp-aggregated histogram increments (match.any)
 };
 
-// Work counter of one segment of a list-kernel launch (zeroed before it).
+// Work counter of one shared segment of a list-kernel launch (zeroed before it), and
+// after those one for the launch's own segments (next: segments handed out).
 struct SegCounter {
   unsigned long long next;  // items claimed
   int32_t attached;         // blocks working on the segment
@@ -207,11 +209,13 @@ struct SegCounter {
 
 struct ListLaunch {
   const ListSegment* segs;
-  SegCounter* ctr;       // one per segment
+  SegCounter* ctr;       // one per shared segment, and one
   int32_t n_segs;
+  int32_t n_shared;      // the first n_shared segments are shared by blocks, each of the others
+                         // is one block's own (list_share_segments)
+  int32_t shared_blocks; // blocks that start on the shared ones
   int32_t hist_width;
-  int64_t n_items;
-  int32_t split;         // items per run pair (1 to 16, a power of two: kRun / split j particles each)
+  int64_t n_items, shared_items;
   int32_t multi;
   int32_t pick;          // frames whose pairs take the shortest of several images (FrameDev.pick)
 };

@@ -20,7 +20,10 @@
 //
 // Warps claim items of one segment (species pair and sweep) straight from its
 // counter; the warps of a block meet only when a segment is exhausted, to merge
-// their shared histogram.
+// their shared histogram.  Large segments are shared by blocks, small ones are one
+// block's own, handed out from one counter: with every block free to choose among all
+// segments, those of equal frames were started one after another (10,000 frames of 200
+// particles, three species: pair kernel 808 -> 4.2 ms, 2,000 of 2,000: 59 -> 4.1 ms).
 //
 // What bounds it: without a box the shared-memory pipe (one increment per pair at
 // 3.5 wavefronts on random banks, 90 % busy at N = 200,000), for periodic frames
@@ -107,6 +110,7 @@ struct SegState {
   const float4 *P4i, *P4j, *bi, *bj;  // positions and run bounds of the i and the j species
   const float2 *P2i, *P2j;
   int i0, j0, ni, nj, n_ti, n_tj, intra;
+  int split, split_log2, part;  // items per run pair, j particles of an item
   int lo, hi;             // the sweep's bins
   float rc_hi2, rc_lo2;   // images kept: nearest distance^2 <= rc_hi2, farthest^2 >= rc_lo2
   float in_hi2, in_lo2;   // every pair in the sweep: farthest^2 <= in_hi2, nearest^2 >= in_lo2
@@ -115,10 +119,20 @@ struct SegState {
   int n_img, all, slow;   // images of a particle; FrameDev list_all; 1: list_slow, 2: some runs are far (slow_item)
   int inner;              // FrameDev in_range: nearly every block is an inner one
   long long items, item_base;
-  long long claimers;     // claims that share the items left: kClaims per warp of the launch
+  long long claimers;     // claims that share the items left: kClaims per warp of the launch (or of the block)
   unsigned long long* next;
+  uint64_t* out;          // the sweep's bins of the species pair's histogram
   float4 V4[27];  // image vectors: high parts on the grid and the rest of x,
   float2 V2[27];  //   the rest of y and z
+};
+
+// What a block keeps between its segments, in shared memory.
+struct BlockState {
+  int seg, len;                  // the segment, and the warps' first claims
+  int next;                      // the segment to go on with, -1: none of its own left; known once asked
+  unsigned since, asked;
+  unsigned long long best, own;  // own: items claimed of a segment of its own
+  long long base, first, seen;   // first claim, items known to be claimed
 };
 
 // d + l as a double-float (d a multiple of the grid, |l| about a step at most).
@@ -655,8 +669,8 @@ __device__ __forceinline__ void merge_count(uint64_t* dst, uint32_t v) {
   if (v) atomicAdd((unsigned long long*)dst, (unsigned long long)(long long)(int32_t)v);
 }
 
-// One thread fills the block's segment state.
-__device__ void enter_segment(const ListSegment& S, SegCounter* ctr, SegState& G) {
+// One thread fills the block's segment state, but for the item counter.
+__device__ void enter_segment(const ListSegment& S, SegState& G) {
   FrameDev* const Fp = S.fd;
   const FrameDev& F = *Fp;
   G.F = Fp;
@@ -673,6 +687,9 @@ __device__ void enter_segment(const ListSegment& S, SegCounter* ctr, SegState& G
   G.n_ti = S.n_ti;
   G.n_tj = S.n_tj;
   G.intra = S.intra;
+  G.split_log2 = S.split_log2;
+  G.split = 1 << S.split_log2;
+  G.part = kRun >> S.split_log2;
   G.lo = S.pass * F.sweep_width;
   G.hi = min(F.nbins, G.lo + F.sweep_width);
   // widened (or narrowed) by 2^-15 and the absolute slack for the float32
@@ -696,16 +713,103 @@ __device__ void enter_segment(const ListSegment& S, SegCounter* ctr, SegState& G
   G.inner = F.in_range;
   G.items = (G.lo < F.nbins && !F.bad) ? S.items : 0;
   G.item_base = S.item_base;
-  G.next = &ctr->next;
-  G.claimers = kClaims * (kListBlock / 32) * (long long)gridDim.x;
+  G.out = F.out + (size_t)S.h * F.nbins + G.lo;
+}
+
+// The work distribution keeps its state in shared memory: whatever of it is in a register
+// across the pair loop is spilled there (as local variables 196 bytes of spills instead
+// of 132, and 1 % of every frame's time).
+
+// The next segment that is one block's own, -1 when all are handed out.
+__device__ __forceinline__ int own_segment(const ListLaunch& L) {
+  if (L.n_shared == L.n_segs) return -1;
+  const unsigned long long t = atomicAdd(&L.ctr[L.n_shared].next, 1ull);
+  return t < (unsigned long long)(L.n_segs - L.n_shared) ? L.n_shared + (int)t : -1;
+}
+
+// Some blocks start spread over the shared segments' items, the others with segments of
+// their own (one thread).
+__device__ __forceinline__ int first_segment(const ListLaunch& L) {
+  int own = -1;
+  if ((int)blockIdx.x >= L.shared_blocks) own = own_segment(L);
+  if (own >= 0 || L.n_shared == 0) return own;
+  const double part = (double)blockIdx.x / ((int)blockIdx.x < L.shared_blocks ? L.shared_blocks : (int)gridDim.x);
+  const long long pos = (long long)((double)L.shared_items * part);
+  int lo = 0, hi = L.n_shared - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (L.segs[mid].item0 <= pos) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// One thread attaches the block to segment B.seg and makes the first claim for all its
+// warps; claims shrink with the items left (a kClaims'th of an even share of them), at
+// first at most the block's share of the launch.
+__device__ __forceinline__ void attach_segment(const ListLaunch& L, BlockState& B, SegState& G) {
+  constexpr int kWarps = kListBlock / 32;
+  const int seg = B.seg;
+  const bool shared = seg < L.n_shared;
+  if (shared) atomicAdd(&L.ctr[seg].attached, 1);
+  enter_segment(L.segs[seg], G);
+  G.next = shared ? &L.ctr[seg].next : &B.own;
+  G.claimers = kClaims * kWarps * (shared ? (long long)gridDim.x : 1LL);
+  B.own = 0ull;
+  B.asked = 0u;
+  B.next = -1;
+  const long long part = max(1LL, min(G.items / G.claimers, 1024LL));
+  const long long share = max(1LL, (L.n_items + gridDim.x - 1) / (long long)gridDim.x);
+  const long long want = min(part * kWarps, share);
+  B.len = (int)part;
+  B.first = want;
+  B.base = G.items ? (long long)atomicAdd(G.next, (unsigned long long)want) : 0LL;
+  B.seen = B.base + want;
+  B.since = 0u;
+}
+
+// The block leaves its segment for B.next, or for the shared segment with the most work
+// left per block; of several, each block takes the first after its own place.
+__device__ __forceinline__ void next_segment(const ListLaunch& L, BlockState& B, const SegState& G, int tid, int lane) {
+  const int next = B.next;
+  if (tid == 0) {
+    const int seg = B.seg;
+    B.best = 0ull;
+    B.seg = next;
+    if (seg < L.n_shared) {
+      atomicAdd(&L.ctr[seg].attached, -1);
+      if (!G.items) L.ctr[seg].next = (unsigned long long)L.segs[seg].items;  // nothing to do for anyone
+    }
+  }
+  __syncthreads();
+  if (next >= 0) return;
+  const int place = (int)((long long)L.n_shared * blockIdx.x / gridDim.x);
+  unsigned long long best = 0ull;
+  for (int k = tid; k < L.n_shared; k += kListBlock) {
+    const int at = k + place < L.n_shared ? k + place : k + place - L.n_shared;
+    const unsigned long long nx = *(volatile unsigned long long*)&L.ctr[at].next;
+    const unsigned long long it = (unsigned long long)L.segs[at].items;
+    if (nx >= it) continue;
+    const int att = *(volatile int32_t*)&L.ctr[at].attached;
+    unsigned long long score = (it - nx) * 16ull / (unsigned long long)(1 + max(att, 0));
+    score = min(max(score, 1ull), (1ull << 40) - 1ull);
+    best = max(best, (score << 24) | (unsigned long long)(L.n_shared - 1 - k));
+  }
+  for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
+  if (lane == 0 && best) atomicMax(&B.best, best);
+  __syncthreads();
+  if (tid == 0 && B.best) {
+    const int at = L.n_shared - 1 - (int)(B.best & 0xFFFFFFull) + place;
+    B.seg = at < L.n_shared ? at : at - L.n_shared;
+  }
+  __syncthreads();
 }
 
 // Item -> (i run, j run, part).  Row a of a species with itself starts at item
 // a n - a (a - 1) / 2; the row is found from the root of that (the discriminant
 // is exact, its float32 root within a row of the truth).
-__device__ __forceinline__ void item_of(const SegState& G, int split, long long u, int& ri, int& rj, int& sub) {
-  const long long v = u + G.item_base, lid = v / split;
-  sub = (int)(v - lid * split);
+__device__ __forceinline__ void item_of(const SegState& G, long long u, int& ri, int& rj, int& sub) {
+  const long long v = u + G.item_base, lid = v >> G.split_log2;
+  sub = (int)v & (G.split - 1);
   if (G.intra) {
     const long long n = G.n_tj, t = 2 * n + 1;
     int a = (int)(0.5f * ((float)t - sqrtf((float)max(t * t - 8 * lid, 0LL))));
@@ -725,16 +829,13 @@ __device__ __forceinline__ void item_of(const SegState& G, int split, long long 
 // PICK: frames whose pairs take the shortest of several images (pick_round).
 // BLK: see kBlk (PICK: 64).
 template <bool MULTI, bool PICK, int BLK>
-__global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
+__global__ void __launch_bounds__(kListBlock, 1) list_kernel(const __grid_constant__ ListLaunch L) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int BLOCK = kListBlock, kWarps = BLOCK / 32, kCap = 2 * BLK;
   WarpList<BLK>* lists = reinterpret_cast<WarpList<BLK>*>(smem);
   PickList* picks = reinterpret_cast<PickList*>(smem + sizeof(WarpList<BLK>) * kWarps);
   uint32_t* sh = reinterpret_cast<uint32_t*>(picks + (PICK ? kWarps : 0)) + kGuard;
-  __shared__ int s_seg, s_len;
-  __shared__ unsigned s_since;
-  __shared__ unsigned long long s_best;
-  __shared__ long long s_base, s_first, s_seen;  // first claim, items known to be claimed
+  __shared__ BlockState B;
   __shared__ SegState G;
 
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -742,57 +843,32 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
   asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
   WarpList<BLK>& W = lists[warp];
   const unsigned lt_mask = (1u << lane) - 1u;
-  if (tid == 0) {
-    // blocks start spread over the launch's items
-    const long long pos = (long long)((double)L.n_items * ((double)blockIdx.x / (double)gridDim.x));
-    int lo = 0, hi = L.n_segs - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (L.segs[mid].item0 <= pos) lo = mid; else hi = mid - 1;
-    }
-    s_seg = lo;
-  }
+  if (tid == 0) B.seg = first_segment(L);
   for (int k = tid; k < L.hist_width + 2 * kGuard; k += BLOCK) sh[k - kGuard] = 0u;
   __syncthreads();
 
   for (;;) {
-    const int seg = s_seg;
-    if (seg < 0) break;
-    if (tid == 0) {
-      atomicAdd(&L.ctr[seg].attached, 1);
-      enter_segment(L.segs[seg], L.ctr + seg, G);
-      // the block's first claim, for all its warps; claims shrink with the items
-      // left (a quarter of an even share of them), at first at most the block's
-      // share of the launch
-      const long long part = max(1LL, min(G.items / G.claimers, 1024LL));
-      const long long share = max(1LL, (L.n_items + gridDim.x - 1) / (long long)gridDim.x);
-      const long long want = min(part * kWarps, share);
-      s_len = (int)part;
-      s_first = want;
-      s_base = G.items ? (long long)atomicAdd(G.next, (unsigned long long)want) : 0LL;
-      s_seen = s_base + want;
-      s_since = 0u;
-    }
+    if (B.seg < 0) break;
+    if (tid == 0) attach_segment(L, B, G);
     __syncthreads();
-    const FrameDev& F = *G.F;
     if (tid < 27) {
-      const Pos v = image_vector(F, tid, G.grid);
+      const Pos v = image_vector(*G.F, tid, G.grid);
       G.V4[tid] = make_float4(v.h.x, v.h.y, v.h.z, v.l.x);
       G.V2[tid] = make_float2(v.l.y, v.l.z);
     }
     __syncthreads();
     int qcount = 0;
     if (lane == 0) W.uni = W.axis = W.cull = 0ull;
-    long long u = s_base + (long long)warp * s_len;
-    int len = (int)min((long long)s_len, min(s_first - (long long)warp * s_len, G.items - u));
+    long long u = B.base + (long long)warp * B.len;
+    int len = (int)min((long long)B.len, min(B.first - (long long)warp * B.len, G.items - u));
 
     for (;;) {
       if (len <= 0) {
         if (lane == 0) {
-          const long long part = (G.items - *(volatile long long*)&s_seen) / G.claimers;
+          const long long part = (G.items - *(volatile long long*)&B.seen) / G.claimers;
           len = (int)max(1LL, min(part, 1024LL));
           u = G.items ? (long long)atomicAdd(G.next, (unsigned long long)len) : 0LL;
-          *(volatile long long*)&s_seen = u + len;
+          *(volatile long long*)&B.seen = u + len;
           len = (int)min((long long)len, G.items - u);
         }
         len = __shfl_sync(kFull, len, 0);
@@ -802,14 +878,14 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
 
       unsigned listed = 0;
       int ri, rj, sub;
-      item_of(G, L.split, u, ri, rj, sub);
+      item_of(G, u, ri, rj, sub);
 
       while (len > 0) {
-        const int row = min(len, (G.n_tj - rj) * L.split - sub);
+        const int row = min(len, (G.n_tj - rj) * G.split - sub);
         len -= row;
         // ---- the run: state and factors
         const int i_begin = ri * kRun, ni = min(kRun, G.ni - i_begin), nj = G.nj;
-        const int part = kRun / L.split;
+        const int part = G.part;
         IRegs I;
         int pf = rj * kRun + sub * part;
         float4 pa = __ldg(G.P4j + min(pf + lane, nj - 1));
@@ -984,7 +1060,7 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
               break;
             }
           }
-          if (++sub == L.split) {
+          if (++sub == G.split) {
             sub = 0;
             ++rj;
           }
@@ -997,13 +1073,14 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
       // flush before a shared count can pass 2^31: a warp that takes the total past a
       // multiple of kFlushPairs moves every word (the others keep counting)
       unsigned before = 0;
-      if (lane == 0) before = atomicAdd(&s_since, listed);
+      if (lane == 0) before = atomicAdd(&B.since, listed);
       before = __shfl_sync(kFull, before, 0);
       if ((before ^ (before + listed)) >= kFlushPairs) {
-        uint64_t* const dst = F.out + (size_t)L.segs[seg].h * F.nbins + G.lo;
-        for (int k = lane; k < G.hi - G.lo; k += 32) merge_count(dst + k, atomicExch(sh + k, 0u));
+        for (int k = lane; k < G.hi - G.lo; k += 32) merge_count(G.out + k, atomicExch(sh + k, 0u));
       }
     }
+    // the first warp without items asks for the block's next segment
+    if (lane == 0 && atomicExch(&B.asked, 1u) == 0u) B.next = own_segment(L);
     while (qcount > 0) qcount = list_drain(G, W.queue, qcount, sh, lane);
     if (lane == 0) {
       if (W.uni) atomicAdd(&G.F->uniform_pairs, W.uni);
@@ -1012,37 +1089,17 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(ListLaunch L) {
     }
 
     __syncthreads();
-    // ---- merge, then attach to the segment with the most work left per block
+    // ---- merge
     const int width = G.hi - G.lo;
     if (G.items) {
-      uint64_t* const dst = F.out + (size_t)L.segs[seg].h * F.nbins + G.lo;
+      uint64_t* const dst = G.out;
       for (int k = tid; k < width; k += BLOCK) {
         merge_count(dst + k, sh[k]);
         sh[k] = 0u;
       }
       for (int k = tid; k < 2 * kGuard; k += BLOCK) sh[k < kGuard ? k - kGuard : width + k - kGuard] = 0u;
     }
-    if (tid == 0) {
-      s_best = 0ull;
-      atomicAdd(&L.ctr[seg].attached, -1);
-      if (!G.items) L.ctr[seg].next = (unsigned long long)L.segs[seg].items;  // nothing to do for anyone
-    }
-    __syncthreads();
-    unsigned long long best = 0ull;
-    for (int k = tid; k < L.n_segs; k += BLOCK) {
-      const unsigned long long nx = *(volatile unsigned long long*)&L.ctr[k].next;
-      const unsigned long long it = (unsigned long long)L.segs[k].items;
-      if (nx >= it) continue;
-      const int att = *(volatile int32_t*)&L.ctr[k].attached;
-      unsigned long long score = (it - nx) * 16ull / (unsigned long long)(1 + max(att, 0));
-      score = min(max(score, 1ull), (1ull << 40) - 1ull);
-      best = max(best, (score << 24) | (unsigned long long)k);
-    }
-    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
-    if (lane == 0 && best) atomicMax(&s_best, best);
-    __syncthreads();
-    if (tid == 0) s_seg = s_best ? (int)(s_best & 0xFFFFFFull) : -1;
-    __syncthreads();
+    next_segment(L, B, G, tid, lane);
   }
 }
 

@@ -56,7 +56,8 @@ struct NaListPlan {
   std::vector<SortSeg> sorts;
   std::vector<ListSegment> segs;
   int64_t items = 0;
-  int split = 1, strips = 0;
+  int split = 1, strips = 0, grid = 0;
+  ListLaunch launch;
   size_t sort_at = 0, seg_at = 0, ctr_at = 0, T_at = 0, bnd_at = 0, P4_at = 0, P2_at = 0, X_at = 0, cells_at = 0;
 };
 
@@ -69,7 +70,10 @@ bool plan_list(const dh_frame* f, int max_width, int num_sms, unsigned char* bas
   p.strips = sort.max_keys[0] > 0;
   if (!prep_fits(f->n, sort.keys)) return false;
   p.split = list_split_for((double)p.pf.pairs / ((double)kRun * kRun) * p.pf.sweeps, num_sms);
-  p.items = add_list_segments(p.pf, fd, 0, p.segs, p.split);
+  p.items = add_list_segments(p.pf, fd, 0, p.segs, p.split, kListLeast);
+  p.grid = pair_grid(num_sms, 1, p.items);
+  std::memset(&p.launch, 0, sizeof p.launch);
+  list_share_segments(p.segs.data(), p.segs.size(), p.grid, p.launch);
   size_t at = kNaOffSegs;
   auto part = [&at](size_t bytes) {
     const size_t here = at;
@@ -78,7 +82,7 @@ bool plan_list(const dh_frame* f, int max_width, int num_sms, unsigned char* bas
   };
   p.sort_at = part(sizeof(SortSeg) * p.sorts.size());
   p.seg_at = part(sizeof(ListSegment) * p.segs.size());
-  p.ctr_at = part(sizeof(SegCounter) * p.segs.size());
+  p.ctr_at = part(sizeof(SegCounter) * ((size_t)p.launch.n_shared + 1));
   p.T_at = part(16 * ((size_t)f->nbins + 1));
   p.bnd_at = part(2 * sizeof(float4) * (size_t)frame_runs(f));
   p.P4_at = part(sizeof(float4) * (size_t)f->n);
@@ -197,17 +201,13 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   if (list) {
     DH_CUDA_TRY(launch_prep(job, 1, frame->n, lp.strips != 0, (const SortSeg*)(base + lp.sort_at), (uint32_t*)(base + lp.cells_at), st));
     if (lp.items > 0) {
-      ListLaunch L;
-      std::memset(&L, 0, sizeof L);
+      ListLaunch L = lp.launch;
       L.segs = (const ListSegment*)(base + lp.seg_at);
       L.ctr = (SegCounter*)(base + lp.ctr_at);
-      L.n_segs = (int32_t)lp.segs.size();
       L.hist_width = lp.pf.sweep_width;
-      L.n_items = lp.items;
-      L.split = lp.split;
       L.multi = lp.pf.sweeps > 1;
       L.pick = lp.pf.pick;
-      DH_CUDA_TRY(launch_list(L, pair_grid(num_sms, 1, lp.items), st));
+      DH_CUDA_TRY(launch_list(L, lp.grid, st));
     }
   } else {
     if (clear) DH_CUDA_TRY(cudaMemsetAsync(frame->out, 0, sizeof(uint64_t) * out_words, st));

@@ -469,7 +469,7 @@ int64_t add_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, std::v
 // One segment per species pair and sweep; the larger species is the i side (its
 // runs have the smaller bounds).  Items are numbered from item0.
 int64_t add_list_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, std::vector<ListSegment>& segs,
-                          int split) {
+                          int split, int least) {
   const dh_frame* f = pf.src;
   const int64_t* o = f->species_offsets;
   const int S = f->n_species;
@@ -498,12 +498,30 @@ int64_t add_list_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, s
         s.i_run0 = run0[i];
         s.j_run0 = run0[j];
         s.item0 = item0 + items;
-        s.items = split * (s.intra ? (int64_t)s.n_ti * (s.n_ti + 1) / 2 : (int64_t)s.n_ti * s.n_tj);
+        const int64_t run_pairs = s.intra ? (int64_t)s.n_ti * (s.n_ti + 1) / 2 : (int64_t)s.n_ti * s.n_tj;
+        while ((1 << s.split_log2) < split || (s.split_log2 < 4 && run_pairs << s.split_log2 < least)) ++s.split_log2;
+        s.items = run_pairs << s.split_log2;
         items += s.items;
         segs.push_back(s);
       }
   }
   return items;
+}
+
+void list_share_segments(ListSegment* segs, size_t n, int grid, ListLaunch& L) {
+  int64_t items = 0, shared = 0;
+  for (size_t q = 0; q < n; ++q) items += segs[q].items;
+  ListSegment* const own = std::stable_partition(
+      segs, segs + n, [&](const ListSegment& s) { return s.items * 32 * grid > items; });
+  for (ListSegment* s = segs; s != own; ++s) {
+    s->item0 = shared;
+    shared += s->items;
+  }
+  L.n_segs = (int32_t)n;
+  L.n_shared = (int32_t)(own - segs);
+  L.n_items = items;
+  L.shared_items = shared;
+  L.shared_blocks = shared == 0 ? 0 : std::max(1, (int)std::lround((double)grid * (double)shared / (double)items));
 }
 
 int list_split_for(double run_pairs, int num_sms) {
@@ -582,16 +600,17 @@ struct CallPlan {
   int launched = 0;
   size_t seg_bytes = 0;          // Segment array in the metadata
   size_t lseg_bytes = 0;         // ListSegment array after it,
-  size_t sort_bytes = 0;         // then the SortSeg array and a zeroed SegCounter per list segment
-  int n_lsegs = 0;
+  size_t sort_bytes = 0;         // then the SortSeg array and the zeroed SegCounters of the list launches
   // list-kernel launches: frames with one image of a pair inside r_max, and the
   // others (PlannedFrame.pick): first segment and segments, items, widest sweep,
   // some sweep above bin 0, blocks, items per run pair
   struct ListPlan {
-    int seg0 = 0, n_segs = 0;
+    int seg0 = 0, ctr0 = 0;
     int64_t items = 0;
     int width = 1, multi = 0, grid = 0, split = 1;
+    ListLaunch launch;
   } list[2];
+  int n_ctr = 0;                 // SegCounters of both
   bool prep = false;             // frames prepared by one launch (launch_prep)
   int n_sort = 0;                // spatial-order segments (after the segments in the metadata)
   SortPlan sort;                 // what they need
@@ -663,25 +682,29 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     segs.clear();
     lsegs.clear();
     P.n_items = 0;
+    P.n_ctr = 0;
     for (int g = 0; g < 2; ++g) {
       CallPlan::ListPlan& lp = P.list[g];
       lp.seg0 = (int)lsegs.size();
       lp.items = 0;
       for (int f = 0; f < k; ++f)
-        if (on_list(f) && (int)pfs[f].pick == g) lp.items += add_list_segments(pfs[f], dF + f, lp.items, lsegs, lp.split);
-      lp.n_segs = (int)lsegs.size() - lp.seg0;
+        if (on_list(f) && (int)pfs[f].pick == g) lp.items += add_list_segments(pfs[f], dF + f, lp.items, lsegs, lp.split, kListLeast);
+      const int n_segs = (int)lsegs.size() - lp.seg0;
       if (c->tune_forced && c->tune_cap_pairs > 0.0) {  // a measurement: the first items only
-        int64_t left = (int64_t)std::ceil(c->tune_cap_pairs / ((double)kRun * kRun)) * lp.split;
+        int64_t left = (int64_t)std::ceil(c->tune_cap_pairs / ((double)kRun * kRun));
         lp.items = 0;
-        for (int q = lp.seg0; q < lp.seg0 + lp.n_segs; ++q) {
-          lsegs[q].items = std::min(lsegs[q].items, left);
-          left -= lsegs[q].items;
+        for (int q = lp.seg0; q < lp.seg0 + n_segs; ++q) {
+          lsegs[q].items = std::min(lsegs[q].items, left << lsegs[q].split_log2);
+          left -= lsegs[q].items >> lsegs[q].split_log2;
           lp.items += lsegs[q].items;
         }
       }
+      std::memset(&lp.launch, 0, sizeof lp.launch);
+      list_share_segments(lsegs.data() + lp.seg0, (size_t)n_segs, pair_grid(c->num_sms, 1, lp.items), lp.launch);
+      lp.ctr0 = P.n_ctr;
+      P.n_ctr += lp.launch.n_shared + 1;
       P.n_items += lp.items;
     }
-    P.n_lsegs = (int)lsegs.size();
     for (int v = 0; v < kNumVariants; ++v) {
       P.vseg0[v] = segs.size();
       P.vitems[v] = 0;
@@ -719,7 +742,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   P.lseg_bytes = sizeof(ListSegment) * lsegs.size();
   P.sort_bytes = sizeof(SortSeg) * sorts.size();
   P.meta_bytes = sizeof(FrameDev) * (size_t)k + sizeof(StageJob) * (size_t)k + P.seg_bytes + P.lseg_bytes +
-                 P.sort_bytes + sizeof(SegCounter) * lsegs.size();
+                 P.sort_bytes + sizeof(SegCounter) * (size_t)P.n_ctr;
   void* before = c->meta.p;
   DH_CUDA_TRY(c->meta.ensure(P.meta_bytes));
   DH_CUDA_TRY(c->hmeta.ensure(P.meta_bytes));
@@ -781,7 +804,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   if (!lsegs.empty()) std::memcpy((unsigned char*)hS + P.seg_bytes, lsegs.data(), P.lseg_bytes);
   if (!sorts.empty())
     std::memcpy((unsigned char*)hS + P.seg_bytes + P.lseg_bytes, sorts.data(), sizeof(SortSeg) * sorts.size());
-  std::memset((unsigned char*)hS + P.seg_bytes + P.lseg_bytes + P.sort_bytes, 0, sizeof(SegCounter) * lsegs.size());
+  std::memset((unsigned char*)hS + P.seg_bytes + P.lseg_bytes + P.sort_bytes, 0, sizeof(SegCounter) * (size_t)P.n_ctr);
   // launch shapes (occupancy queries and kernel attributes stay outside any stream capture)
   for (int v = 0; v < kNumVariants; ++v) {
     P.vgrid[v] = 0;
@@ -865,14 +888,10 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
     for (int g = 0; g < 2; ++g) {
       const CallPlan::ListPlan& lp = P.list[g];
       if (lp.grid == 0) continue;
-      ListLaunch L;
-      std::memset(&L, 0, sizeof L);
+      ListLaunch L = lp.launch;
       L.segs = (const ListSegment*)((unsigned char*)dS + P.seg_bytes) + lp.seg0;
-      L.ctr = (SegCounter*)((unsigned char*)dSort + P.sort_bytes) + lp.seg0;
-      L.n_segs = lp.n_segs;
+      L.ctr = (SegCounter*)((unsigned char*)dSort + P.sort_bytes) + lp.ctr0;
       L.hist_width = lp.width;
-      L.n_items = lp.items;
-      L.split = lp.split;
       L.multi = lp.multi;
       L.pick = g;
       DH_CUDA_TRY(launch_list(L, lp.grid, st));

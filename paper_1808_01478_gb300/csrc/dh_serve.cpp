@@ -478,7 +478,7 @@ void Server::admit() {
     }
     r.segs.clear();
     r.lsegs.clear();
-    r.n_items = r.pf.list ? add_list_segments(r.pf, r.fd, 0, r.lsegs, 1) : add_segments(r.pf, r.fd, 0, r.segs);
+    r.n_items = r.pf.list ? add_list_segments(r.pf, r.fd, 0, r.lsegs, 1, 1) : add_segments(r.pf, r.fd, 0, r.segs);
     r.pairs_per_item = r.pf.list ? (double)kRun * kRun : (double)kTile * kTile;
     r.next = 0;
     r.state = Q_ACTIVE;
@@ -667,7 +667,15 @@ bool Server::launch_wave(int v) {
   for (int q = 0; q < kWidthClasses; ++q) nseg += csegs[q].size();
   for (const auto& l : lsegs) nlseg += l.size();
   const size_t bytes = sizeof(Segment) * nseg + sizeof(ListSegment) * nlseg;
-  const size_t ctl_bytes = sizeof(Control) * kWidthClasses + sizeof(SegCounter) * nlseg;
+  ListLaunch launches[2 * kWidthClasses];
+  std::memset(launches, 0, sizeof launches);
+  size_t nctr = 0;
+  for (int q = 0; q < 2 * kWidthClasses; ++q) {
+    if (lsegs[q].empty()) continue;
+    list_share_segments(lsegs[q].data(), lsegs[q].size(), pair_grid(ctx_->num_sms, 1, litems[q]), launches[q]);
+    nctr += (size_t)launches[q].n_shared + 1;
+  }
+  const size_t ctl_bytes = sizeof(Control) * kWidthClasses + sizeof(SegCounter) * nctr;
   if (W.segs.ensure(bytes) != cudaSuccess || W.hsegs.ensure(bytes) != cudaSuccess ||
       W.ctl.ensure(ctl_bytes) != cudaSuccess) {
     thread_error_ = "out of memory for wave descriptors";
@@ -689,20 +697,18 @@ bool Server::launch_wave(int v) {
   cudaEventRecord(W.ev0, ln.stream);
   cudaError_t e = cudaSuccess;
   at = 0;
+  SegCounter* ctr = (SegCounter*)((Control*)W.ctl.p + kWidthClasses);
   for (int q = 0; q < 2 * kWidthClasses && e == cudaSuccess; ++q) {
     if (lsegs[q].empty()) continue;
-    ListLaunch L;
-    std::memset(&L, 0, sizeof L);
+    ListLaunch L = launches[q];
     L.segs = (const ListSegment*)((const Segment*)W.segs.p + nseg) + at;
-    L.ctr = (SegCounter*)((Control*)W.ctl.p + kWidthClasses) + at;
-    L.n_segs = (int32_t)lsegs[q].size();
+    L.ctr = ctr;
     L.hist_width = lwidth[q];
-    L.n_items = litems[q];
-    L.split = 1;
     L.multi = lmulti[q];
     L.pick = q >= kWidthClasses;
     e = launch_list(L, pair_grid(ctx_->num_sms, 1, litems[q]), ln.stream);
     at += lsegs[q].size();
+    ctr += launches[q].n_shared + 1;
   }
   at = 0;
   for (int q = 0; q < kWidthClasses && e == cudaSuccess; ++q) {

@@ -40,3 +40,42 @@ def test_more_species_than_a_launch_dimension(torch_mod, oracle_mod, odd):
     assert np.array_equal(got[:, 0, 0], near) and np.array_equal(got[:, 0, 1], 3 - near)
     if odd != "none":
         assert np.array_equal(fas[frames // 2].out.cpu().numpy().view(np.uint64), want)
+
+
+@pytest.mark.parametrize("box", ["none", "ortho"])
+def test_segments_of_one_block_and_of_many(torch_mod, oracle_mod, box):
+    # 300 frames of three species, each species pair one block's own, and a frame whose
+    # species pairs are shared by blocks; the smallest have one particle a species
+    rng = w.rng_for(42)
+    frames = []
+    for k in range(300):
+        n = 20_000 if k == 170 else int(rng.integers(3, 700))
+        side = (n / 0.1) ** (1.0 / 3.0)
+        b = w.ortho_box(side)
+        kind, r = (w.BOX_NONE, 2.0 * side) if box == "none" else (w.BOX_ORTHO, 0.5 * side)
+        cuts = [0, n // 3, n // 2, n]
+        frames.append(w.frame_from((rng.random((n, 3)) * side).astype(np.float32), cuts, kind, b, r, 400, str(k)))
+    fas = [dh.FrameArgs(torch_mod.from_numpy(f.coords).cuda(), f.offsets, f.box_type, f.box, f.r_max, f.nbins)
+           for f in frames]
+    with dh.Context(0) as ctx:
+        ctx.histogram_batch(fas)
+    for fa, f in zip(fas, frames):
+        assert np.array_equal(fa.out.cpu().numpy().view(np.uint64), oracle_mod.histogram_frame(f)), f.name
+
+
+def test_time_of_a_batch_is_linear_in_its_frames(torch_mod):
+    # four times the frames take four times as long (2 at most for the rest), not sixteen
+    n, most = 600, 2000
+    x = torch_mod.from_numpy((w.rng_for(43).random((most, n, 3)) * 18.0).astype(np.float32)).cuda()
+    out = torch_mod.zeros((most, 6, 300), dtype=torch_mod.int64, device="cuda")
+    ms = {}
+    with dh.Context(0, flags=dh.DH_CFG_TIMING) as ctx:
+        for frames in (most // 4, most):
+            fas = [dh.FrameArgs(x[k], [0, 200, 400, n], w.BOX_NONE, None, 32.0, 300, out[k]) for k in range(frames)]
+            runs = []
+            for _ in range(4):
+                ctx.histogram_batch(fas)
+                runs.append(ctx.stats()["pair_kernel_ms"])
+            ms[frames] = min(runs)
+    assert int(out.sum()) == most * (n * (n - 1) // 2)
+    assert ms[most] < 8.0 * ms[most // 4], ms
