@@ -721,7 +721,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   auto plan_sorts = [&](FrameDev* dF) {
     sorts.clear();
     P.sort = SortPlan();
-    P.prep = with_pairs;
+    P.prep = with_pairs && xoff[k] > 0;
     for (int f = 0; f < k; ++f) {
       SortPlan fp;
       std::vector<SortSeg> fs = plan_spatial_order(pfs[f], on_list(f), dF + f, xoff[f], P.sort.keys, &fp);
@@ -729,7 +729,8 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
       P.sort.add(fp);
       strips[f] = fp.max_keys[0] > 0;
       sort0[f + 1] = (int)sorts.size();
-      P.prep = P.prep && on_list(f) && xoff[f + 1] - xoff[f] <= kPrepBestN && prep_fits(xoff[f + 1] - xoff[f], fp.keys);
+      const int64_t n = pfs[f].src->n;
+      if (n > 0) P.prep = P.prep && on_list(f) && n <= kPrepBestN && prep_fits(n, fp.keys);
     }
     P.n_sort = (int)sorts.size();
     number_sort_blocks(sorts.data(), sorts.size(), P.sort);
@@ -852,7 +853,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   if (P.prep) {
     int64_t max_n = 0;
     for (auto& pf : pfs) max_n = std::max(max_n, pf.src->n);
-    DH_CUDA_TRY(launch_prep(dJ, k, max_n, P.sort.max_keys[0] > 0, dSort, (uint32_t*)c->sortC.p, st));
+    DH_CUDA_TRY(launch_prep(dJ, P.n_jobs, max_n, P.sort.max_keys[0] > 0, dSort, (uint32_t*)c->sortC.p, st));
     ++launched;
   } else {
     if (P.n_jobs > 0) {
@@ -1031,14 +1032,14 @@ dh_status run_frames(dh_ctx* c, const dh_frame* frames, int k, bool wait, bool u
   }
   if (s == DH_OK) {
     cudaError_t e = cudaSuccess;
-    if (P.prep) {
-      // cleared by the preparation
-    } else if (dev) {
-      for (int f = 0; f < k && e == cudaSuccess; ++f)
-        if (!(frames[f].flags & DH_ACCUMULATE))
-          e = cudaMemsetAsync(frames[f].out, 0, sizeof(uint64_t) * (hoff[f + 1] - hoff[f]), st);
-    } else {
+    if (!dev && !P.prep) {
       e = cudaMemsetAsync(c->hist.p, 0, sizeof(uint64_t) * hoff[k], st);
+    } else {
+      for (int f = 0; f < k && e == cudaSuccess; ++f) {
+        if (P.prep && frames[f].n > 0) continue;  // cleared by the preparation
+        if (!dev || !(frames[f].flags & DH_ACCUMULATE))
+          e = cudaMemsetAsync(dev_out[f], 0, sizeof(uint64_t) * (hoff[f + 1] - hoff[f]), st);
+      }
     }
     if (e != cudaSuccess) s = fail(DH_ERR_CUDA, "output memset: %s", cudaGetErrorString(e));
     if (s == DH_OK) s = record_frames(c, pfs, P);

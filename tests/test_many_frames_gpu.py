@@ -79,3 +79,45 @@ def test_time_of_a_batch_is_linear_in_its_frames(torch_mod):
             ms[frames] = min(runs)
     assert int(out.sum()) == most * (n * (n - 1) // 2)
     assert ms[most] < 8.0 * ms[most // 4], ms
+
+
+@pytest.mark.parametrize("where", ["device", "host"])
+def test_empty_frames_leave_the_preparation_of_the_others_alone(torch_mod, oracle_mod, where):
+    # the first, one between and the last frame empty: their outputs are cleared (or left, to
+    # be added to), the others are prepared in the one launch they take without them
+    rng = w.rng_for(44)
+    sizes = [0, 700, 0, 1300, 40, 0]
+    xs = [(rng.random((n, 3)) * 9.0).astype(np.float32) for n in sizes]
+    box = w.ortho_box(9.0)
+    offs = [np.array([0, n // 4, n]) for n in sizes]
+    want = [oracle_mod.histogram(x, o, w.BOX_ORTHO, box, 4.0, 90) for x, o in zip(xs, offs)]
+
+    def frames(accumulate, outs, which):
+        return [dh.FrameArgs(torch_mod.from_numpy(xs[k]).cuda() if where == "device" else xs[k], offs[k], w.BOX_ORTHO,
+                             box, 4.0, 90, outs[k], accumulate) for k in which]
+
+    def fresh():
+        if where == "device":
+            return [torch_mod.full((3, 90), 5, dtype=torch_mod.int64, device="cuda") for _ in sizes]
+        return [np.full((3, 90), 5, dtype=np.uint64) for _ in sizes]
+
+    def values(out):
+        return out.cpu().numpy().view(np.uint64) if where == "device" else out
+
+    full = [k for k, n in enumerate(sizes) if n]
+    with dh.Context(0) as ctx:
+        outs = fresh()
+        for _ in range(2):  # (the first call also builds the bin thresholds)
+            ctx.histogram_batch(frames(False, outs, full))
+        launches = ctx.stats()["kernel_launches"]
+        outs = fresh()
+        ctx.histogram_batch(frames(False, outs, range(len(sizes))))
+        assert ctx.stats()["kernel_launches"] == launches
+        for k, out in enumerate(outs):
+            assert np.array_equal(values(out), want[k]), k
+        ctx.histogram_batch(frames(True, outs, range(len(sizes))))
+        for k, out in enumerate(outs):
+            assert np.array_equal(values(out), 2 * want[k]), k
+        outs = fresh()
+        ctx.histogram_batch(frames(False, outs, [0, 2]))  # nothing but empty frames
+        assert not values(outs[0]).any() and not values(outs[2]).any()
