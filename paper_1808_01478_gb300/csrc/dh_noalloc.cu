@@ -172,6 +172,7 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   float4* X = (float4*)(base + (list ? lp.X_at : kNaOffX));
   const bool clear = !(frame->flags & DH_ACCUMULATE);
   const size_t out_words = (size_t)pf.n_hist * (size_t)frame->nbins;
+  const bool prep_clear = list && clear && (int64_t)out_words <= prep_clears(frame->n);
 
   // The descriptors, uploaded in one copy that has read them when it returns; what
   // must start at zero is part of it.
@@ -190,7 +191,7 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
     hF.P2 = (float2*)(base + lp.P2_at);
     hJ.n_sort = (int32_t)lp.sorts.size();
     hJ.strips = lp.strips;
-    hJ.clear = clear ? (int64_t)out_words : 0;
+    hJ.clear = prep_clear ? (int64_t)out_words : 0;
     std::memcpy(up.data() + lp.sort_at, lp.sorts.data(), sizeof(SortSeg) * lp.sorts.size());
     if (!lp.segs.empty()) std::memcpy(up.data() + lp.seg_at, lp.segs.data(), sizeof(ListSegment) * lp.segs.size());
   } else if (n_segs > 0) {
@@ -198,6 +199,7 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   }
   DH_CUDA_TRY(cudaMemcpyAsync(base, up.data(), up.size(), cudaMemcpyHostToDevice, st));
   DH_CUDA_TRY(launch_thresholds(frame->r_max, frame->nbins, T, &ctl->status, st));
+  if (clear && !prep_clear) DH_CUDA_TRY(cudaMemsetAsync(frame->out, 0, sizeof(uint64_t) * out_words, st));
   if (list) {
     DH_CUDA_TRY(launch_prep(job, 1, frame->n, lp.strips != 0, (const SortSeg*)(base + lp.sort_at), (uint32_t*)(base + lp.cells_at), st));
     if (lp.items > 0) {
@@ -210,7 +212,6 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
       DH_CUDA_TRY(launch_list(L, lp.grid, st));
     }
   } else {
-    if (clear) DH_CUDA_TRY(cudaMemsetAsync(frame->out, 0, sizeof(uint64_t) * out_words, st));
     int64_t chunks = (frame->n + kStageChunk - 1) / kStageChunk;
     if (chunks > 0) DH_CUDA_TRY(launch_stage(job, 1, chunks, st));
     DH_CUDA_TRY(launch_frame_setup(fd, 1, false, false, st));

@@ -612,6 +612,8 @@ struct CallPlan {
   } list[2];
   int n_ctr = 0;                 // SegCounters of both
   bool prep = false;             // frames prepared by one launch (launch_prep)
+  int64_t max_n = 0;             // particles of the largest
+  std::vector<char> cleared;     // per frame: its output is cleared by that launch
   int n_sort = 0;                // spatial-order segments (after the segments in the metadata)
   SortPlan sort;                 // what they need
   int64_t sort_particles = 0;    // particles of the frames (index space of keys and the scratch copy)
@@ -781,6 +783,9 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
   // A1 staging jobs
   P.n_jobs = 0;
   P.n_chunks = 0;
+  P.max_n = 0;
+  for (auto& pf : pfs) P.max_n = std::max(P.max_n, pf.src->n);
+  P.cleared.assign((size_t)k, 0);
   for (int f = 0; f < k; ++f) {
     const dh_frame* fr = pfs[f].src;
     if (fr->n == 0) continue;
@@ -797,7 +802,9 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     J.sort0 = sort0[f];
     J.n_sort = sort0[f + 1] - sort0[f];
     J.strips = strips[f];
-    J.clear = host_coords || !(fr->flags & DH_ACCUMULATE) ? (int64_t)pfs[f].n_hist * fr->nbins : 0;
+    const int64_t words = host_coords || !(fr->flags & DH_ACCUMULATE) ? (int64_t)pfs[f].n_hist * fr->nbins : 0;
+    P.cleared[f] = P.prep && words <= prep_clears(P.max_n);
+    J.clear = P.cleared[f] ? words : 0;
     J.chunk0 = (int32_t)P.n_chunks;
     P.n_chunks += (fr->n + kStageChunk - 1) / kStageChunk;
   }
@@ -851,9 +858,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   DH_CUDA_TRY(cudaMemcpyAsync(dF, c->hmeta.p, P.meta_bytes, cudaMemcpyHostToDevice, st));
   const SortSeg* dSort = (const SortSeg*)((unsigned char*)dS + P.seg_bytes + P.lseg_bytes);
   if (P.prep) {
-    int64_t max_n = 0;
-    for (auto& pf : pfs) max_n = std::max(max_n, pf.src->n);
-    DH_CUDA_TRY(launch_prep(dJ, P.n_jobs, max_n, P.sort.max_keys[0] > 0, dSort, (uint32_t*)c->sortC.p, st));
+    DH_CUDA_TRY(launch_prep(dJ, P.n_jobs, P.max_n, P.sort.max_keys[0] > 0, dSort, (uint32_t*)c->sortC.p, st));
     ++launched;
   } else {
     if (P.n_jobs > 0) {
@@ -1036,7 +1041,7 @@ dh_status run_frames(dh_ctx* c, const dh_frame* frames, int k, bool wait, bool u
       e = cudaMemsetAsync(c->hist.p, 0, sizeof(uint64_t) * hoff[k], st);
     } else {
       for (int f = 0; f < k && e == cudaSuccess; ++f) {
-        if (P.prep && frames[f].n > 0) continue;  // cleared by the preparation
+        if (P.cleared[f]) continue;
         if (!dev || !(frames[f].flags & DH_ACCUMULATE))
           e = cudaMemsetAsync(dev_out[f], 0, sizeof(uint64_t) * (hoff[f + 1] - hoff[f]), st);
       }

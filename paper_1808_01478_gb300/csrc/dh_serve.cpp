@@ -505,7 +505,8 @@ dh_status Server::prep(Request& r) {
   r.job_pin->dst = r.sorts.empty() || fused ? r.X : r.sort_X;
   r.job_pin->n_sort = (int32_t)r.sorts.size();
   r.job_pin->strips = r.sort.max_keys[0] > 0;
-  r.job_pin->clear = clear ? (int64_t)r.res_count : 0;
+  const bool prep_clear = fused && clear && (int64_t)r.res_count <= prep_clears(r.frame.n);
+  r.job_pin->clear = prep_clear ? (int64_t)r.res_count : 0;
   r.job_pin->fd = r.fd;
   r.job_pin->n = r.frame.n;
   r.job_pin->stride = r.stride;
@@ -520,10 +521,10 @@ dh_status Server::prep(Request& r) {
   if (!r.dev_ptrs && r.frame.n > 0)
     DH_CUDA_TRY(cudaMemcpyAsync(r.raw, r.raw_pin, 4 * (size_t)r.stride * (size_t)r.frame.n,
                                 cudaMemcpyHostToDevice, st));
+  if (clear && !prep_clear) DH_CUDA_TRY(cudaMemsetAsync(r.hist, 0, 8 * r.res_count, st));
   if (fused) {
     DH_CUDA_TRY(launch_prep(r.job_dev, 1, r.frame.n, r.sort.max_keys[0] > 0, r.sort_dev, r.sort_C, st));
   } else {
-    if (clear) DH_CUDA_TRY(cudaMemsetAsync(r.hist, 0, 8 * r.res_count, st));
     int64_t chunks = (r.frame.n + kStageChunk - 1) / kStageChunk;
     if (chunks > 0) DH_CUDA_TRY(launch_stage(r.job_dev, 1, chunks, st));
     DH_CUDA_TRY(launch_frame_setup(r.fd, 1, true, false, st));

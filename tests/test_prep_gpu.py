@@ -136,3 +136,25 @@ def test_served_request_without_room_for_the_order(torch_mod, box):
         with pytest.raises(dh.DHError) as e:
             c.submit(dh.FrameArgs(big, [0, 60_000], box_type, B, 5.0, nbins))
         assert e.value.status == dh.DH_ERR_NOMEM
+
+
+@pytest.mark.parametrize("species,nbins", [(1, 16384), (1, 16385), (3, 16384), (16, 2000)])
+@pytest.mark.parametrize("n", [90, 1100])
+def test_outputs_cleared_by_the_preparation_or_by_a_fill(torch_mod, oracle_mod, n, species, nbins):
+    # 16,384 words per block of the launch (one block for 90 particles, two for 1,100) and one more
+    x = (w.rng_for(92).random((n, 3)) * 8.0).astype(np.float32)
+    offs = np.array([n * k // species for k in range(species + 1)], dtype=np.int64)
+    want = oracle_mod.histogram(x, offs, w.BOX_NONE, np.zeros(9), 14.0, nbins)
+    dev = torch_mod.from_numpy(x).cuda()
+    with dh.Context(0, pool_bytes=256 << 20) as ctx:
+        for accumulate in (False, True):
+            fas = [dh.FrameArgs(dev, offs, w.BOX_NONE, None, 14.0, nbins,
+                                torch_mod.full(want.shape, 3, dtype=torch_mod.int64, device="cuda"), accumulate)
+                   for _ in range(5)]
+            ctx.histogram(dev, offs, w.BOX_NONE, None, 14.0, nbins, fas[0].out, accumulate=accumulate)
+            ctx.histogram_batch(fas[1:3])
+            assert ctx.wait(ctx.submit(fas[3])) == dh.DH_OK
+            dh.dh_histogram_noalloc(fas[4].frame)
+            for k, fa in enumerate(fas):
+                assert np.array_equal(fa.out.cpu().numpy().view(np.uint64), want + (3 if accumulate else 0)), (k, accumulate)
+        assert np.array_equal(ctx.histogram(x, offs, w.BOX_NONE, None, 14.0, nbins), want)  # host arrays
