@@ -87,6 +87,7 @@ struct FrameDev {
   float2* P2;         //   the rest of y and z
   float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz; w of the
                       // first: 1 if some coordinate is beyond list_far)
+  const float4* staged;  // the coordinates before they are ordered (bulk_box; not in launch_prep)
   float S_l;          // nbins / r_max - S
   float img_h[27][3], img_l[27][3];  // image vectors -B k as double-floats (index as tshift)
   float period[3];    // a_x, b_y, c_z

@@ -545,8 +545,8 @@ __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {
   // of bins their finite range.  From 2^16 r_max on, where float32 coordinates are a
   // 256th of r_max apart, a run's pairs are compared in binary64 and the others' grid
   // does not reach; frames within 2^17 r_max, wherever they are, need none of this.
-  // One particle of N = 100,000 parked at 1e8: pair kernel 16.0 -> 5.6 ms; at 1e20, where
-  // every pair was replayed and many were lost, 200.8 -> 5.6 ms.
+  // One particle of N = 100,000 parked at 1e8: pair kernel 16.0 -> 4.2 ms; at 1e20, where
+  // every pair was replayed and many were lost, 200.8 -> 4.2 ms.
   F.list_far = INFINITY;
   if (F.variant == V_NONE && fmax(R[0], fmax(R[1], R[2])) > 131072.0 * F.r_max) {
     F.list_far = 65536.0f * (float)F.nbins;
@@ -792,6 +792,40 @@ __device__ __forceinline__ void frame_ranges(const FrameDev& F, double* R, doubl
   }
 }
 
+// The spatial order's box of a frame without a box whose range is far beyond r_max, by
+// one warp after list_setup, from the coordinates at x or x64.  A few particles far
+// away would put all the others into one cell, and runs without an order have large
+// bounds: windows as wide as the frame, no pairs left out (one particle of N = 100,000
+// at 1e5: pair kernel 4.6 ms, ordered 3.1 ms).  So the box holds the bulk: the third
+// smallest to the third largest of 32 particles, 30 % wider on each side.
+__device__ __noinline__ void bulk_box(FrameDev& F, int lane, const float* x, const double* x64, int stride) {
+  float lo[3], hi[3], range = 0.0f, side = 0.0f;
+  for (int c = 0; c < 3; ++c) range = fmaxf(range, float_of_ord(F.cmax[c]) - float_of_ord(F.cmin[c]));
+  if (!(range > 16.0f * F.rmax_f)) return;
+  const int i = (int)((int64_t)lane * (F.n - 1) / 31);
+  for (int c = 0; c < 3; ++c) {
+    const int64_t at = (int64_t)i * stride + c;
+    const float v = x64 ? __double2float_rn(x64[at]) : x[at];
+    int rank = 0;
+    for (int k = 0; k < 32; ++k) {
+      const float o = __shfl_sync(kFull, v, k);
+      rank += o < v || (o == v && k < lane);
+    }
+    const unsigned at_lo = __ballot_sync(kFull, rank == 2), at_hi = __ballot_sync(kFull, rank == 29);
+    lo[c] = __shfl_sync(kFull, v, (__ffs(at_lo) - 1) & 31);
+    hi[c] = __shfl_sync(kFull, v, (__ffs(at_hi) - 1) & 31);
+    const float more = 0.3f * (hi[c] - lo[c]);
+    lo[c] = fmaxf(lo[c] - more, float_of_ord(F.cmin[c]));
+    hi[c] = fminf(hi[c] + more, float_of_ord(F.cmax[c]));
+    side = fmaxf(side, hi[c] - lo[c]);
+  }
+  if (!(side > 0.0f && side < 0.5f * range)) return;
+  __syncwarp();
+  if (lane < 3) F.key_lo[lane] = lo[lane];
+  if (lane == 0) F.key_inv = 0.99999f / side;
+  __syncwarp();
+}
+
 // One block per frame: its descriptor in shared memory, where one thread's chain of
 // dependent accesses costs a tenth of what it does in global memory, and of the two
 // setups those that the frame needs: order (spatial order, list kernel) and the
@@ -809,6 +843,9 @@ __global__ void frame_setup_kernel(FrameDev* frames, int order, int windows) {
     if (order) list_setup(F, R, Xm);
     if (windows || !F.P4) window_setup(F, R, Xm);
   }
+  __syncwarp();
+  if (order && threadIdx.x < 32 && F.variant == V_NONE && F.n > kRun)
+    bulk_box(F, threadIdx.x, reinterpret_cast<const float*>(F.staged), nullptr, 4);
   __syncthreads();
   for (int k = threadIdx.x; k < (int)(sizeof(FrameDev) / 4); k += blockDim.x) dev[k] = own[k];
 }
@@ -933,6 +970,8 @@ __global__ void __launch_bounds__(kPrepBlock, 1)
     frame_ranges(F, R, Xm);
     list_setup(F, R, Xm);
   }
+  __syncwarp();
+  if (warp == 0 && F.variant == V_NONE && n > kRun) bulk_box(F, lane, J.src, src64, stride);
   __syncthreads();
   if (block == 0 && tid < fwords) reinterpret_cast<uint32_t*>(dev)[tid] = reinterpret_cast<const uint32_t*>(&F)[tid];
 

@@ -797,6 +797,7 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     const bool sorted = !P.prep && (pfs[f].variant != V_TRIC_SEARCH || pfs[f].list);
     J.dst = (float4*)(sorted ? c->sortX.p : c->X.p) + xoff[f];
     J.dst64 = (fr->flags & DH_COORDS_F64) ? (double4*)(sorted ? c->sortX64.p : c->X64.p) + xoff[f] : nullptr;
+    hF[f].staged = J.dst;
     J.fd = dF + f;
     J.n = fr->n;
     J.sort0 = sort0[f];

@@ -503,6 +503,7 @@ dh_status Server::prep(Request& r) {
   const bool clear = !r.dev_ptrs || !(r.frame.flags & DH_ACCUMULATE);
   const bool fused = r.pf.list && r.frame.n <= kPrepBestN && prep_fits(r.frame.n, r.sort.keys);
   r.job_pin->dst = r.sorts.empty() || fused ? r.X : r.sort_X;
+  r.fd_pin->staged = r.job_pin->dst;
   r.job_pin->n_sort = (int32_t)r.sorts.size();
   r.job_pin->strips = r.sort.max_keys[0] > 0;
   const bool prep_clear = fused && clear && (int64_t)r.res_count <= prep_clears(r.frame.n);

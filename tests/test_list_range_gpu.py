@@ -72,3 +72,36 @@ def test_a_box_far_longer_than_wide(torch_mod, oracle_mod):
     x = (w.rng_for(24).random((500, 3)) * 10.0).astype(np.float32)
     x[:, 0] = w.rng_for(25).choice(np.array([0.0, 1e24, 5e24, 9e24]), 500)
     check(torch_mod, oracle_mod, x, [0, 200, 500], w.BOX_ORTHO, box, 5.0, 300)
+
+
+@pytest.mark.parametrize("n,cuts", [(3000, []), (3000, [1000]), (40_000, [20_000]), (210_000, [])])
+def test_few_far_particles_leave_the_order_of_the_others(torch_mod, n, cuts):
+    # runs stay compact, so hardly more pairs are re-decided than without them: three far
+    # particles' runs with every other pair, and 3 times the rest
+    x = (w.rng_for(28).random((n, 3)) * 30.0).astype(np.float32)
+    far = x.copy()
+    far[[5, n // 2, n - 1], [0, 1, 2]] = (1e20, -7e4, 2e6)
+    offs = np.array([0, *cuts, n])
+    share = {}
+    with dh.Context(0) as ctx:
+        for name, y in (("near", x), ("far", far)):
+            ctx.histogram(torch_mod.from_numpy(y).cuda(), offs, w.BOX_NONE, None, 52.0, 5000)
+            st = ctx.stats()
+            share[name] = st["deferred"] / st["pairs"]
+    assert share["far"] < 3.0 * share["near"] + 3 * 128 / n * 2, share
+
+
+@pytest.mark.parametrize("nbins", [1, 700, 300_000])
+def test_pairs_of_a_far_particle_s_run(torch_mod, oracle_mod, nbins):
+    # decided in float32 where that is enough: lattice distances on the bin edges, particles
+    # in one place, and pairs beyond r_max among them
+    g = np.arange(9, dtype=np.float32) * 0.5
+    x = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3)
+    x = np.concatenate([x, x[::3], np.array([[1e12, 0, 0], [1e12, 0.5, 0], [0, -2e15, 1e9]], np.float32)])
+    x = x[w.rng_for(29).permutation(len(x))]
+    check(torch_mod, oracle_mod, x, [0, 300, len(x)], w.BOX_NONE, np.zeros(9), 3.5, min(nbins, 60_000))
+    if nbins > 60_000:  # (beyond the allocation-free limit)
+        want = oracle_mod.histogram(x, np.array([0, 300, len(x)]), w.BOX_NONE, np.zeros(9), 3.5, nbins)
+        with dh.Context(0) as ctx:
+            got = ctx.histogram(torch_mod.from_numpy(x).cuda(), [0, 300, len(x)], w.BOX_NONE, None, 3.5, nbins)
+        assert np.array_equal(got.cpu().numpy().view(np.uint64), want)
