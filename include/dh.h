@@ -224,7 +224,7 @@ dh_status dh_bin_thresholds(double r_max, int32_t nbins, double* thresholds);
  * that dh_create reads and the autotuner rewrites (DH_CFG_AUTOTUNE with
  * dh_config.tune_cache): lines starting with '#' are comments, every other line
  * is one launch key and its measured shape,
- *   sms variant width_log2 n_log2 frames_log4 tile_j block depth bps gpairs_s [agg]
+ *   sms variant width_log2 n_log2 frames_log4 tile_j block depth bps gpairs_s [agg [list]]
  * (variant: 0 none, 1 orthorhombic, 2 triclinic, 3 triclinic with the
  * 27-image search; width_log2 = ceil(log2 of the shared-memory histogram
  * width); n_log2 = round(log2 of the mean particles per frame); frames_log4 =
@@ -233,7 +233,11 @@ dh_status dh_bin_thresholds(double r_max, int32_t nbins, double* thresholds);
  * blocks per SM, >= 1 (at most what fits is used); gpairs_s > 0; agg, optional,
  * 1 for warp-aggregated histogram increments (match.any: the lanes of a warp
  * that hit one bin add their count once), only with 256-thread blocks and a
- * single bin sweep, else 0).  *n_entries receives the number
+ * single bin sweep, else 0; list, optional, 1 where the list kernel was the
+ * fastest, else the tiled shape is used.  Files whose first line is this
+ * library's but has no list column are from before that kernel: their lines are
+ * counted but not used, and replaced when the key is measured again).
+ * *n_entries receives the number
  * of distinct launch keys with a well-formed line for a GPU with sm_count SMs
  * (a later line replaces an earlier one of the same key); lines for other SM
  * counts and malformed lines are skipped.  DH_ERR_NOTFOUND if the file cannot

@@ -621,7 +621,7 @@ struct CallPlan {
 
 
 
-dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const std::vector<uint64_t*>& dev_out,
+dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::vector<uint64_t*>& dev_out,
                          bool host_coords, bool with_pairs, CallPlan& P) {
   cudaStream_t st = c->stream();
   int k = (int)pfs.size();
@@ -657,8 +657,14 @@ dh_status prepare_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const 
     vsum[v] = summarize(pfs, v);
     P.vparams[v] = launch_params(c, vsum[v], v);
   }
-  // frames the list kernel takes: those it can run, unless a measured shape says otherwise
-  auto on_list = [&](int f) { return pfs[f].list && P.vparams[pfs[f].variant].list; };
+  // frames the list kernel takes: those it can run, unless a measured shape says otherwise;
+  // the others' sweeps are planned anew, for the tiled kernel's histogram
+  for (int f = 0; f < k; ++f)
+    if (pfs[f].list && !P.vparams[pfs[f].variant].list) {
+      const dh_status s = check_frame(pfs[f].src, pfs[f], c->max_width, 0);
+      if (s != DH_OK) return s;
+    }
+  auto on_list = [&](int f) { return pfs[f].list; };
   double lrun_pairs[2] = {0.0, 0.0};
   for (int f = 0; f < k; ++f)
     if (on_list(f)) {
@@ -959,7 +965,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
   return DH_OK;
 }
 
-dh_status enqueue_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, const std::vector<uint64_t*>& dev_out,
+dh_status enqueue_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::vector<uint64_t*>& dev_out,
                          bool host_coords, bool with_pairs = true) {
   CallPlan P;
   dh_status s = prepare_frames(c, pfs, dev_out, host_coords, with_pairs, P);

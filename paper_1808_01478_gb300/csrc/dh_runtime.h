@@ -139,6 +139,7 @@ struct TuneKey {
 struct TuneEntry {
   LaunchParams p;
   double gpairs_s = 0.0;
+  bool old = false;  // measured before there was a list kernel to compare with: counted, but not used
 };
 TuneKey make_tune_key(int variant, int width, double mean_pairs_per_frame, int frames);
 

@@ -28,6 +28,15 @@ bool valid_shape(const LaunchParams& p) {
          (p.agg == 0 || (p.agg == 1 && p.block == kBlockSmall)) && (p.list == 0 || (p.list == 1 && !p.agg));
 }
 
+// First line of the files written here.  Without the last column a file is from before
+// the list kernel: its shapes were measured against each other only.  (Lines without that
+// column are as good as any in a file without such a first line: somebody's choice.)
+constexpr char kHeader[] = "# dh autotune cache:", kListColumn[] = " list";
+
+bool old_header(const char* line) {
+  return std::strncmp(line, kHeader, sizeof kHeader - 1) == 0 && !std::strstr(line, kListColumn);
+}
+
 // One cache line -> (sms, key, entry); false if malformed.
 bool parse_line(const char* line, int* sms, TuneKey* k, TuneEntry* e) {
   int tile_j = 0, agg = 0, list = 0;
@@ -64,7 +73,7 @@ TuneKey make_tune_key(int variant, int width, double mean_pairs_per_frame, int f
 bool Tuner::lookup(const TuneKey& k, LaunchParams* p) {
   std::lock_guard<std::mutex> g(mu_);
   auto it = map_.find(k);
-  if (it == map_.end()) return false;
+  if (it == map_.end() || it->second.old) return false;
   *p = it->second.p;
   return true;
 }
@@ -84,13 +93,18 @@ int Tuner::load(const std::string& path, int sms) {
   if (!fp) return -1;
   char line[512];
   int n = 0;
+  bool old = false;
   std::lock_guard<std::mutex> g(mu_);
   while (std::fgets(line, sizeof line, fp)) {
-    if (line[0] == '#') continue;
+    if (line[0] == '#') {
+      old = old || old_header(line);
+      continue;
+    }
     int s = 0;
     TuneKey k;
     TuneEntry e;
     if (!parse_line(line, &s, &k, &e) || s != sms) continue;
+    e.old = old;
     map_[k] = e;
     ++n;
   }
@@ -98,28 +112,31 @@ int Tuner::load(const std::string& path, int sms) {
   return n;
 }
 
-// Rewrites the file: entries of other SM counts already in it are kept.
+// Rewrites the file: entries of other SM counts already in it are kept, unless they are old.
 bool Tuner::save(const std::string& path, int sms) {
   std::string keep;
   if (FILE* fp = std::fopen(path.c_str(), "r")) {
     char line[512];
+    bool old = false;
     while (std::fgets(line, sizeof line, fp)) {
       int s = 0;
       TuneKey k;
       TuneEntry e;
-      if (line[0] != '#' && parse_line(line, &s, &k, &e) && s != sms) keep += line;
+      old = old || old_header(line);
+      if (line[0] != '#' && !old && parse_line(line, &s, &k, &e) && s != sms) keep += line;
     }
     std::fclose(fp);
   }
   std::string tmp = path + ".tmp";
   FILE* fp = std::fopen(tmp.c_str(), "w");
   if (!fp) return false;
-  std::fprintf(fp, "# dh autotune cache: sms variant width_log2 n_log2 frames_log4 tile_j block depth bps gpairs_s agg list\n");
+  std::fprintf(fp, "%s sms variant width_log2 n_log2 frames_log4 tile_j block depth bps gpairs_s agg%s\n", kHeader, kListColumn);
   std::fputs(keep.c_str(), fp);
   {
     std::lock_guard<std::mutex> g(mu_);
     for (const auto& kv : map_)
-      std::fprintf(fp, "%d %d %d %d %d %d %d %d %d %.3f %d %d\n", sms, kv.first.variant, kv.first.width_log2,
+      if (!kv.second.old)
+        std::fprintf(fp, "%d %d %d %d %d %d %d %d %d %.3f %d %d\n", sms, kv.first.variant, kv.first.width_log2,
                    kv.first.n_log2, kv.first.frames_log4, kTile / kv.second.p.jm, kv.second.p.block,
                    kv.second.p.depth, kv.second.p.bps, kv.second.gpairs_s, kv.second.p.agg, kv.second.p.list);
   }

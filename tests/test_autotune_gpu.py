@@ -164,3 +164,42 @@ def test_autotune_measures_once_and_reuses_the_file(torch_mod, oracle_mod, tmp_p
         assert (st["tile_j"], st["hist_depth"], st["blocks_per_sm"], st["block_threads"]) == shape
         for fa, fb in zip(fas, fas2):
             assert np.array_equal(result(fa), result(fb))
+
+
+def test_sweeps_of_a_tiled_shape_are_its_own(torch_mod, oracle_mod, tmp_path):
+    # 50,000 bins: one sweep of the tiled kernel, two of the list kernel
+    f = w.uniform_frame(38, 2500, w.BOX_ORTHO, w.ortho_box(30.0), 14.0, 50_000)
+    v, _, nl, f4 = tune_key([f])
+    path = tmp_path / "tune.txt"
+    write_cache(path, sm_count(torch_mod), [(v, wl, nl, f4) for wl in (15, 16)], 1024, 1, 1, 1024)
+    x = torch_mod.from_numpy(f.coords).cuda()
+    with dh.Context(0, tune_cache=str(path)) as ctx:
+        got = ctx.histogram(x, f.offsets, f.box_type, f.box, f.r_max, f.nbins).cpu().numpy().view(np.uint64)
+        st = ctx.stats()
+    assert st["block_threads"] == 1024 and st["sweeps"] == 1, st
+    assert np.array_equal(got, oracle_mod.histogram_frame(f))
+
+
+def test_cache_files_from_before_the_list_kernel_are_measured_again(torch_mod, tmp_path):
+    # a file this library wrote without the list column pins nobody to the shapes in it;
+    # the same lines without that first line are a choice
+    f = FRAMES["ortho_3species"]
+    sms = sm_count(torch_mod)
+    path = tmp_path / "tune.txt"
+    write_cache(path, sms, [tune_key([f])], 256, 4, 1, 256)
+    chosen = path.read_text()
+    old = "# dh autotune cache: sms variant width_log2 n_log2 frames_log4 tile_j block depth bps gpairs_s agg\n"
+    x = torch_mod.from_numpy(f.coords).cuda()
+    shapes = []
+    for text in (chosen, old + chosen):
+        path.write_text(text)
+        assert dh.dh_tune_cache_count(str(path), sms) == 1
+        with dh.Context(0, tune_cache=str(path)) as ctx:
+            ctx.histogram(x, f.offsets, f.box_type, f.box, f.r_max, f.nbins)
+            shapes.append((ctx.stats()["tile_j"], ctx.stats()["hist_depth"]))
+    assert shapes[0] == (256, 4) and shapes[1] != (256, 4), shapes
+    path.write_text(old + chosen)
+    with dh.Context(0, flags=dh.DH_CFG_AUTOTUNE, tune_cache=str(path)) as ctx:
+        ctx.histogram(x, f.offsets, f.box_type, f.box, f.r_max, f.nbins)
+        assert ctx.stats()["tune_runs"] > 1
+    assert path.read_text().splitlines()[0].endswith(" list") and dh.dh_tune_cache_count(str(path), sms) == 1
