@@ -87,6 +87,7 @@ struct FrameDev {
   float2* P2;         //   the rest of y and z
   float4* bnd;        // bounds of each run of kRun particles (two float4: min, max xyz; w of the
                       // first: 1 if some coordinate is beyond list_far)
+  int32_t clear;      // words of output to clear in frame_setup_kernel (at most kSetupClears)
   const float4* staged;  // the coordinates before they are ordered (bulk_box; not in launch_prep)
   float S_l;          // nbins / r_max - S
   float img_h[27][3], img_l[27][3];  // image vectors -B k as double-floats (index as tshift)
@@ -250,6 +251,7 @@ inline bool prep_fits(int64_t n, int64_t keys) {
 constexpr int64_t kPrepBestN = 32768;
 // order: the spatial order's grid and the list kernel's window too; windows: the tiled
 // kernel's window also for frames of the list kernel.
+constexpr int64_t kSetupClears = 65536;
 cudaError_t launch_frame_setup(FrameDev* frames, int n_frames, bool order, bool windows, cudaStream_t stream);
 // What a set of SortSeg needs.
 struct SortPlan {

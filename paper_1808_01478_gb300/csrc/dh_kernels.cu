@@ -843,6 +843,7 @@ __global__ void frame_setup_kernel(FrameDev* frames, int order, int windows) {
     if (order) list_setup(F, R, Xm);
     if (windows || !F.P4) window_setup(F, R, Xm);
   }
+  for (int k = threadIdx.x; k < F.clear; k += blockDim.x) F.out[k] = 0ull;
   __syncwarp();
   if (order && threadIdx.x < 32 && F.variant == V_NONE && F.n > kRun)
     bulk_box(F, threadIdx.x, reinterpret_cast<const float*>(F.staged), nullptr, 4);

@@ -365,8 +365,13 @@ std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, bool list, const
                                         SortPlan* plan) {
   std::vector<SortSeg> out;
   *plan = SortPlan();
-  if (pf.variant == V_TRIC_SEARCH && !pf.list) return out;
   const int64_t* o = pf.src->species_offsets;
+  // the tiled kernel's frames: not with the search, nor when every species is within two tiles
+  if (!list) {
+    int64_t most = 0;
+    for (int a = 0; a < pf.src->n_species; ++a) most = std::max(most, o[a + 1] - o[a]);
+    if (pf.variant == V_TRIC_SEARCH || most < kSortMinTiled) return out;
+  }
   const double* B = pf.src->box;
   const double cube[3] = {1.0, 1.0, 1.0}, box[3] = {B[0], B[4], B[8]};
   const bool strips = list && pf.src->n >= (pf.variant == V_NONE ? kStripMinNoBoxN : kStripMinN);
@@ -511,8 +516,9 @@ int64_t add_list_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, s
 void list_share_segments(ListSegment* segs, size_t n, int grid, ListLaunch& L) {
   int64_t items = 0, shared = 0;
   for (size_t q = 0; q < n; ++q) items += segs[q].items;
-  ListSegment* const own = std::stable_partition(
-      segs, segs + n, [&](const ListSegment& s) { return s.items * 32 * grid > items; });
+  auto is_shared = [&](const ListSegment& s) { return s.items * 32 * grid > items; };
+  ListSegment* own = std::find_if_not(segs, segs + n, is_shared);
+  if (own != segs + n) own = std::stable_partition(own, segs + n, is_shared);
   for (ListSegment* s = segs; s != own; ++s) {
     s->item0 = shared;
     shared += s->items;
@@ -522,6 +528,53 @@ void list_share_segments(ListSegment* segs, size_t n, int grid, ListLaunch& L) {
   L.n_items = items;
   L.shared_items = shared;
   L.shared_blocks = shared == 0 ? 0 : std::max(1, (int)std::lround((double)grid * (double)shared / (double)items));
+}
+
+FrameCost frame_cost(const PlannedFrame& pf, int num_sms) {
+  const dh_frame* f = pf.src;
+  const int64_t* o = f->species_offsets;
+  const int S = f->n_species;
+  const bool box = pf.variant != V_NONE;
+  const double rho = box ? f->r_max / std::cbrt(f->box[0] * f->box[4] * f->box[8]) : 0.0;
+  std::vector<double> images((size_t)S);  // with the species on the i side, and the padding of its runs
+  for (int a = 0; a < S; ++a) {
+    const double na = (double)(o[a + 1] - o[a]);
+    if (na == 0.0) continue;
+    const double side = na <= kRun ? 1.0 : std::cbrt(kRun / na);
+    const double v = side * side * (side + 6.0 * rho) + rho * rho * (9.42 * side + 4.19 * rho);
+    images[a] = (box ? std::min(27.0, v) * (pf.variant == V_ORTHO ? 1.0 : 1.25) : 1.0) * kRun * std::ceil(na / kRun) / na;
+  }
+  FrameCost t;
+  for (int a = 0; a < S; ++a)
+    for (int b = a; b < S; ++b) {
+      const double na = (double)(o[a + 1] - o[a]), nb = (double)(o[b + 1] - o[b]);
+      const double pairs = a == b ? 0.5 * na * (na - 1.0) : na * nb;
+      if (pairs == 0.0) continue;
+      const double ta = std::min(na, (double)kTile), tb = std::min(nb, (double)kTile);
+      t.list += (box ? 20.0 : 9.0) + 1.1e-4 * pairs * images[na >= nb ? a : b];
+      t.tiled += 2.5 + 1.25e-4 * (a == b ? 0.5 * na * (na + ta) : pairs);
+      t.tile = std::max(t.tile, 24.0 + 1.3e-4 * ta * tb);
+    }
+  t.list *= (double)pf.sweeps / num_sms;
+  t.tiled *= (double)pf.sweeps / num_sms;
+  return t;
+}
+
+bool choose_tiled(const std::vector<FrameCost>& costs, size_t others, std::vector<char>* tiled) {
+  double gain = 0.0, tile = 0.0;
+  size_t n = 0;
+  tiled->assign(costs.size(), 0);
+  for (size_t f = 0; f < costs.size(); ++f)
+    if (costs[f].tiled < 0.9 * costs[f].list) {
+      (*tiled)[f] = 1;
+      ++n;
+      gain += costs[f].list - costs[f].tiled;
+      tile = std::max(tile, costs[f].tile);
+    }
+  // 20 us for the window and the kernels in place of the one preparation launch; 26 us, the
+  // list kernel's shortest launch, are saved when no frame is left to it
+  const double cost = 20.0 + tile - (n == costs.size() && others == 0 ? 26.0 : 0.0);
+  return n > 0 && gain > 0.7 * cost;  // (few frames keep the list kernel's blocks less evenly busy)
 }
 
 int list_split_for(double run_pairs, int num_sms) {
@@ -569,10 +622,12 @@ TuneKey variant_key(const VariantSummary& s, int v) {
 // Launch shape for a variant: forced during a measurement, else the tuned
 // shape of its key, else one j tile per i tile, one histogram copy and as
 // many blocks per SM as fit.
-LaunchParams launch_params(dh_ctx* c, const VariantSummary& s, int v) {
+LaunchParams launch_params(dh_ctx* c, const VariantSummary& s, int v, bool* measured) {
+  *measured = true;
   if (c->tune_forced) return c->tune_force;
   LaunchParams p;
   if (c->tuner.lookup(variant_key(s, v), &p)) return p;
+  *measured = false;
   p.list = s.list;
   p.block = default_block(v, s.width);
   return p;
@@ -653,14 +708,38 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
   std::vector<Segment> segs;
   std::vector<ListSegment> lsegs;
   VariantSummary vsum[kNumVariants];
+  bool measured[kNumVariants];
   for (int v = 0; v < kNumVariants; ++v) {
     vsum[v] = summarize(pfs, v);
-    P.vparams[v] = launch_params(c, vsum[v], v);
+    P.vparams[v] = launch_params(c, vsum[v], v, &measured[v]);
   }
-  // frames the list kernel takes: those it can run, unless a measured shape says otherwise;
-  // the others' sweeps are planned anew, for the tiled kernel's histogram
+  // frames the list kernel takes: those it can run, unless a measured shape says otherwise
+  // or, without one, the tiled kernel is the faster (the shortest of several images is left
+  // to the list kernel: no estimate); the others' sweeps are planned anew, for the tiled
+  // kernel's histogram
+  std::vector<FrameCost> costs;
+  std::vector<int> choosing;
+  std::vector<char> tiled, to_tiled;
+  size_t others = 0;
+  // (no estimate where the list kernel's time cannot pay for the other's launch)
+  double most = 0.0;
+  for (const PlannedFrame& pf : pfs)
+    most += pf.sweeps * (20.0 * pf.n_hist + 1e-3 * (double)pf.pairs) / c->num_sms;
+  for (int f = 0; f < k && most > 12.0; ++f) {
+    if (pfs[f].src->n == 0) continue;
+    if (!pfs[f].list || pfs[f].pick || measured[pfs[f].variant]) {
+      ++others;
+      continue;
+    }
+    costs.push_back(frame_cost(pfs[f], c->num_sms));
+    choosing.push_back(f);
+  }
+  if (!costs.empty() && choose_tiled(costs, others, &tiled)) {
+    to_tiled.assign((size_t)k, 0);
+    for (size_t q = 0; q < choosing.size(); ++q) to_tiled[choosing[q]] = tiled[q];
+  }
   for (int f = 0; f < k; ++f)
-    if (pfs[f].list && !P.vparams[pfs[f].variant].list) {
+    if (pfs[f].list && (!P.vparams[pfs[f].variant].list || (!to_tiled.empty() && to_tiled[f]))) {
       const dh_status s = check_frame(pfs[f].src, pfs[f], c->max_width, 0);
       if (s != DH_OK) return s;
     }
@@ -800,7 +879,7 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
     J.stride = (fr->flags & DH_COORDS_F4) ? 4 : 3;
     J.src = host_coords ? (const float*)((const unsigned char*)c->raw.p + P.raw_off[f]) : fr->coords;
     // staged for the spatial order, or in place where there is none
-    const bool sorted = !P.prep && (pfs[f].variant != V_TRIC_SEARCH || pfs[f].list);
+    const bool sorted = !P.prep && sort0[f + 1] > sort0[f];
     J.dst = (float4*)(sorted ? c->sortX.p : c->X.p) + xoff[f];
     J.dst64 = (fr->flags & DH_COORDS_F64) ? (double4*)(sorted ? c->sortX64.p : c->X64.p) + xoff[f] : nullptr;
     hF[f].staged = J.dst;
@@ -812,6 +891,11 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
     const int64_t words = host_coords || !(fr->flags & DH_ACCUMULATE) ? (int64_t)pfs[f].n_hist * fr->nbins : 0;
     P.cleared[f] = P.prep && words <= prep_clears(P.max_n);
     J.clear = P.cleared[f] ? words : 0;
+    // (a fill costs the graph of a large batch 1 us each)
+    if (!P.prep && !host_coords && k >= 8 && words <= kSetupClears) {
+      hF[f].clear = (int32_t)words;
+      P.cleared[f] = 1;
+    }
     J.chunk0 = (int32_t)P.n_chunks;
     P.n_chunks += (fr->n + kStageChunk - 1) / kStageChunk;
   }

@@ -112,6 +112,28 @@ int64_t add_list_segments(const PlannedFrame& pf, FrameDev* fd, int64_t item0, s
 // 8.4 -> 8.6 ms, served requests of mixed sizes 6.03 -> 6.20 ms).
 void list_share_segments(ListSegment* segs, size_t n, int grid, ListLaunch& L);
 int64_t frame_runs(const dh_frame* f);  // runs of kRun particles over its species
+// Estimated time of a frame's species pairs in a launch that fills `num_sms` SMs, in
+// microseconds, on the list kernel and on the tiled kernel, and of the latter's longest item.
+//
+// The list kernel evaluates a particle's images against whole runs of 128, whose boxes are
+// large parts of the cell when a species is small: of the cell's volume, a box with sides f
+// widened by r_max = rho cells all around takes V = f^3 + 6 f^2 rho + 3 pi f rho^2 + 4/3 pi rho^3,
+// as many pairs per pair of particles (6.9 for species of one run and rho = 1/2; a quarter
+// more in a skewed cell).  The tiled
+// kernel evaluates every pair once, in whole tiles.  So a species pair takes
+//   list:  9 us (20 with a box) + 0.11 ns V per pair, padded to runs,
+//   tiled: 2.5 us + 0.125 ns per pair of its tiles; a tile 24 us + 0.13 ns per pair on its own,
+// fitted to calls of 1 to 3,000 frames of 100 to 12,000 particles in 1 to 100 species, of all
+// box types, which they meet within a third.  N = 1,500 in 8 species, orthorhombic, 1,777
+// frames: list 22.6 ms, tiled 4.4 ms; N = 6,000 in one species, 111 frames: 1.85 and 1.88 ms;
+// N = 12,000 in 3, 27 frames: 2.05 and 1.67 ms, with r_max a third of that half as much as tiled.
+struct FrameCost {
+  double list = 0.0, tiled = 0.0, tile = 0.0;
+};
+FrameCost frame_cost(const PlannedFrame& pf, int num_sms);
+// Marks the frames of a call for which the tiled kernel is worth its launch, its setup and
+// the wait for its last tile (costs: of the frames that may choose; n of all others).
+bool choose_tiled(const std::vector<FrameCost>& costs, size_t others, std::vector<char>* tiled);
 // Items per run pair: one item per warp where the frames are that small, else
 // enough for an even end.
 int list_split_for(double run_pairs, int num_sms);
@@ -149,7 +171,8 @@ size_t coord_bytes(const dh_frame* f);
 // Species are put in spatial order before the pair kernel, over the frame's
 // bounding box or its home cell (SortSeg).  plan_spatial_order lists the species of
 // one frame (its particles from x0 in the packed coordinates, its counters from
-// key0); frames of the search that are not for the list kernel keep their order.
+// key0); not for the list kernel, frames of the search and those of species below
+// kSortMinTiled keep their order.
 // list: the list kernel runs the frame, and its larger species are ordered in strips.
 std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, bool list, const FrameDev* fd, int64_t x0, int64_t key0,
                                         SortPlan* plan);
@@ -161,6 +184,7 @@ std::vector<SortSeg> plan_spatial_order(const PlannedFrame& pf, bool list, const
 // 190 against 191 orthorhombic, at N = 12,000 144 against 153.  Without a box nothing is
 // gained where r_max holds the whole frame: N = 60,000 1.01 against 1.03 ms, from
 // N = 200,000 on even.  Species of a few runs have nothing to gain either way.
+constexpr int64_t kSortMinTiled = 2048;
 constexpr int64_t kStripMinN = 16000, kStripMinNoBoxN = 200000, kStripMinSpecies = 2048;
 
 // Threads per block for a launch without a measured shape: from 16,384 bins on,

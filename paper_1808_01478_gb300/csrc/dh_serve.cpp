@@ -308,6 +308,12 @@ dh_status Server::submit(const dh_frame* f, uint64_t* ticket) {
     return fail(DH_ERR_INVALID, "the served path takes float32 coordinates (DH_COORDS_F64: use dh_histogram)");
   dh_status s = check_frame(&r->frame, r->pf, ctx_->max_width, ctx_->list_width);
   if (s != DH_OK) return s;
+  std::vector<char> tiled;
+  if (r->pf.list && !r->pf.pick && r->frame.n > 0 &&
+      choose_tiled({frame_cost(r->pf, ctx_->num_sms)}, 1, &tiled)) {  // (other requests share the waves)
+    s = check_frame(&r->frame, r->pf, ctx_->max_width, 0);
+    if (s != DH_OK) return s;
+  }
   r->pf.src = &r->frame;
   r->dev_ptrs = (f->flags & DH_DEVICE_PTRS) != 0;
   r->stride = (f->flags & DH_COORDS_F4) ? 4 : 3;

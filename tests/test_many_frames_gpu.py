@@ -121,3 +121,51 @@ def test_empty_frames_leave_the_preparation_of_the_others_alone(torch_mod, oracl
         outs = fresh()
         ctx.histogram_batch(frames(False, outs, [0, 2]))  # nothing but empty frames
         assert not values(outs[0]).any() and not values(outs[2]).any()
+
+
+@pytest.mark.parametrize("box", ["none", "ortho", "triclinic"])
+def test_small_species_go_to_the_tiled_kernel(torch_mod, oracle_mod, box):
+    # a batch of small frames of eight species (tiled, several to a launch), with one large frame
+    # (list kernel) and one beyond half the box among them; outputs overwritten and added to
+    rng = w.rng_for(45)
+    kinds = {"none": (w.BOX_NONE, lambda s: np.zeros(9)), "ortho": (w.BOX_ORTHO, lambda s: w.ortho_box(s, s, 1.2 * s)),
+             "triclinic": (w.BOX_TRICLINIC, lambda s: w.triclinic_box(s, s, s, *w.C3_ANGLES))}
+    kind, make = kinds[box]
+    frames = []
+    for k in range(120):
+        n, species = (30_000, 1) if k == 50 else (int(rng.integers(8, 900)), 8)
+        side = (n / 0.1) ** (1.0 / 3.0)
+        b = make(side)
+        m = np.eye(3) * side if box == "none" else w.box_matrix(b)
+        r = 1.8 * side if box == "none" else (1.5 if k == 51 else 0.95) * float(w.box_heights(b).min()) / 2.0
+        cuts = [n * q // species for q in range(species + 1)]
+        frames.append(w.frame_from((rng.random((n, 3)) @ m.T).astype(np.float32), cuts, kind, b, r, 300, str(k)))
+    fas = [dh.FrameArgs(torch_mod.from_numpy(f.coords).cuda(), f.offsets, f.box_type, f.box, f.r_max, f.nbins,
+                        torch_mod.full((f.n_hist, f.nbins), 3, dtype=torch_mod.int64, device="cuda")) for f in frames]
+    with dh.Context(0) as ctx:
+        for _ in range(2):
+            ctx.histogram_batch(fas)
+        assert ctx.stats()["block_threads"] == 256, ctx.stats()  # the tiled kernel's shape
+    for fa, f in zip(fas, frames):
+        assert np.array_equal(fa.out.cpu().numpy().view(np.uint64), oracle_mod.histogram_frame(f)), f.name
+
+
+@pytest.mark.parametrize("box", ["none", "ortho"])
+def test_one_frame_of_many_species(torch_mod, oracle_mod, box):
+    n, species = 2400, 60
+    x = (w.rng_for(46).random((n, 3)) * 28.0).astype(np.float32)
+    kind, b, r = (w.BOX_NONE, np.zeros(9), 50.0) if box == "none" else (w.BOX_ORTHO, w.ortho_box(28.0), 13.0)
+    offs = np.array([n * q // species for q in range(species + 1)], dtype=np.int64)
+    want = oracle_mod.histogram(x, offs, kind, b, r, 200)
+    dev = torch_mod.from_numpy(x).cuda()
+    with dh.Context(0, pool_bytes=256 << 20) as ctx:
+        got = ctx.histogram(dev, offs, kind, b, r, 200)
+        assert ctx.stats()["block_threads"] == 256, ctx.stats()
+        fa = dh.FrameArgs(dev, offs, kind, b, r, 200)
+        assert ctx.wait(ctx.submit(fa)) == dh.DH_OK
+    assert np.array_equal(got.cpu().numpy().view(np.uint64), want)
+    assert torch_mod.equal(fa.out, got)
+    few = np.array([n * q // 15 for q in range(16)], dtype=np.int64)  # the allocation-free entry's most
+    out = dh.FrameArgs(dev, few, kind, b, r, 200)
+    dh.dh_histogram_noalloc(out.frame)
+    assert np.array_equal(out.out.cpu().numpy().view(np.uint64), oracle_mod.histogram(x, few, kind, b, r, 200))
