@@ -638,7 +638,7 @@ LaunchParams launch_params(dh_ctx* c, const VariantSummary& s, int v, bool* meas
 // Nothing in it enqueues work except threshold tables that are not cached yet.
 struct CallPlan {
   int k = 0;
-  bool host_coords = false, with_pairs = true;
+  bool host_coords = false, with_pairs = true, async = false;
   size_t meta_bytes = 0;
   int n_jobs = 0;
   int64_t n_chunks = 0;
@@ -683,6 +683,11 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
   P.k = k;
   P.host_coords = host_coords;
   P.with_pairs = with_pairs;
+  if (c->async_in_flight) {  // (before a buffer grows, too)
+    DH_CUDA_TRY(cudaEventSynchronize(c->ev_meta));
+    DH_CUDA_TRY(cudaStreamWaitEvent(st, c->ev_async, 0));
+    c->async_in_flight = false;
+  }
   std::vector<int64_t> xoff(k + 1, 0);
   size_t raw_bytes = 0;
   P.raw_off.assign((size_t)k, 0);
@@ -947,6 +952,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
                                   cudaMemcpyHostToDevice, st));
     }
   DH_CUDA_TRY(cudaMemcpyAsync(dF, c->hmeta.p, P.meta_bytes, cudaMemcpyHostToDevice, st));
+  if (P.async) DH_CUDA_TRY(cudaEventRecord(c->ev_meta, st));
   const SortSeg* dSort = (const SortSeg*)((unsigned char*)dS + P.seg_bytes + P.lseg_bytes);
   if (P.prep) {
     DH_CUDA_TRY(launch_prep(dJ, P.n_jobs, P.max_n, P.sort.max_keys[0] > 0, dSort, (uint32_t*)c->sortC.p, st));
@@ -1121,6 +1127,7 @@ dh_status run_frames(dh_ctx* c, const dh_frame* frames, int k, bool wait, bool u
     for (int f = 0; f < k; ++f) dev_out[f] = (uint64_t*)c->hist.p + hoff[f];
   }
   CallPlan P;
+  P.async = !wait && dev;
   dh_status s = prepare_frames(c, pfs, dev_out, !dev, true, P);
   if (s == DH_OK && graph) {
     cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
@@ -1190,8 +1197,10 @@ dh_status run_frames(dh_ctx* c, const dh_frame* frames, int k, bool wait, bool u
         DH_CUDA_TRY(cudaMemcpyAsync(frames[f].out, dev_out[f], sizeof(uint64_t) * cnt, cudaMemcpyDeviceToHost, st));
     }
   }
-  if (!wait && dev) {
+  if (P.async) {
     c->pending_async = true;
+    DH_CUDA_TRY(cudaEventRecord(c->ev_async, st));
+    c->async_in_flight = true;
     return DH_OK;
   }
   s = finish_frames(c, k);
@@ -1500,6 +1509,8 @@ dh_status dh_create(const dh_config* config, dh_ctx** out) {
   c->max_width = pair_kernel_max_width();
   c->list_width = list_kernel_max_width();
   if (c->max_width < 1024) return fail(DH_ERR_CUDA, "not enough shared memory per block");
+  DH_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_meta, cudaEventDisableTiming));
+  DH_CUDA_TRY(cudaEventCreateWithFlags(&c->ev_async, cudaEventDisableTiming));
   DH_CUDA_TRY(c->ctl.ensure(sizeof(Control) * kNumVariants));
   DH_CUDA_TRY(c->tstat.ensure(64));
   DH_CUDA_TRY(cudaMemset(c->tstat.p, 0, sizeof(int32_t)));
@@ -1547,6 +1558,8 @@ dh_status dh_destroy(dh_ctx* c) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   if (c->ev_pair0) cudaEventDestroy(c->ev_pair0);
   if (c->ev_pair1) cudaEventDestroy(c->ev_pair1);
+  if (c->ev_meta) cudaEventDestroy(c->ev_meta);
+  if (c->ev_async) cudaEventDestroy(c->ev_async);
   if (c->own_stream) cudaStreamDestroy(c->own_stream);
   delete c;
   return DH_OK;

@@ -261,6 +261,10 @@ struct dh_ctx {
   cudaEvent_t ev_pair0 = nullptr, ev_pair1 = nullptr;  // pair-kernel timing (DH_CFG_TIMING)
   bool timed = false;
   bool pending_async = false;
+  // of the last asynchronous call: its descriptors are uploaded (the pinned copy may be
+  // written again), and all of it is done (the workspace may be used on another stream)
+  cudaEvent_t ev_meta = nullptr, ev_async = nullptr;
+  bool async_in_flight = false;
   cudaGraphExec_t gexec = nullptr;  // batched path: executable graph, updated per call
 
   std::mutex server_mu;
