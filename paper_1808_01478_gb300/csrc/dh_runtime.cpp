@@ -701,12 +701,7 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
   }
   DH_CUDA_TRY(c->X.ensure(sizeof(float4) * (size_t)std::max<int64_t>(xoff[k], 1)));
   if (P.any_f64) DH_CUDA_TRY(c->X64.ensure(sizeof(double4) * (size_t)std::max<int64_t>(xoff[k], 1)));
-  DH_CUDA_TRY(c->P4.ensure(sizeof(float4) * (size_t)std::max<int64_t>(xoff[k], 1)));
-  DH_CUDA_TRY(c->P2.ensure(sizeof(float2) * (size_t)std::max<int64_t>(xoff[k], 1)));
   if (host_coords) DH_CUDA_TRY(c->raw.ensure(std::max<size_t>(raw_bytes, 16)));
-  std::vector<int64_t> runs((size_t)k + 1, 0);
-  for (int f = 0; f < k; ++f) runs[f + 1] = runs[f] + frame_runs(pfs[f].src);
-  DH_CUDA_TRY(c->bnd.ensure(2 * sizeof(float4) * (size_t)std::max<int64_t>(runs[k], 1)));
   // device metadata: FrameDev[k] | StageJob[k] | Segment[m] | ListSegment[l] |
   // SortSeg[s] | SegCounter[l], uploaded in one copy; segments are grouped by minimum-image
   // variant (one pair-kernel launch each), those of the list kernel together
@@ -749,6 +744,15 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
       if (s != DH_OK) return s;
     }
   auto on_list = [&](int f) { return pfs[f].list; };
+  // positions and run bounds, for these frames only (24 of the 64 bytes a particle takes)
+  std::vector<int64_t> loff((size_t)k + 1, 0), runs((size_t)k + 1, 0);
+  for (int f = 0; f < k; ++f) {
+    loff[f + 1] = loff[f] + (on_list(f) ? pfs[f].src->n : 0);
+    runs[f + 1] = runs[f] + (on_list(f) ? frame_runs(pfs[f].src) : 0);
+  }
+  DH_CUDA_TRY(c->P4.ensure(sizeof(float4) * (size_t)loff[k]));
+  DH_CUDA_TRY(c->P2.ensure(sizeof(float2) * (size_t)loff[k]));
+  DH_CUDA_TRY(c->bnd.ensure(2 * sizeof(float4) * (size_t)runs[k]));
   double lrun_pairs[2] = {0.0, 0.0};
   for (int f = 0; f < k; ++f)
     if (on_list(f)) {
@@ -864,8 +868,8 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
     fill_frame_dev(pfs[f], hF[f], (const float4*)c->X.p + xoff[f], dev_out[f], T);
     if (pfs[f].src->flags & DH_COORDS_F64) hF[f].X64 = (const double4*)c->X64.p + xoff[f];
     if (on_list(f)) {
-      hF[f].P4 = (float4*)c->P4.p + xoff[f];
-      hF[f].P2 = (float2*)c->P2.p + xoff[f];
+      hF[f].P4 = (float4*)c->P4.p + loff[f];
+      hF[f].P2 = (float2*)c->P2.p + loff[f];
       hF[f].bnd = (float4*)c->bnd.p + 2 * runs[f];
     }
     P.max_pass = std::max(P.max_pass, pfs[f].sweeps);
