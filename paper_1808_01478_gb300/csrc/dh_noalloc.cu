@@ -20,6 +20,7 @@
 
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "dh_runtime.h"
@@ -123,7 +124,7 @@ dh_status scratch_for_current_device(unsigned char** out) {
 
 using namespace dh;
 
-extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_ptr) {
+static dh_status histogram_noalloc(const dh_frame* frame, void* stream_ptr) {
   if (!frame) return fail(DH_ERR_INVALID, "frame is NULL");
   if (!(frame->flags & DH_DEVICE_PTRS))
     return fail(DH_ERR_INVALID, "dh_histogram_noalloc needs DH_DEVICE_PTRS (device coords and out)");
@@ -237,4 +238,13 @@ extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_pt
   if (((const Control*)up.data())->status != 0) return fail(DH_ERR_CUDA, "bin threshold table did not converge");
   if (hF.bad) return fail(DH_ERR_INVALID, "frame has non-finite coordinates");
   return DH_OK;
+}
+
+// (the descriptors are kept in host vectors, all of them made before the first enqueued operation)
+extern "C" dh_status dh_histogram_noalloc(const dh_frame* frame, void* stream_ptr) {
+  try {
+    return histogram_noalloc(frame, stream_ptr);
+  } catch (const std::bad_alloc&) {
+    return DH_ERR_NOMEM;
+  }
 }
