@@ -363,10 +363,12 @@ __global__ void sort_count_kernel(const SortSeg* segs, int n_segs, int pass, con
 }
 
 // Exclusive prefix sum of each segment's counters (counts -> cursors), one block
-// per kScanTile of them.  A block sums the counters before its tile itself: at
-// most a few MB from L2 in 16-byte loads, cheaper than a second launch or a wait
-// on the blocks before it (a single block per segment took 0.42 ms at 2^18
-// counters, one tenth of what the whole frame's other preparation took).
+// per kScanTile of them.  A block sums the counters before its tile itself, from L2
+// in 16-byte loads: up to 6 MB at N = 1,000,000 (1.5 counters a particle, 1.1 GB over
+// all blocks), cheaper than a second launch or a wait on the blocks before it (a single
+// block per segment took 0.42 ms at 2^18 counters, one tenth of what the whole frame's
+// other preparation took).  The sum grows with the square of the counters: at N = 10^7
+// 60 MB a block and 110 GB over all of them, from where on a second level would pay.
 __global__ void __launch_bounds__(1024) sort_scan_kernel(const SortSeg* segs, int n_segs, int pass,
                                                          const uint32_t* __restrict__ counts,
                                                          uint32_t* __restrict__ cursors) {
@@ -493,7 +495,7 @@ __device__ __forceinline__ bool inside_one_sweep(const FrameDev& F, double D) {
 //   three FMAs, results below 2 TH + H^2    6u TH + 3u H^2
 //   last add                                u (T + H)^2
 // in all u (2 T^2 + 12 TH + 5 H^2) <= u ((2 + 6l) T^2 + (5 + 6/l) H^2) for any
-// l > 0 (run_window takes l = H over a typical T).  list_c0 covers what the
+// l > 0 (run_state takes l = H over a typical T).  list_c0 covers what the
 // double-floats leave out (a0: positions, 2^-47 each and per axis, the products
 // with S and the image vectors) and the binary64 definition's own rounding of t.
 __device__ void list_setup(FrameDev& F, const double* R, const double* Xm) {

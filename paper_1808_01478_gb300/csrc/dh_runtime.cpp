@@ -334,7 +334,7 @@ int sort_grid_bits(int64_t n) {
 
 // Slabs, columns and cells of the strip order of a species of n particles in a box
 // with sides L (any scale): runs of about equal sides, with 32 to 64 cells along each
-// (the blur of a run's ends), and at most 1.5 counters per particle.
+// (the blur of a run's ends), and at most 1.5 counters per particle and pass.
 void plan_strips(SortSeg& g, int64_t n, const double* L) {
   const double runs = (double)((n + kRun - 1) / kRun), side = std::cbrt(L[0] * L[1] * L[2] / runs);
   const double n_slab = std::min(runs, std::max(1.0, std::round(L[0] / side)));
@@ -349,8 +349,12 @@ void plan_strips(SortSeg& g, int64_t n, const double* L) {
   const double want = 32.0 * std::max(L[0], std::max(L[1], L[2])) / side;
   g.nb[2] = 32;
   while (g.nb[2] < 4096 && g.nb[2] < want && 2.0 * g.nb[2] <= most) g.nb[2] *= 2;
-  g.nb[1] = std::min(4 * g.nb[2], 4096);  // few slabs, few counters: more cells, not more increments of each
+  // few slabs, few counters: more cells, not more increments of each (but no more of them
+  // than that where there are few columns to a slab, as in a long box)
+  g.nb[1] = std::min(4 * g.nb[2], 4096);
+  while (g.nb[1] > 32 && (double)g.nb[1] * g.n_slab > 1.5 * (double)n) g.nb[1] /= 2;
   g.nb[0] = std::min(16 * g.nb[2], 8192);
+  while (g.nb[0] > 32 && (double)g.nb[0] > 1.5 * (double)n) g.nb[0] /= 2;
 }
 }  // namespace
 

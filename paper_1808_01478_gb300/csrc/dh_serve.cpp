@@ -39,7 +39,8 @@ using Clock = std::chrono::steady_clock;
 
 constexpr size_t kAlign = 256;
 constexpr int kWaveSlots = 4;          // waves that may be in flight at once
-// Histogram-width classes of a wave: one pair-kernel launch per class,
+// Histogram-width classes of a wave: one pair-kernel launch per class and kernel
+// (tiled, list, list with the shortest of several images),
 // ceil(log2 of the sweep width) up to 16 and one class above it.
 constexpr int kWidthClasses = 8;
 int width_class(int width) {
@@ -563,7 +564,7 @@ dh_status Server::finalize_enqueue(Request& r) {
 
 // One wave of lane v: the lane's pair budget over the running requests of that
 // variant, the least work left first (the order is stated below), as one
-// pair-kernel launch per histogram-width class.
+// pair-kernel launch per histogram-width class and kernel.
 bool Server::launch_wave(int v) {
   Lane& ln = lanes_[v];
   int slot = -1;
