@@ -254,6 +254,9 @@ dh_status dh_tune_cache_count(const char* path, int32_t sm_count, int32_t* n_ent
  *    binary64 (definition) and delta is the frame's decision window (must be
  *    < 1); out[1] = sampled pairs the float32 path would decide whose bin differs
  *    from the binary64 bin (must be 0); out[2] = pairs compared; out[3] = delta.
+ *    Frames that dh_histogram runs on the list kernel: the same for that kernel's
+ *    window (of the squared distance) and its double-float tier, on as many more
+ *    sampled pairs of the ordered species; out[0] the larger of the two ratios.
  *  what = DH_CHECK_TILES (orthorhombic or triclinic frames without search):
  *    stages `frame` and draws n_samples tiles with splitmix64 from `seed`, each
  *    a run of 128 consecutive particles against a run of 256 (the pair kernel's

@@ -293,6 +293,8 @@ cudaError_t launch_thresholds(double r_max, int32_t nbins, double* T, int32_t* s
 cudaError_t launch_pairs(const PairLaunch& p, int variant, int grid, size_t smem, cudaStream_t stream);
 // The list kernel (dh_list.cu): segments of any frames planned for it.
 cudaError_t launch_list(const ListLaunch& p, int grid, cudaStream_t stream);
+cudaError_t launch_check_list(const ListSegment* segs, int n_segs, uint64_t n_samples, uint64_t seed,
+                              unsigned long long* out, cudaStream_t stream);
 int list_kernel_max_width();  // widest sweep of the list kernel on the current device,
 constexpr int kPickWords = 12288;  //   less these bins for frames that need the shortest image
 cudaError_t launch_check_sqrt(unsigned long long* out, cudaStream_t stream);

@@ -1125,6 +1125,88 @@ __global__ void __launch_bounds__(kListBlock, 1) list_kernel(const __grid_consta
   }
 }
 
+// ------------------------------------------------------------------ self check
+
+// Sampled pairs of a frame (a block takes segment after segment of it) with the pair
+// loop's arithmetic for their shortest image, against the binary64 definition: out[0] =
+// largest |q - t64^2| / W over pairs inside the sweep (below 1), out[1] = pairs whose
+// bin, as decided in float32 or by the double-float tier, is another (0), out[2] = pairs.
+__device__ void check_listed_pair(const SegState& G, int i, int j, int lane, double* worst, unsigned long long* viol,
+                                  unsigned long long* checked) {
+  const FrameDev& F = *G.F;
+  const int m = F.variant == V_NONE ? kHome : picked_image(F, G.i0 + i, G.j0 + j);
+  if (m < 0) return;  // two images within rounding: re-decided in binary64
+  const RunState R = run_state(G, __ldg(G.bi + 2 * (i / kRun)), __ldg(G.bi + 2 * (i / kRun) + 1));
+  const float4 x = run_factor(G, i, i + 1, R.c);
+  const float4 y = j_image(unpack(__ldg(G.P4j + j), __ldg(G.P2j + j)), image_origin(G, m, R.c), R.c1, R.c0);
+  const float nq = __fadd_rn(__fmaf_rn(y.x, x.x, __fmaf_rn(y.y, x.y, __fmaf_rn(y.z, x.z, x.w))), y.w);
+  const float w2 = __fmaf_rn(y.w, -2.0f * R.c1 * (1.0f + 0x1p-10f), 2.0f * R.c0 * (1.0f + 0x1p-10f));
+  const double3 pi = coords64(F, G.i0 + i), pj = coords64(F, G.j0 + j);
+  const double r2 = F.variant == V_NONE    ? exact_r2<V_NONE>(F, pi, pj)
+                    : F.variant == V_ORTHO ? exact_r2<V_ORTHO>(F, pi, pj)
+                    : F.variant == V_TRIC ? exact_r2<V_TRIC>(F, pi, pj)
+                                          : exact_r2<V_TRIC_SEARCH>(F, pi, pj);
+  const int k64 = bin_from_thresholds(F.T, F.S, F.nbins, r2);
+  const double t64 = sqrt(r2) * ((double)F.nbins / F.r_max);
+  if (t64 >= (double)G.lo && t64 < (double)G.hi) {
+    *worst = fmax(*worst, fabs(0.5 * (double)w2 - (double)nq - t64 * t64) / (0.5 * (double)w2));
+    ++*checked;
+  }
+  float sc = fminf(sqrt_approx(-nq), (float)(G.hi + 1 + lane));
+  if (G.lo > 0) sc = fmaxf(sc, (float)(G.lo - lane));
+  const float sm = __fadd_rn(sc, kMagicRound), n = __fadd_rn(sm, -kMagicRound), e = __fmaf_rn(n, n, nq);
+  int bin;
+  if (G.all || -nq < (w2 + 1.0f) * (w2 + 1.0f) || __float_as_uint(e) < __float_as_uint(w2)) {
+    float edge;
+    unsigned nexact = 0;
+    bin = listed_bin(G, i, j, m, edge, nexact);
+  } else {
+    bin = G.lo + (__float_as_int(sm) + (int)(__float_as_uint(e) >> 31) - (__float_as_int(kMagicRound) + G.lo + 1));
+  }
+  const bool in = bin >= G.lo && bin < G.hi, in64 = k64 >= G.lo && k64 < G.hi;
+  if (in != in64 || (in && bin != k64)) ++*viol;
+}
+
+__global__ void check_list_kernel(const ListSegment* segs, int n_segs, uint64_t n_samples, uint64_t seed,
+                                  unsigned long long* out) {
+  __shared__ SegState G;
+  const int tid = threadIdx.x, lane = tid & 31;
+  double worst = 0.0;
+  unsigned long long viol = 0, checked = 0;
+  const uint64_t each = (n_samples + n_segs - 1) / n_segs;
+  for (int seg = 0; seg < n_segs; ++seg) {
+    __syncthreads();
+    if (tid == 0) enter_segment(segs[seg], G);
+    __syncthreads();
+    if (tid < 27) {
+      const Pos v = image_vector(*G.F, tid, G.grid);
+      G.V4[tid] = make_float4(v.h.x, v.h.y, v.h.z, v.l.x);
+      G.V2[tid] = make_float2(v.l.y, v.l.z);
+    }
+    __syncthreads();
+    if (G.slow || G.items == 0) continue;  // (binary64)
+    for (uint64_t s = blockIdx.x * (uint64_t)blockDim.x + tid; s < each; s += (uint64_t)gridDim.x * blockDim.x) {
+      uint64_t h = (seed + s + (uint64_t)seg * each) * 0x9E3779B97F4A7C15ull;
+      h = (h ^ (h >> 30)) * 0xBF58476D1CE4E5B9ull;
+      h = (h ^ (h >> 27)) * 0x94D049BB133111EBull;
+      h ^= h >> 31;
+      const int i = (int)(h % (uint64_t)G.ni), j = (int)((h >> 32) % (uint64_t)G.nj);
+      if (G.intra && i == j) continue;
+      check_listed_pair(G, i, j, lane, &worst, &viol, &checked);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    worst = fmax(worst, __shfl_xor_sync(kFull, worst, o));
+    viol += __shfl_xor_sync(kFull, viol, o);
+    checked += __shfl_xor_sync(kFull, checked, o);
+  }
+  if (lane == 0) {
+    atomicMax(out, (unsigned long long)__double_as_longlong(worst));
+    atomicAdd(out + 1, viol);
+    atomicAdd(out + 2, checked);
+  }
+}
+
 size_t smem_of(size_t list_bytes, int hist_width) {
   return list_bytes * (kListBlock / 32) + 4 * ((size_t)hist_width + 2 * kGuard);
 }
@@ -1152,6 +1234,14 @@ cudaError_t launch_list_t(const ListLaunch& p, int grid, cudaStream_t stream) {
 int list_kernel_max_width() {
   const size_t limit = smem_limit(), fixed = smem_of(sizeof(WarpList<kBlkNarrow>), 0);
   return limit <= fixed ? 0 : (int)((limit - fixed) / 4) & ~3;
+}
+
+cudaError_t launch_check_list(const ListSegment* segs, int n_segs, uint64_t n_samples, uint64_t seed,
+                              unsigned long long* out, cudaStream_t stream) {
+  (void)cudaGetLastError();
+  if (n_segs <= 0) return cudaSuccess;
+  check_list_kernel<<<1024, 256, 0, stream>>>(segs, n_segs, n_samples, seed, out);
+  return cudaGetLastError();
 }
 
 // Blocks of 64 images where the histogram leaves room for their lists, else of 32,

@@ -1064,8 +1064,7 @@ dh_status record_frames(dh_ctx* c, const std::vector<PlannedFrame>& pfs, CallPla
 }
 
 dh_status enqueue_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::vector<uint64_t*>& dev_out,
-                         bool host_coords, bool with_pairs = true) {
-  CallPlan P;
+                         bool host_coords, bool with_pairs, CallPlan& P) {
   dh_status s = prepare_frames(c, pfs, dev_out, host_coords, with_pairs, P);
   if (s != DH_OK) return s;
   return record_frames(c, pfs, P);
@@ -1435,13 +1434,20 @@ dh_status selfcheck(dh_ctx* c, int32_t what, const dh_frame* frame, uint64_t n_s
   DH_CUDA_TRY(c->hist.ensure(sizeof(uint64_t) * (size_t)pfs[0].n_hist * frame->nbins));
   dev_out[0] = (uint64_t*)c->hist.p;
   DH_CUDA_TRY(cudaMemsetAsync(c->tstat.p, 0, sizeof(int32_t), st));
-  s = enqueue_frames(c, pfs, dev_out, !dev, false);
+  CallPlan P;
+  s = enqueue_frames(c, pfs, dev_out, !dev, false, P);
   if (s == DH_OK) {
     cudaError_t e =
         what == DH_CHECK_TILES
             ? launch_check_tiles((const FrameDev*)c->meta.p, pfs[0].variant, n_samples, seed,
                                  (unsigned long long*)res.p, st)
             : launch_check_window((const FrameDev*)c->meta.p, n_samples, seed, (unsigned long long*)res.p, st);
+    // a frame of the list kernel: that kernel's window too
+    if (e == cudaSuccess && what == DH_CHECK_WINDOW && pfs[0].list) {
+      const Segment* dS = (const Segment*)((StageJob*)((FrameDev*)c->meta.p + 1) + 1);
+      e = launch_check_list((const ListSegment*)((const unsigned char*)dS + P.seg_bytes),
+                            (int)(P.lseg_bytes / sizeof(ListSegment)), n_samples, seed, (unsigned long long*)res.p, st);
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, res.p, sizeof h, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) s = fail(DH_ERR_CUDA, "self check: %s", cudaGetErrorString(e));
   }

@@ -100,3 +100,32 @@ def test_window_bound_holds_for_binary64_input(ctx, name):
     assert res["checked"] > 1 << 20
     assert res["violations"] == 0, res
     assert res["max_ratio"] < 1.0, res
+
+
+def test_window_check_covers_the_list_kernel(ctx):
+    # no box, every pair in range: as many pairs again as the tiled kernel's window is checked on
+    f = w.headline_frame(w.BOX_NONE, seed=18, n=50_000)
+    n_samples = 1 << 20
+    res = ctx.check_window(f.coords, f.offsets, f.box_type, f.box, f.r_max, f.nbins, n_samples=n_samples, seed=3)
+    assert res["checked"] > 1.9 * n_samples, res
+    assert res["violations"] == 0 and 0.01 < res["max_ratio"] < 1.0, res
+
+
+@pytest.mark.parametrize("name", ["ortho_beyond", "several_cells", "far", "one_bin"])
+def test_list_window_holds_at_its_edges(ctx, name):
+    rng = w.rng_for(19)
+    box = w.ortho_box(30.0, 26.0, 34.0)
+    x = rng.random((30_000, 3)) * np.array([30.0, 26.0, 34.0])
+    r_max, nbins = 12.9, 4000
+    if name == "ortho_beyond":
+        r_max = 19.0
+    elif name == "several_cells":
+        x = x + rng.integers(-40, 41, (30_000, 3)) * np.array([30.0, 26.0, 34.0])
+    elif name == "far":
+        x = x + 4000.0
+    else:
+        nbins = 1
+    res = ctx.check_window(x.astype(np.float32), [0, 9000, 30_000], w.BOX_ORTHO, box, r_max, nbins, n_samples=1 << 21,
+                           seed=4)
+    assert res["checked"] > 1 << 18
+    assert res["violations"] == 0 and res["max_ratio"] < 1.0, res
