@@ -66,7 +66,7 @@ struct NaListPlan {
 bool plan_list(const dh_frame* f, int max_width, int num_sms, unsigned char* base, NaListPlan& p) {
   if (check_frame(f, p.pf, max_width, list_kernel_max_width()) != DH_OK || !p.pf.list) return false;
   std::vector<char> tiled;
-  if (!p.pf.pick && choose_tiled({frame_cost(p.pf, num_sms)}, 0, &tiled)) return false;
+  if (may_be_tiled(p.pf) && choose_tiled({frame_cost(p.pf, num_sms)}, 0, &tiled)) return false;
   FrameDev* fd = (FrameDev*)(base + kNaOffFrame);
   SortPlan sort;
   p.sorts = plan_spatial_order(p.pf, true, fd, 0, 0, &sort);

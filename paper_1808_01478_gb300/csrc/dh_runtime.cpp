@@ -540,13 +540,15 @@ FrameCost frame_cost(const PlannedFrame& pf, int num_sms) {
   const int S = f->n_species;
   const bool box = pf.variant != V_NONE;
   const double rho = box ? f->r_max / std::cbrt(f->box[0] * f->box[4] * f->box[8]) : 0.0;
-  std::vector<double> images((size_t)S);  // with the species on the i side, and the padding of its runs
+  std::vector<double> per_pair((size_t)S);  // list kernel, with the species on the i side: us
   for (int a = 0; a < S; ++a) {
     const double na = (double)(o[a + 1] - o[a]);
     if (na == 0.0) continue;
     const double side = na <= kRun ? 1.0 : std::cbrt(kRun / na);
     const double v = side * side * (side + 6.0 * rho) + rho * rho * (9.42 * side + 4.19 * rho);
-    images[a] = (box ? std::min(27.0, v) * (pf.variant == V_ORTHO ? 1.0 : 1.25) : 1.0) * kRun * std::ceil(na / kRun) / na;
+    const double seen = pf.pick ? (0.1 + 2.4 * side) * std::min(1.0, v)
+                        : !box ? 0.11 : 0.11 * std::min(27.0, v) * (pf.variant == V_ORTHO ? 1.0 : 1.25);
+    per_pair[a] = 1e-3 * seen * kRun * std::ceil(na / kRun) / na;  // (padded to whole runs)
   }
   FrameCost t;
   for (int a = 0; a < S; ++a)
@@ -555,7 +557,7 @@ FrameCost frame_cost(const PlannedFrame& pf, int num_sms) {
       const double pairs = a == b ? 0.5 * na * (na - 1.0) : na * nb;
       if (pairs == 0.0) continue;
       const double ta = std::min(na, (double)kTile), tb = std::min(nb, (double)kTile);
-      t.list += (box ? 20.0 : 9.0) + 1.1e-4 * pairs * images[na >= nb ? a : b];
+      t.list += (box ? 20.0 : 9.0) + pairs * per_pair[na >= nb ? a : b];
       t.tiled += 2.5 + 1.25e-4 * (a == b ? 0.5 * na * (na + ta) : pairs);
       t.tile = std::max(t.tile, 24.0 + 1.3e-4 * ta * tb);
     }
@@ -718,9 +720,8 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
     P.vparams[v] = launch_params(c, vsum[v], v, &measured[v]);
   }
   // frames the list kernel takes: those it can run, unless a measured shape says otherwise
-  // or, without one, the tiled kernel is the faster (the shortest of several images is left
-  // to the list kernel: no estimate); the others' sweeps are planned anew, for the tiled
-  // kernel's histogram
+  // or, without one, the tiled kernel is the faster; the others' sweeps are planned anew,
+  // for the tiled kernel's histogram
   std::vector<FrameCost> costs;
   std::vector<int> choosing;
   std::vector<char> tiled, to_tiled;
@@ -728,10 +729,10 @@ dh_status prepare_frames(dh_ctx* c, std::vector<PlannedFrame>& pfs, const std::v
   // (no estimate where the list kernel's time cannot pay for the other's launch)
   double most = 0.0;
   for (const PlannedFrame& pf : pfs)
-    most += pf.sweeps * (20.0 * pf.n_hist + 1e-3 * (double)pf.pairs) / c->num_sms;
+    most += pf.sweeps * (20.0 * pf.n_hist + (pf.pick ? 3e-3 : 1e-3) * (double)pf.pairs) / c->num_sms;
   for (int f = 0; f < k && most > 12.0; ++f) {
     if (pfs[f].src->n == 0) continue;
-    if (!pfs[f].list || pfs[f].pick || measured[pfs[f].variant]) {
+    if (!may_be_tiled(pfs[f]) || measured[pfs[f].variant]) {
       ++others;
       continue;
     }

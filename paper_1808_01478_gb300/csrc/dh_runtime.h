@@ -122,8 +122,14 @@ int64_t frame_runs(const dh_frame* f);  // runs of kRun particles over its speci
 // more in a skewed cell).  The tiled
 // kernel evaluates every pair once, in whole tiles.  So a species pair takes
 //   list:  9 us (20 with a box) + 0.11 ns V per pair, padded to runs,
-//   tiled: 2.5 us + 0.125 ns per pair of its tiles; a tile 24 us + 0.13 ns per pair on its own,
-// fitted to calls of 1 to 3,000 frames of 100 to 12,000 particles in 1 to 100 species, of all
+//   tiled: 2.5 us + 0.125 ns per pair of its tiles; a tile 24 us + 0.13 ns per pair on its own.
+// Where the shortest of several images counts (PlannedFrame.pick), particles with more than
+// one candidate are evaluated image by image: 0.1 + 2.4 f ns per pair on the list kernel,
+// times V where r_max holds only a part of the cell.  Orthorhombic, r_max = 0.85 L,
+// N = 40,000: list 2.27 ms, tiled 0.66; N = 500,000: 185 and 69 ms; a rod of 1 : 1 : 50, N =
+// 200,000: 144 and 11.5 ms; N = 1,500: 43 and 160 us; r_max = 0.75 of the short side of a
+// 1 : 10 : 10 slab, N = 200,000: 2.2 and 2.6 ms.
+// All fitted to calls of 1 to 3,000 frames of 100 to 12,000 particles in 1 to 100 species, of all
 // box types, which they meet within a third.  N = 1,500 in 8 species, orthorhombic, 1,777
 // frames: list 22.6 ms, tiled 4.4 ms; N = 6,000 in one species, 111 frames: 1.85 and 1.88 ms;
 // N = 12,000 in 3, 27 frames: 2.05 and 1.67 ms, with r_max a third of that half as much as tiled.
@@ -131,6 +137,8 @@ struct FrameCost {
   double list = 0.0, tiled = 0.0, tile = 0.0;
 };
 FrameCost frame_cost(const PlannedFrame& pf, int num_sms);
+// Frames that may choose: the tiled kernel takes the 27-image search several times slower.
+inline bool may_be_tiled(const PlannedFrame& pf) { return pf.list && pf.variant != V_TRIC_SEARCH; }
 // Marks the frames of a call for which the tiled kernel is worth its launch, its setup and
 // the wait for its last tile (costs: of the frames that may choose; n of all others).
 bool choose_tiled(const std::vector<FrameCost>& costs, size_t others, std::vector<char>* tiled);

@@ -310,7 +310,7 @@ dh_status Server::submit(const dh_frame* f, uint64_t* ticket) {
   dh_status s = check_frame(&r->frame, r->pf, ctx_->max_width, ctx_->list_width);
   if (s != DH_OK) return s;
   std::vector<char> tiled;
-  if (r->pf.list && !r->pf.pick && r->frame.n > 0 &&
+  if (may_be_tiled(r->pf) && r->frame.n > 0 &&
       choose_tiled({frame_cost(r->pf, ctx_->num_sms)}, 1, &tiled)) {  // (other requests share the waves)
     s = check_frame(&r->frame, r->pf, ctx_->max_width, 0);
     if (s != DH_OK) return s;

@@ -11,7 +11,7 @@ import workloads as w
 pytestmark = pytest.mark.gpu
 
 
-def test_chosen_images_are_flushed_too():
+def test_chosen_images_are_flushed_too(tmp_path):
     # a slab so thin that every pair has several images to choose from, and one bin
     # that takes every pair: each of the blocks counts about 3.3e9 of them
     torch = pytest.importorskip("torch")
@@ -22,8 +22,10 @@ def test_chosen_images_are_flushed_too():
     x = torch.from_numpy((w.rng_for(31).random((n, 3)) * box).astype(np.float32)).cuda()
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     assert n * (n - 1) // 2 // sms > 2 ** 31
-    with dh.Context(0) as ctx:
+    path = tmp_path / "tune.txt"  # the list kernel, by the last column
+    path.write_text("".join(f"{sms} 1 {wl} 20 0 1024 256 1 1 1.0 0 1\n" for wl in range(3)))
+    with dh.Context(0, tune_cache=str(path)) as ctx:
         out = ctx.histogram(x, [0, n], w.BOX_ORTHO, w.ortho_box(*box), 710.0, 1)
         st = ctx.stats()
-    assert st["blocks"] <= sms
+    assert st["blocks"] <= sms and st["block_threads"] == 512, st
     assert int(out.cpu().numpy().view(np.uint64)[0, 0]) == n * (n - 1) // 2

@@ -169,3 +169,23 @@ def test_one_frame_of_many_species(torch_mod, oracle_mod, box):
     out = dh.FrameArgs(dev, few, kind, b, r, 200)
     dh.dh_histogram_noalloc(out.frame)
     assert np.array_equal(out.out.cpu().numpy().view(np.uint64), oracle_mod.histogram(x, few, kind, b, r, 200))
+
+
+@pytest.mark.parametrize("n,species,reach,threads", [(1500, 1, 1.7, 512), (30_000, 1, 1.2, 256), (30_000, 2, 1.7, 256),
+                                                     (30_000, 1, 2.2, 256)])
+def test_r_max_beyond_half_an_orthorhombic_box(torch_mod, oracle_mod, n, species, reach, threads):
+    # the shortest of several images: the list kernel only where a frame is too small for the tiled one
+    side = (n / 0.1) ** (1.0 / 3.0)
+    f = w.uniform_frame(47, n, w.BOX_ORTHO, w.ortho_box(side, 1.1 * side, side), 0.5 * reach * side, 500,
+                        n_species=species)
+    dev = torch_mod.from_numpy(f.coords).cuda()
+    want = oracle_mod.histogram_frame(f)
+    with dh.Context(0, pool_bytes=256 << 20) as ctx:
+        got = ctx.histogram(dev, f.offsets, f.box_type, f.box, f.r_max, f.nbins)
+        assert ctx.stats()["block_threads"] == threads, ctx.stats()
+        fa = dh.FrameArgs(dev, f.offsets, f.box_type, f.box, f.r_max, f.nbins)
+        assert ctx.wait(ctx.submit(fa)) == dh.DH_OK
+    out = dh.FrameArgs(dev, f.offsets, f.box_type, f.box, f.r_max, f.nbins)
+    dh.dh_histogram_noalloc(out.frame)
+    for o in (got, fa.out, out.out):
+        assert np.array_equal(o.cpu().numpy().view(np.uint64), want)
